@@ -69,7 +69,10 @@ typedef enum {
     MM_ERR_UNSUPPORTED = -7     /* valid but outside what this build supports (see mm_setup_geometry) */
 } mm_status;
 
-/* Element type and arithmetic of the field path.  MM_F32X2 (an extension):
+/* Element type and arithmetic of the field path.  MM_FP64: double fields,
+ * local terms, step and sums; the FFTs and the demagnetisation convolution run
+ * in 64-bit block fixed point on the integer pipes, with a smaller error than
+ * the same transforms in double.  MM_F32X2 (an extension):
  * the caller's arrays are double as for MM_FP64; inside, the iterates, the
  * FFTs, the demagnetisation convolution, the local terms, the step and the
  * per-CTA sums use double-float arithmetic (pairs of floats, about 48

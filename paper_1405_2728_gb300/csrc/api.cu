@@ -60,11 +60,11 @@ namespace {
 
 int next_pow2(int v) { int p = 1; while (p < v) p <<= 1; return p; }
 
-// stored tensor: film layout C * max(1, Pz/2) * 6 * (Py/2+1), bulk layout C * (Pz/2+1) * (Py/2+1) * 6
-size_t tensor_bytes(const Geom &g, size_t esz)
+// stored tensor: film layout C * mm_film_coefs * (Py/2+1), bulk layout C * (Pz/2+1) * (Py/2+1) * 6
+size_t tensor_bytes(const Geom &g, int precision, size_t esz)
 {
     return (g.bulk ? (size_t)g.C * (g.Pz / 2 + 1) * (g.Py / 2 + 1) * 6
-                   : (size_t)g.C * (g.Pz > 1 ? g.Pz / 2 : 1) * 6 * (g.Py / 2 + 1)) * esz;
+                   : (size_t)g.C * mm_film_coefs(g, precision) * (g.Py / 2 + 1)) * esz;
 }
 int ilog2i(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 
@@ -137,7 +137,7 @@ void free_problem(mm_problem *p)
     mm_adjoint_invalidate(p);
     void *bufs[] = {p->mbuf[0], p->mbuf[1], p->gbuf[0], p->gbuf[1], p->W, p->Nhat, p->tw_px, p->tw_py,
                     p->tw_pz, p->W2, p->Kc, p->uc, p->partials, p->st, p->Hext_dev, p->stage_in, p->stage_out,
-                    p->rec_dev, p->counter, p->adj[0], p->adj[1], p->adj_state, p->adj_partials};
+                    p->rec_dev, p->counter, p->fexp, p->adj[0], p->adj[1], p->adj_state, p->adj_partials};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (p->st_host) cudaFreeHost(p->st_host);
@@ -234,6 +234,9 @@ int plan(mm_problem *p)
         if (g.RBZ * g.Gz > maxT) g.RBZ = maxT / g.Gz;
     }
     g.nbody = g.bulk ? 5 : 3;
+    if (!g.bulk) { g.ZB = g.nz; g.KB = g.Py; }
+    g.nzb = (g.nz + g.ZB - 1) / g.ZB;
+    g.nkb = (g.Py + g.KB - 1) / g.KB;
     // y rows per CTA in the x kernels: powers of two up to 16 (and up to the
     // next power of two of ny) within 768 threads and the shared-memory cap
     p->nty = 0;
@@ -400,7 +403,7 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
     const size_t F = 3 * (size_t)g.N * p->esz;
     const size_t vsz = 2 * p->esz;
     const size_t Wb = (size_t)g.C * 3 * g.nz * g.ny * vsz;
-    const size_t Tb = tensor_bytes(g, p->esz);
+    const size_t Tb = tensor_bytes(g, p->precision, p->esz);
     do {
         if ((rc = dalloc(p, &p->mbuf[0], F)) || (rc = dalloc(p, &p->mbuf[1], F)) ||
             (rc = dalloc(p, &p->gbuf[0], F)) || (rc = dalloc(p, &p->gbuf[1], F)) ||
@@ -408,6 +411,7 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
             (g.bulk && (rc = dalloc(p, &p->W2, (size_t)g.C * 3 * g.nz * g.Py * vsz))) ||
             (rc = dalloc(p, &p->tw_px, g.Px * vsz)) || (rc = dalloc(p, &p->tw_py, g.Py * vsz)) ||
             (rc = dalloc(p, &p->tw_pz, g.Pz * vsz)) ||
+            (precision == MM_FP64 && (rc = dalloc(p, (void **)&p->fexp, sizeof(int) * mm_scale_count(g)))) ||
             (rc = dalloc(p, (void **)&p->partials, sizeof(double) * RED_NSLOT * (size_t)p->nblk_x)) ||
             (rc = dalloc(p, (void **)&p->st, sizeof(MinState))) ||
             (rc = dalloc(p, (void **)&p->counter, 64)) ||
@@ -418,6 +422,10 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
         if ((ce = cudaMallocHost((void **)&p->st_host, sizeof(MinState)))) { rc = failed(ce, "cudaMallocHost", MM_ERR_OOM); break; }
         if ((ce = cudaMemsetAsync(p->st, 0, sizeof(MinState), s)) || (ce = cudaMemsetAsync(p->counter, 0, 64, s)) ||
             (ce = cudaMemsetAsync(p->gbuf[0], 0, F, s)) || (ce = cudaMemsetAsync(p->gbuf[1], 0, F, s))) {
+            rc = failed(ce, "cudaMemsetAsync", MM_ERR_CUDA);
+            break;
+        }
+        if (p->fexp && (ce = cudaMemsetAsync(p->fexp, 0, sizeof(int) * mm_scale_count(g), s))) {
             rc = failed(ce, "cudaMemsetAsync", MM_ERR_CUDA);
             break;
         }
@@ -488,7 +496,7 @@ extern "C" int mm_problem_info(const mm_problem *p, mm_info *info)
     info->cells = g.N;
     info->workspace_bytes = p->bytes;
     info->spectrum_bytes = (long)g.C * 3 * g.nz * g.ny * 2 * (long)p->esz;
-    info->tensor_bytes = (long)tensor_bytes(g, p->esz);
+    info->tensor_bytes = (long)tensor_bytes(g, p->precision, p->esz);
     info->x_tile_rows = g.TY;
     info->yz_batch_rows = g.RB;
     info->bulk_layout = g.bulk;

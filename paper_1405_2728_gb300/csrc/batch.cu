@@ -39,6 +39,15 @@
 
 namespace {
 
+// the FFT arithmetic of a group's fields, and its y-z stage
+template <typename T> using FA = typename fft_of<T>::type;
+template <typename T, int PZ, int L>
+__device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int tid, int nth, int kx)
+{
+    if constexpr (!is_fx<FA<T>>) yz_body<T, FA<T>, PZ, L>(g, P, tid, nth, kx);
+    else if constexpr (L == 0) yz_body_fx<PZ, 0>(g, P, tid, nth, kx);
+}
+
 // one problem of a grouped launch, as the grouped kernels read it
 template <typename T>
 struct GFilm {
@@ -135,22 +144,25 @@ __global__ void __launch_bounds__(768) k_xfwd_group(const GFilm<T> *films, const
 {
     MM_GROUP_LOOP(0)
         switch (lc_of(f.g.lhx)) {
-#define C(L) case L: xfwd_body<T, T, true, L>(f.g, f.P, threadIdx.x, f.nth_xf, it.bx, it.by); break;
+#define C(L) case L: xfwd_body<T, FA<T>, true, L>(f.g, f.P, threadIdx.x, f.nth_xf, it.bx, it.by); break;
             MM_LC_CASES(C)
 #undef C
         }
     }
 }
 
+// Block fixed point takes the code for any row length here: integer results do
+// not depend on the instance, and its compiled lengths in one kernel with
+// three layer counts took four minutes to build.
 template <typename T>
 __global__ void __launch_bounds__(YZBound<T>::v) k_yz_group(const GFilm<T> *films, const GItem *items,
                                                             const int *first_of, GActive A)
 {
     MM_GROUP_LOOP(1)
-    switch (f.g.Pz * 16 + lc_of(f.g.lpy)) {
-#define C(L) case 1 * 16 + L: yz_body<T, T, 1, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 4 * 16 + L: yz_body<T, T, 4, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 8 * 16 + L: yz_body<T, T, 8, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break;
+    switch (f.g.Pz * 16 + (is_fx<FA<T>> ? 0 : lc_of(f.g.lpy))) {
+#define C(L) case 1 * 16 + L: yz_of<T, 1, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
+             case 4 * 16 + L: yz_of<T, 4, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
+             case 8 * 16 + L: yz_of<T, 8, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break;
         MM_LC_CASES(C)
 #undef C
     }
@@ -164,7 +176,7 @@ __global__ void __launch_bounds__(768) k_xinv_group(const GFilm<T> *films, const
     MM_GROUP_LOOP(2)
         const int bid = it.by * f.gx_x + it.bx;
         switch (lc_of(f.g.lhx)) {
-#define C(L) case L: xinv_body<T, T, MODE_MIN, L>(f.g, f.P, 0.0, 0.0, 0.0, 0, 0, threadIdx.x, f.nth_x, it.bx, it.by, \
+#define C(L) case L: xinv_body<T, FA<T>, MODE_MIN, L>(f.g, f.P, 0.0, 0.0, 0.0, 0, 0, threadIdx.x, f.nth_x, it.bx, it.by, \
                                                     bid, f.nblk_x); break;
             MM_LC_CASES(C)
 #undef C

@@ -21,20 +21,54 @@
 
 namespace {
 
+template <typename V> __device__ __forceinline__ V load_cg(const V *p) { return __ldcg(p); }
+template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
+{
+    const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(p));
+    return fxc{fx(v.x), fx(v.y)};
+}
+
 template <typename T> struct BulkBound { static constexpr int v = sizeof(T) == 8 ? 384 : 512; };
 
+// In block fixed point (double fields, F = fx) every CTA of a pass brings its
+// block to full magnitude when it loads it and when it stores it, with the
+// scale of a block per (kx, ZB planes) after the y passes and per (kx, KB
+// y-frequencies) after the z convolution.
 template <typename T, bool INV, int LY>
 __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> P)
 {
-    typedef typename cvec<T>::type V;
+    typedef typename FieldPtrs<T>::V V;
+    typedef typename FieldPtrs<T>::TW TW;
+    constexpr bool FX = std::is_same<V, fxc>::value;
+    __shared__ int s_e;
+    __shared__ unsigned s_r[3];  // flags, magnitudes in and out
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
     const int ny = g.ny, nz = g.nz, Py = g.Py, ZB = g.ZB, rs = g.rsy;
     const int kx = blockIdx.x, z0 = blockIdx.y * ZB;
     const int zb = min(ZB, nz - z0);
-    V *tw = S + 3 * ZB * rs;
+    TW *tw = reinterpret_cast<TW *>(S + 3 * ZB * rs);
     load_twiddles_async(tw, P.tw_py, Py);
+    int emax = FX_ZERO;
+    unsigned mag = 0;
+    const int *scales = nullptr;   // of the values read: one per (z, y) row of W, or per KB y-frequencies of W2
+    if constexpr (FX) {
+        if (tid == 0) s_e = FX_ZERO;
+        if (tid < 3) s_r[tid] = 0;
+        __syncthreads();
+        scales = INV ? P.feb + (long)kx * g.nkb : P.fe1 + (long)z0 * ny;
+        const int n = INV ? g.nkb : zb * ny;
+        unsigned fl = 0;
+        for (int i = tid; i < n; i += nth) {
+            emax = max(emax, fx_exp(scales[i]));
+            fl |= fx_flags(scales[i]);
+        }
+        fx_cta_max(&s_e, emax);
+        fx_cta_or(&s_r[0], fl);
+        __syncthreads();
+        emax = s_e;
+    }
     const long first = (long)kx * nz + z0;  // first (kx, z) row pair of this CTA
     const int lin = INV ? Py : ny;           // input length per (z, c) row
     const V *src = INV ? P.W2 + first * Py * 3 : P.W + first * ny * 3;
@@ -46,13 +80,17 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
-            if (e < tot) v[i] = __ldcg(src + e);
+            if (e < tot) v[i] = load_cg(src + e);
         }
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zl = rest / lin, y = rest - zl * lin;
+            if constexpr (FX) {
+                v[i] = fx_scale(v[i], fx_exp(scales[INV ? y / g.KB : rest]) - emax);
+                mag |= fx_mag(v[i]);
+            }
             S[(c * ZB + zl) * rs + spos<V>(y)] = v[i];
         }
     }
@@ -64,36 +102,78 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
             S[(c * ZB + zl) * rs + spos<V>(y)] = czero<V>();
         }
     }
+    if constexpr (FX) fx_cta_or(&s_r[1], mag);
     cp_async_wait_all();
     __syncthreads();
     const int Gy = g.Gy, RB = g.RBY;
     const int rb = tid / Gy, j = tid - rb * Gy;
+    const int pre = FX ? (INV ? 58 : 59) - fx_bits(s_r[1]) : 0;
+    int sh = 0;
+    mag = 0;
     for (int r0 = 0; r0 < 3 * ZB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * ZB && (r % ZB) < zb;
-        fft_row<INV, !INV, INV, 1, LY>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act);
+        if constexpr (FX)
+            sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, pre, 64, mag);
+        else
+            fft_row<INV, !INV, INV, 1, LY>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act);
     }
-    __syncthreads();
+    int post = 0;
+    if constexpr (FX) {
+        fx_cta_or(&s_r[2], mag);
+        __syncthreads();
+        post = 60 - fx_bits(s_r[2]);
+        if (tid == 0)
+            (INV ? P.fe2 : P.fea)[(long)kx * g.nzb + blockIdx.y] =
+                fx_pack(emax - pre + sh - post, s_r[0] ? 3 : 0);  // the tensor mixes all components
+    } else {
+        __syncthreads();
+    }
     const int lout = INV ? ny : Py;
     V *dst = INV ? P.W + first * ny * 3 : P.W2 + first * Py * 3;
     for (int e = tid; e < zb * lout * 3; e += nth) {
         const int c = e % 3, rest = e / 3, zl = rest / lout, y = rest - zl * lout;
-        dst[e] = S[(c * ZB + zl) * rs + spos<V>(y)];
+        V r = S[(c * ZB + zl) * rs + spos<V>(y)];
+        if constexpr (FX) r = fx_scale(r, post);
+        dst[e] = r;
     }
 }
 
 template <typename T, int LZ>
 __global__ void __launch_bounds__(BulkBound<T>::v) k_zconv(Geom g, FieldPtrs<T> P)
 {
-    typedef typename cvec<T>::type V;
+    typedef typename FieldPtrs<T>::V V;
+    typedef typename FieldPtrs<T>::TW TW;
+    constexpr bool FX = std::is_same<V, fxc>::value;
+    __shared__ int s_e;
+    __shared__ int s_top;
+    __shared__ unsigned s_r[4];  // flags, magnitudes in and out, sum of the frequencies' scales over the largest
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
     const int nz = g.nz, Py = g.Py, Pz = g.Pz, KB = g.KB, rs = g.rsz;
     const int kx = blockIdx.x, ky0 = blockIdx.y * KB;
     const int kb = min(KB, Py - ky0);
-    V *tw = S + 3 * KB * rs;
+    TW *tw = reinterpret_cast<TW *>(S + 3 * KB * rs);
     load_twiddles_async(tw, P.tw_pz, Pz);
+    int emax = FX_ZERO;
+    unsigned mag = 0;
+    const int *scales = nullptr;
+    if constexpr (FX) {
+        if (tid == 0) { s_e = FX_ZERO; s_top = FX_ZERO; }
+        if (tid < 4) s_r[tid] = 0;
+        __syncthreads();
+        scales = P.fea + (long)kx * g.nzb;
+        unsigned fl = 0;
+        for (int i = tid; i < g.nzb; i += nth) {
+            emax = max(emax, fx_exp(scales[i]));
+            fl |= fx_flags(scales[i]);
+        }
+        fx_cta_max(&s_e, emax);
+        fx_cta_or(&s_r[0], fl);
+        __syncthreads();
+        emax = s_e;
+    }
     // W2[kx][z][ky0 + kyl][c], z < nz -> row (c, kyl), element z; PF loads
     // per thread in flight before use
     V *base = P.W2 + ((long)kx * nz * Py + ky0) * 3;
@@ -107,7 +187,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_zconv(Geom g, FieldPtrs<T> 
             const int e = e0 + i * nth;
             if (e < tot) {
                 const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
-                v[i] = __ldcg(base + (long)z * zs + kyl * 3 + c);
+                v[i] = load_cg(base + (long)z * zs + kyl * 3 + c);
             }
         }
 #pragma unroll
@@ -115,6 +195,10 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_zconv(Geom g, FieldPtrs<T> 
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
+            if constexpr (FX) {
+                v[i] = fx_scale(v[i], fx_exp(scales[z / g.ZB]) - emax);
+                mag |= fx_mag(v[i]);
+            }
             S[(c * KB + kyl) * rs + spos<V>(z)] = v[i];
         }
     }
@@ -124,47 +208,112 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_zconv(Geom g, FieldPtrs<T> 
         const int c = r / kb, kyl = r - c * kb;
         S[(c * KB + kyl) * rs + spos<V>(z)] = czero<V>();
     }
+    if constexpr (FX) fx_cta_or(&s_r[1], mag);
     cp_async_wait_all();
     __syncthreads();
     const int Gz = g.Gz, RB = g.RBZ;
     const int rb = tid / Gz, j = tid - rb * Gz;
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + Pz);  // [2][KB][Pz]: scale and top bit of a frequency
+    int pre = FX ? 59 - fx_bits(s_r[1]) : 0, sh = 0, top = FX_ZERO;
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
-        fft_row<false, true, false, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
+        if constexpr (FX)
+            sh = fft_row_fx<false, true, false, 1, LZ, false>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, pre, 64, mag);
+        else
+            fft_row<false, true, false, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
     }
     __syncthreads();
+    if constexpr (FX) emax += sh - pre + P.fek[kx];
     // tensor product per (ky, kz); octant storage [kx][kzr][kyr][6] with the
     // off-diagonal signs of the reflected frequencies
     const int hy = Py / 2, hz = Pz / 2;
-    const T *Nk = P.Nhat + (long)kx * (hz + 1) * (hy + 1) * 6;
+    const typename coef<typename fft_of<T>::type>::type *Nk = P.Nhat + (long)kx * (hz + 1) * (hy + 1) * 6;
     for (int e = tid; e < kb * Pz; e += nth) {
         const int kyl = e % kb, kz = e / kb, ky = ky0 + kyl;
         const int kyr = ky <= hy ? ky : Py - ky, kzr = kz <= hz ? kz : Pz - kz;
-        const T sy = ky <= hy ? (T)1 : (T)-1, sz = kz <= hz ? (T)1 : (T)-1;
-        const T *n6 = Nk + ((long)kzr * (hy + 1) + kyr) * 6;
-        const T nxx = __ldg(n6 + 0), nyy = __ldg(n6 + 1), nzz = __ldg(n6 + 2);
-        const T nxy = sy * __ldg(n6 + 3), nxz = sz * __ldg(n6 + 4), nyz = sy * sz * __ldg(n6 + 5);
+        const auto *n6 = Nk + ((long)kzr * (hy + 1) + kyr) * 6;
         V *a0 = S + (0 * KB + kyl) * rs + spos<V>(kz);
         V *a1 = S + (1 * KB + kyl) * rs + spos<V>(kz);
         V *a2 = S + (2 * KB + kyl) * rs + spos<V>(kz);
+        if constexpr (FX) {
+            // one scale per frequency: inputs below 2^59, outputs below 2^59
+            auto element = [&](int c, bool neg) {
+                const int2 w = __ldg(reinterpret_cast<const int2 *>(n6 + c));
+                return fxk(fxk(fxm{w.x, w.y}), neg);
+            };
+            const fxk k[6] = {element(0, false), element(1, false), element(2, false), element(3, ky > hy),
+                              element(4, kz > hz), element(5, (ky > hy) != (kz > hz))};
+            fxc m0 = *a0, m1 = *a1, m2 = *a2;
+            const int sc = 59 - fx_bits(fx_mag(m0) | fx_mag(m1) | fx_mag(m2));
+            m0 = fx_scale(m0, sc); m1 = fx_scale(m1, sc); m2 = fx_scale(m2, sc);
+            auto row = [&](const fxk &p, const fxk &q, const fxk &r, fx x, fx y, fx z) {
+                fxdot h;
+                h.zero();
+                h.mad(fx_split(x), p);
+                h.mad(fx_split(y), q);
+                h.mad(fx_split(z), r);
+                return h.value();
+            };
+            const fxc h0{row(k[0], k[3], k[4], m0.x, m1.x, m2.x), row(k[0], k[3], k[4], m0.y, m1.y, m2.y)};
+            const fxc h1{row(k[3], k[1], k[5], m0.x, m1.x, m2.x), row(k[3], k[1], k[5], m0.y, m1.y, m2.y)};
+            const fxc h2{row(k[4], k[5], k[2], m0.x, m1.x, m2.x), row(k[4], k[5], k[2], m0.y, m1.y, m2.y)};
+            const int tk = fx_bits(fx_mag(h0) | fx_mag(h1) | fx_mag(h2)) - sc;
+            s_sc[kyl * Pz + kz] = (signed char)sc;
+            s_sc[(KB + kyl) * Pz + kz] = (signed char)tk;
+            top = max(top, tk);
+            *a0 = h0; *a1 = h1; *a2 = h2;
+        } else {
+        const T sy = ky <= hy ? (T)1 : (T)-1, sz = kz <= hz ? (T)1 : (T)-1;
+        const T nxx = __ldg(n6 + 0), nyy = __ldg(n6 + 1), nzz = __ldg(n6 + 2);
+        const T nxy = sy * __ldg(n6 + 3), nxz = sz * __ldg(n6 + 4), nyz = sy * sz * __ldg(n6 + 5);
         const V m0 = *a0, m1 = *a1, m2 = *a2;
         V h0, h1, h2;
         h0.x = nxx * m0.x + nxy * m1.x + nxz * m2.x; h0.y = nxx * m0.y + nxy * m1.y + nxz * m2.y;
         h1.x = nxy * m0.x + nyy * m1.x + nyz * m2.x; h1.y = nxy * m0.y + nyy * m1.y + nyz * m2.y;
         h2.x = nxz * m0.x + nyz * m1.x + nzz * m2.x; h2.y = nxz * m0.y + nyz * m1.y + nzz * m2.y;
         *a0 = h0; *a1 = h1; *a2 = h2;
+        }
     }
+    int t = 64;
+    if constexpr (FX) fx_cta_max(&s_top, top);
     __syncthreads();
+    if constexpr (FX) {
+        // no partial sum of an inverse transform exceeds the sum of the largest moduli over kz
+        top = s_top;
+        unsigned sum = 0;
+        for (int e = tid; e < Pz; e += nth) {
+            int tk = FX_ZERO;
+            for (int kyl = 0; kyl < kb; ++kyl) tk = max(tk, (int)s_sc[(KB + kyl) * Pz + e]);
+            sum += ((1u << 18) >> min(top - tk, 18)) + 1;
+        }
+        fx_cta_add(&s_r[3], sum);
+        __syncthreads();
+        pre = 58 - top;
+        t = max(0, fx_log2_up(s_r[3]) - 18);
+        mag = 0;
+    }
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
-        fft_row<true, false, true, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
+        if constexpr (FX)
+            sh = fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, pre, t,
+                                                                  mag, s_sc + (act ? r % KB : 0) * Pz);
+        else
+            fft_row<true, false, true, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
     }
+    if constexpr (FX) fx_cta_or(&s_r[2], mag);
     __syncthreads();
+    int post = 0;
+    if constexpr (FX) {
+        post = 60 - fx_bits(s_r[2]);
+        if (tid == 0) P.feb[(long)kx * g.nkb + blockIdx.y] = fx_pack(emax + sh - pre - post, s_r[0] ? 3 : 0);
+    }
     for (int e = tid; e < nz * kb * 3; e += nth) {
         const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
-        base[(long)z * zs + kyl * 3 + c] = S[(c * KB + kyl) * rs + spos<V>(z)];
+        V r = S[(c * KB + kyl) * rs + spos<V>(z)];
+        if constexpr (FX) r = fx_scale(r, post);
+        base[(long)z * zs + kyl * 3 + c] = r;
     }
 }
 
@@ -178,7 +327,8 @@ template <typename T> size_t smem_y_t(const Geom &g, int zb)
 template <typename T> size_t smem_z_t(const Geom &g, int kb)
 {
     typedef typename cvec<T>::type V;
-    return ((size_t)3 * kb * g.rsz + g.Pz) * sizeof(V);
+    // and two bytes per frequency of a block fixed-point transform
+    return ((size_t)3 * kb * g.rsz + g.Pz) * sizeof(V) + (sizeof(T) == 8 ? (size_t)2 * kb * g.Pz : 0);
 }
 
 inline int lc_of(int logL) { return MM_FFT_SPECIALISED(logL) ? logL : 0; }

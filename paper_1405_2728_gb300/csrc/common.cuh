@@ -9,6 +9,7 @@
 
 #include "../../include/mm.h"
 #include "dfloat.cuh"
+#include "fixed.cuh"
 
 #define MM_MU0 (4e-7 * 3.14159265358979323846)
 
@@ -19,6 +20,15 @@ template <typename T> struct cvec;
 template <> struct cvec<double> { typedef double2 type; };
 template <> struct cvec<float> { typedef float2 type; };
 template <> struct cvec<dfloat> { typedef dcomplex type; };
+template <> struct cvec<fx> { typedef fxc type; };
+// twiddle and tensor element of an FFT arithmetic
+template <typename F> struct twvec { typedef typename cvec<F>::type type; };
+template <> struct twvec<fx> { typedef fxmc type; };
+template <typename F> struct coef { typedef F type; };
+template <> struct coef<fx> { typedef fxm type; };
+// FFT arithmetic of a field type: double fields are convolved in block fixed point
+template <typename T> struct fft_of { typedef T type; };
+template <> struct fft_of<double> { typedef fx type; };
 
 template <typename V> __device__ __forceinline__ V cmake(decltype(V().x) a, decltype(V().x) b) { V r; r.x = a; r.y = b; return r; }
 template <typename V> __device__ __forceinline__ V cadd(V a, V b) { V r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
@@ -137,6 +147,7 @@ struct Geom {
     int RBY;               // y rows transformed at once in the y passes
     int KB;                // y frequencies per CTA of the z pass
     int RBZ;               // z rows transformed at once in the z pass
+    int nzb, nkb;          // blocks of ZB z planes (film layout: one block of all), of KB y frequencies
     int lpz, Gz, rsz;      // log2(Pz), threads per z row, smem stride of a z row
     int nbody;             // kernels per minimiser iteration (3 film, 5 bulk)
     long N;                // cells
@@ -214,9 +225,10 @@ template <> struct io_of<dfloat> { typedef double type; };
 // the convolution, whose complex values fill the spectrum buffers and the
 // tensor; IO: the caller's element type (m for MODE_HEFF/ENERGY, H, per-cell
 // material)
-template <typename T, typename F = T>
+template <typename T, typename F = typename fft_of<T>::type>
 struct FieldPtrs {
     typedef typename cvec<F>::type V;
+    typedef typename twvec<F>::type TW;
     typedef typename io_of<T>::type IO;
     const IO *m_src;       // field input for MODE_HEFF/ENERGY, or NULL (then mbuf by state)
     IO *H_out;             // MODE_HEFF output
@@ -224,12 +236,18 @@ struct FieldPtrs {
     T *gbuf[2];            // projected-gradient buffers
     V *W;                  // spectrum [C][nz][ny][3] (x-frequency slowest, component fastest)
     V *W2;                 // bulk layout only: y-transformed spectrum [C][nz][Py][3]
-    const F *Nhat;         // tensor: film [C][max(1,Pz/2)][6][Py/2+1] (x-y transform at real z offsets, scaled by
+    const typename coef<F>::type *Nhat;  // tensor: film [C][max(1,Pz/2)][6][Py/2+1] (x-y transform at real z offsets, scaled by
                            // -Ms/(Px Py)); bulk [C][Pz/2+1][Py/2+1][6] (octant of the 3-D spectrum,
                            // scaled by -Ms/(Px Py Pz))
-    const V *tw_px;        // exp(-2 pi i t/Px), t < Px
-    const V *tw_py;        // exp(-2 pi i t/Py), t < Py
-    const V *tw_pz;        // exp(-2 pi i t/Pz), t < Pz
+    const TW *tw_px;       // exp(-2 pi i t/Px), t < Px
+    const TW *tw_py;       // exp(-2 pi i t/Py), t < Py
+    const TW *tw_pz;       // exp(-2 pi i t/Pz), t < Pz
+    // block fixed point only (F = fx): the scales of the blocks (fx_pack)
+    int *fe1;              // [nz][ny] of W as the x-forward kernel writes it
+    int *fea;              // [C][nzb] bulk: of W2 after the y transform
+    int *feb;              // [C][nkb] bulk: of W2 after the z convolution
+    int *fe2;              // [C][nzb] of W as the y-z stage leaves it
+    const int *fek;        // [C] exponents of the tensor
     const IO *Kc;          // per-cell K or NULL
     const IO *uc;          // per-cell axis [3][N] or NULL
     double *partials;      // [nblocks][RED_NSLOT]
@@ -252,6 +270,7 @@ struct mm_problem {
     void *W;
     void *W2;              // bulk layout only
     void *Nhat;
+    int *fexp;             // block scales of the fixed-point convolution: fe1, fea, feb, fe2, fek in one buffer
     void *tw_px, *tw_py, *tw_pz;
     void *Kc, *uc;
     double *partials;
@@ -312,6 +331,22 @@ MM_DECLARE_FIELD_ENTRIES(f32x2)
 // problems configured before it.  It only permits launches; nothing is
 // reserved by it.
 #define MM_SMEM_CAP (200 * 1024)
+
+// tensor elements per (kx, ky) of the film layout: six components at
+// max(1, Pz/2) z offsets, or the combinations of them that the block
+// fixed-point z convolution multiplies with (ZConv)
+inline int mm_film_coefs(const Geom &g, int precision)
+{
+    const int nzm = g.Pz > 1 ? g.Pz / 2 : 1;
+    if (precision != MM_FP64) return 6 * nzm;
+    return nzm == 1 ? 4 : (nzm == 2 ? 10 : 32);
+}
+
+// ints of mm_problem::fexp
+inline size_t mm_scale_count(const Geom &g)
+{
+    return (size_t)g.nz * g.ny + (size_t)g.C * (2 * g.nzb + g.nkb + 1);
+}
 
 // launchers implemented in heff.cu
 int mm_launch_min_body(mm_problem *p, cudaGraphConditionalHandle h, cudaStream_t s, int use_cond);

@@ -126,8 +126,8 @@ template <bool INV, bool HIN, typename V> __device__ __forceinline__ void dft8(V
 
 template <int R, bool INV, bool HIN, typename V> __device__ __forceinline__ void dftR(V *a)
 {
-    if (R == 2) dft2<HIN>(a[0], a[1]);
-    else if (R == 4) dft4<INV, HIN>(a[0], a[1], a[2], a[3]);
+    if constexpr (R == 2) dft2<HIN>(a[0], a[1]);
+    else if constexpr (R == 4) dft4<INV, HIN>(a[0], a[1], a[2], a[3]);
     else dft8<INV, HIN>(a);
 }
 
@@ -294,6 +294,193 @@ __device__ __forceinline__ void fft_row(V *row, int L, int logL, int j, const V 
 {
     if constexpr (LC > 0) fft_row_c<LC, INV, HIN, HOUT, TS>(row, j, tw, active);
     else fft_row_n<INV, HIN, HOUT, TS>(row, L, logL, j, tw, active);
+}
+
+// ---------------------------------------------------------------------------
+// The same transforms in block fixed point (fixed.cuh)
+// ---------------------------------------------------------------------------
+// Scaling: the first pass takes its inputs times 2^pre, which the caller
+// chooses so that their components stay below 2^58 (2^59 with HIN, whose
+// first pass adds half as many).  A value after passes of total radix 2^q is
+// a sum of at most 2^q inputs, and at most 2^t times the largest input when
+// the caller knows that all inputs of a row together are no larger (t >= log2 L
+// says nothing).  Moduli then stay below 2^61.5 when
+// fx_cum(q, t) = max(0, min(q, t) - 3) bits have been shifted out by then; each
+// later pass folds its share into the rounding of the twiddle products.
+// Sums of two such values stay below 2^63.
+// With VAR, element i of the row is scaled by 2^(pre - var[i]) instead.
+// fft_row_fx returns the bits shifted out in all; `mag` collects the magnitude
+// bits of the outputs (fx_mag).
+__host__ __device__ __forceinline__ constexpr int fx_cum(int q, int t)
+{
+    const int m = q < t ? q : t;
+    return m > 3 ? m - 3 : 0;
+}
+
+template <bool INV, bool HIN> __device__ __forceinline__ void dft8_fx(fxc *a)
+{
+    // sqrt(1/2) in units of 2^-61
+    constexpr fxm r = fx_multiplier(1630477228166597777ll);
+    fxc u0, u1, u2, u3, d0, d1, d2, d3;
+    if (HIN) {
+        u0 = a[0]; u1 = a[1]; u2 = a[2]; u3 = a[3];
+        d0 = a[0]; d1 = a[1]; d2 = a[2]; d3 = a[3];
+    } else {
+        u0 = cadd(a[0], a[4]); d0 = csub(a[0], a[4]);
+        u1 = cadd(a[1], a[5]); d1 = csub(a[1], a[5]);
+        u2 = cadd(a[2], a[6]); d2 = csub(a[2], a[6]);
+        u3 = cadd(a[3], a[7]); d3 = csub(a[3], a[7]);
+    }
+    fxc v1, v2, v3;
+    if (INV) {
+        v1.x = fx_mulc(r, d1.x - d1.y); v1.y = fx_mulc(r, d1.x + d1.y);
+        v2.x = -d2.y;                   v2.y = d2.x;
+        v3.x = fx_mulc(r, -(d3.x + d3.y)); v3.y = fx_mulc(r, d3.x - d3.y);
+    } else {
+        v1.x = fx_mulc(r, d1.x + d1.y); v1.y = fx_mulc(r, d1.y - d1.x);
+        v2.x = d2.y;                    v2.y = -d2.x;
+        v3.x = fx_mulc(r, d3.y - d3.x); v3.y = fx_mulc(r, -(d3.x + d3.y));
+    }
+    dft4<INV, false>(u0, u1, u2, u3);
+    dft4<INV, false>(d0, v1, v2, v3);
+    a[0] = u0; a[1] = d0; a[2] = u1; a[3] = v1;
+    a[4] = u2; a[5] = v2; a[6] = u3; a[7] = v3;
+}
+
+template <int R, bool INV, bool HIN, bool HOUT, bool FIRST, bool MAG, bool VAR>
+__device__ __forceinline__ void stockham_pass_fx(fxc *row, int L, int Ns, int j, int G, const fxmc *__restrict__ tw,
+                                                 int ts, bool active, int sh, unsigned &mag,
+                                                 const signed char *var)
+{
+    constexpr int NB = 8 / R;
+    fxc v[8];
+    const int LR = L / R;
+    const int ld9 = LR + (LR >> 3);
+    const int tstep0 = (L / (Ns * R)) * ts;
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            const int p0 = pidx(b);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (HIN && r >= R / 2) { v[q * R + r] = czero<fxc>(); continue; }
+                v[q * R + r] = row[(LR & 7) ? pidx(b + r * LR) : p0 + r * ld9];
+            }
+            if (FIRST && VAR) {
+#pragma unroll
+                for (int r = 0; r < (HIN ? R / 2 : R); ++r)
+                    v[q * R + r] = fx_scale(v[q * R + r], sh - var[b + r * LR]);
+            } else if (FIRST && sh > 0) {
+#pragma unroll
+                for (int r = 0; r < (HIN ? R / 2 : R); ++r) {
+                    v[q * R + r].x.v <<= sh;
+                    v[q * R + r].y.v <<= sh;
+                }
+            }
+            if (FIRST && !VAR && sh < 0) {
+#pragma unroll
+                for (int r = 0; r < (HIN ? R / 2 : R); ++r) v[q * R + r] = fx_scale(v[q * R + r], sh);
+            }
+            if (!FIRST) {
+                const int step = tstep0 * (b & (Ns - 1));
+                v[q * R].x = fx_shr(v[q * R].x, sh);
+                v[q * R].y = fx_shr(v[q * R].y, sh);
+                int t = step;
+#pragma unroll
+                for (int r = 1; r < R; ++r, t += step) v[q * R + r] = fx_cmul<INV>(v[q * R + r], tw[t], sh);
+            }
+            if constexpr (R == 8) dft8_fx<INV, HIN>(&v[q * R]);
+            else dftR<R, INV, HIN>(&v[q * R]);
+        }
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            const int k = b & (Ns - 1);
+            const int hi = (b - k) * R;
+            const int s0 = (R == 8) ? hi + (hi >> 3) + k + (k >> 3) : 0;
+#pragma unroll
+            for (int r = 0; r < (HOUT ? R / 2 : R); ++r) {
+                const int rn = r * Ns;
+                row[(R == 8) ? s0 + rn + (rn >> 3) : pidx(hi + k + rn)] = v[q * R + r];
+                if (MAG) mag |= fx_mag(v[q * R + r]);
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// one pass of a row: FIRST with the scale `pre`, later ones with their share of the shift
+template <int R, bool INV, bool HIN, bool HOUT, bool FIRST, bool MAG, bool VAR>
+__device__ __forceinline__ void fx_pass(fxc *row, int L, int Ns, int j, int G, const fxmc *tw, int ts, bool active,
+                                        int pre, int q, int t, unsigned &mag, const signed char *var)
+{
+    const int lr = R == 8 ? 3 : (R == 4 ? 2 : 1);
+    const int sh = FIRST ? pre : fx_cum(q, t) - fx_cum(q - lr, t);
+    stockham_pass_fx<R, INV, HIN, HOUT, FIRST, MAG, VAR>(row, L, Ns, j, G, tw, ts, active, sh, mag, var);
+}
+
+template <bool INV, bool HIN, bool HOUT, int TS, int LC, bool MAG, bool VAR = false>
+__device__ __forceinline__ int fft_row_fx(fxc *row, int L, int logL, int j, const fxmc *__restrict__ tw, bool active,
+                                          int pre, int t, unsigned &mag, const signed char *var = nullptr)
+{
+    if constexpr (LC > 0) {
+        constexpr int LL = 1 << LC, G = LL >> 3, rem = LC % 3, n8 = LC / 3;
+        constexpr int NS0 = rem == 1 ? 2 : (rem == 2 ? 4 : 1);
+        if constexpr (rem == 1) fx_pass<2, INV, HIN, false, true, false, VAR>(row, LL, 1, j, G, tw, TS, active, pre, 1, t, mag, var);
+        if constexpr (rem == 2) fx_pass<4, INV, HIN, false, true, false, VAR>(row, LL, 1, j, G, tw, TS, active, pre, 2, t, mag, var);
+#pragma unroll
+        for (int p = 0; p < n8; ++p) {
+            const int Ns = NS0 << (3 * p), q = rem + 3 * (p + 1);
+            const bool last = (p == n8 - 1), first = (p == 0 && rem == 0);
+            if (first && last) fx_pass<8, INV, HIN, HOUT, true, MAG, VAR>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else if (first) fx_pass<8, INV, HIN, false, true, false, VAR>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else if (last) fx_pass<8, INV, false, HOUT, false, MAG, false>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else fx_pass<8, INV, false, false, false, false, false>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+        }
+        return fx_cum(LC, t);
+    } else {
+        if (L < 8) {
+            fxc a[4];
+            if (active) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    a[i] = czero<fxc>();
+                    if (i < L && !(HIN && 2 * i >= L && L > 1)) a[i] = fx_scale(row[i], VAR ? pre - var[i] : pre);
+                }
+                if (L == 2) dft2<false>(a[0], a[1]);
+                if (L == 4) dft4<INV, false>(a[0], a[1], a[2], a[3]);
+            }
+            __syncthreads();
+            if (active) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < L && !(HOUT && 2 * i >= L && L > 1)) {
+                        row[i] = a[i];
+                        if (MAG) mag |= fx_mag(a[i]);
+                    }
+            }
+            __syncthreads();
+            return 0;
+        }
+        const int G = L >> 3, rem = logL % 3, n8 = logL / 3;
+        int Ns = 1, q = 0;
+        if (rem == 1) { fx_pass<2, INV, HIN, false, true, false, VAR>(row, L, 1, j, G, tw, TS, active, pre, 1, t, mag, var); Ns = 2; q = 1; }
+        else if (rem == 2) { fx_pass<4, INV, HIN, false, true, false, VAR>(row, L, 1, j, G, tw, TS, active, pre, 2, t, mag, var); Ns = 4; q = 2; }
+        for (int p = 0; p < n8; ++p) {
+            const bool last = p == n8 - 1, first = q == 0;
+            q += 3;
+            if (first && last) fx_pass<8, INV, HIN, HOUT, true, MAG, VAR>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else if (first) fx_pass<8, INV, HIN, false, true, false, VAR>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else if (last) fx_pass<8, INV, false, HOUT, false, MAG, false>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            else fx_pass<8, INV, false, false, false, false, false>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
+            Ns <<= 3;
+        }
+        return fx_cum(logL, t);
+    }
 }
 
 // Row lengths with compiled specialisations in the field kernels (log2 of

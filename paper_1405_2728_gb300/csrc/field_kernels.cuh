@@ -31,6 +31,17 @@ template <> __device__ __forceinline__ dcomplex ld_cg(const dcomplex *p)
     const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
     return dcomplex{dfloat(v.x, v.y), dfloat(v.z, v.w)};
 }
+template <> __device__ __forceinline__ fxc ld_nc(const fxc *p)
+{
+    const longlong2 v = __ldg(reinterpret_cast<const longlong2 *>(p));
+    return fxc{fx(v.x), fx(v.y)};
+}
+template <> __device__ __forceinline__ fxc ld_cg(const fxc *p)
+{
+    const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(p));
+    return fxc{fx(v.x), fx(v.y)};
+}
+template <typename F> constexpr bool is_fx = std::is_same<F, fx>::value;
 // a value of the FFT arithmetic F read back in the field type T
 template <typename T, typename F> __device__ __forceinline__ T to_field(F v) { return (T)v; }
 template <> __device__ __forceinline__ double to_field<double, dfloat>(dfloat v) { return df_to_double(v); }
@@ -95,14 +106,21 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
                                           const int bx, const int by)
 {
     typedef typename cvec<F>::type V;
+    typedef typename twvec<F>::type TW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int TY = g.TYF, y0 = bx * TY, z = by;
     const int nx = g.nx, ny = g.ny, Px = g.Px;
     const long N = g.N;
-    V *tw = S + 3 * TY * g.rsx;  // Px twiddles exp(-2 pi i t / Px)
+    TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);  // Px twiddles exp(-2 pi i t / Px)
     for (int i = tt; i < Px; i += nth) tw[i] = P.tw_px[i];
+    __shared__ int s_max[2];       // block fixed point: high words of the tile's largest |m_x|, |m_y| and |m_z|
+    int max_xy = 0, max_z = 0;
+    if constexpr (is_fx<F>) {
+        if (tid < 2) s_max[tid] = 0;
+        __syncthreads();
+    }
 
     typedef typename io_of<T>::type IO;
     const T *src = nullptr;        // minimiser mode: the iterate buffers
@@ -164,9 +182,39 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
                 dst[n] = m0; dst[N + n] = m1; dst[2 * N + n] = m2;
             }
         }
-        rel<F>(S + (0 * TY + yl) * g.rsx, x) = F(m0);
-        rel<F>(S + (1 * TY + yl) * g.rsx, x) = F(m1);
-        rel<F>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
+        if constexpr (is_fx<F>) {  // as they are, until the tile's scale is known
+            max_xy = max(max_xy, max(__double2hiint(m0) & 0x7fffffff, __double2hiint(m1) & 0x7fffffff));
+            max_z = max(max_z, __double2hiint(m2) & 0x7fffffff);
+            rel<double>(S + (0 * TY + yl) * g.rsx, x) = m0;
+            rel<double>(S + (1 * TY + yl) * g.rsx, x) = m1;
+            rel<double>(S + (2 * TY + yl) * g.rsx, x) = m2;
+        } else {
+            rel<F>(S + (0 * TY + yl) * g.rsx, x) = F(m0);
+            rel<F>(S + (1 * TY + yl) * g.rsx, x) = F(m1);
+            rel<F>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
+        }
+    }
+    int e1 = 0;
+    if constexpr (is_fx<F>) {
+        // the tile's scale 2^s: its largest component becomes 2^57 .. 2^58 (one up to 1 + 2^-8 counts as 1, so that
+        // unit vectors and their rounding share one scale); non-finite components are taken as zero and flagged
+        fx_cta_max(&s_max[0], max_xy);
+        fx_cta_max(&s_max[1], max_z);
+        __syncthreads();
+        const int inf = 0x7ff00000;
+        const bool bad_xy = s_max[0] >= inf, bad_z = s_max[1] >= inf;
+        const int top = max(bad_xy ? 0 : s_max[0], bad_z ? 0 : s_max[1]);
+        const int sc = min(58 - (((top - 0x1000) >> 20) - 1022), 1000);
+        e1 = fx_pack(top > 0 ? -sc - 1 : FX_ZERO, (bad_xy ? 1 : 0) | (bad_z ? 2 : 0));
+        const double scale = top > 0 ? fx_pow2(sc) : 0.0;
+        for (int e = tt; e < TY * nx; e += nth) {  // the elements this thread stored
+            const int yl = g.fd_nx.div(e), x = e - yl * nx;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                fx &q = rel<F>(S + (c * TY + yl) * g.rsx, x);
+                q.v = (c < 2 ? bad_xy : bad_z) ? 0 : __double2ll_rn(__longlong_as_double(q.v) * scale);
+            }
+        }
     }
     const int npad = Px - nx;
     for (int e = tt; e < 3 * TY * npad; e += nth) {
@@ -179,7 +227,14 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
     {
         const int row = tid / g.Gx, j = tid - row * g.Gx;
         const bool act = row < 3 * TY;
-        fft_row<false, true, false, 2, LX>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j, tw, act);
+        if constexpr (is_fx<F>) {
+            unsigned none = 0;
+            e1 += fx_pack(fft_row_fx<false, true, false, 2, LX, false>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j,
+                                                                       tw, act, 0, 64, none), 0);
+            if (tid < TY && y0 + tid < ny) P.fe1[z * ny + y0 + tid] = e1;
+        } else {
+            fft_row<false, true, false, 2, LX>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j, tw, act);
+        }
     }
 
     // unpack to the real-input spectrum X[k], k = 0..Hx, and store transposed.
@@ -193,6 +248,15 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         const V *row = S + (c * TY + yl) * g.rsx;
         const V Zk = row[spos<V>(k)];
         const V Zm = cconj(row[spos<V>(k == 0 ? 0 : Hx - k)]);
+        if constexpr (is_fx<F>) {  // 2 X is stored: |Zk|, |Zm| < 2^60.5, so |2 X| < 2^62
+            const V sum = cadd(Zk, Zm), wd = fx_cmul<false>(csub(Zk, Zm), tw[k], 0);
+            if (y < ny) {
+                P.W[(((long)k * g.nz + z) * ny + y) * 3 + c] = V{sum.x + wd.y, sum.y - wd.x};
+                if (Hx - k != k)
+                    P.W[(((long)(Hx - k) * g.nz + z) * ny + y) * 3 + c] = V{sum.x - wd.y, -(sum.y + wd.x)};
+            }
+            continue;
+        } else {
         const V sum = cadd(Zk, Zm), dif = csub(Zk, Zm);
         const V wd = cmul(tw[k], dif);
         if (y < ny) {
@@ -205,6 +269,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
                 X.y = F(0.5) * (-sum.y - wd.x);
                 P.W[(((long)(Hx - k) * g.nz + z) * ny + y) * 3 + c] = X;
             }
+        }
         }
     }
 }
@@ -221,6 +286,237 @@ __global__ void __launch_bounds__(768) k_xfwd(Geom g, FieldPtrs<T, F> P)
 // the double kernel runs fewer, fatter threads (its z-phase keeps ~100
 // doubles live); the y rows are then transformed in batches of RB rows
 template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ? 512 : 768; };
+
+// Block fixed point: the z convolution of one (kx, ky), NZM layers, both
+// parts of three components.  The tensor is a Toeplitz matrix along z, even
+// (xx, yy, zz, xy) or odd (xz, yz, times i) in z - z', so with
+// up_j = m_j + m_{NZM-1-j} and um_j = m_j - m_{NZM-1-j} the sums S_i and
+// differences D_i of the outputs i and NZM-1-i come from half-size products:
+// 8 multiplications a component pair and part for 4 layers instead of 16
+// (even) or 12 (odd).  Outputs carry a factor 2 for NZM > 1.
+// The coefficients, combinations of the tensor at the z offsets K0 .. K3, are
+// stored [coefficient][ky], 4 NE + 2 NO of them (k_tensor_fixed):
+//  even  S: [K0+K3 K1+K2; K1+K2 K0+K1] up,  D: the same with minus, um
+//  odd   S: [K3 K2-K1; K1+K2 K1] um,        D: [-K3 -(K1+K2); K1-K2 -K1] up
+// so that each is loaded where it is used.
+template <int NZM> struct ZConv {
+    static constexpr int H = NZM > 1 ? NZM / 2 : 1;
+    static constexpr int NE = NZM == 1 ? 1 : (NZM == 2 ? 2 : 6), NO = NZM == 1 ? 0 : (NZM == 2 ? 1 : 4);
+    int2 up[3][H][2], um[3][H][2];   // split words, [component][j][part]
+    const fxm *K;                    // this (kx, ky)'s first coefficient
+    int kst;
+
+    __device__ __forceinline__ fxk coefficient(int i) const
+    {
+        const int2 w = __ldg(reinterpret_cast<const int2 *>(K + (long)i * kst));
+        return fxk(fxm{w.x, w.y});
+    }
+    // component e (xx, yy, zz, xy = 0 .. 3) from source b, into S_i (D false) or D_i
+    template <bool D> __device__ __forceinline__ void even(fxdot (&a)[2], int e, int b, int i) const
+    {
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const fxk w = coefficient(e * NE + (NZM == 1 ? 0 : (NZM == 2 ? D : (D ? 3 : 0) + i + j)));
+            a[0].mad(D ? um[b][j][0] : up[b][j][0], w);
+            a[1].mad(D ? um[b][j][1] : up[b][j][1], w);
+        }
+    }
+    // component o (xz, yz = 0, 1): times i
+    template <bool D> __device__ __forceinline__ void odd(fxdot (&a)[2], int o, int b, int i) const
+    {
+        if constexpr (NZM > 1) {
+#pragma unroll
+            for (int j = 0; j < H; ++j) {
+                // NZM = 4: rows (K3, -(K1-K2)), (K1+K2, K1) of S; (-K3, -(K1+K2)), (K1-K2, -K1) of D
+                const int at = NZM == 2 ? 0 : (i == j ? 3 * i : (D ? 1 + j : 2 - j));
+                const bool neg = NZM == 2 ? D : (D ? !(i == 1 && j == 0) : (i == 0 && j == 1));
+                const fxk w = coefficient(4 * NE + o * NO + at), p(w, neg), n(w, !neg);
+                a[0].mad(D ? up[b][j][1] : um[b][j][1], n);
+                a[1].mad(D ? up[b][j][0] : um[b][j][0], p);
+            }
+        }
+    }
+    template <bool D> __device__ __forceinline__ fxc sum(int comp, int i) const
+    {
+        fxdot t[2];
+        t[0].zero();
+        t[1].zero();
+        if (comp == 0) { even<D>(t, 0, 0, i); even<D>(t, 3, 1, i); odd<D>(t, 0, 2, i); }
+        if (comp == 1) { even<D>(t, 3, 0, i); even<D>(t, 1, 1, i); odd<D>(t, 1, 2, i); }
+        if (comp == 2) { odd<D>(t, 0, 0, i); odd<D>(t, 1, 1, i); even<D>(t, 2, 2, i); }
+        return fxc{t[0].value(), t[1].value()};
+    }
+    // output component comp: store(layer, value)
+    template <typename St> __device__ __forceinline__ void output(int comp, St store) const
+    {
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const fxc S = sum<false>(comp, i);
+            if constexpr (NZM == 1) {
+                store(0, S);
+            } else {
+                const fxc D = sum<true>(comp, i);
+                store(i, cadd(S, D));
+                store(NZM - 1 - i, csub(S, D));
+            }
+        }
+    }
+};
+
+// The same stage in block fixed point (F = fx), one scale per x-frequency.
+// The plane is brought to full magnitude when it is loaded, before the inverse
+// transform and when it is stored; the z convolution, where the tensor scales
+// each frequency differently, has a scale per ky.
+template <int PZ, int LY>
+__device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double, fx> &P, const int tid, const int nth,
+                                           const int kx)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fxc *S = reinterpret_cast<fxc *>(smem_raw);
+    __shared__ int s_e, s_top;
+    __shared__ unsigned s_r[4];   // flags, magnitudes in and out, sum of the frequencies' scales over the largest
+    const int tt = tid < nth ? tid : MM_IDLE_START;
+    const int ny = g.ny, nz = g.nz, Py = g.Py, nrow = 3 * nz;
+    signed char *s_sc = reinterpret_cast<signed char *>(S + nrow * g.rsy);  // [2][Py]: scale and top bit of every ky
+    fxc *Wk = P.W + (long)kx * nrow * ny;
+    const fxmc *tw = P.tw_py;
+    if (tid == 0) { s_e = FX_ZERO; s_top = FX_ZERO; }
+    if (tid < 4) s_r[tid] = 0;
+    __syncthreads();
+
+    // Wk[z][y][c] -> row (c, z); the first loads are issued before the rows' scales are looked at
+    constexpr int PF = 4;
+    const int tot = nrow * ny;
+    fxc v[PF];
+    auto load = [&](int e0) {
+#pragma unroll
+        for (int i = 0; i < PF; ++i)
+            if (e0 + i * nth < tot) v[i] = ld_cg(Wk + e0 + i * nth);
+    };
+    if (tt < tot) load(tt);
+    int emax = FX_ZERO;
+    unsigned fl = 0;
+    for (int i = tt; i < nz * ny; i += nth) {
+        const int p = P.fe1[i];
+        emax = max(emax, fx_exp(p));
+        fl |= fx_flags(p);
+    }
+    fx_cta_max(&s_e, emax);
+    fx_cta_or(&s_r[0], fl);
+    __syncthreads();
+    emax = s_e;
+    unsigned mag = 0;
+    for (int e0 = tt; e0 < tot;) {
+#pragma unroll
+        for (int i = 0; i < PF; ++i) {
+            const int e = e0 + i * nth;
+            if (e >= tot) break;
+            const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
+            const int d = fx_exp(P.fe1[rest]) - emax;
+            if (d) v[i] = fx_scale(v[i], d);
+            mag |= fx_mag(v[i]);
+            S[(c * nz + zz) * g.rsy + pidx(y)] = v[i];
+        }
+        e0 += PF * nth;
+        if (e0 < tot) load(e0);
+    }
+    fx_cta_or(&s_r[1], mag);
+    const int npad = Py - ny;
+    for (int e = tt; e < nrow * npad; e += nth) {
+        const int row = g.fd_pady.div(e), y = ny + (e - row * npad);
+        S[row * g.rsy + pidx(y)] = czero<fxc>();
+    }
+    __syncthreads();
+    const int rb = tid / g.Gy, j = tid - rb * g.Gy;  // row within a batch of g.RB rows
+    const bool act = rb < g.RB;
+    int pre = 59 - fx_bits(s_r[1]), e = emax - pre, sh = 0;
+    for (int r0 = 0; r0 < nrow; r0 += g.RB)
+        sh = fft_row_fx<false, true, false, 1, LY, false>(S + (act ? r0 + rb : 0) * g.rsy, Py, g.lpy, j, tw, act, pre,
+                                                          64, mag);
+    // z convolution: inputs of a ky below 2^59, so sums and differences below
+    // 2^60; outputs below 2^60 (the tensor's terms of an output sum to less
+    // than 2^62 units, and the factor 2)
+    constexpr int NZM = PZ > 1 ? PZ / 2 : 1;
+    const int hy = Py / 2, kst = hy + 1;
+    constexpr int NC = 4 * ZConv<NZM>::NE + 2 * ZConv<NZM>::NO;
+    e += sh + P.fek[kx] - (NZM > 1 ? 1 : 0);
+    int top = FX_ZERO;
+    for (int ky = tt; ky < Py; ky += nth) {
+        const int pky = pidx(ky), kyr = ky <= hy ? ky : Py - ky;
+        const bool flip = ky > hy;   // xy and yz are odd in ky: m_y and H_y change sign
+        ZConv<NZM> z;
+        z.K = P.Nhat + (long)kx * NC * kst + kyr;
+        z.kst = kst;
+        int sc;
+        {
+            fxc m[3][NZM];
+            unsigned mk = 0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int n = 0; n < NZM; ++n) {
+                    m[c][n] = n < nz ? S[(c * nz + n) * g.rsy + pky] : czero<fxc>();
+                    mk |= fx_mag(m[c][n]);
+                }
+            sc = 59 - fx_bits(mk);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int n = 0; n < NZM; ++n) {
+                    m[c][n] = fx_scale(m[c][n], sc);
+                    if (c == 1 && flip) m[c][n] = fxc{-m[c][n].x, -m[c][n].y};
+                }
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int i = 0; i < ZConv<NZM>::H; ++i) {
+                    const fxc a = m[c][i], b = m[c][NZM - 1 - i];
+                    z.up[c][i][0] = fx_split(NZM > 1 ? a.x + b.x : a.x);
+                    z.up[c][i][1] = fx_split(NZM > 1 ? a.y + b.y : a.y);
+                    z.um[c][i][0] = fx_split(a.x - b.x);
+                    z.um[c][i][1] = fx_split(a.y - b.y);
+                }
+        }
+        mag = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            z.output(c, [&](int n, fxc r) {
+                if (n >= nz) return;
+                if (c == 1 && flip) r = fxc{-r.x, -r.y};
+                mag |= fx_mag(r);
+                S[(c * nz + n) * g.rsy + pky] = r;
+            });
+        const int tk = fx_bits(mag) - sc;  // values of this ky: stored * 2^-sc, below 2^tk
+        s_sc[ky] = (signed char)sc;
+        s_sc[Py + ky] = (signed char)tk;
+        top = max(top, tk);
+    }
+    fx_cta_max(&s_top, top);
+    __syncthreads();
+    top = s_top;
+    // no partial sum of an inverse transform exceeds the sum of the largest moduli over ky
+    unsigned sum = 0;
+    for (int ky = tt; ky < Py; ky += nth) sum += ((1u << 18) >> min(top - s_sc[Py + ky], 18)) + 1;
+    fx_cta_add(&s_r[3], sum);
+    __syncthreads();
+    pre = 58 - top;
+    const int t = max(0, fx_log2_up(s_r[3]) - 18);
+    mag = 0;
+    for (int r0 = 0; r0 < nrow; r0 += g.RB)
+        sh = fft_row_fx<true, false, true, 1, LY, true, true>(S + (act ? r0 + rb : 0) * g.rsy, Py, g.lpy, j, tw, act, pre,
+                                                              t, mag, s_sc);
+    fx_cta_or(&s_r[2], mag);
+    __syncthreads();
+    const int post = 60 - fx_bits(s_r[2]);
+    e += sh - pre - post;
+    for (int i = tt; i < tot; i += nth) {
+        const int c = i % 3, rest = i / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
+        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + pidx(y)], post);
+    }
+    // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
+    const int flags = (int)s_r[0];
+    if (tid == 0) P.fe2[kx] = fx_pack(e, (nz == 1 || !flags) ? flags : 3);
+}
 
 template <typename T, typename F, int PZ, int LY>
 __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<T, F> &P, const int tid, const int nth,
@@ -342,9 +638,10 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<T, F> &P,
 }
 
 template <typename T, typename F, int PZ, int LY>
-__global__ void __launch_bounds__(YZBound<T>::v) k_yz(Geom g, FieldPtrs<T, F> P)
+__global__ void __launch_bounds__(YZBound<T>::v, 1) k_yz(Geom g, FieldPtrs<T, F> P)
 {
-    yz_body<T, F, PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
+    if constexpr (is_fx<F>) yz_body_fx<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
+    else yz_body<T, F, PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -551,13 +848,35 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
                                           const int bx, const int by, const int bid, const int nblk)
 {
     typedef typename cvec<F>::type V;
+    typedef typename twvec<F>::type TW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int TY = g.TY, y0 = bx * TY, z = by;
     const int nx = g.nx, ny = g.ny, nz = g.nz, Hx = g.Hx;
     const long N = g.N;
-    V *tw = S + 3 * TY * g.rsx;
+    TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);
+    // block fixed point: largest scale and flags of the x-frequencies, the sum of their scales over the largest, and
+    // the magnitude of this CTA's rows
+    __shared__ int s_e;
+    __shared__ unsigned s_r[3];
+    unsigned mag = 0;
+    const int *fe2 = nullptr;
+    int emax = FX_ZERO;
+    if constexpr (is_fx<F>) {
+        fe2 = P.fe2 + z / g.ZB;
+        if (tid == 0) s_e = FX_ZERO;
+        if (tid < 3) s_r[tid] = 0;
+        __syncthreads();
+        unsigned fl = 0;
+        for (int i = tt; i < g.C; i += nth) {
+            const int p = fe2[i * g.nzb];
+            emax = max(emax, fx_exp(p));
+            fl |= fx_flags(p);
+        }
+        fx_cta_max(&s_e, emax);
+        fx_cta_or(&s_r[0], fl);
+    }
 
     MinState *st = P.st;
     long k = 0;
@@ -629,32 +948,61 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         if (g0 == 0) {  // the twiddles (first commit group) are needed from here on
             cp_async_wait_group<1>();
             __syncthreads();
+            if constexpr (is_fx<F>) {
+                emax = s_e;
+                unsigned sum = 0;
+                for (int i = tt; i < g.C; i += nth) sum += ((1u << 18) >> min(emax - fx_exp(fe2[i * g.nzb]), 18)) + 1;
+                fx_cta_add(&s_r[1], sum);
+            }
         }
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= nel) break;
             const int c = e % 3, rest = e / 3, yl = rest & (TY - 1), kk = rest >> g.lty;
-            const V Xk = xa[i], Xm = cconj(xb[i]);
-            const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
-            const V t = cmulc(dif, tw[kk]);  // conj(w^k) dif
             V *row = S + (c * TY + yl) * g.rsx;
             V Z;
+            V Xk = xa[i], Xm = cconj(xb[i]);
+            if constexpr (is_fx<F>) {  // components below 2^60: |Z| < 2^62
+                Xk = fx_scale(Xk, fx_exp(fe2[kk * g.nzb]) - emax);
+                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * g.nzb]) - emax);
+            }
+            const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
+            V t;
+            if constexpr (is_fx<F>) t = fx_cmul<true>(dif, tw[kk], 0);
+            else t = cmulc(dif, tw[kk]);  // conj(w^k) dif
             Z.x = sum.x - t.y;
             Z.y = sum.y + t.x;
             row[spos<V>(kk)] = Z;
+            if constexpr (is_fx<F>) mag |= fx_mag(Z);
             if (kk != 0 && Hx - kk != kk) {
                 Z.x = sum.x + t.y;
                 Z.y = t.x - sum.y;
                 row[spos<V>(Hx - kk)] = Z;
+                if constexpr (is_fx<F>) mag |= fx_mag(Z);
             }
         }
     }
+    if constexpr (is_fx<F>) fx_cta_or(&s_r[2], mag);
     __syncthreads();
     {
         const int row = tid / g.Gx, j = tid - row * g.Gx;
         const bool act = row < 3 * TY;
-        fft_row<true, false, true, 2, LX>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act);
+        if constexpr (is_fx<F>) {
+            // the moduli of a row sum to at most 2^62 times the frequencies' scales over the largest
+            const int bits = fx_bits(s_r[2]), pre = 58 - bits;
+            unsigned none = 0;
+            emax += fft_row_fx<true, false, true, 2, LX, false>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act, pre,
+                                                                max(0, fx_log2_up(s_r[1]) - 18 + 62 - bits), none) - pre;
+        } else {
+            fft_row<true, false, true, 2, LX>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act);
+        }
+    }
+    double dscale = 0.0;   // block fixed point: one unit of the rows' values, in A/m
+    int bad = 0;
+    if constexpr (is_fx<F>) {
+        dscale = fx_pow2(emax);
+        bad = (int)s_r[0];
     }
     cp_async_wait_all();
     if (stg) __syncthreads();
@@ -683,9 +1031,21 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         const int yl = g.fd_nx.div(e), x = e - yl * nx, y = y0 + yl;
         if (y >= ny) continue;
         const long n = ((long)z * ny + y) * nx + x;
-        const T d0 = to_field<T>(rel<F>(S + (0 * TY + yl) * g.rsx, x));
-        const T d1 = to_field<T>(rel<F>(S + (1 * TY + yl) * g.rsx, x));
-        const T d2 = to_field<T>(rel<F>(S + (2 * TY + yl) * g.rsx, x));
+        T d0, d1, d2;
+        if constexpr (is_fx<F>) {
+            d0 = __ll2double_rn(rel<F>(S + (0 * TY + yl) * g.rsx, x).v) * dscale;
+            d1 = __ll2double_rn(rel<F>(S + (1 * TY + yl) * g.rsx, x).v) * dscale;
+            d2 = __ll2double_rn(rel<F>(S + (2 * TY + yl) * g.rsx, x).v) * dscale;
+            if (bad) {  // uniform over the CTA
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                if (bad & 1) d0 = d1 = nan;
+                if (bad & 2) d2 = nan;
+            }
+        } else {
+            d0 = to_field<T>(rel<F>(S + (0 * TY + yl) * g.rsx, x));
+            d1 = to_field<T>(rel<F>(S + (1 * TY + yl) * g.rsx, x));
+            d2 = to_field<T>(rel<F>(S + (2 * TY + yl) * g.rsx, x));
+        }
         // exchange: sum over present neighbours of (m_j - m_i) / d^2 (free faces)
         T m0, m1, m2, e0 = 0, e1 = 0, e2 = 0;
         if (stg) {
@@ -838,15 +1198,22 @@ __global__ void __launch_bounds__(768) k_xinv(Geom g, FieldPtrs<T, F> P, double 
 // ---------------------------------------------------------------------------
 // launch shapes and buffers of a problem's field kernels
 // ---------------------------------------------------------------------------
-template <typename T, typename F = T> FieldPtrs<T, F> make_ptrs(mm_problem *p)
+template <typename T, typename F = typename fft_of<T>::type> FieldPtrs<T, F> make_ptrs(mm_problem *p)
 {
     typedef typename cvec<F>::type V;
+    typedef typename twvec<F>::type TW;
+    const Geom &g = p->g;
     FieldPtrs<T, F> P;
     P.m_src = nullptr; P.H_out = nullptr;
     P.mbuf[0] = (T *)p->mbuf[0]; P.mbuf[1] = (T *)p->mbuf[1];
     P.gbuf[0] = (T *)p->gbuf[0]; P.gbuf[1] = (T *)p->gbuf[1];
-    P.W = (V *)p->W; P.W2 = (V *)p->W2; P.Nhat = (const F *)p->Nhat;
-    P.tw_px = (const V *)p->tw_px; P.tw_py = (const V *)p->tw_py; P.tw_pz = (const V *)p->tw_pz;
+    P.W = (V *)p->W; P.W2 = (V *)p->W2; P.Nhat = (const typename coef<F>::type *)p->Nhat;
+    P.tw_px = (const TW *)p->tw_px; P.tw_py = (const TW *)p->tw_py; P.tw_pz = (const TW *)p->tw_pz;
+    P.fe1 = p->fexp;
+    P.fea = p->fexp + (long)g.nz * g.ny;
+    P.feb = P.fea + (long)g.C * g.nzb;
+    P.fe2 = P.feb + (long)g.C * g.nkb;
+    P.fek = P.fe2 + (long)g.C * g.nzb;
     typedef typename io_of<T>::type IO;
     P.Kc = (const IO *)p->Kc; P.uc = (const IO *)p->uc;
     P.partials = p->partials; P.st = p->st; P.counter = p->counter;
@@ -876,7 +1243,8 @@ template <typename T> size_t smem_yz_t(const Geom &g)
 {
     typedef typename cvec<T>::type V;
     // the float kernel also holds the Py twiddles (the double kernel reads them from global memory)
-    return (size_t)3 * g.nz * g.rsy * sizeof(V) + (sizeof(T) == 4 ? (size_t)g.Py * sizeof(V) : 0);
+    // and the block fixed-point kernel two bytes per y-frequency
+    return (size_t)3 * g.nz * g.rsy * sizeof(V) + (sizeof(T) == 4 ? (size_t)g.Py * sizeof(V) : 2 * (size_t)g.Py);
 }
 
 // The field kernels are compiled for FFT row lengths 2^6 .. 2^10 (template

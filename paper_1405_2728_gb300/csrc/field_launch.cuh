@@ -72,7 +72,7 @@ cudaError_t launch_yz_any(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t 
 // the bulk layout's passes exist for double and float (double-word problems
 // are film-layout only: the planner refuses bulk grids for them)
 template <typename T, typename F>
-constexpr bool has_bulk = std::is_same<T, F>::value && !std::is_same<F, dfloat>::value;
+constexpr bool has_bulk = !std::is_same<F, dfloat>::value;
 
 // the y-z stage: the film kernel, or the three passes of the bulk layout
 template <typename T, typename F>

@@ -1,0 +1,201 @@
+// Block fixed-point arithmetic of the MM_FP64 convolution: 64-bit integers
+// with one power-of-two scale per block of values (a tile of rows, an
+// x-frequency), run on the integer pipes.
+//
+// Why: this GPU has 2 FP64 lanes per SM (measured 1.68 FMA per clock and SM),
+// against 42 64-bit integer additions and 24-32 wide multiply-adds per clock
+// and SM.  A radix-8 butterfly with its twiddles is 84 FP64 instructions, 50
+// clocks of an SM, or about 6 clocks in this arithmetic.  Precision: an FFT's
+// error is relative to the norm of its row, and a value here carries up to 58
+// bits below the largest value of its block, where a double carries 53.
+//
+// A value is v * 2^e with e held per block.  Twiddles are multipliers of type
+// fxm: hi * 2^32 + lo with a signed low word, in units of 2^-61.  Their
+// products with a value leave out the low x low partial product, at most 2
+// units of the result before its scaling, and are rounded.  The tensor is held
+// in units of 2^-62 and multiplied exactly (fxdot).
+// Bounds: values stay below 2^62 in magnitude wherever they are multiplied,
+// and below 2^63 everywhere (see the callers' scaling).
+#pragma once
+
+#include <cuda_runtime.h>
+
+// a value (aligned like the double it takes the place of)
+struct __align__(8) fx {
+    long long v;
+    fx() = default;
+    __host__ __device__ constexpr fx(long long x) : v(x) {}
+    __host__ __device__ constexpr fx(int x) : v(x) {}
+};
+struct __align__(16) fxc {
+    fx x, y;
+};
+// a multiplier: a twiddle in units of 2^-61 or a tensor element in units of 2^-62
+struct __align__(8) fxm {
+    int lo, hi;
+};
+struct __align__(16) fxmc {
+    fxm x, y;
+};
+
+// Scale of a block as the kernels hand it on: e * 4 + flags.  Non-finite
+// inputs have no place in a block; their components are taken as zero and
+// flagged (1: x or y, 2: z), and come out as NaN where the field would.
+#define FX_ZERO (-100000)   // exponent of an all-zero block
+__host__ __device__ __forceinline__ constexpr int fx_pack(int e, int flags) { return e * 4 + flags; }
+__host__ __device__ __forceinline__ constexpr int fx_exp(int p) { return p >> 2; }
+__host__ __device__ __forceinline__ constexpr int fx_flags(int p) { return p & 3; }
+
+__host__ __device__ constexpr fxm fx_multiplier(long long q)
+{
+    // signed low word, never -2^31, so that a multiplier can be negated word by word
+    const int lo = (int)(unsigned)(unsigned long long)q;
+    return lo == (int)0x80000000u ? fxm{lo + 1, (int)((q >> 32) + 1)} : fxm{lo, (int)((q - lo) >> 32)};
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ fx operator+(fx a, fx b) { return fx(a.v + b.v); }
+__device__ __forceinline__ fx operator-(fx a, fx b) { return fx(a.v - b.v); }
+__device__ __forceinline__ fx operator-(fx a) { return fx(-a.v); }
+
+// signed high word of the split v = hi * 2^32 + (signed) lo
+__device__ __forceinline__ int fx_hi(fx a) { return (int)(a.v >> 32) + (int)((unsigned)a.v >> 31); }
+__device__ __forceinline__ int fx_lo(fx a) { return (int)a.v; }
+
+// sum of products of values and twiddles: P holds the high x high products
+// (units of 2^64), c the cross products (units of 2^32)
+struct fxacc {
+    long long P, c;
+    // value(sh) drops `sh` further bits (0..3): the rounding constant enters here
+    __device__ __forceinline__ void zero(int sh) { P = 0; c = 1ll << (28 + sh); }
+    __device__ __forceinline__ void mad(int ah, int al, int bh, int bl)
+    {
+        P += (long long)ah * bh;
+        c += (long long)ah * bl;
+        c += (long long)al * bh;
+    }
+    // (P 2^32 + c) >> (29 + sh)
+    __device__ __forceinline__ fx value(int sh) const
+    {
+        const long long h = P + (c >> 32);
+        const unsigned w0 = (unsigned)c, w1 = (unsigned)h, w2 = (unsigned)(h >> 32);
+        const unsigned lo = __funnelshift_rc(w0, w1, 29 + sh), hi = __funnelshift_rc(w1, w2, 29 + sh);
+        return fx((long long)(((unsigned long long)hi << 32) | lo));
+    }
+};
+
+// a tensor element (units of 2^-62) split for fxdot, and its negative
+struct fxk {
+    int hi, lo, lo3;
+    __device__ __forceinline__ explicit fxk(fxm k) : hi(k.hi), lo(k.lo), lo3(k.lo >> 3) {}
+    __device__ __forceinline__ fxk(const fxk &k, bool neg)
+        : hi(neg ? -k.hi : k.hi), lo(neg ? -k.lo : k.lo), lo3(neg ? -k.lo3 : k.lo3) {}
+};
+// sum of up to 8 products of values below 2^60 and tensor elements, the low x
+// low products included (q, in units of 2^-27 of a unit)
+struct fxdot {
+    long long P, c;
+    int q;
+    __device__ __forceinline__ void zero() { P = 0; c = 1ll << 29; q = 0; }
+    __device__ __forceinline__ void mad(int2 a, const fxk &b)  // a: (low, high) words of a split value
+    {
+        P += (long long)a.y * b.hi;
+        c += (long long)a.y * b.lo;
+        c += (long long)a.x * b.hi;
+        q += __mulhi(a.x, b.lo3);
+    }
+    __device__ __forceinline__ fx value() const
+    {
+        const long long d = c + ((long long)q << 3), h = P + (d >> 32);
+        const unsigned w0 = (unsigned)d, w1 = (unsigned)h, w2 = (unsigned)(h >> 32);
+        const unsigned lo = __funnelshift_r(w0, w1, 30), hi = __funnelshift_r(w1, w2, 30);
+        return fx((long long)(((unsigned long long)hi << 32) | lo));
+    }
+};
+__device__ __forceinline__ int2 fx_split(fx a) { return make_int2(fx_lo(a), fx_hi(a)); }
+
+// a * b for a constant b, |b| <= 1 (rounded)
+__device__ __forceinline__ fx fx_mulc(fxm b, fx a)
+{
+    fxacc s;
+    s.zero(0);
+    s.mad(fx_hi(a), fx_lo(a), b.hi, b.lo);
+    return s.value(0);
+}
+
+// a * w (CONJ: a * conj(w)) divided by 2^sh, sh in 0..3
+template <bool CONJ> __device__ __forceinline__ fxc fx_cmul(fxc a, fxmc w, int sh)
+{
+    const int xh = fx_hi(a.x), xl = fx_lo(a.x), yh = fx_hi(a.y), yl = fx_lo(a.y);
+    fxacc re, im;
+    re.zero(sh);
+    im.zero(sh);
+    re.mad(xh, xl, w.x.hi, w.x.lo);
+    im.mad(yh, yl, w.x.hi, w.x.lo);
+    if (CONJ) {
+        re.mad(yh, yl, w.y.hi, w.y.lo);
+        im.mad(xh, xl, -w.y.hi, -w.y.lo);
+    } else {
+        re.mad(yh, yl, -w.y.hi, -w.y.lo);
+        im.mad(xh, xl, w.y.hi, w.y.lo);
+    }
+    fxc r;
+    r.x = re.value(sh);
+    r.y = im.value(sh);
+    return r;
+}
+
+// v / 2^s rounded to nearest, ties to even, s >= 0: rounding ties up shifts the mean of a row by up to a quarter of a
+// unit, which the next transform gathers in one cell
+__device__ __forceinline__ fx fx_shr(fx a, int s)
+{
+    return s ? fx((a.v + ((1ll << (s - 1)) - 1) + ((a.v >> s) & 1)) >> s) : a;
+}
+// v * 2^d, d of either sign (uniform over a block); large right shifts give 0
+__device__ __forceinline__ fx fx_scale(fx a, int d)
+{
+    if (d >= 0) return fx(a.v << d);
+    return d > -62 ? fx_shr(a, -d) : fx(0);
+}
+__device__ __forceinline__ fxc fx_scale(fxc a, int d)
+{
+    fxc r;
+    r.x = fx_scale(a.x, d);
+    r.y = fx_scale(a.y, d);
+    return r;
+}
+// bits of the high word's magnitude, to be OR-ed over a block; with b the
+// number of bits of the result, every |v| of the block is below 2^(32 + b) + 1
+__device__ __forceinline__ unsigned fx_mag(fx a)
+{
+    const int h = (int)(a.v >> 32);
+    return (unsigned)(h ^ (h >> 31));
+}
+__device__ __forceinline__ unsigned fx_mag(fxc a) { return fx_mag(a.x) | fx_mag(a.y); }
+// OR (or maximum, or sum) over the CTA into *dst in shared memory; a barrier makes it visible
+__device__ __forceinline__ void fx_cta_or(unsigned *dst, unsigned v)
+{
+    v = __reduce_or_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && v) atomicOr(dst, v);
+}
+__device__ __forceinline__ void fx_cta_max(int *dst, int v)
+{
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMax(dst, v);
+}
+__device__ __forceinline__ void fx_cta_add(unsigned *dst, unsigned v)
+{
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicAdd(dst, v);
+}
+// least t >= 0 with 2^t >= v
+__device__ __forceinline__ int fx_log2_up(unsigned v) { return v > 1 ? 32 - __clz((int)(v - 1)) : 0; }
+__device__ __forceinline__ int fx_bits(unsigned mag) { return 64 - __clz((int)mag); }  // 32 + bits of mag
+
+// 2^e as a double, 0 below the smallest normal power
+__device__ __forceinline__ double fx_pow2(int e)
+{
+    if (e < -1022) return 0.0;
+    return __longlong_as_double((long long)(min(e, 1023) + 1023) << 52);
+}
+#endif

@@ -100,6 +100,17 @@ __global__ void k_twiddle(typename cvec<T>::type *tw, int L)
     tw[t] = w;
 }
 
+// the same table as multipliers of the block fixed-point convolution
+__global__ void k_twiddle_fx(fxmc *tw, int L)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= L) return;
+    double s, c;
+    sincospi(2.0 * (double)t / (double)L, &s, &c);
+    const double one = 2305843009213693952.0;  // 2^61
+    tw[t] = fxmc{fx_multiplier(__double2ll_rn(c * one)), fx_multiplier(__double2ll_rn(-s * one))};
+}
+
 template <typename T>
 __global__ void k_convert(T *dst, const double *src, long n)
 {
@@ -234,7 +245,7 @@ int mm_launch_twiddles(mm_problem *p, cudaStream_t s)
     for (int i = 0; i < 3; ++i) {
         const int blocks = (L[i] + 255) / 256;
         if (p->precision == MM_F32X2) k_twiddle<dfloat><<<blocks, 256, 0, s>>>((dcomplex *)dst[i], L[i]);
-        else if (p->precision == MM_FP64) k_twiddle<double><<<blocks, 256, 0, s>>>((double2 *)dst[i], L[i]);
+        else if (p->precision == MM_FP64) k_twiddle_fx<<<blocks, 256, 0, s>>>((fxmc *)dst[i], L[i]);
         else k_twiddle<float><<<blocks, 256, 0, s>>>((float2 *)dst[i], L[i]);
     }
     cudaError_t e = cudaGetLastError();

@@ -167,6 +167,70 @@ __global__ void k_extract_film(int c, int Px, int Py, int nz, int nzf, const dou
     }
 }
 
+// The tensor of the block fixed-point convolution (MM_FP64): one x-frequency
+// per CTA, from doubles to integers in units of 2^(ek - 62).  ek is chosen so
+// that the magnitudes of the terms of any one output value sum to less than 1:
+// over the sources' components and, for films, z offsets (offset 0 once, the
+// others on both sides).
+// Bulk (NZM = 0), in place: K[i * 6 + c], i < n frequencies.
+// Film, from K[(dz * 6 + c) * n + i] to out[coefficient * n + i], i < n ky
+// values: the combinations of the offsets that ZConv multiplies with, formed
+// from the rounded elements so that they are exact.
+template <int NZM>
+__global__ void __launch_bounds__(256) k_tensor_fixed(const double *K, long per_kx, fxm *out, long out_kx, int n,
+                                                      int *ek)
+{
+    const double *Kx = K + blockIdx.x * per_kx;
+    fxm *Ox = out + blockIdx.x * out_kx;
+    __shared__ double s_top[256];
+    double top = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) {
+        double r0 = 0.0, r1 = 0.0, r2 = 0.0;
+        for (int dz = 0; dz < (NZM ? NZM : 1); ++dz) {
+            double k[6];
+            for (int c = 0; c < 6; ++c) k[c] = fabs(NZM ? Kx[((long)dz * 6 + c) * n + i] : Kx[(long)i * 6 + c]);
+            const double w = dz ? 2.0 : 1.0;
+            r0 += w * (k[0] + k[3] + k[4]);
+            r1 += w * (k[3] + k[1] + k[5]);
+            r2 += w * (k[4] + k[5] + k[2]);
+        }
+        top = fmax(top, fmax(r0, fmax(r1, r2)));
+    }
+    s_top[threadIdx.x] = top;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) s_top[threadIdx.x] = fmax(s_top[threadIdx.x], s_top[threadIdx.x + o]);
+        __syncthreads();
+    }
+    top = s_top[0];
+    // one bit to spare for the rounding of the sums above
+    const int e = top > 0.0 && isfinite(top) ? ilogb(top) + 2 : 0;
+    if (threadIdx.x == 0) ek[blockIdx.x] = e;
+    if constexpr (NZM == 0) {
+        for (long q = threadIdx.x; q < per_kx; q += 256) Ox[q] = fx_multiplier(__double2ll_rn(scalbn(Kx[q], 62 - e)));
+    } else {
+        for (int i = threadIdx.x; i < n; i += 256) {
+            fxm *o = Ox + i;
+            for (int c = 0; c < 6; ++c) {
+                long long k[4] = {0, 0, 0, 0};
+                for (int dz = 0; dz < NZM; ++dz) k[dz] = __double2ll_rn(scalbn(Kx[((long)dz * 6 + c) * n + i], 62 - e));
+                auto put = [&](long long v) { *o = fx_multiplier(v); o += n; };
+                if (c < 4) {  // even in z
+                    if (NZM == 1) put(k[0]);
+                    if (NZM == 2) { put(k[0] + k[1]); put(k[0] - k[1]); }
+                    if (NZM == 4) {
+                        put(k[0] + k[3]); put(k[1] + k[2]); put(k[0] + k[1]);
+                        put(k[0] - k[3]); put(k[1] - k[2]); put(k[0] - k[1]);
+                    }
+                } else {      // odd
+                    if (NZM == 2) put(k[1]);
+                    if (NZM == 4) { put(k[3]); put(k[1] - k[2]); put(k[1] + k[2]); put(k[1]); }
+                }
+            }
+        }
+    }
+}
+
 int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 
 } // namespace
@@ -234,6 +298,16 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
     const long fext = (long)(g.Px / 2 + 1) * nzf * (g.Py / 2 + 1);
     long fblocks = (fext + 255) / 256;
     if (fblocks > mm_sm_count() * 32L) fblocks = mm_sm_count() * 32L;
+    // the transformed tensor in the field's precision; for the film layout of block fixed point in a work buffer
+    void *K64 = p->Nhat;
+    if (p->precision == MM_FP64 && !g.bulk) {
+        e = cudaMallocAsync(&K64, sizeof(double) * 6 * (size_t)fext, s);
+        if (e) {
+            cudaFreeAsync(F, s); cudaFreeAsync(tw, s);
+            mm_set_cuda_error(e, "cudaMallocAsync(tensor)");
+            return MM_ERR_OOM;
+        }
+    }
     for (int c = 0; c < 6 && !e; ++c) {
         k_place<<<(int)blocks, 256, 0, s>>>(c, g.nx, g.ny, g.nz, g.Px, g.Py, g.Pz, N_dev, F);
         for (int a = 0; a < naxes; ++a) {
@@ -248,7 +322,7 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
         if (!g.bulk) {
             const double fscale = -g.Ms / ((double)g.Px * g.Py);
             if (p->precision == MM_FP64)
-                k_extract_film<double><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (double *)p->Nhat);
+                k_extract_film<double><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (double *)K64);
             else if (p->precision == MM_F32X2)
                 k_extract_film<dfloat><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (dfloat *)p->Nhat);
             else
@@ -260,6 +334,21 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
         }
         e = cudaGetLastError();
     }
+    if (!e && p->precision == MM_FP64) {
+        const int hy = g.Py / 2;
+        fxm *out = (fxm *)p->Nhat;
+        int *ek = p->fexp + ((long)g.nz * g.ny + (long)g.C * (2 * g.nzb + g.nkb));
+        if (g.bulk) {
+            const int n = (g.Pz / 2 + 1) * (hy + 1);
+            k_tensor_fixed<0><<<g.C, 256, 0, s>>>((const double *)K64, (long)n * 6, out, (long)n * 6, n, ek);
+        } else {
+            const long in = (long)nzf * 6 * (hy + 1), no = (long)mm_film_coefs(g, p->precision) * (hy + 1);
+            auto *k = nzf == 1 ? k_tensor_fixed<1> : (nzf == 2 ? k_tensor_fixed<2> : k_tensor_fixed<4>);
+            k<<<g.C, 256, 0, s>>>((const double *)K64, in, out, no, hy + 1, ek);
+        }
+        e = cudaGetLastError();
+    }
+    if (K64 != p->Nhat) cudaFreeAsync(K64, s);
     cudaFreeAsync(F, s);
     cudaFreeAsync(tw, s);
     if (e) { mm_set_cuda_error(e, "tensor spectrum"); return MM_ERR_CUDA; }
