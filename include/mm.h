@@ -142,8 +142,10 @@ MM_API int mm_newell_static(const mm_grid *grid, double *N_dev, void *stream);
 /*
  * mm_setup_geometry -- create a problem: validates the grid and material,
  * allocates device workspaces, computes the Newell tensor (as mm_newell), its
- * Fourier spectrum on the zero-padded grid (padded size per axis: the smallest
- * power of two >= 2n-1, and >= 2 along x), times the admissible launch
+ * Fourier spectrum on the zero-padded grid (padded size per axis: the power of
+ * two P >= 2n-1 (and >= 2 along x) or, in MM_FP64 and MM_FP32, a shorter length
+ * >= 2n-1: 5/8 or 3/4 of P = 512 or 1024 along x and along y of films, 5/8, 3/4
+ * or 25/32 of P = 128 .. 1024 along y and z of bulk grids), times the admissible launch
  * shapes of the field kernels on this problem and keeps the fastest, and
  * captures the minimiser's CUDA graph.  precision = MM_FP64 or MM_FP32: element type of m/H and of the FFT
  * and stencil arithmetic; MM_F32X2: double arrays, double-float arithmetic
@@ -160,6 +162,8 @@ MM_API int mm_newell_static(const mm_grid *grid, double *N_dev, void *stream);
  * 1024 x 512 x 4 in FP32): one kernel per x-frequency.  Bulk layout (every
  * other grid, e.g. 256^3 cubes): separate y, z and inverse-y passes through
  * an extra spectrum buffer of C * nz * Py * 3 complex values.
+ * Both the layout and what is supported are decided with every axis padded to
+ * its power of two.
  * Supported in this build (else MM_ERR_UNSUPPORTED): every padded length
  * <= 4096 (nx, ny, nz <= 2048) and one padded y row or z row, with its
  * twiddles, within 200 KiB of shared memory.

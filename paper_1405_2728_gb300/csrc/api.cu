@@ -66,7 +66,6 @@ size_t tensor_bytes(const Geom &g, int precision, size_t esz)
     return (g.bulk ? (size_t)g.C * (g.Pz / 2 + 1) * (g.Py / 2 + 1) * 6
                    : (size_t)g.C * mm_film_coefs(g, precision) * (g.Py / 2 + 1)) * esz;
 }
-int ilog2i(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 
 bool grid_ok(const mm_grid *g)
 {
@@ -144,19 +143,51 @@ void free_problem(mm_problem *p)
     delete p;
 }
 
+// Padded FFT length of an axis of n cells: the power of two P >= 2n - 1, or a
+// shorter length with an odd part where that is compiled (fft.cuh) and pays:
+// the first of 5/8, 3/4 and 25/32 of P that reaches 2n - 1 (bulk y and z: P from
+// 128 to 1024, 25/32 too; x and the film y-z kernel: 320, 384, 640 and 768).
+// Work and traffic of an axis go with its padded length: a 160^3 cube's z pass
+// takes 2045 us at 512 x 512 x 512 and 550 us at 320 x 320 x 320 (FP32).  Films
+// of up to 128 cells an axis stay on powers of two, their kernels being bound by
+// latency, and 25/32 loses there: its 25 x 8 points take five passes' barriers
+// (200 x 100 x 2, FP64 y-z stage: 20.6 us at 256, 31.8 us at 200).
+int padded_length(int n, bool bulk_axis)
+{
+    const int P = next_pow2(2 * n - 1);
+    if (P > 1024 || P < (bulk_axis ? 128 : 512)) return P;
+    const int cand[3] = {P / 8 * 5, P / 4 * 3, P / 32 * 25};
+    for (int i = 0; i < (bulk_axis ? 3 : 2); ++i)
+        if (cand[i] >= 2 * n - 1 && cand[i] % 8 == 0) return cand[i];
+    return P;
+}
+
 // Geometry and launch shape; returns MM_ERR_UNSUPPORTED outside this build's envelope.
 int plan(mm_problem *p)
 {
     Geom &g = p->g;
     const mm_grid &gr = p->grid;
     g.nx = gr.nx; g.ny = gr.ny; g.nz = gr.nz;
-    g.Px = next_pow2(2 * gr.nx - 1); if (g.Px < 2) g.Px = 2;
-    g.Py = next_pow2(2 * gr.ny - 1);
-    g.Pz = next_pow2(2 * gr.nz - 1);
-    g.Hx = g.Px / 2; g.C = g.Hx + 1;
-    g.lhx = ilog2i(g.Hx); g.lpy = ilog2i(g.Py);
-    g.Gx = g.Hx >= 8 ? g.Hx / 8 : 1;
-    g.Gy = g.Py >= 8 ? g.Py / 8 : 1;
+    // what is supported, and in which layout, is decided on powers of two
+    const int P2[3] = {next_pow2(2 * gr.nx - 1), next_pow2(2 * gr.ny - 1), next_pow2(2 * gr.nz - 1)};
+    auto lengths = [&](int Px, int Py, int Pz) {
+        const int vsz = p->precision == MM_FP32 ? 8 : 16;  // bytes per complex element
+        g.Px = Px < 2 ? 2 : Px; g.Py = Py; g.Pz = Pz;
+        g.Hx = g.Px / 2; g.C = g.Hx + 1;
+        g.lhx = pow2_part(g.Hx); g.lpy = pow2_part(g.Py); g.lpz = pow2_part(g.Pz);
+        g.Gx = g.Hx >= 8 ? g.Hx / 8 : 1;
+        g.Gy = g.Py >= 8 ? g.Py / 8 : 1;
+        g.Gz = g.Pz >= 8 ? g.Pz / 8 : 1;
+        // shared-memory row strides: 16-byte rows pad one element per 8, float
+        // rows are XOR-swizzled within groups of 16 (fft.cuh)
+        g.rsx = row_stride(g.Hx, vsz);
+        g.rsy = row_stride(g.Py, vsz);
+        g.rsz = row_stride(g.Pz, vsz);
+        g.fd_padx.init(g.Px - gr.nx > 0 ? g.Px - gr.nx : 1);
+        g.fd_pady.init(g.Py - gr.ny > 0 ? g.Py - gr.ny : 1);
+    };
+    if (P2[0] > 4096 || P2[1] > 4096 || P2[2] > 4096) return MM_ERR_UNSUPPORTED;
+    lengths(P2[0], P2[1], P2[2]);
     g.N = (long)gr.nx * gr.ny * gr.nz;
     g.dx = gr.dx; g.dy = gr.dy; g.dz = gr.dz;
     g.Ms = p->mat.Ms;
@@ -172,45 +203,36 @@ int plan(mm_problem *p)
     g.wcan = dfloat(g.can); g.wK = dfloat(g.K);
     for (int c = 0; c < 3; ++c) g.wu[c] = dfloat(g.u[c]);
     g.fd_nx.init(gr.nx); g.fd_ny.init(gr.ny);
-    g.fd_padx.init(g.Px - gr.nx > 0 ? g.Px - gr.nx : 1);
-    g.fd_pady.init(g.Py - gr.ny > 0 ? g.Py - gr.ny : 1);
     // the float x-inverse kernel stages its stencil rows with 16-byte copies
     g.stage = p->precision == MM_FP32 && gr.nx % 4 == 0;
     g.fd_nc.init(g.stage ? gr.nx / 4 : 1);
-    if (g.Px > 4096 || g.Py > 4096 || g.Pz > 4096) return MM_ERR_UNSUPPORTED;
-    // shared-memory row strides: double rows pad one element per 8, float rows
-    // are XOR-swizzled within a stride of L+1 (fft.cuh)
-    const int vsz = p->precision == MM_FP32 ? 8 : 16;  // bytes per complex element
-    g.rsx = row_stride(g.Hx, vsz);
-    g.rsy = row_stride(g.Py, vsz);
-    g.rsz = row_stride(g.Pz, vsz);
-    if (g.rsx <= g.Hx || g.rsy <= g.Py || g.rsz <= g.Pz) return MM_ERR_UNSUPPORTED;  // the kernels index rows with these strides
-    g.lpz = ilog2i(g.Pz);
-    g.Gz = g.Pz >= 8 ? g.Pz / 8 : 1;
     // admissible launch shapes; mm_autotune picks among them after setup
     const size_t smax = MM_SMEM_CAP;
     g.bulk = 0;
     p->nrb = 0;
-    if (g.Pz <= 8) {
+    const int maxT = g.Pz <= 8 ? mm_yz_thread_bound(p) : 0, nrow = 3 * g.nz;
+    bool film = g.Gy <= maxT && mm_smem_yz_for(p) <= smax;
+    if (!film) {
+        // bulk layout: separate y and z passes (double and float only)
+        if (p->precision == MM_F32X2 || g.Gy > mm_bulk_thread_bound(p) || g.Gz > mm_bulk_thread_bound(p) ||
+            mm_bulk_smem_y(p, 1) > smax || mm_bulk_smem_z(p, 1) > smax)
+            return MM_ERR_UNSUPPORTED;
+    }
+    // films keep their few layers' power of two: the z direction is a direct convolution
+    if (p->precision != MM_F32X2)
+        lengths(padded_length(gr.nx, false), padded_length(gr.ny, !film), film ? P2[2] : padded_length(gr.nz, true));
+    if (film) {
         // film layout: y rows per batch in the y-z kernel, divisors of 3 nz
         // with RB*Gy threads within the kernel's bound
-        const int maxT = mm_yz_thread_bound(p), nrow = 3 * g.nz;
         for (int rb = nrow; rb >= 1 && p->nrb < 16; --rb)
             if (nrow % rb == 0 && rb * g.Gy <= maxT) p->rbs[p->nrb++] = rb;
-        if (p->nrb) {
-            g.RB = p->rbs[0];
-            if (mm_smem_yz_for(p) > smax) p->nrb = 0;
-        }
-    }
-    if (!p->nrb) {
-        // bulk layout: separate y and z passes (double and float only)
-        if (p->precision == MM_F32X2) return MM_ERR_UNSUPPORTED;
+        g.RB = p->rbs[0];
+    } else {
         g.bulk = 1;
         g.RB = 1;
         p->rbs[0] = 1;
         p->nrb = 1;
         const int maxT = mm_bulk_thread_bound(p);
-        if (g.Gy > maxT || g.Gz > maxT) return MM_ERR_UNSUPPORTED;
         // z planes per y-pass CTA: up to 4, as many rows as one pass of threads covers
         g.ZB = 0;
         for (int zb = 4; zb >= 1; zb /= 2)
@@ -248,7 +270,7 @@ int plan(mm_problem *p)
     // (the 32 x 16 x 1 film: 49 us per evaluation against 69 us with the
     // widest tile); the autotuner replaces it on larger problems
     g.TY = g.TYF = p->tys[0];
-    g.lty = g.ltyf = ilog2i(g.TY);
+    g.lty = g.ltyf = mm_ilog2(g.TY);
     // partial sums are sized for the smallest tile (most CTAs)
     p->nblk_x = ((gr.ny + p->tys[0] - 1) / p->tys[0]) * gr.nz;
     return MM_OK;

@@ -35,43 +35,23 @@
 #include <vector>
 
 #include "common.cuh"
-#include "field_kernels.cuh"
+#include "batch_kernels.cuh"
+
+// the grouped kernels' addresses (group_*.cu)
+#define MM_DECLARE_GROUP(SFX) \
+    const void *mm_group_xfwd_##SFX(); \
+    const void *mm_group_yz_##SFX(); \
+    const void *mm_group_xinv_##SFX();
+MM_DECLARE_GROUP(fp64)
+MM_DECLARE_GROUP(fp32)
 
 namespace {
 
-// the FFT arithmetic of a group's fields, and its y-z stage
-template <typename T> using FA = typename fft_of<T>::type;
-template <typename T, int PZ, int L>
-__device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int tid, int nth, int kx)
+template <typename T> const void *group_kernel(int stage)
 {
-    if constexpr (!is_fx<FA<T>>) yz_body<T, FA<T>, PZ, L>(g, P, tid, nth, kx);
-    else if constexpr (L == 0) yz_body_fx<PZ, 0>(g, P, tid, nth, kx);
+    if constexpr (sizeof(T) == 8) return stage == 0 ? mm_group_xfwd_fp64() : (stage == 1 ? mm_group_yz_fp64() : mm_group_xinv_fp64());
+    else return stage == 0 ? mm_group_xfwd_fp32() : (stage == 1 ? mm_group_yz_fp32() : mm_group_xinv_fp32());
 }
-
-// one problem of a grouped launch, as the grouped kernels read it
-template <typename T>
-struct GFilm {
-    Geom g;
-    FieldPtrs<T> P;
-    int nth_xf, nth_x, nth_yz;   // working threads of the three stages (the problem's own launch shapes)
-    int gx_x, nblk_x;            // x-inverse grid: CTAs along y, CTAs in all
-    int first[3], count[3];      // the problem's work items of each stage (x-forward, y-z, x-inverse)
-};
-
-// Problems still running in this iteration, as a compacted work list: the
-// grouped kernels are persistent and walk virtual item indices 0 ..
-// prefix[s][nact] - 1 of stage s; index v belongs to films[a] for the a with
-// prefix[s][a] <= v < prefix[s][a + 1].  Layout in device memory:
-// nact, films[nf], prefix[3][nf + 1] (ints).
-struct GActive {
-    int *base;
-    int nf;
-    __device__ int &nact() const { return base[0]; }
-    __device__ int *films() const { return base + 1; }
-    __device__ int *prefix(int s) const { return base + 1 + nf + s * (nf + 1); }
-};
-
-struct GItem { int film, bx, by; };
 
 // A problem group as the init and advance kernels see it.  The descriptor
 // layout does not depend on the field type (Geom, then pointers), so both
@@ -96,93 +76,12 @@ struct GCtl {
     double kappa;
 };
 
-template <typename T>
-__device__ __forceinline__ void load_film(GFilm<T> &f, const GFilm<T> *src)
-{
-    const int nw = (int)(sizeof(GFilm<T>) / sizeof(int));
-    for (int i = threadIdx.x; i < nw; i += blockDim.x)
-        reinterpret_cast<int *>(&f)[i] = reinterpret_cast<const int *>(src)[i];
-    __syncthreads();
-}
-
-// the work item behind virtual index v of stage s (binary search over the
-// active problems' prefix sums)
 struct GRef {
     const GFilm<double> *films;
     int nf;
     GActive act;
 };
 static_assert(sizeof(GFilm<double>) == sizeof(GFilm<float>), "descriptor layout is precision independent");
-
-__device__ __forceinline__ GItem active_item(const GActive &A, const int *first, const GItem *items, int s, int v)
-// first[s * nf + f]: where problem f's items start in stage s's item array
-{
-    const int *pre = A.prefix(s);
-    int lo = 0, hi = A.nact() - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre[mid] <= v) lo = mid; else hi = mid - 1;
-    }
-    const int f = A.films()[lo];
-    return items[first[s * A.nf + f] + (v - pre[lo])];
-}
-
-// Persistent grouped kernels: CTA b takes virtual items b, b + gridDim.x, ...
-// of the problems still running.  Items of a stage are independent, so the
-// order does not matter; the shared memory is reused item after item.
-#define MM_GROUP_LOOP(STAGE)                                                                  \
-    __shared__ __align__(16) GFilm<T> f;                                                      \
-    const int total = A.prefix(STAGE)[A.nact()];                                              \
-    for (int v = blockIdx.x; v < total; v += gridDim.x) {                                    \
-        __syncthreads();                                                                      \
-        const GItem it = active_item(A, first_of, items, STAGE, v);                           \
-        load_film(f, films + it.film);
-
-template <typename T>
-__global__ void __launch_bounds__(768) k_xfwd_group(const GFilm<T> *films, const GItem *items, const int *first_of,
-                                                    GActive A)
-{
-    MM_GROUP_LOOP(0)
-        switch (lc_of(f.g.lhx)) {
-#define C(L) case L: xfwd_body<T, FA<T>, true, L>(f.g, f.P, threadIdx.x, f.nth_xf, it.bx, it.by); break;
-            MM_LC_CASES(C)
-#undef C
-        }
-    }
-}
-
-// Block fixed point takes the code for any row length here: integer results do
-// not depend on the instance, and its compiled lengths in one kernel with
-// three layer counts took four minutes to build.
-template <typename T>
-__global__ void __launch_bounds__(YZBound<T>::v) k_yz_group(const GFilm<T> *films, const GItem *items,
-                                                            const int *first_of, GActive A)
-{
-    MM_GROUP_LOOP(1)
-    switch (f.g.Pz * 16 + (is_fx<FA<T>> ? 0 : lc_of(f.g.lpy))) {
-#define C(L) case 1 * 16 + L: yz_of<T, 1, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 4 * 16 + L: yz_of<T, 4, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 8 * 16 + L: yz_of<T, 8, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break;
-        MM_LC_CASES(C)
-#undef C
-    }
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(768) k_xinv_group(const GFilm<T> *films, const GItem *items, const int *first_of,
-                                                    GActive A)
-{
-    MM_GROUP_LOOP(2)
-        const int bid = it.by * f.gx_x + it.bx;
-        switch (lc_of(f.g.lhx)) {
-#define C(L) case L: xinv_body<T, FA<T>, MODE_MIN, L>(f.g, f.P, 0.0, 0.0, 0.0, 0, 0, threadIdx.x, f.nth_x, it.bx, it.by, \
-                                                    bid, f.nblk_x); break;
-            MM_LC_CASES(C)
-#undef C
-        }
-    }
-}
 
 // compacted work lists of the problems still running (one CTA); `first`
 // lists, per problem, where its items start in each stage's item array
@@ -444,15 +343,15 @@ template <typename T> cudaError_t build_group(mm_batch *b, Group<T> &G)
     if ((e = cudaMemset(G.act.base, 0, sizeof(int) * (1 + nf + 3 * ((size_t)nf + 1))))) return e;
     if (nf == 0) return cudaSuccess;
     if (G.sm_xf > MM_SMEM_CAP || G.sm_yz > MM_SMEM_CAP || G.sm_x > MM_SMEM_CAP) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(k_xfwd_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
-        (e = cudaFuncSetAttribute(k_yz_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
-        (e = cudaFuncSetAttribute(k_xinv_group<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)))
+    if ((e = cudaFuncSetAttribute(group_kernel<T>(0), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
+        (e = cudaFuncSetAttribute(group_kernel<T>(1), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
+        (e = cudaFuncSetAttribute(group_kernel<T>(2), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)))
         return e;
     // persistent grids: as many CTAs as are resident on all SMs at once
     int r0 = 0, r1 = 0, r2 = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r0, k_xfwd_group<T>, G.thr_xf, G.sm_xf)) ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r1, k_yz_group<T>, G.thr_yz, G.sm_yz)) ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r2, k_xinv_group<T>, G.thr_x, G.sm_x)))
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r0, group_kernel<T>(0), G.thr_xf, G.sm_xf)) ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r1, group_kernel<T>(1), G.thr_yz, G.sm_yz)) ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r2, group_kernel<T>(2), G.thr_x, G.sm_x)))
         return e;
     const int sms = mm_sm_count();
     G.grid_xf = std::max(1, std::min(G.n_xf, sms * std::max(1, r0)));
@@ -473,9 +372,17 @@ template <typename T> cudaError_t refresh_group(mm_batch *b, Group<T> &G, cudaSt
 template <typename T> void launch_group(const Group<T> &G, cudaStream_t s)
 {
     if (G.members.empty()) return;
-    k_xfwd_group<T><<<G.grid_xf, G.thr_xf, G.sm_xf, s>>>(G.films, G.items_xf, G.first, G.act);
-    k_yz_group<T><<<G.grid_yz, G.thr_yz, G.sm_yz, s>>>(G.films, G.items_yz, G.first, G.act);
-    k_xinv_group<T><<<G.grid_x, G.thr_x, G.sm_x, s>>>(G.films, G.items_x, G.first, G.act);
+    // a failed launch is found by the caller's cudaGetLastError
+    auto launch = [&](int stage, int grid, int threads, size_t smem, const GItem *items) {
+        const GFilm<T> *films = G.films;
+        const int *first = G.first;
+        GActive act = G.act;
+        void *args[] = {&films, &items, &first, &act};
+        cudaLaunchKernel(group_kernel<T>(stage), dim3(grid), dim3(threads), args, smem, s);
+    };
+    launch(0, G.grid_xf, G.thr_xf, G.sm_xf, G.items_xf);
+    launch(1, G.grid_yz, G.thr_yz, G.sm_yz, G.items_yz);
+    launch(2, G.grid_x, G.thr_x, G.sm_x, G.items_x);
 }
 
 // graph of a whole sweep call: init -> WHILE { grouped stages of both

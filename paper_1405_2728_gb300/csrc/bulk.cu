@@ -29,6 +29,8 @@ template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
 }
 
 template <typename T> struct BulkBound { static constexpr int v = sizeof(T) == 8 ? 384 : 512; };
+// two float CTAs of the z pass per SM: its odd radices would otherwise take 121 registers
+template <typename T> struct BulkCtas { static constexpr int v = sizeof(T) == 8 ? 1 : 2; };
 
 // In block fixed point (double fields, F = fx) every CTA of a pass brings its
 // block to full magnitude when it loads it and when it stores it, with the
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
 }
 
 template <typename T, int LZ>
-__global__ void __launch_bounds__(BulkBound<T>::v) k_zconv(Geom g, FieldPtrs<T> P)
+__global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom g, FieldPtrs<T> P)
 {
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
@@ -331,34 +333,34 @@ template <typename T> size_t smem_z_t(const Geom &g, int kb)
     return ((size_t)3 * kb * g.rsz + g.Pz) * sizeof(V) + (sizeof(T) == 8 ? (size_t)2 * kb * g.Pz : 0);
 }
 
-inline int lc_of(int logL) { return MM_FFT_SPECIALISED(logL) ? logL : 0; }
-#define MM_LC_CASES(X) X(0) X(6) X(7) X(8) X(9) X(10)
-
 template <typename T> cudaError_t bulk_conv_t(const Geom &g, const FieldPtrs<T> &P, cudaStream_t s, int pass)
 {
     const dim3 gy(g.C, (g.nz + g.ZB - 1) / g.ZB), gz(g.C, (g.Py + g.KB - 1) / g.KB);
     const int ty = round32(g.RBY * g.Gy), tz = round32(g.RBZ * g.Gz);
     const size_t sy = smem_y_t<T>(g, g.ZB), sz = smem_z_t<T>(g, g.KB);
-    const int ly = lc_of(g.lpy), lz = lc_of(g.lpz);
+    const int ly = lb_of(g.Py), lz = lb_of(g.Pz);
     if (pass < 0 || pass == 0) {
         switch (ly) {
 #define C(L) case L: k_ypass<T, false, L><<<gy, ty, sy, s>>>(g, P); break;
-            MM_LC_CASES(C)
+            MM_LB_CASES(C)
 #undef C
+        default: return cudaErrorInvalidValue;
         }
     }
     if (pass < 0 || pass == 1) {
         switch (lz) {
 #define C(L) case L: k_zconv<T, L><<<gz, tz, sz, s>>>(g, P); break;
-            MM_LC_CASES(C)
+            MM_LB_CASES(C)
 #undef C
+        default: return cudaErrorInvalidValue;
         }
     }
     if (pass < 0 || pass == 2) {
         switch (ly) {
 #define C(L) case L: k_ypass<T, true, L><<<gy, ty, sy, s>>>(g, P); break;
-            MM_LC_CASES(C)
+            MM_LB_CASES(C)
 #undef C
+        default: return cudaErrorInvalidValue;
         }
     }
     return cudaGetLastError();
@@ -375,14 +377,14 @@ template <typename T> cudaError_t configure_t(const Geom &g)
 {
     cudaError_t e = cudaSuccess;
     const size_t sy = smem_y_t<T>(g, g.ZB), sz = smem_z_t<T>(g, g.KB);
-    switch (lc_of(g.lpy)) {
+    switch (lb_of(g.Py)) {
 #define C(L) case L: if ((e = smem_attr(k_ypass<T, false, L>, sy)) || (e = smem_attr(k_ypass<T, true, L>, sy))) return e; break;
-        MM_LC_CASES(C)
+        MM_LB_CASES(C)
 #undef C
     }
-    switch (lc_of(g.lpz)) {
+    switch (lb_of(g.Pz)) {
 #define C(L) case L: return smem_attr(k_zconv<T, L>, sz);
-        MM_LC_CASES(C)
+        MM_LB_CASES(C)
 #undef C
     }
     return cudaErrorInvalidValue;

@@ -134,7 +134,7 @@ struct Geom {
     int nx, ny, nz;
     int Px, Py, Pz;        // padded FFT lengths
     int Hx, C;             // Hx = Px/2 (packed complex length), C = Hx + 1 x-frequencies
-    int lhx, lpy;          // log2(Hx), log2(Py)
+    int lhx, lpy;          // log2 of the power of two in Hx, Py (their odd parts are 1, 3, 5 or 25)
     int Gx, Gy;            // threads per FFT row: max(1, L/8)
     int TY;                // y rows per CTA of the x-inverse kernel
     int TYF, ltyf;         // y rows per CTA of the x-forward kernel, log2
@@ -148,7 +148,7 @@ struct Geom {
     int KB;                // y frequencies per CTA of the z pass
     int RBZ;               // z rows transformed at once in the z pass
     int nzb, nkb;          // blocks of ZB z planes (film layout: one block of all), of KB y frequencies
-    int lpz, Gz, rsz;      // log2(Pz), threads per z row, smem stride of a z row
+    int lpz, Gz, rsz;      // likewise of Pz, threads per z row, smem stride of a z row
     int nbody;             // kernels per minimiser iteration (3 film, 5 bulk)
     long N;                // cells
     double dx, dy, dz;

@@ -1,12 +1,13 @@
 // Shared-memory FFT building blocks for the zero-padded demagnetisation
 // convolution (the "FFT accelerated convolution" of Section 3).
 //
-// A row of L = 2^l complex values lives in shared memory and is transformed
-// in place by G = max(1, L/8) threads with self-sorting Stockham passes
-// (Stockham; Cochran et al., Proc. IEEE 55 (1967) 1664): an optional first
-// pass of radix 2 or 4 and then radix-8 passes.  Each thread keeps one radix-8
-// butterfly (or two radix-4 / four radix-2 ones) in registers per pass; a
-// barrier separates the loads of a pass from its stores, which makes the
+// A row of L complex values, L = 2^l or 2^l times 3, 5 or 25 with l >= 3,
+// lives in shared memory and is transformed in place by G = max(1, L/8)
+// threads with self-sorting Stockham passes (Stockham; Cochran et al., Proc.
+// IEEE 55 (1967) 1664): an optional first pass of radix 2 or 4, then radix-8
+// passes, then the odd radices.  Each thread keeps one radix-8 butterfly (or
+// two radix-4 or -5, three radix-3, four radix-2 ones) in registers per pass;
+// a barrier separates the loads of a pass from its stores, which makes the
 // in-place update safe.  Twiddles come from a table tw[t] = exp(-2 pi i t/L')
 // read with stride ts = L'/L.
 //
@@ -47,7 +48,15 @@ template <typename V> __host__ __device__ __forceinline__ int spos(int i)
 }
 __host__ __device__ __forceinline__ int row_stride(int L, int esz)
 {
-    return esz == 8 ? L + 1 : padded_row(L);
+    return esz == 8 ? (L <= 8 ? L : (L + 15) / 16 * 16) + 1 : padded_row(L);
+}
+
+// L = 2^l (times an odd part): l
+__host__ __device__ constexpr int pow2_part(int L)
+{
+    int l = 0;
+    while (!((L >> l) & 1)) ++l;
+    return l;
 }
 
 // copy a twiddle table of n complex values into shared memory (all threads)
@@ -131,6 +140,93 @@ template <int R, bool INV, bool HIN, typename V> __device__ __forceinline__ void
     else dft8<INV, HIN>(a);
 }
 
+// r times i (inverse) or -i (forward) added to and taken from u: the outputs
+// n and R - n of an odd-length DFT
+template <bool INV, typename V> __device__ __forceinline__ void odd_pair(V u, V r, V &lo, V &hi)
+{
+    const V w = cmul_mi<INV>(r);
+    lo = cadd(u, w);
+    hi = csub(u, w);
+}
+template <typename V, typename T> __device__ __forceinline__ V caxpy(V a, T c, V b)
+{
+    V r;
+    r.x = a.x + c * b.x;
+    r.y = a.y + c * b.y;
+    return r;
+}
+// 3-point and 5-point DFTs from the sums and differences of a_n and a_{R-n}
+template <bool INV, typename V> __device__ __forceinline__ void dft3(V *a)
+{
+    typedef decltype(a[0].x) T;
+    const T s = (T)0.86602540378443864676372317075294;
+    const V t = cadd(a[1], a[2]), d = csub(a[1], a[2]);
+    const V u = caxpy(a[0], (T)-0.5, t);
+    V r;
+    r.x = s * d.x; r.y = s * d.y;
+    a[0] = cadd(a[0], t);
+    odd_pair<INV>(u, r, a[1], a[2]);
+}
+template <bool INV, typename V> __device__ __forceinline__ void dft5(V *a)
+{
+    typedef decltype(a[0].x) T;
+    const T c1 = (T)0.30901699437494742410229341718282, c2 = (T)-0.80901699437494742410229341718282;
+    const T s1 = (T)0.95105651629515357211643933337938, s2 = (T)0.58778525229247312916870595463907;
+    const V t1 = cadd(a[1], a[4]), t2 = cadd(a[2], a[3]), d1 = csub(a[1], a[4]), d2 = csub(a[2], a[3]);
+    const V u1 = caxpy(caxpy(a[0], c1, t1), c2, t2), u2 = caxpy(caxpy(a[0], c2, t1), c1, t2);
+    V r1, r2;
+    r1.x = s1 * d1.x + s2 * d2.x; r1.y = s1 * d1.y + s2 * d2.y;
+    r2.x = s2 * d1.x - s1 * d2.x; r2.y = s2 * d1.y - s1 * d2.y;
+    a[0] = cadd(a[0], cadd(t1, t2));
+    odd_pair<INV>(u1, r1, a[1], a[4]);
+    odd_pair<INV>(u2, r2, a[2], a[3]);
+}
+
+// One Stockham pass of odd radix R (3 or 5) over a row of length L: L/R
+// butterflies, thread j takes j, j + G, ...  Ns is a power of two or L/R.  With
+// HOUT only the outputs below L/2 are stored.
+template <int R, bool INV, bool HOUT, typename V>
+__device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G, const V *__restrict__ tw, int ts,
+                                             bool active)
+{
+    constexpr int NB = (8 + R - 1) / R;
+    V v[NB * R];
+    const int LR = L / R, tstep0 = (L / (Ns * R)) * ts;
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            if (b >= LR) break;
+            const int step = tstep0 * (Ns == LR ? b : b & (Ns - 1));
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                v[q * R + r] = row[spos<V>(b + r * LR)];
+                if (r > 0) {
+                    const V w = tw[r * step];
+                    v[q * R + r] = INV ? cmulc(v[q * R + r], w) : cmul(v[q * R + r], w);
+                }
+            }
+            if constexpr (R == 3) dft3<INV>(&v[q * R]);
+            else dft5<INV>(&v[q * R]);
+        }
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            if (b >= LR) break;
+            const int k = Ns == LR ? b : b & (Ns - 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = (b - k) * R + k + r * Ns;
+                if (!HOUT || 2 * i < L) row[spos<V>(i)] = v[q * R + r];
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // One Stockham pass of radix R over a row of length L (Ns = product of the
 // radices of the previous passes).  Thread j handles butterflies j + q G,
 // q < 8/R.  Caller guarantees visibility of the row before the call; the
@@ -193,8 +289,8 @@ __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int 
     __syncthreads();
 }
 
-// In-place FFT of one shared-memory row of length L = 2^logL (forward:
-// exp(-i...), inverse: exp(+i...), unnormalised).  Every thread of the CTA
+// In-place FFT of one shared-memory row of length L, 2^logL times 1, 3, 5 or
+// 25 (forward: exp(-i...), inverse: exp(+i...), unnormalised).  Every thread of the CTA
 // must call this with the same L (it contains barriers); thread j in [0, G)
 // of the row's group works on it.  Threads with active == false (padding
 // threads of the CTA) only take part in the barriers.  The caller
@@ -206,7 +302,7 @@ __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int 
 // pass count folds into the instructions.  Kernels are instantiated for the
 // common lengths (template parameter LC of fft_row) and the host launches
 // the matching instance.
-template <bool INV, bool HIN, bool HOUT, int TS, typename V>
+template <bool INV, bool HIN, bool HOUT, int TS, bool ODD, typename V>
 __device__ __forceinline__ void fft_row_n(V *row, int L, int logL, int j, const V *__restrict__ tw, bool active)
 {
     if (L == 1) return;
@@ -242,6 +338,7 @@ __device__ __forceinline__ void fft_row_n(V *row, int L, int logL, int j, const 
     const int G = L >> 3;
     const int rem = logL % 3;
     const int n8 = logL / 3;
+    int odd = ODD ? L >> logL : 1;
     int Ns = 1;
     bool first = true;
     if (rem == 1) {
@@ -252,7 +349,7 @@ __device__ __forceinline__ void fft_row_n(V *row, int L, int logL, int j, const 
         Ns = 4; first = false;
     }
     for (int p = 0; p < n8; ++p) {
-        const bool last = (p == n8 - 1);
+        const bool last = (p == n8 - 1) && odd == 1;
         if (first && HIN) {
             if (last && HOUT) stockham_pass<8, INV, true, true>(row, L, Ns, j, G, tw, TS, active);
             else stockham_pass<8, INV, true, false>(row, L, Ns, j, G, tw, TS, active);
@@ -263,20 +360,29 @@ __device__ __forceinline__ void fft_row_n(V *row, int L, int logL, int j, const 
         Ns <<= 3;
         first = false;
     }
+    if constexpr (ODD) {
+        if (odd == 25) {
+            stockham_odd<5, INV, false>(row, L, Ns, j, G, tw, TS, active);
+            Ns *= 5;
+            odd = 5;
+        }
+        if (odd == 5) stockham_odd<5, INV, HOUT>(row, L, Ns, j, G, tw, TS, active);
+        else if (odd == 3) stockham_odd<3, INV, HOUT>(row, L, Ns, j, G, tw, TS, active);
+    }
 }
 
-template <int LOGL, bool INV, bool HIN, bool HOUT, int TS, typename V>
+template <int L, bool INV, bool HIN, bool HOUT, int TS, typename V>
 __device__ __forceinline__ void fft_row_c(V *row, int j, const V *__restrict__ tw, bool active)
 {
-    static_assert(LOGL >= 3, "compile-time rows have at least 8 elements");
-    constexpr int L = 1 << LOGL, G = L >> 3, rem = LOGL % 3, n8 = LOGL / 3;
+    static_assert(L >= 8 && L % 8 == 0, "compile-time rows have at least 8 elements");
+    constexpr int LOGL = pow2_part(L), odd = L >> LOGL, G = L >> 3, rem = LOGL % 3, n8 = LOGL / 3;
     constexpr int NS0 = rem == 1 ? 2 : (rem == 2 ? 4 : 1);
     if constexpr (rem == 1) stockham_pass<2, INV, HIN, false>(row, L, 1, j, G, tw, TS, active);
     if constexpr (rem == 2) stockham_pass<4, INV, HIN, false>(row, L, 1, j, G, tw, TS, active);
 #pragma unroll
     for (int p = 0; p < n8; ++p) {
         const int Ns = NS0 << (3 * p);
-        const bool last = (p == n8 - 1), first = (p == 0 && rem == 0);
+        const bool last = (p == n8 - 1) && odd == 1, first = (p == 0 && rem == 0);
         if (first && HIN) {
             if (last && HOUT) stockham_pass<8, INV, true, true>(row, L, Ns, j, G, tw, TS, active);
             else stockham_pass<8, INV, true, false>(row, L, Ns, j, G, tw, TS, active);
@@ -285,15 +391,19 @@ __device__ __forceinline__ void fft_row_c(V *row, int j, const V *__restrict__ t
             else stockham_pass<8, INV, false, false>(row, L, Ns, j, G, tw, TS, active);
         }
     }
+    if constexpr (odd == 25) stockham_odd<5, INV, false>(row, L, L / 25, j, G, tw, TS, active);
+    if constexpr (odd == 25 || odd == 5) stockham_odd<5, INV, HOUT>(row, L, L / 5, j, G, tw, TS, active);
+    if constexpr (odd == 3) stockham_odd<3, INV, HOUT>(row, L, L / 3, j, G, tw, TS, active);
 }
 
-// LC > 0: the kernel was compiled for rows of length 2^LC (L, logL unused);
-// LC == 0: any length
+// LC > 0: the kernel was compiled for rows of length 2^LC, or LC above 16
+// (L, logL unused); LC == 0: any power of two; LC == -1: any length
+constexpr int fft_length(int LC) { return LC > 16 ? LC : 1 << LC; }
 template <bool INV, bool HIN, bool HOUT, int TS, int LC, typename V>
 __device__ __forceinline__ void fft_row(V *row, int L, int logL, int j, const V *__restrict__ tw, bool active)
 {
-    if constexpr (LC > 0) fft_row_c<LC, INV, HIN, HOUT, TS>(row, j, tw, active);
-    else fft_row_n<INV, HIN, HOUT, TS>(row, L, logL, j, tw, active);
+    if constexpr (LC > 0) fft_row_c<fft_length(LC), INV, HIN, HOUT, TS>(row, j, tw, active);
+    else fft_row_n<INV, HIN, HOUT, TS, LC < 0>(row, L, logL, j, tw, active);
 }
 
 // ---------------------------------------------------------------------------
@@ -413,6 +523,79 @@ __device__ __forceinline__ void stockham_pass_fx(fxc *row, int L, int Ns, int j,
     __syncthreads();
 }
 
+// a + c1 t1 + c2 t2 (constants in units of 2^-61)
+__device__ __forceinline__ fx fx_axpy2(fx a, fxm c1, fx t1, fxm c2, fx t2)
+{
+    fxacc s;
+    s.zero(0);
+    s.mad(fx_hi(t1), fx_lo(t1), c1.hi, c1.lo);
+    s.mad(fx_hi(t2), fx_lo(t2), c2.hi, c2.lo);
+    return a + s.value(0);
+}
+template <bool INV> __device__ __forceinline__ void dft3_fx(fxc *a)
+{
+    constexpr fxm s = fx_multiplier(1996918623117814388ll);   // sqrt(3)/2
+    const fxc t = cadd(a[1], a[2]), d = csub(a[1], a[2]);
+    const fxc u{a[0].x - fx_shr(t.x, 1), a[0].y - fx_shr(t.y, 1)}, r{fx_mulc(s, d.x), fx_mulc(s, d.y)};
+    a[0] = cadd(a[0], t);
+    odd_pair<INV>(u, r, a[1], a[2]);
+}
+template <bool INV> __device__ __forceinline__ void dft5_fx(fxc *a)
+{
+    constexpr fxm c1 = fx_multiplier(712544676207699905ll), c2 = fx_multiplier(-1865466180814546881ll);  // cos(2 pi n/5)
+    constexpr fxm s1 = fx_multiplier(2192987019466309470ll), s2 = fx_multiplier(1355340514917506542ll);  // sin(2 pi n/5)
+    constexpr fxm n1{-s1.lo, -s1.hi};
+    const fxc t1 = cadd(a[1], a[4]), t2 = cadd(a[2], a[3]), d1 = csub(a[1], a[4]), d2 = csub(a[2], a[3]);
+    const fxc u1{fx_axpy2(a[0].x, c1, t1.x, c2, t2.x), fx_axpy2(a[0].y, c1, t1.y, c2, t2.y)};
+    const fxc u2{fx_axpy2(a[0].x, c2, t1.x, c1, t2.x), fx_axpy2(a[0].y, c2, t1.y, c1, t2.y)};
+    const fxc r1{fx_axpy2(fx(0), s1, d1.x, s2, d2.x), fx_axpy2(fx(0), s1, d1.y, s2, d2.y)};
+    const fxc r2{fx_axpy2(fx(0), s2, d1.x, n1, d2.x), fx_axpy2(fx(0), s2, d1.y, n1, d2.y)};
+    a[0] = cadd(a[0], cadd(t1, t2));
+    odd_pair<INV>(u1, r1, a[1], a[4]);
+    odd_pair<INV>(u2, r2, a[2], a[3]);
+}
+template <int R, bool INV, bool HOUT, bool MAG>
+__device__ __forceinline__ void stockham_odd_fx(fxc *row, int L, int Ns, int j, int G, const fxmc *__restrict__ tw, int ts,
+                                                bool active, int sh, unsigned &mag)
+{
+    constexpr int NB = (8 + R - 1) / R;
+    fxc v[NB * R];
+    const int LR = L / R, tstep0 = (L / (Ns * R)) * ts;
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            if (b >= LR) break;
+            const int step = tstep0 * (Ns == LR ? b : b & (Ns - 1));
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const fxc a = row[pidx(b + r * LR)];
+                v[q * R + r] = r ? fx_cmul<INV>(a, tw[r * step], sh) : fxc{fx_shr(a.x, sh), fx_shr(a.y, sh)};
+            }
+            if constexpr (R == 3) dft3_fx<INV>(&v[q * R]);
+            else dft5_fx<INV>(&v[q * R]);
+        }
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const int b = j + q * G;
+            if (b >= LR) break;
+            const int k = Ns == LR ? b : b & (Ns - 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = (b - k) * R + k + r * Ns;
+                if (!HOUT || 2 * i < L) {
+                    row[pidx(i)] = v[q * R + r];
+                    if (MAG) mag |= fx_mag(v[q * R + r]);
+                }
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // one pass of a row: FIRST with the scale `pre`, later ones with their share of the shift
 template <int R, bool INV, bool HIN, bool HOUT, bool FIRST, bool MAG, bool VAR>
 __device__ __forceinline__ void fx_pass(fxc *row, int L, int Ns, int j, int G, const fxmc *tw, int ts, bool active,
@@ -428,20 +611,28 @@ __device__ __forceinline__ int fft_row_fx(fxc *row, int L, int logL, int j, cons
                                           int pre, int t, unsigned &mag, const signed char *var = nullptr)
 {
     if constexpr (LC > 0) {
-        constexpr int LL = 1 << LC, G = LL >> 3, rem = LC % 3, n8 = LC / 3;
+        constexpr int LL = fft_length(LC), LG = pow2_part(LL), odd = LL >> LG, G = LL >> 3, rem = LG % 3, n8 = LG / 3;
         constexpr int NS0 = rem == 1 ? 2 : (rem == 2 ? 4 : 1);
         if constexpr (rem == 1) fx_pass<2, INV, HIN, false, true, false, VAR>(row, LL, 1, j, G, tw, TS, active, pre, 1, t, mag, var);
         if constexpr (rem == 2) fx_pass<4, INV, HIN, false, true, false, VAR>(row, LL, 1, j, G, tw, TS, active, pre, 2, t, mag, var);
 #pragma unroll
         for (int p = 0; p < n8; ++p) {
             const int Ns = NS0 << (3 * p), q = rem + 3 * (p + 1);
-            const bool last = (p == n8 - 1), first = (p == 0 && rem == 0);
+            const bool last = (p == n8 - 1) && odd == 1, first = (p == 0 && rem == 0);
             if (first && last) fx_pass<8, INV, HIN, HOUT, true, MAG, VAR>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
             else if (first) fx_pass<8, INV, HIN, false, true, false, VAR>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
             else if (last) fx_pass<8, INV, false, HOUT, false, MAG, false>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
             else fx_pass<8, INV, false, false, false, false, false>(row, LL, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
         }
-        return fx_cum(LC, t);
+        if constexpr (odd == 25) {
+            stockham_odd_fx<5, INV, false, false>(row, LL, LL / 25, j, G, tw, TS, active, fx_cum(LG + 3, t) - fx_cum(LG, t), mag);
+            stockham_odd_fx<5, INV, HOUT, MAG>(row, LL, LL / 5, j, G, tw, TS, active, fx_cum(LG + 5, t) - fx_cum(LG + 3, t), mag);
+        }
+        if constexpr (odd == 5)
+            stockham_odd_fx<5, INV, HOUT, MAG>(row, LL, LL / 5, j, G, tw, TS, active, fx_cum(LG + 3, t) - fx_cum(LG, t), mag);
+        if constexpr (odd == 3)
+            stockham_odd_fx<3, INV, HOUT, MAG>(row, LL, LL / 3, j, G, tw, TS, active, fx_cum(LG + 2, t) - fx_cum(LG, t), mag);
+        return fx_cum(LG + (odd == 25 ? 5 : (odd == 5 ? 3 : (odd == 3 ? 2 : 0))), t);
     } else {
         if (L < 8) {
             fxc a[4];
@@ -467,11 +658,11 @@ __device__ __forceinline__ int fft_row_fx(fxc *row, int L, int logL, int j, cons
             return 0;
         }
         const int G = L >> 3, rem = logL % 3, n8 = logL / 3;
-        int Ns = 1, q = 0;
+        int Ns = 1, q = 0, odd = LC < 0 ? L >> logL : 1;
         if (rem == 1) { fx_pass<2, INV, HIN, false, true, false, VAR>(row, L, 1, j, G, tw, TS, active, pre, 1, t, mag, var); Ns = 2; q = 1; }
         else if (rem == 2) { fx_pass<4, INV, HIN, false, true, false, VAR>(row, L, 1, j, G, tw, TS, active, pre, 2, t, mag, var); Ns = 4; q = 2; }
         for (int p = 0; p < n8; ++p) {
-            const bool last = p == n8 - 1, first = q == 0;
+            const bool last = p == n8 - 1 && odd == 1, first = q == 0;
             q += 3;
             if (first && last) fx_pass<8, INV, HIN, HOUT, true, MAG, VAR>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
             else if (first) fx_pass<8, INV, HIN, false, true, false, VAR>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
@@ -479,10 +670,51 @@ __device__ __forceinline__ int fft_row_fx(fxc *row, int L, int logL, int j, cons
             else fx_pass<8, INV, false, false, false, false, false>(row, L, Ns, j, G, tw, TS, active, pre, q, t, mag, var);
             Ns <<= 3;
         }
-        return fx_cum(logL, t);
+        // the odd passes: q bits rounded up from the radices so far (40 = 8 x 5: 6; 25 x 2^l: l + 5)
+        if constexpr (LC < 0) {
+            if (odd == 25) {
+                stockham_odd_fx<5, INV, false, false>(row, L, Ns, j, G, tw, TS, active, fx_cum(q + 3, t) - fx_cum(q, t), mag);
+                q += 3;
+                Ns *= 5;
+                const int q2 = logL + 5;
+                stockham_odd_fx<5, INV, HOUT, MAG>(row, L, Ns, j, G, tw, TS, active, fx_cum(q2, t) - fx_cum(q, t), mag);
+                q = q2;
+            } else if (odd == 5) {
+                stockham_odd_fx<5, INV, HOUT, MAG>(row, L, Ns, j, G, tw, TS, active, fx_cum(q + 3, t) - fx_cum(q, t), mag);
+                q += 3;
+            } else if (odd == 3) {
+                stockham_odd_fx<3, INV, HOUT, MAG>(row, L, Ns, j, G, tw, TS, active, fx_cum(q + 2, t) - fx_cum(q, t), mag);
+                q += 2;
+            }
+        }
+        return fx_cum(q, t);
     }
 }
 
-// Row lengths with compiled specialisations in the field kernels (log2 of
-// 64 .. 1024); other lengths take the generic code.
-#define MM_FFT_SPECIALISED(logL) ((logL) >= 6 && (logL) <= 10)
+// Row lengths with compiled code: the powers of two 64 .. 1024 in every kernel,
+// and the lengths with an odd part that the planner gives an axis (LC of
+// fft_row; X(LC)): the x rows hold half the padded length, the y-z kernel of
+// films the whole one, and the passes of bulk grids have all of them.
+#define MM_LC_POW2(X) X(6) X(7) X(8) X(9) X(10)
+#define MM_LX_ODD(X) X(160) X(192) X(320) X(384)
+#define MM_LY_ODD(X) X(320) X(384) X(640) X(768)
+#define MM_LB_ODD(X) X(80) X(96) X(160) X(192) X(200) X(320) X(384) X(400) X(640) X(768) X(800)
+#define MM_LX_CASES(X) X(0) MM_LC_POW2(X) MM_LX_ODD(X)
+#define MM_LY_CASES(X) X(0) MM_LC_POW2(X) MM_LY_ODD(X)
+#define MM_LB_CASES(X) X(-1) MM_LC_POW2(X) MM_LB_ODD(X)
+__host__ __device__ inline int lc_pow2(int L, int other)
+{
+    return L >= 64 && L <= 1024 && (L & (L - 1)) == 0 ? pow2_part(L) : other;
+}
+#define MM_LC_OF(name, ODD, other)           \
+    __host__ __device__ inline int name(int L) \
+    {                                         \
+        switch (L) {                          \
+            ODD(MM_LC_CASE) return L;         \
+        }                                     \
+        return lc_pow2(L, other);             \
+    }
+#define MM_LC_CASE(N) case N:
+MM_LC_OF(lx_of, MM_LX_ODD, 0)
+MM_LC_OF(ly_of, MM_LY_ODD, 0)
+MM_LC_OF(lb_of, MM_LB_ODD, -1)

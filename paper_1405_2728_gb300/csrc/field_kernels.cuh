@@ -1247,20 +1247,24 @@ template <typename T> size_t smem_yz_t(const Geom &g)
     return (size_t)3 * g.nz * g.rsy * sizeof(V) + (sizeof(T) == 4 ? (size_t)g.Py * sizeof(V) : 2 * (size_t)g.Py);
 }
 
-// The field kernels are compiled for FFT row lengths 2^6 .. 2^10 (template
-// parameter LX of the x kernels: log2 Hx; LY of the y-z kernel: log2 Py) and
-// once for any length (0); these launchers pick the instance.
-__host__ __device__ inline int lc_of(int logL) { return MM_FFT_SPECIALISED(logL) ? logL : 0; }
-#define MM_LC_CASES(X) X(0) X(6) X(7) X(8) X(9) X(10)
+// The field kernels are compiled for a set of FFT row lengths (template
+// parameter LX of the x kernels, LY of the y-z kernel; MM_LX_CASES,
+// MM_LY_CASES) and once for any power of two (0); the launchers pick the
+// instance.
 // Double-word (F = dfloat) kernels are compiled for the lengths 512 and 1024
 // only (rows of films 257 .. 1024 cells long, and 129 .. 512 wide), other
 // lengths take the generic code: their unrolled double-word arithmetic makes
 // every compiled length expensive to build.
 template <typename F> constexpr bool lc_compiled(int L) { return true; }
 template <> constexpr bool lc_compiled<dfloat>(int L) { return L == 0 || L == 9 || L == 10; }
-template <typename F> __host__ __device__ inline int lc_of_f(int logL)
+template <typename F> __host__ __device__ inline int lx_of_f(int length)
 {
-    const int L = lc_of(logL);
+    const int L = lx_of(length);
+    return lc_compiled<F>(L) ? L : 0;
+}
+template <typename F> __host__ __device__ inline int ly_of_f(int length)
+{
+    const int L = ly_of(length);
     return lc_compiled<F>(L) ? L : 0;
 }
 

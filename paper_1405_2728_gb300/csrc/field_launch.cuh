@@ -23,10 +23,11 @@ cudaError_t launch_xfwd(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
     const dim3 grid((g.ny + g.TYF - 1) / g.TYF, g.nz);
     const int thr = threads_xf<T>(g);
     const size_t sm = smem_xf_t<T>(g);
-    switch (lc_of_f<F>(g.lhx)) {
+    switch (lx_of_f<F>(g.Hx)) {
 #define C(L) case L: if constexpr (lc_compiled<F>(L)) k_xfwd<T, F, MIN, L><<<grid, thr, sm, s>>>(g, P); break;
-        MM_LC_CASES(C)
+        MM_LX_CASES(C)
 #undef C
+    default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
@@ -39,10 +40,11 @@ cudaError_t launch_xinv(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s,
     const int thr = threads_x<T>(g);
     const size_t sm = smem_x_t<T>(g);
     const double h0 = hext ? hext[0] : 0.0, h1 = hext ? hext[1] : 0.0, h2 = hext ? hext[2] : 0.0;
-    switch (lc_of_f<F>(g.lhx)) {
+    switch (lx_of_f<F>(g.Hx)) {
 #define C(L) case L: if constexpr (lc_compiled<F>(L)) k_xinv<T, F, MODE, L><<<grid, thr, sm, s>>>(g, P, h0, h1, h2, h, use_cond); break;
-        MM_LC_CASES(C)
+        MM_LX_CASES(C)
 #undef C
+    default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
@@ -50,10 +52,11 @@ cudaError_t launch_xinv(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s,
 template <typename T, typename F, int PZ>
 cudaError_t launch_yz(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
 {
-    switch (lc_of_f<F>(g.lpy)) {
+    switch (ly_of_f<F>(g.Py)) {
 #define C(L) case L: if constexpr (lc_compiled<F>(L)) k_yz<T, F, PZ, L><<<g.C, threads_yz<T>(g), smem_yz_t<T>(g), s>>>(g, P); break;
-        MM_LC_CASES(C)
+        MM_LY_CASES(C)
 #undef C
+    default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
@@ -95,7 +98,7 @@ template <typename K> cudaError_t smem_attr(K *f, size_t bytes)
 template <typename T, typename F> cudaError_t configure_t(const Geom &g, size_t sxf, size_t sx, size_t syz)
 {
     cudaError_t e = cudaSuccess;
-    switch (lc_of_f<F>(g.lhx)) {
+    switch (lx_of_f<F>(g.Hx)) {
 #define C(L)                                                                                     \
     case L:                                                                                      \
         if constexpr (lc_compiled<F>(L)) {                                                       \
@@ -105,11 +108,11 @@ template <typename T, typename F> cudaError_t configure_t(const Geom &g, size_t 
                 return e;                                                                        \
         }                                                                                        \
         break;
-        MM_LC_CASES(C)
+        MM_LX_CASES(C)
 #undef C
     }
     if (g.bulk) return cudaSuccess;
-    switch (lc_of_f<F>(g.lpy)) {
+    switch (ly_of_f<F>(g.Py)) {
 #define C(L)                                                                                     \
     case L:                                                                                      \
         if constexpr (lc_compiled<F>(L)) {                                                       \
@@ -118,7 +121,7 @@ template <typename T, typename F> cudaError_t configure_t(const Geom &g, size_t 
             if (g.Pz == 8) return smem_attr(k_yz<T, F, 8, L>, syz);                              \
         }                                                                                        \
         return cudaErrorInvalidValue;
-        MM_LC_CASES(C)
+        MM_LY_CASES(C)
 #undef C
     }
     return cudaErrorInvalidValue;

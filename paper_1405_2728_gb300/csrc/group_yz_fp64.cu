@@ -1,0 +1,4 @@
+// The grouped batch's y-z kernel (MM_FP64).
+#include "batch_kernels.cuh"
+
+const void *mm_group_yz_fp64() { return (const void *)k_yz_group<double>; }

@@ -128,7 +128,7 @@ __global__ void k_fft_strided(double2 *F, int L, int logL, long stride, long inn
     __syncthreads();
     const int G = L >= 8 ? L / 8 : 1;
     const bool act = threadIdx.x < G;
-    fft_row<false, false, false, 1, 0>(S, L, logL, act ? (int)threadIdx.x : 0, tw, act);
+    fft_row<false, false, false, 1, -1>(S, L, logL, act ? (int)threadIdx.x : 0, tw, act);
     __syncthreads();
     for (int t = threadIdx.x; t < L; t += blockDim.x) F[base + t * stride] = S[pidx(t)];
 }
@@ -231,8 +231,6 @@ __global__ void __launch_bounds__(256) k_tensor_fixed(const double *K, long per_
     }
 }
 
-int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
-
 } // namespace
 
 // Newell octant on the device: N_dev [6][nz][ny][nx] doubles.
@@ -316,7 +314,7 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
             const size_t sm = sizeof(double2) * padded_row(L[a]);
             if (sm > 48 * 1024)
                 cudaFuncSetAttribute(k_fft_strided, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            k_fft_strided<<<(unsigned)rows[a], thr, sm, s>>>(F, L[a], ilog2(L[a]), stride[a], inner[a],
+            k_fft_strided<<<(unsigned)rows[a], thr, sm, s>>>(F, L[a], pow2_part(L[a]), stride[a], inner[a],
                                                              outer[a] ? outer[a] : 1, tws[a]);
         }
         if (!g.bulk) {
