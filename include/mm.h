@@ -72,13 +72,12 @@ typedef enum {
 /* Element type and arithmetic of the field path.  MM_FP64: double fields,
  * local terms, step and sums; the FFTs and the demagnetisation convolution run
  * in 64-bit block fixed point on the integer pipes, with a smaller error than
- * the same transforms in double.  MM_F32X2 (an extension):
- * the caller's arrays are double as for MM_FP64; inside, the iterates, the
- * FFTs, the demagnetisation convolution, the local terms, the step and the
- * per-CTA sums use double-float arithmetic (pairs of floats, about 48
- * significant bits, run on the FP32 pipes), and the sums across CTAs,
- * the step size and the stop rule are double; film-layout grids only (see
- * mm_setup_geometry). */
+ * the same transforms in double.  MM_F32X2 (an extension): the caller's arrays
+ * are double as for MM_FP64; inside, the iterates, the local terms, the step
+ * and the per-CTA sums use double-float arithmetic (pairs of floats, about 48
+ * significant bits, run on the FP32 pipes), the FFTs and the convolution the
+ * block fixed point of MM_FP64, and the sums across CTAs, the step size and
+ * the stop rule are double; film-layout grids only (see mm_setup_geometry). */
 enum { MM_FP64 = 0, MM_FP32 = 1, MM_F32X2 = 2 };
 enum { MM_STEP_CAYLEY = 0, MM_STEP_NORMALIZE = 1 };  /* update rule, see mm_min_opts */
 enum { MM_TAU_ALTERNATE = 0, MM_TAU_ADAPTIVE = 1 };  /* step-size rule, see mm_min_opts */
@@ -143,7 +142,7 @@ MM_API int mm_newell_static(const mm_grid *grid, double *N_dev, void *stream);
  * mm_setup_geometry -- create a problem: validates the grid and material,
  * allocates device workspaces, computes the Newell tensor (as mm_newell), its
  * Fourier spectrum on the zero-padded grid (padded size per axis: the power of
- * two P >= 2n-1 (and >= 2 along x) or, in MM_FP64 and MM_FP32, a shorter length
+ * two P >= 2n-1 (and >= 2 along x) or a shorter length
  * >= 2n-1: 5/8 or 3/4 of P = 512 or 1024 along x and along y of films, 5/8, 3/4
  * or 25/32 of P = 128 .. 1024 along y and z of bulk grids), times the admissible launch
  * shapes of the field kernels on this problem and keeps the fastest, and

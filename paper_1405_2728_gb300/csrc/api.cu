@@ -219,8 +219,7 @@ int plan(mm_problem *p)
             return MM_ERR_UNSUPPORTED;
     }
     // films keep their few layers' power of two: the z direction is a direct convolution
-    if (p->precision != MM_F32X2)
-        lengths(padded_length(gr.nx, false), padded_length(gr.ny, !film), film ? P2[2] : padded_length(gr.nz, true));
+    lengths(padded_length(gr.nx, false), padded_length(gr.ny, !film), film ? P2[2] : padded_length(gr.nz, true));
     if (film) {
         // film layout: y rows per batch in the y-z kernel, divisors of 3 nz
         // with RB*Gy threads within the kernel's bound
@@ -433,7 +432,7 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
             (g.bulk && (rc = dalloc(p, &p->W2, (size_t)g.C * 3 * g.nz * g.Py * vsz))) ||
             (rc = dalloc(p, &p->tw_px, g.Px * vsz)) || (rc = dalloc(p, &p->tw_py, g.Py * vsz)) ||
             (rc = dalloc(p, &p->tw_pz, g.Pz * vsz)) ||
-            (precision == MM_FP64 && (rc = dalloc(p, (void **)&p->fexp, sizeof(int) * mm_scale_count(g)))) ||
+            (precision != MM_FP32 && (rc = dalloc(p, (void **)&p->fexp, sizeof(int) * mm_scale_count(g)))) ||
             (rc = dalloc(p, (void **)&p->partials, sizeof(double) * RED_NSLOT * (size_t)p->nblk_x)) ||
             (rc = dalloc(p, (void **)&p->st, sizeof(MinState))) ||
             (rc = dalloc(p, (void **)&p->counter, 64)) ||

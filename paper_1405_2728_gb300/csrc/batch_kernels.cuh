@@ -14,7 +14,7 @@ template <typename T> using FA = typename fft_of<T>::type;
 template <typename T, int PZ, int L>
 __device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int tid, int nth, int kx)
 {
-    if constexpr (!is_fx<FA<T>>) yz_body<T, FA<T>, PZ, L>(g, P, tid, nth, kx);
+    if constexpr (!is_fx<FA<T>>) yz_body<PZ, L>(g, P, tid, nth, kx);
     else if constexpr (L == 0) yz_body_fx<PZ, 0>(g, P, tid, nth, kx);
 }
 

@@ -19,16 +19,15 @@
 template <typename T> struct cvec;
 template <> struct cvec<double> { typedef double2 type; };
 template <> struct cvec<float> { typedef float2 type; };
-template <> struct cvec<dfloat> { typedef dcomplex type; };
 template <> struct cvec<fx> { typedef fxc type; };
 // twiddle and tensor element of an FFT arithmetic
 template <typename F> struct twvec { typedef typename cvec<F>::type type; };
 template <> struct twvec<fx> { typedef fxmc type; };
 template <typename F> struct coef { typedef F type; };
 template <> struct coef<fx> { typedef fxm type; };
-// FFT arithmetic of a field type: double fields are convolved in block fixed point
-template <typename T> struct fft_of { typedef T type; };
-template <> struct fft_of<double> { typedef fx type; };
+// FFT arithmetic of a field type: double and double-word fields are convolved in block fixed point
+template <typename T> struct fft_of { typedef fx type; };
+template <> struct fft_of<float> { typedef float type; };
 
 template <typename V> __device__ __forceinline__ V cmake(decltype(V().x) a, decltype(V().x) b) { V r; r.x = a; r.y = b; return r; }
 template <typename V> __device__ __forceinline__ V cadd(V a, V b) { V r; r.x = a.x + b.x; r.y = a.y + b.y; return r; }
@@ -222,8 +221,8 @@ template <> struct io_of<dfloat> { typedef double type; };
 
 // T: element type of the minimiser's fields m and g and of the local terms
 // (double, float, or dfloat for MM_F32X2); F: arithmetic type of the FFTs and
-// the convolution, whose complex values fill the spectrum buffers and the
-// tensor; IO: the caller's element type (m for MODE_HEFF/ENERGY, H, per-cell
+// the convolution (float, or fx for the other two), whose complex values fill
+// the spectrum buffers; IO: the caller's element type (m for MODE_HEFF/ENERGY, H, per-cell
 // material)
 template <typename T, typename F = typename fft_of<T>::type>
 struct FieldPtrs {
@@ -338,7 +337,7 @@ MM_DECLARE_FIELD_ENTRIES(f32x2)
 inline int mm_film_coefs(const Geom &g, int precision)
 {
     const int nzm = g.Pz > 1 ? g.Pz / 2 : 1;
-    if (precision != MM_FP64) return 6 * nzm;
+    if (precision == MM_FP32) return 6 * nzm;
     return nzm == 1 ? 4 : (nzm == 2 ? 10 : 32);
 }
 
@@ -369,6 +368,10 @@ int mm_launch_convert(mm_problem *p, void *dst, const double *src, long n, cudaS
 int mm_launch_iterate_in(mm_problem *p, void *dst, const double *src, long n, cudaStream_t s);
 int mm_launch_iterate_out(mm_problem *p, double *dst, const void *src, long n, cudaStream_t s);
 int mm_rebuild_graph(mm_problem *p);
+// implemented in yz_fixed.cu: the film y-z kernel in block fixed point, which
+// does not depend on the field type
+cudaError_t mm_yz_fixed(const Geom &g, const FieldPtrs<double, fx> &P, cudaStream_t s);
+cudaError_t mm_yz_fixed_configure(const Geom &g, size_t smem);
 // implemented in bulk.cu: the three y-z passes of the bulk layout (pass -1:
 // all three in order; 0, 1, 2: only that one)
 cudaError_t mm_bulk_conv(const Geom &g, const FieldPtrs<double> &P, cudaStream_t s, int pass);

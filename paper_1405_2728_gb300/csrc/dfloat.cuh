@@ -1,5 +1,5 @@
 // Double-float ("double-word") arithmetic of the MM_F32X2 precision (its
-// fields, FFTs, convolution and local terms): a value is the unevaluated sum hi + lo of two
+// fields, step and local terms): a value is the unevaluated sum hi + lo of two
 // floats with |lo| <= ulp(hi)/2, about 48 significant bits, computed on the
 // FP32 pipes (64 times the FP64 FMA rate on this GPU).
 //
@@ -7,8 +7,7 @@
 // Math. 18 (1971) 224) and the exact product with one FMA.  Addition is the
 // double-word sum that adds the two high parts exactly, the low parts with
 // one rounding and renormalises ("SloppyDWPlusDW"); its error is a small
-// multiple of u^2 (|a| + |b|), u = 2^-24, which is the norm-wise bound an
-// FFT error analysis needs.  Multiplication is the double-word product with
+// multiple of u^2 (|a| + |b|), u = 2^-24, a norm-wise bound.  Multiplication is the double-word product with
 // FMA ("DWTimesDW"), relative error a small multiple of u^2.  Both are
 // analysed by Joldes, Muller and Popescu, ACM Trans. Math. Softw. 44 (2017)
 // 15.  Intrinsics with explicit rounding keep the compiler from contracting
@@ -17,8 +16,8 @@
 
 #include <cuda_runtime.h>
 
-// aligned like float2 / float4, so that loads and stores of a value (or a
-// complex value) are single vector accesses in shared and global memory
+// aligned like float2, so that loads and stores of a value are single vector
+// accesses in shared and global memory
 struct __align__(8) dfloat {
     float hi, lo;
     dfloat() = default;
@@ -26,10 +25,6 @@ struct __align__(8) dfloat {
     // nearest double-word of a double (hi = rounded value, lo = rounded remainder)
     __host__ __device__ constexpr dfloat(double d) : hi((float)d), lo((float)(d - (double)(float)d)) {}
     __host__ __device__ constexpr dfloat(int i) : hi((float)i), lo(0.0f) {}
-};
-
-struct __align__(16) dcomplex {
-    dfloat x, y;
 };
 
 #ifdef __CUDACC__

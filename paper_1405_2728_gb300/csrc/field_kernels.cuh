@@ -20,17 +20,7 @@ template <> __device__ __forceinline__ dfloat ldg(const dfloat *p)
 }
 // complex loads through the read-only path (ld_nc) or cached in L2 only (ld_cg)
 template <typename V> __device__ __forceinline__ V ld_nc(const V *p) { return __ldg(p); }
-template <> __device__ __forceinline__ dcomplex ld_nc(const dcomplex *p)
-{
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-    return dcomplex{dfloat(v.x, v.y), dfloat(v.z, v.w)};
-}
 template <typename V> __device__ __forceinline__ V ld_cg(const V *p) { return __ldcg(p); }
-template <> __device__ __forceinline__ dcomplex ld_cg(const dcomplex *p)
-{
-    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
-    return dcomplex{dfloat(v.x, v.y), dfloat(v.z, v.w)};
-}
 template <> __device__ __forceinline__ fxc ld_nc(const fxc *p)
 {
     const longlong2 v = __ldg(reinterpret_cast<const longlong2 *>(p));
@@ -44,7 +34,6 @@ template <> __device__ __forceinline__ fxc ld_cg(const fxc *p)
 template <typename F> constexpr bool is_fx = std::is_same<F, fx>::value;
 // a value of the FFT arithmetic F read back in the field type T
 template <typename T, typename F> __device__ __forceinline__ T to_field(F v) { return (T)v; }
-template <> __device__ __forceinline__ double to_field<double, dfloat>(dfloat v) { return df_to_double(v); }
 // a caller's value (double for double-word fields) in the field type T, and back
 template <typename T> __device__ __forceinline__ T from_io(typename io_of<T>::type v) { return (T)v; }
 template <typename T> __device__ __forceinline__ typename io_of<T>::type to_io(T v) { return v; }
@@ -56,6 +45,11 @@ template <> __device__ __forceinline__ dfloat inv_sqrt<dfloat>(dfloat x) { retur
 // reciprocal square root, ~2 ulp; double-word: one Newton step, ~2^-47)
 __device__ __forceinline__ float renorm_scale(float s) { return rsqrtf(s); }
 __device__ __forceinline__ dfloat renorm_scale(dfloat s) { return df_rsqrt(s); }
+
+// ordered bits of |x|'s high part, at or above those of infinity if x is not finite
+__device__ __forceinline__ int magnitude(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int magnitude(dfloat x) { return __float_as_int(x.hi) & 0x7fffffff; }
+__device__ __forceinline__ int magnitude(float) { return 0; }   // floats keep their own scale
 
 // real element x of a padded complex row holding Px reals
 template <typename T, typename V> __device__ __forceinline__ T &rel(V *row, int x)
@@ -183,11 +177,11 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             }
         }
         if constexpr (is_fx<F>) {  // as they are, until the tile's scale is known
-            max_xy = max(max_xy, max(__double2hiint(m0) & 0x7fffffff, __double2hiint(m1) & 0x7fffffff));
-            max_z = max(max_z, __double2hiint(m2) & 0x7fffffff);
-            rel<double>(S + (0 * TY + yl) * g.rsx, x) = m0;
-            rel<double>(S + (1 * TY + yl) * g.rsx, x) = m1;
-            rel<double>(S + (2 * TY + yl) * g.rsx, x) = m2;
+            max_xy = max(max_xy, max(magnitude(m0), magnitude(m1)));
+            max_z = max(max_z, magnitude(m2));
+            rel<T>(S + (0 * TY + yl) * g.rsx, x) = m0;
+            rel<T>(S + (1 * TY + yl) * g.rsx, x) = m1;
+            rel<T>(S + (2 * TY + yl) * g.rsx, x) = m2;
         } else {
             rel<F>(S + (0 * TY + yl) * g.rsx, x) = F(m0);
             rel<F>(S + (1 * TY + yl) * g.rsx, x) = F(m1);
@@ -201,18 +195,27 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         fx_cta_max(&s_max[0], max_xy);
         fx_cta_max(&s_max[1], max_z);
         __syncthreads();
-        const int inf = 0x7ff00000;
+        constexpr bool DW = std::is_same<T, dfloat>::value;
+        constexpr int inf = DW ? 0x7f800000 : 0x7ff00000, mant = DW ? 23 : 20, bias = DW ? 126 : 1022;
         const bool bad_xy = s_max[0] >= inf, bad_z = s_max[1] >= inf;
         const int top = max(bad_xy ? 0 : s_max[0], bad_z ? 0 : s_max[1]);
-        const int sc = min(58 - (((top - 0x1000) >> 20) - 1022), 1000);
+        const int top_e = ((top - (1 << (mant - 8))) >> mant) - bias, sc = min(58 - top_e, DW ? 150 : 1000);
         e1 = fx_pack(top > 0 ? -sc - 1 : FX_ZERO, (bad_xy ? 1 : 0) | (bad_z ? 2 : 0));
-        const double scale = top > 0 ? fx_pow2(sc) : 0.0;
+        double scale = 0.0;
+        float scalef = 0.0f;
+        if constexpr (DW) scalef = top > 0 ? fx_pow2f(sc - 28) : 0.0f;
+        else scale = top > 0 ? fx_pow2(sc) : 0.0;
         for (int e = tt; e < TY * nx; e += nth) {  // the elements this thread stored
             const int yl = g.fd_nx.div(e), x = e - yl * nx;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                fx &q = rel<F>(S + (c * TY + yl) * g.rsx, x);
-                q.v = (c < 2 ? bad_xy : bad_z) ? 0 : __double2ll_rn(__longlong_as_double(q.v) * scale);
+                const T a = rel<T>(S + (c * TY + yl) * g.rsx, x);
+                fx q(0);
+                if (!(c < 2 ? bad_xy : bad_z)) {
+                    if constexpr (DW) q = fx_from(a, scalef);
+                    else q = fx(__double2ll_rn(a * scale));
+                }
+                rel<fx>(S + (c * TY + yl) * g.rsx, x) = q;
             }
         }
     }
@@ -283,8 +286,8 @@ __global__ void __launch_bounds__(768) k_xfwd(Geom g, FieldPtrs<T, F> P)
 // ---------------------------------------------------------------------------
 // k_yz
 // ---------------------------------------------------------------------------
-// the double kernel runs fewer, fatter threads (its z-phase keeps ~100
-// doubles live); the y rows are then transformed in batches of RB rows
+// The fixed-point kernel runs fewer, fatter threads; the y rows are then
+// transformed in batches of RB rows.
 template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ? 512 : 768; };
 
 // Block fixed point: the z convolution of one (kx, ky), NZM layers, both
@@ -518,30 +521,23 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     if (tid == 0) P.fe2[kx] = fx_pack(e, (nz == 1 || !flags) ? flags : 3);
 }
 
-template <typename T, typename F, int PZ, int LY>
-__device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<T, F> &P, const int tid, const int nth,
+template <int PZ, int LY>
+__device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<float> &P, const int tid, const int nth,
                                         const int kx)
 {
-    typedef typename cvec<F>::type V;
+    typedef float F;
+    typedef float2 V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int ny = g.ny, nz = g.nz, Py = g.Py;
     const int nrow = 3 * nz;
     V *Wk = P.W + (long)kx * nrow * ny;
-    // Py twiddles: a shared copy in float; the double kernel reads them from
-    // global memory (L1), which keeps its shared memory within two CTAs per SM
-    const V *tw;
-    if constexpr (sizeof(V) == 8) {
-        V *tws = S + nrow * g.rsy;
-        for (int i = tt; i < Py; i += nth) cp_async8(tws + i, P.tw_py + i);
-        tw = tws;
-    } else {
-        tw = P.tw_py;
-    }
+    V *tw = S + nrow * g.rsy;
+    for (int i = tt; i < Py; i += nth) cp_async8(tw + i, P.tw_py + i);
 
     // Wk[z][y][c] -> row (c, z); PF loads per thread in flight before use
-    constexpr int PF = sizeof(V) == 8 ? 8 : 4;
+    constexpr int PF = 8;
     const int tot = nrow * ny;
     for (int e0 = tt; e0 < tot; e0 += PF * nth) {
         V v[PF];
@@ -637,11 +633,16 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<T, F> &P,
     }
 }
 
-template <typename T, typename F, int PZ, int LY>
-__global__ void __launch_bounds__(YZBound<T>::v, 1) k_yz(Geom g, FieldPtrs<T, F> P)
+template <int PZ, int LY>
+__global__ void __launch_bounds__(YZBound<float>::v, 1) k_yz(Geom g, FieldPtrs<float> P)
 {
-    if constexpr (is_fx<F>) yz_body_fx<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
-    else yz_body<T, F, PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
+    yz_body<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
+}
+
+template <int PZ, int LY>
+__global__ void __launch_bounds__(YZBound<double>::v, 1) k_yz_fx(Geom g, FieldPtrs<double, fx> P)
+{
+    yz_body_fx<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -998,10 +999,13 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             fft_row<true, false, true, 2, LX>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act);
         }
     }
+    constexpr bool DW = std::is_same<T, dfloat>::value;
     double dscale = 0.0;   // block fixed point: one unit of the rows' values, in A/m
+    float dscalef = 0.0f;
     int bad = 0;
     if constexpr (is_fx<F>) {
-        dscale = fx_pow2(emax);
+        if constexpr (DW) dscalef = fx_pow2f(emax);
+        else dscale = fx_pow2(emax);
         bad = (int)s_r[0];
     }
     cp_async_wait_all();
@@ -1033,11 +1037,21 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         const long n = ((long)z * ny + y) * nx + x;
         T d0, d1, d2;
         if constexpr (is_fx<F>) {
-            d0 = __ll2double_rn(rel<F>(S + (0 * TY + yl) * g.rsx, x).v) * dscale;
-            d1 = __ll2double_rn(rel<F>(S + (1 * TY + yl) * g.rsx, x).v) * dscale;
-            d2 = __ll2double_rn(rel<F>(S + (2 * TY + yl) * g.rsx, x).v) * dscale;
+            const fx q0 = rel<F>(S + (0 * TY + yl) * g.rsx, x), q1 = rel<F>(S + (1 * TY + yl) * g.rsx, x),
+                     q2 = rel<F>(S + (2 * TY + yl) * g.rsx, x);
+            if constexpr (DW) {
+                d0 = fx_to_dfloat(q0, dscalef);
+                d1 = fx_to_dfloat(q1, dscalef);
+                d2 = fx_to_dfloat(q2, dscalef);
+            } else {
+                d0 = __ll2double_rn(q0.v) * dscale;
+                d1 = __ll2double_rn(q1.v) * dscale;
+                d2 = __ll2double_rn(q2.v) * dscale;
+            }
             if (bad) {  // uniform over the CTA
-                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                T nan;
+                if constexpr (DW) nan = dfloat(__int_as_float(0x7fc00000), 0.0f);
+                else nan = __longlong_as_double(0x7ff8000000000000ll);
                 if (bad & 1) d0 = d1 = nan;
                 if (bad & 2) d2 = nan;
             }
@@ -1226,14 +1240,14 @@ template <typename T> int threads_x(const Geom &g) { return round32(3 * g.TY * g
 template <typename T> int threads_xf(const Geom &g) { return round32(3 * g.TYF * g.Gx); }
 template <typename T> size_t smem_xf_t(const Geom &g)
 {
-    typedef typename cvec<T>::type V;
+    typedef typename cvec<typename fft_of<T>::type>::type V;
     return (size_t)3 * g.TYF * g.rsx * sizeof(V) + (size_t)g.Px * sizeof(V);
 }
 template <typename T> int threads_yz(const Geom &g) { return round32(g.RB * g.Gy); }
 
 template <typename T> size_t smem_x_t(const Geom &g)
 {
-    typedef typename cvec<T>::type V;
+    typedef typename cvec<typename fft_of<T>::type>::type V;
     size_t rows = (size_t)3 * g.TY * g.rsx * sizeof(V) + (size_t)g.Px * sizeof(V);
     if (sizeof(T) == 4 && g.stage) rows = stage_offset<T>(g) + (size_t)(15 * g.TY + 6) * g.nx * sizeof(T);
     const size_t stage = (size_t)NSL * threads_x<T>(g) * sizeof(Acc<T>);
@@ -1241,7 +1255,7 @@ template <typename T> size_t smem_x_t(const Geom &g)
 }
 template <typename T> size_t smem_yz_t(const Geom &g)
 {
-    typedef typename cvec<T>::type V;
+    typedef typename cvec<typename fft_of<T>::type>::type V;
     // the float kernel also holds the Py twiddles (the double kernel reads them from global memory)
     // and the block fixed-point kernel two bytes per y-frequency
     return (size_t)3 * g.nz * g.rsy * sizeof(V) + (sizeof(T) == 4 ? (size_t)g.Py * sizeof(V) : 2 * (size_t)g.Py);
@@ -1250,22 +1264,13 @@ template <typename T> size_t smem_yz_t(const Geom &g)
 // The field kernels are compiled for a set of FFT row lengths (template
 // parameter LX of the x kernels, LY of the y-z kernel; MM_LX_CASES,
 // MM_LY_CASES) and once for any power of two (0); the launchers pick the
-// instance.
-// Double-word (F = dfloat) kernels are compiled for the lengths 512 and 1024
-// only (rows of films 257 .. 1024 cells long, and 129 .. 512 wide), other
-// lengths take the generic code: their unrolled double-word arithmetic makes
-// every compiled length expensive to build.
-template <typename F> constexpr bool lc_compiled(int L) { return true; }
-template <> constexpr bool lc_compiled<dfloat>(int L) { return L == 0 || L == 9 || L == 10; }
-template <typename F> __host__ __device__ inline int lx_of_f(int length)
+// instance (lx_of, ly_of).
+
+// the bytes a launch needs must fit the common cap, which every kernel is given
+template <typename K> cudaError_t smem_attr(K *f, size_t bytes)
 {
-    const int L = lx_of(length);
-    return lc_compiled<F>(L) ? L : 0;
-}
-template <typename F> __host__ __device__ inline int ly_of_f(int length)
-{
-    const int L = ly_of(length);
-    return lc_compiled<F>(L) ? L : 0;
+    if (bytes > (size_t)MM_SMEM_CAP) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP);
 }
 
 } // namespace

@@ -23,8 +23,8 @@ cudaError_t launch_xfwd(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
     const dim3 grid((g.ny + g.TYF - 1) / g.TYF, g.nz);
     const int thr = threads_xf<T>(g);
     const size_t sm = smem_xf_t<T>(g);
-    switch (lx_of_f<F>(g.Hx)) {
-#define C(L) case L: if constexpr (lc_compiled<F>(L)) k_xfwd<T, F, MIN, L><<<grid, thr, sm, s>>>(g, P); break;
+    switch (lx_of(g.Hx)) {
+#define C(L) case L: k_xfwd<T, F, MIN, L><<<grid, thr, sm, s>>>(g, P); break;
         MM_LX_CASES(C)
 #undef C
     default: return cudaErrorInvalidValue;
@@ -40,8 +40,8 @@ cudaError_t launch_xinv(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s,
     const int thr = threads_x<T>(g);
     const size_t sm = smem_x_t<T>(g);
     const double h0 = hext ? hext[0] : 0.0, h1 = hext ? hext[1] : 0.0, h2 = hext ? hext[2] : 0.0;
-    switch (lx_of_f<F>(g.Hx)) {
-#define C(L) case L: if constexpr (lc_compiled<F>(L)) k_xinv<T, F, MODE, L><<<grid, thr, sm, s>>>(g, P, h0, h1, h2, h, use_cond); break;
+    switch (lx_of(g.Hx)) {
+#define C(L) case L: k_xinv<T, F, MODE, L><<<grid, thr, sm, s>>>(g, P, h0, h1, h2, h, use_cond); break;
         MM_LX_CASES(C)
 #undef C
     default: return cudaErrorInvalidValue;
@@ -49,11 +49,12 @@ cudaError_t launch_xinv(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s,
     return cudaGetLastError();
 }
 
-template <typename T, typename F, int PZ>
-cudaError_t launch_yz(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
+// the film y-z kernel: float, or block fixed point (yz_fixed.cu), whose
+// buffers and scales do not depend on the field type
+template <int PZ> cudaError_t launch_yz(const Geom &g, const FieldPtrs<float> &P, cudaStream_t s)
 {
-    switch (ly_of_f<F>(g.Py)) {
-#define C(L) case L: if constexpr (lc_compiled<F>(L)) k_yz<T, F, PZ, L><<<g.C, threads_yz<T>(g), smem_yz_t<T>(g), s>>>(g, P); break;
+    switch (ly_of(g.Py)) {
+#define C(L) case L: k_yz<PZ, L><<<g.C, threads_yz<float>(g), smem_yz_t<float>(g), s>>>(g, P); break;
         MM_LY_CASES(C)
 #undef C
     default: return cudaErrorInvalidValue;
@@ -64,18 +65,26 @@ cudaError_t launch_yz(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
 template <typename T, typename F>
 cudaError_t launch_yz_any(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
 {
-    switch (g.Pz) {
-    case 1: return launch_yz<T, F, 1>(g, P, s);
-    case 4: return launch_yz<T, F, 4>(g, P, s);
-    case 8: return launch_yz<T, F, 8>(g, P, s);
-    default: return cudaErrorInvalidValue;  // Pz = 2 does not occur (nz = 1 gives 1, nz = 2 gives 4)
+    if constexpr (is_fx<F>) {
+        FieldPtrs<double, fx> Q;
+        memset((void *)&Q, 0, sizeof Q);
+        Q.W = P.W; Q.Nhat = P.Nhat; Q.tw_py = P.tw_py;
+        Q.fe1 = P.fe1; Q.fe2 = P.fe2; Q.fek = P.fek;
+        return mm_yz_fixed(g, Q, s);
+    } else {
+        switch (g.Pz) {
+        case 1: return launch_yz<1>(g, P, s);
+        case 4: return launch_yz<4>(g, P, s);
+        case 8: return launch_yz<8>(g, P, s);
+        default: return cudaErrorInvalidValue;  // Pz = 2 does not occur (nz = 1 gives 1, nz = 2 gives 4)
+        }
     }
 }
 
 // the bulk layout's passes exist for double and float (double-word problems
 // are film-layout only: the planner refuses bulk grids for them)
 template <typename T, typename F>
-constexpr bool has_bulk = !std::is_same<F, dfloat>::value;
+constexpr bool has_bulk = !std::is_same<T, dfloat>::value;
 
 // the y-z stage: the film kernel, or the three passes of the bulk layout
 template <typename T, typename F>
@@ -87,44 +96,38 @@ cudaError_t launch_conv(const Geom &g, const FieldPtrs<T, F> &P, cudaStream_t s)
     return launch_yz_any<T, F>(g, P, s);
 }
 
-// the bytes a launch needs must fit the common cap, which every kernel is given
-template <typename K> cudaError_t smem_attr(K *f, size_t bytes)
-{
-    if (bytes > (size_t)MM_SMEM_CAP) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP);
-}
-
 // dynamic shared memory limits of the instances this geometry launches
 template <typename T, typename F> cudaError_t configure_t(const Geom &g, size_t sxf, size_t sx, size_t syz)
 {
     cudaError_t e = cudaSuccess;
-    switch (lx_of_f<F>(g.Hx)) {
+    switch (lx_of(g.Hx)) {
 #define C(L)                                                                                     \
     case L:                                                                                      \
-        if constexpr (lc_compiled<F>(L)) {                                                       \
-            if ((e = smem_attr(k_xfwd<T, F, false, L>, sxf)) || (e = smem_attr(k_xfwd<T, F, true, L>, sxf)) || \
-                (e = smem_attr(k_xinv<T, F, MODE_HEFF, L>, sx)) || (e = smem_attr(k_xinv<T, F, MODE_ENERGY, L>, sx)) || \
-                (e = smem_attr(k_xinv<T, F, MODE_MIN, L>, sx)))                                     \
-                return e;                                                                        \
-        }                                                                                        \
+        if ((e = smem_attr(k_xfwd<T, F, false, L>, sxf)) || (e = smem_attr(k_xfwd<T, F, true, L>, sxf)) || \
+            (e = smem_attr(k_xinv<T, F, MODE_HEFF, L>, sx)) || (e = smem_attr(k_xinv<T, F, MODE_ENERGY, L>, sx)) || \
+            (e = smem_attr(k_xinv<T, F, MODE_MIN, L>, sx)))                                      \
+            return e;                                                                            \
         break;
         MM_LX_CASES(C)
 #undef C
+    default: return cudaErrorInvalidValue;
     }
     if (g.bulk) return cudaSuccess;
-    switch (ly_of_f<F>(g.Py)) {
+    if constexpr (is_fx<F>) {
+        return mm_yz_fixed_configure(g, syz);
+    } else {
+        switch (ly_of(g.Py)) {
 #define C(L)                                                                                     \
     case L:                                                                                      \
-        if constexpr (lc_compiled<F>(L)) {                                                       \
-            if (g.Pz == 1) return smem_attr(k_yz<T, F, 1, L>, syz);                              \
-            if (g.Pz == 4) return smem_attr(k_yz<T, F, 4, L>, syz);                              \
-            if (g.Pz == 8) return smem_attr(k_yz<T, F, 8, L>, syz);                              \
-        }                                                                                        \
+        if (g.Pz == 1) return smem_attr(k_yz<1, L>, syz);                                        \
+        if (g.Pz == 4) return smem_attr(k_yz<4, L>, syz);                                        \
+        if (g.Pz == 8) return smem_attr(k_yz<8, L>, syz);                                        \
         return cudaErrorInvalidValue;
-        MM_LY_CASES(C)
+            MM_LY_CASES(C)
 #undef C
+        }
+        return cudaErrorInvalidValue;
     }
-    return cudaErrorInvalidValue;
 }
 
 // Launch-shape autotuner: time every admissible rows-per-tile of the

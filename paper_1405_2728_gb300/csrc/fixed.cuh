@@ -1,4 +1,4 @@
-// Block fixed-point arithmetic of the MM_FP64 convolution: 64-bit integers
+// Block fixed-point arithmetic of the MM_FP64 and MM_F32X2 convolution: 64-bit integers
 // with one power-of-two scale per block of values (a tile of rows, an
 // x-frequency), run on the integer pipes.
 //
@@ -54,6 +54,17 @@ __host__ __device__ constexpr fxm fx_multiplier(long long q)
 }
 
 #ifdef __CUDACC__
+// double-word value * 2^s, s = 58 - E, for |hi| <= (1 + 2^-8) 2^E, on the FP32
+// pipes (f = 2^(30 - E)): the high part to 2^-28 of its integer unit exactly,
+// the low part (at most 2^34 units) to a multiple of 16 units
+__device__ __forceinline__ fx fx_from(dfloat a, float f)
+{
+    const float h = __fmul_rn(a.hi, f);
+    const int i = __float2int_rn(h);
+    const float rest = __fmul_rn(__fsub_rn(h, (float)i), 268435456.0f);                 // 2^28
+    const float low = __fmul_rn(__fmul_rn(a.lo, f), 16777216.0f);                       // 2^24
+    return fx(((long long)i << 28) + __float2int_rn(rest) + ((long long)__float2int_rn(low) << 4));
+}
 __device__ __forceinline__ fx operator+(fx a, fx b) { return fx(a.v + b.v); }
 __device__ __forceinline__ fx operator-(fx a, fx b) { return fx(a.v - b.v); }
 __device__ __forceinline__ fx operator-(fx a) { return fx(-a.v); }
@@ -172,6 +183,16 @@ __device__ __forceinline__ unsigned fx_mag(fx a)
     return (unsigned)(h ^ (h >> 31));
 }
 __device__ __forceinline__ unsigned fx_mag(fxc a) { return fx_mag(a.x) | fx_mag(a.y); }
+// v * f as a double-word, f a power of two: the high word's leading 24 bits,
+// then what they leave with the low word
+__device__ __forceinline__ dfloat fx_to_dfloat(fx a, float f)
+{
+    const int h = fx_hi(a);
+    const float top = (float)h;
+    const float rest = fmaf((float)(h - (int)top), 4294967296.0f, (float)fx_lo(a));     // 2^32
+    return df_fast2sum(__fmul_rn(__fmul_rn(top, 65536.0f), __fmul_rn(f, 65536.0f)), __fmul_rn(rest, f));
+}
+
 // OR (or maximum, or sum) over the CTA into *dst in shared memory; a barrier makes it visible
 __device__ __forceinline__ void fx_cta_or(unsigned *dst, unsigned v)
 {
@@ -192,6 +213,10 @@ __device__ __forceinline__ void fx_cta_add(unsigned *dst, unsigned v)
 __device__ __forceinline__ int fx_log2_up(unsigned v) { return v > 1 ? 32 - __clz((int)(v - 1)) : 0; }
 __device__ __forceinline__ int fx_bits(unsigned mag) { return 64 - __clz((int)mag); }  // 32 + bits of mag
 
+__device__ __forceinline__ float fx_pow2f(int e)
+{
+    return e < -126 ? 0.0f : __int_as_float((min(e, 127) + 127) << 23);
+}
 // 2^e as a double, 0 below the smallest normal power
 __device__ __forceinline__ double fx_pow2(int e)
 {

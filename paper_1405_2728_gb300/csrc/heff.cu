@@ -88,16 +88,13 @@ __global__ void k_dfloat_to_double(double *dst, const dfloat *src, long n)
         dst[i] = df_to_double(src[i]);
 }
 
-template <typename T>
-__global__ void k_twiddle(typename cvec<T>::type *tw, int L)
+__global__ void k_twiddle(float2 *tw, int L)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L) return;
     double s, c;
     sincospi(2.0 * (double)t / (double)L, &s, &c);
-    typename cvec<T>::type w;
-    w.x = (T)c; w.y = (T)(-s);
-    tw[t] = w;
+    tw[t] = make_float2((float)c, (float)(-s));
 }
 
 // the same table as multipliers of the block fixed-point convolution
@@ -244,9 +241,8 @@ int mm_launch_twiddles(mm_problem *p, cudaStream_t s)
     void *dst[3] = {p->tw_px, p->tw_py, p->tw_pz};
     for (int i = 0; i < 3; ++i) {
         const int blocks = (L[i] + 255) / 256;
-        if (p->precision == MM_F32X2) k_twiddle<dfloat><<<blocks, 256, 0, s>>>((dcomplex *)dst[i], L[i]);
-        else if (p->precision == MM_FP64) k_twiddle_fx<<<blocks, 256, 0, s>>>((fxmc *)dst[i], L[i]);
-        else k_twiddle<float><<<blocks, 256, 0, s>>>((float2 *)dst[i], L[i]);
+        if (p->precision != MM_FP32) k_twiddle_fx<<<blocks, 256, 0, s>>>((fxmc *)dst[i], L[i]);
+        else k_twiddle<<<blocks, 256, 0, s>>>((float2 *)dst[i], L[i]);
     }
     cudaError_t e = cudaGetLastError();
     if (e) { mm_set_cuda_error(e, "k_twiddle"); return MM_ERR_CUDA; }

@@ -167,7 +167,7 @@ __global__ void k_extract_film(int c, int Px, int Py, int nz, int nzf, const dou
     }
 }
 
-// The tensor of the block fixed-point convolution (MM_FP64): one x-frequency
+// The tensor of the block fixed-point convolution: one x-frequency
 // per CTA, from doubles to integers in units of 2^(ek - 62).  ek is chosen so
 // that the magnitudes of the terms of any one output value sum to less than 1:
 // over the sources' components and, for films, z offsets (offset 0 once, the
@@ -298,7 +298,7 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
     if (fblocks > mm_sm_count() * 32L) fblocks = mm_sm_count() * 32L;
     // the transformed tensor in the field's precision; for the film layout of block fixed point in a work buffer
     void *K64 = p->Nhat;
-    if (p->precision == MM_FP64 && !g.bulk) {
+    if (p->precision != MM_FP32 && !g.bulk) {
         e = cudaMallocAsync(&K64, sizeof(double) * 6 * (size_t)fext, s);
         if (e) {
             cudaFreeAsync(F, s); cudaFreeAsync(tw, s);
@@ -319,10 +319,8 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
         }
         if (!g.bulk) {
             const double fscale = -g.Ms / ((double)g.Px * g.Py);
-            if (p->precision == MM_FP64)
+            if (p->precision != MM_FP32)
                 k_extract_film<double><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (double *)K64);
-            else if (p->precision == MM_F32X2)
-                k_extract_film<dfloat><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (dfloat *)p->Nhat);
             else
                 k_extract_film<float><<<(int)fblocks, 256, 0, s>>>(c, g.Px, g.Py, g.nz, nzf, F, fscale, (float *)p->Nhat);
         } else if (p->precision == MM_FP64) {
@@ -332,7 +330,7 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
         }
         e = cudaGetLastError();
     }
-    if (!e && p->precision == MM_FP64) {
+    if (!e && p->precision != MM_FP32) {
         const int hy = g.Py / 2;
         fxm *out = (fxm *)p->Nhat;
         int *ek = p->fexp + ((long)g.nz * g.ny + (long)g.C * (2 * g.nzb + g.nkb));

@@ -15,7 +15,7 @@ from gpu_cases import dev, make_pair, rel_l2
 
 pytestmark = pytest.mark.gpu
 CELL = (3.90625e-9, 3.90625e-9, 5e-9)
-# cells -> padded length: x, and y of films (double-word keeps powers of two); y and z of bulk grids
+# cells -> padded length: x, and y of films; y and z of bulk grids
 FILM = {128: 256, 129: 320, 160: 320, 161: 384, 192: 384, 193: 512, 257: 640, 320: 640, 384: 768, 385: 1024}
 BULK = {32: 64, 33: 80, 40: 80, 48: 96, 49: 128, 80: 160, 96: 192, 100: 200, 101: 256, 160: 320, 192: 384, 200: 400, 320: 640,
         384: 768, 400: 800}
@@ -41,13 +41,11 @@ BAR = {"MM_FP64": 2e-15, "MM_FP32": 3e-6, "MM_F32X2": 1e-13}
 @pytest.mark.parametrize("prec", ["MM_FP64", "MM_FP32", "MM_F32X2"])
 @pytest.mark.parametrize("n", sorted(FILM))
 def test_film_axes(mmlib, n, prec):
-    def want(n):
-        return FILM[n] if prec != "MM_F32X2" else 1 << (2 * n - 2).bit_length()
     err, info = demag_error(mmlib, (n, 5, 1 + n % 4), prec)
-    assert info["px"] == want(n) and info["bulk_layout"] == 0
+    assert info["px"] == FILM[n] and info["bulk_layout"] == 0
     assert err <= BAR[prec]
     err, info = demag_error(mmlib, (6, n, 1 + n % 3), prec)
-    assert info["py"] == want(n) and info["bulk_layout"] == 0
+    assert info["py"] == FILM[n] and info["bulk_layout"] == 0
     assert err <= BAR[prec]
 
 
