@@ -171,18 +171,17 @@ int plan(mm_problem *p)
     // what is supported, and in which layout, is decided on powers of two
     const int P2[3] = {next_pow2(2 * gr.nx - 1), next_pow2(2 * gr.ny - 1), next_pow2(2 * gr.nz - 1)};
     auto lengths = [&](int Px, int Py, int Pz) {
-        const int vsz = p->precision == MM_FP32 ? 8 : 16;  // bytes per complex element
         g.Px = Px < 2 ? 2 : Px; g.Py = Py; g.Pz = Pz;
         g.Hx = g.Px / 2; g.C = g.Hx + 1;
         g.lhx = pow2_part(g.Hx); g.lpy = pow2_part(g.Py); g.lpz = pow2_part(g.Pz);
         g.Gx = g.Hx >= 8 ? g.Hx / 8 : 1;
         g.Gy = g.Py >= 8 ? g.Py / 8 : 1;
         g.Gz = g.Pz >= 8 ? g.Pz / 8 : 1;
-        // shared-memory row strides: 16-byte rows pad one element per 8, float
-        // rows are XOR-swizzled within groups of 16 (fft.cuh)
-        g.rsx = row_stride(g.Hx, vsz);
-        g.rsy = row_stride(g.Py, vsz);
-        g.rsz = row_stride(g.Pz, vsz);
+        // shared-memory row strides (swizzled rows, fft.cuh)
+        const bool f = p->precision == MM_FP32;
+        g.rsx = f ? row_stride(g.Hx, 8) : row_stride_fx(g.Hx);
+        g.rsy = f ? row_stride(g.Py, 8) : row_stride_fx(g.Py);
+        g.rsz = f ? row_stride(g.Pz, 8) : row_stride_fx(g.Pz);
         g.fd_padx.init(g.Px - gr.nx > 0 ? g.Px - gr.nx : 1);
         g.fd_pady.init(g.Py - gr.ny > 0 ? g.Py - gr.ny : 1);
     };

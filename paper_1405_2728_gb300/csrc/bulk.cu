@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
     const int kx = blockIdx.x, z0 = blockIdx.y * ZB;
     const int zb = min(ZB, nz - z0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * ZB * rs);
-    load_twiddles_async(tw, P.tw_py, Py);
+    load_twiddles_async(tw, P.tw_py, Py, Py, tid, nth);
     int emax = FX_ZERO;
     unsigned mag = 0;
     const int *scales = nullptr;   // of the values read: one per (z, y) row of W, or per KB y-frequencies of W2
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
     const int kx = blockIdx.x, ky0 = blockIdx.y * KB;
     const int kb = min(KB, Py - ky0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * KB * rs);
-    load_twiddles_async(tw, P.tw_pz, Pz);
+    load_twiddles_async(tw, P.tw_pz, Pz, Pz, tid, nth);
     int emax = FX_ZERO;
     unsigned mag = 0;
     const int *scales = nullptr;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
     __syncthreads();
     const int Gz = g.Gz, RB = g.RBZ;
     const int rb = tid / Gz, j = tid - rb * Gz;
-    signed char *s_sc = reinterpret_cast<signed char *>(tw + Pz);  // [2][KB][Pz]: scale and top bit of a frequency
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));  // [2][KB][Pz]: scale and top bit of a frequency
     int pre = FX ? 59 - fx_bits(s_r[1]) : 0, sh = 0, top = FX_ZERO;
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
@@ -324,13 +324,13 @@ inline int round32(int n) { return (n + 31) & ~31; }
 template <typename T> size_t smem_y_t(const Geom &g, int zb)
 {
     typedef typename cvec<T>::type V;
-    return ((size_t)3 * zb * g.rsy + g.Py) * sizeof(V);
+    return ((size_t)3 * zb * g.rsy + tw_slots(g.Py)) * sizeof(V);
 }
 template <typename T> size_t smem_z_t(const Geom &g, int kb)
 {
     typedef typename cvec<T>::type V;
     // and two bytes per frequency of a block fixed-point transform
-    return ((size_t)3 * kb * g.rsz + g.Pz) * sizeof(V) + (sizeof(T) == 8 ? (size_t)2 * kb * g.Pz : 0);
+    return ((size_t)3 * kb * g.rsz + tw_slots(g.Pz)) * sizeof(V) + (sizeof(T) == 8 ? (size_t)2 * kb * g.Pz : 0);
 }
 
 template <typename T> cudaError_t bulk_conv_t(const Geom &g, const FieldPtrs<T> &P, cudaStream_t s, int pass)

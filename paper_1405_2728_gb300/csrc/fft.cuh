@@ -41,15 +41,23 @@ __host__ __device__ __forceinline__ int padded_row(int L) { return L + (L >> 3) 
 // first pass and the grouped stores of the later passes at 2 wavefronts
 // (L = 512, 4096).  It is a permutation of every aligned group of 16, so a
 // row of L elements needs only L slots, plus one between rows.
+// Block fixed-point rows (16-byte elements, 8 per wavefront) are swizzled
+// within aligned groups of 8 for the same reason, which leaves room for the
+// twiddles of the y-z kernel beside its rows: 12 rows of 512 and the table take
+// 108 KiB, two CTAs an SM.
 template <typename V> __host__ __device__ __forceinline__ int spos(int i)
 {
-    if constexpr (sizeof(V) == 8) return i ^ (((i >> 4) & 7) | (((i >> 6) & 1) << 3));
+    if constexpr (std::is_same<V, fxc>::value) return i ^ ((i >> 3) & 7);
+    else if constexpr (sizeof(V) == 8) return i ^ (((i >> 4) & 7) | (((i >> 6) & 1) << 3));
     else return i + (i >> 3);
 }
 __host__ __device__ __forceinline__ int row_stride(int L, int esz)
 {
     return esz == 8 ? (L <= 8 ? L : (L + 15) / 16 * 16) + 1 : padded_row(L);
 }
+
+// the same for block fixed-point rows
+__host__ __device__ __forceinline__ int row_stride_fx(int L) { return (L <= 8 ? L : (L + 7) / 8 * 8) + 1; }
 
 // L = 2^l (times an odd part): l
 __host__ __device__ constexpr int pow2_part(int L)
@@ -59,19 +67,32 @@ __host__ __device__ constexpr int pow2_part(int L)
     return l;
 }
 
-// copy a twiddle table of n complex values into shared memory (all threads)
-template <typename V> __device__ __forceinline__ void load_twiddles(V *dst, const V *src, int n)
+// Twiddle t of a table in shared memory lives at tpos(t, L), L the row length.
+// A pass reads multiples of L/(Ns R) r; unswizzled, the eight different ones of
+// a pass with Ns = 8 over a power of two lie 128 bytes apart, in one bank group
+// (512 x 256 x 4: FP32 y-z kernel 37 -> 32.5 us,
+// x-forward 20.7 -> 19.5 us).  Lengths with an odd part
+// spread by themselves.  Double tables (the tensor setup) stay in global
+// memory, in order.
+template <typename W> __host__ __device__ __forceinline__ int tpos(int t, int L)
 {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+    if constexpr (std::is_same<W, double2>::value) return t;
+    else if (L & (L - 1)) return t;
+    else if constexpr (std::is_same<W, fxmc>::value) return spos<fxc>(t);
+    else return spos<W>(t);
 }
 
-// the same, issued as asynchronous copies (8 or 16 bytes per element);
-// complete at cp_async_wait_all() of each thread, then a barrier
-template <typename V> __device__ __forceinline__ void load_twiddles_async(V *dst, const V *src, int n)
+// slots of such a table of n: whole swizzle groups
+__host__ __device__ constexpr int tw_slots(int n) { return n <= 16 ? n : (n + 15) / 16 * 16; }
+
+// copy a twiddle table of n complex values for rows of length L into shared memory (threads tid of
+// nth), issued as asynchronous copies (8 or 16 bytes per element); complete at cp_async_wait_all() of each thread, then a barrier
+template <typename W>
+__device__ __forceinline__ void load_twiddles_async(W *dst, const W *src, int n, int L, int tid, int nth)
 {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        if constexpr (sizeof(V) == 16) cp_async16(dst + i, src + i);
-        else cp_async8(dst + i, src + i);
+    for (int i = tid; i < n; i += nth) {
+        if constexpr (sizeof(W) == 16) cp_async16(dst + tpos<W>(i, L), src + i);
+        else cp_async8(dst + tpos<W>(i, L), src + i);
     }
 }
 
@@ -191,6 +212,8 @@ __device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G
 {
     constexpr int NB = (8 + R - 1) / R;
     V v[NB * R];
+#pragma unroll
+    for (int i = 0; i < NB * R; ++i) v[i] = czero<V>();
     const int LR = L / R, tstep0 = (L / (Ns * R)) * ts;
     if (active) {
 #pragma unroll
@@ -202,7 +225,7 @@ __device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G
             for (int r = 0; r < R; ++r) {
                 v[q * R + r] = row[spos<V>(b + r * LR)];
                 if (r > 0) {
-                    const V w = tw[r * step];
+                    const V w = tw[tpos<V>(r * step, L)];
                     v[q * R + r] = INV ? cmulc(v[q * R + r], w) : cmul(v[q * R + r], w);
                 }
             }
@@ -263,12 +286,17 @@ __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int 
                 int t = step;
 #pragma unroll
                 for (int r = 1; r < R; ++r, t += step) {
-                    const V w = tw[t];
+                    const V w = tw[tpos<V>(t, L)];
                     v[q * R + r] = INV ? cmulc(v[q * R + r], w) : cmul(v[q * R + r], w);
                 }
             }
             dftR<R, INV, HIN>(&v[q * R]);
         }
+    } else {
+        // (defined for idle threads too: in a loop over rows an undefined value would be carried round it, 32 registers
+        // and more a pass)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = czero<V>();
     }
     __syncthreads();
     if (active) {
@@ -465,17 +493,16 @@ __device__ __forceinline__ void stockham_pass_fx(fxc *row, int L, int Ns, int j,
     constexpr int NB = 8 / R;
     fxc v[8];
     const int LR = L / R;
-    const int ld9 = LR + (LR >> 3);
     const int tstep0 = (L / (Ns * R)) * ts;
     if (active) {
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
             const int b = j + q * G;
-            const int p0 = pidx(b);
+            const int p0 = spos<fxc>(b);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (HIN && r >= R / 2) { v[q * R + r] = czero<fxc>(); continue; }
-                v[q * R + r] = row[(LR & 7) ? pidx(b + r * LR) : p0 + r * ld9];
+                v[q * R + r] = row[(LR & 63) ? spos<fxc>(b + r * LR) : p0 + r * LR];
             }
             if (FIRST && VAR) {
 #pragma unroll
@@ -498,11 +525,14 @@ __device__ __forceinline__ void stockham_pass_fx(fxc *row, int L, int Ns, int j,
                 v[q * R].y = fx_shr(v[q * R].y, sh);
                 int t = step;
 #pragma unroll
-                for (int r = 1; r < R; ++r, t += step) v[q * R + r] = fx_cmul<INV>(v[q * R + r], tw[t], sh);
+                for (int r = 1; r < R; ++r, t += step) v[q * R + r] = fx_cmul<INV>(v[q * R + r], tw[tpos<fxmc>(t, L)], sh);
             }
             if constexpr (R == 8) dft8_fx<INV, HIN>(&v[q * R]);
             else dftR<R, INV, HIN>(&v[q * R]);
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = czero<fxc>();
     }
     __syncthreads();
     if (active) {
@@ -510,12 +540,11 @@ __device__ __forceinline__ void stockham_pass_fx(fxc *row, int L, int Ns, int j,
         for (int q = 0; q < NB; ++q) {
             const int b = j + q * G;
             const int k = b & (Ns - 1);
-            const int hi = (b - k) * R;
-            const int s0 = (R == 8) ? hi + (hi >> 3) + k + (k >> 3) : 0;
+            const int i0 = (b - k) * R + k, p0 = spos<fxc>(i0);
 #pragma unroll
             for (int r = 0; r < (HOUT ? R / 2 : R); ++r) {
                 const int rn = r * Ns;
-                row[(R == 8) ? s0 + rn + (rn >> 3) : pidx(hi + k + rn)] = v[q * R + r];
+                row[(Ns & 63) ? spos<fxc>(i0 + rn) : p0 + rn] = v[q * R + r];
                 if (MAG) mag |= fx_mag(v[q * R + r]);
             }
         }
@@ -560,6 +589,8 @@ __device__ __forceinline__ void stockham_odd_fx(fxc *row, int L, int Ns, int j, 
 {
     constexpr int NB = (8 + R - 1) / R;
     fxc v[NB * R];
+#pragma unroll
+    for (int i = 0; i < NB * R; ++i) v[i] = czero<fxc>();
     const int LR = L / R, tstep0 = (L / (Ns * R)) * ts;
     if (active) {
 #pragma unroll
@@ -569,8 +600,8 @@ __device__ __forceinline__ void stockham_odd_fx(fxc *row, int L, int Ns, int j, 
             const int step = tstep0 * (Ns == LR ? b : b & (Ns - 1));
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const fxc a = row[pidx(b + r * LR)];
-                v[q * R + r] = r ? fx_cmul<INV>(a, tw[r * step], sh) : fxc{fx_shr(a.x, sh), fx_shr(a.y, sh)};
+                const fxc a = row[spos<fxc>(b + r * LR)];
+                v[q * R + r] = r ? fx_cmul<INV>(a, tw[tpos<fxmc>(r * step, L)], sh) : fxc{fx_shr(a.x, sh), fx_shr(a.y, sh)};
             }
             if constexpr (R == 3) dft3_fx<INV>(&v[q * R]);
             else dft5_fx<INV>(&v[q * R]);
@@ -587,7 +618,7 @@ __device__ __forceinline__ void stockham_odd_fx(fxc *row, int L, int Ns, int j, 
             for (int r = 0; r < R; ++r) {
                 const int i = (b - k) * R + k + r * Ns;
                 if (!HOUT || 2 * i < L) {
-                    row[pidx(i)] = v[q * R + r];
+                    row[spos<fxc>(i)] = v[q * R + r];
                     if (MAG) mag |= fx_mag(v[q * R + r]);
                 }
             }

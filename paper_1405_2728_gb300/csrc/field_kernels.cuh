@@ -108,7 +108,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
     const int nx = g.nx, ny = g.ny, Px = g.Px;
     const long N = g.N;
     TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);  // Px twiddles exp(-2 pi i t / Px)
-    for (int i = tt; i < Px; i += nth) tw[i] = P.tw_px[i];
+    for (int i = tt; i < Px; i += nth) tw[tpos<TW>(i, g.Hx)] = P.tw_px[i];
     __shared__ int s_max[2];       // block fixed point: high words of the tile's largest |m_x|, |m_y| and |m_z|
     int max_xy = 0, max_z = 0;
     if constexpr (is_fx<F>) {
@@ -252,7 +252,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         const V Zk = row[spos<V>(k)];
         const V Zm = cconj(row[spos<V>(k == 0 ? 0 : Hx - k)]);
         if constexpr (is_fx<F>) {  // 2 X is stored: |Zk|, |Zm| < 2^60.5, so |2 X| < 2^62
-            const V sum = cadd(Zk, Zm), wd = fx_cmul<false>(csub(Zk, Zm), tw[k], 0);
+            const V sum = cadd(Zk, Zm), wd = fx_cmul<false>(csub(Zk, Zm), tw[tpos<TW>(k, g.Hx)], 0);
             if (y < ny) {
                 P.W[(((long)k * g.nz + z) * ny + y) * 3 + c] = V{sum.x + wd.y, sum.y - wd.x};
                 if (Hx - k != k)
@@ -261,7 +261,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             continue;
         } else {
         const V sum = cadd(Zk, Zm), dif = csub(Zk, Zm);
-        const V wd = cmul(tw[k], dif);
+        const V wd = cmul(tw[tpos<TW>(k, g.Hx)], dif);
         if (y < ny) {
             V X;
             X.x = F(0.5) * (sum.x + wd.y);
@@ -286,16 +286,22 @@ __global__ void __launch_bounds__(768) k_xfwd(Geom g, FieldPtrs<T, F> P)
 // ---------------------------------------------------------------------------
 // k_yz
 // ---------------------------------------------------------------------------
-// The fixed-point kernel runs fewer, fatter threads; the y rows are then
-// transformed in batches of RB rows.
-template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ? 512 : 768; };
+// The fixed-point kernel runs fewer, fatter threads (128 registers, two CTAs an
+// SM); the y rows are then transformed in batches of RB rows.  384 threads of
+// 80 registers took 156 us at 512 x 256 x 4 where 256 took 141: the z
+// convolution then keeps too few coefficients in flight.
+template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ? 256 : 768; };
 
-// Block fixed point: the z convolution of one (kx, ky), NZM layers, both
-// parts of three components.  The tensor is a Toeplitz matrix along z, even
-// (xx, yy, zz, xy) or odd (xz, yz, times i) in z - z', so with
-// up_j = m_j + m_{NZM-1-j} and um_j = m_j - m_{NZM-1-j} the sums S_i and
-// differences D_i of the outputs i and NZM-1-i come from half-size products:
-// 8 multiplications a component pair and part for 4 layers instead of 16
+// Block fixed point: the z convolution of one (kx, ky), NZM layers.  The
+// tensor's xz and yz transforms are imaginary, so with i m_z in the place of
+// m_z and -i H_z in that of H_z its matrix is real,
+//   [xx xy xz; xy yy yz; xz yz -zz],
+// and the real and the imaginary part are convolved apart, by two threads: half
+// the registers, which lets the kernel run 24 warps an SM instead of 16.
+// Along z the tensor is a Toeplitz matrix, even (xx, yy, zz, xy) or odd (xz,
+// yz) in z - z', so with up_j = m_j + m_{NZM-1-j} and um_j = m_j - m_{NZM-1-j} the
+// sums S_i and differences D_i of the outputs i and NZM-1-i come from half-size
+// products: 8 multiplications a component pair for 4 layers instead of 16
 // (even) or 12 (odd).  Outputs carry a factor 2 for NZM > 1.
 // The coefficients, combinations of the tensor at the z offsets K0 .. K3, are
 // stored [coefficient][ky], 4 NE + 2 NO of them (k_tensor_fixed):
@@ -305,27 +311,28 @@ template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ?
 template <int NZM> struct ZConv {
     static constexpr int H = NZM > 1 ? NZM / 2 : 1;
     static constexpr int NE = NZM == 1 ? 1 : (NZM == 2 ? 2 : 6), NO = NZM == 1 ? 0 : (NZM == 2 ? 1 : 4);
-    int2 up[3][H][2], um[3][H][2];   // split words, [component][j][part]
-    const fxm *K;                    // this (kx, ky)'s first coefficient
+    int2 up[3][H], um[3][H];   // split words, [component][j]
+    const fxm *K;              // this (kx, ky)'s first coefficient
     int kst;
 
-    __device__ __forceinline__ fxk coefficient(int i) const
-    {
-        const int2 w = __ldg(reinterpret_cast<const int2 *>(K + (long)i * kst));
-        return fxk(fxm{w.x, w.y});
-    }
-    // component e (xx, yy, zz, xy = 0 .. 3) from source b, into S_i (D false) or D_i
-    template <bool D> __device__ __forceinline__ void even(fxdot (&a)[2], int e, int b, int i) const
+    // n coefficients from the table's index `first`
+    template <int N> __device__ __forceinline__ void load(fxm (&k)[N], int first) const
     {
 #pragma unroll
-        for (int j = 0; j < H; ++j) {
-            const fxk w = coefficient(e * NE + (NZM == 1 ? 0 : (NZM == 2 ? D : (D ? 3 : 0) + i + j)));
-            a[0].mad(D ? um[b][j][0] : up[b][j][0], w);
-            a[1].mad(D ? um[b][j][1] : up[b][j][1], w);
+        for (int i = 0; i < N; ++i) {
+            const int2 w = __ldg(reinterpret_cast<const int2 *>(K + (long)(first + i) * kst));
+            k[i] = fxm{w.x, w.y};
         }
     }
-    // component o (xz, yz = 0, 1): times i
-    template <bool D> __device__ __forceinline__ void odd(fxdot (&a)[2], int o, int b, int i) const
+    // an even component's coefficients k from source b, into S_i (D false) or D_i
+    template <bool D> __device__ __forceinline__ void even(fxdot &a, const fxm (&k)[NE], bool neg, int b, int i) const
+    {
+#pragma unroll
+        for (int j = 0; j < H; ++j)
+            a.mad(D ? um[b][j] : up[b][j], fxk(fxk(k[NZM == 1 ? 0 : (NZM == 2 ? D : (D ? 3 : 0) + i + j)]), neg));
+    }
+    // an odd one's
+    template <bool D> __device__ __forceinline__ void odd(fxdot &a, const fxm (&k)[NO ? NO : 1], int b, int i) const
     {
         if constexpr (NZM > 1) {
 #pragma unroll
@@ -333,34 +340,45 @@ template <int NZM> struct ZConv {
                 // NZM = 4: rows (K3, -(K1-K2)), (K1+K2, K1) of S; (-K3, -(K1+K2)), (K1-K2, -K1) of D
                 const int at = NZM == 2 ? 0 : (i == j ? 3 * i : (D ? 1 + j : 2 - j));
                 const bool neg = NZM == 2 ? D : (D ? !(i == 1 && j == 0) : (i == 0 && j == 1));
-                const fxk w = coefficient(4 * NE + o * NO + at), p(w, neg), n(w, !neg);
-                a[0].mad(D ? up[b][j][1] : um[b][j][1], n);
-                a[1].mad(D ? up[b][j][0] : um[b][j][0], p);
+                a.mad(D ? up[b][j] : um[b][j], fxk(fxk(k[at]), neg));
             }
         }
     }
-    template <bool D> __device__ __forceinline__ fxc sum(int comp, int i) const
+    // outputs of component comp from two components of one parity and one of the other: store(layer, value).  Their
+    // coefficients are loaded together: the loads come from L2, and one at a time they would be waited for.
+    template <int COMP, typename St> __device__ __forceinline__ void output(St store) const
     {
-        fxdot t[2];
-        t[0].zero();
-        t[1].zero();
-        if (comp == 0) { even<D>(t, 0, 0, i); even<D>(t, 3, 1, i); odd<D>(t, 0, 2, i); }
-        if (comp == 1) { even<D>(t, 3, 0, i); even<D>(t, 1, 1, i); odd<D>(t, 1, 2, i); }
-        if (comp == 2) { odd<D>(t, 0, 0, i); odd<D>(t, 1, 1, i); even<D>(t, 2, 2, i); }
-        return fxc{t[0].value(), t[1].value()};
-    }
-    // output component comp: store(layer, value)
-    template <typename St> __device__ __forceinline__ void output(int comp, St store) const
-    {
+        constexpr int XZ = 4 * NE, YZ = 4 * NE + NO;
+        fxm e0[NE], e1[NE], o0[NO ? NO : 1], o1[NO ? NO : 1];
+        if constexpr (COMP == 0) { load(e0, 0); load(e1, 3 * NE); if constexpr (NO > 0) load(o0, XZ); }
+        if constexpr (COMP == 1) { load(e0, 3 * NE); load(e1, NE); if constexpr (NO > 0) load(o0, YZ); }
+        if constexpr (COMP == 2) { load(e0, 2 * NE); if constexpr (NO > 0) { load(o0, XZ); load(o1, YZ); } }
 #pragma unroll
         for (int i = 0; i < H; ++i) {
-            const fxc S = sum<false>(comp, i);
+            fx sd[2];
+#pragma unroll
+            for (int w = 0; w < (NZM > 1 ? 2 : 1); ++w) {
+                fxdot t;
+                t.zero();
+                auto add = [&](auto D) {
+                    if constexpr (COMP < 2) {
+                        even<D.value>(t, e0, false, 0, i);
+                        even<D.value>(t, e1, false, 1, i);
+                        odd<D.value>(t, o0, 2, i);
+                    } else {
+                        odd<D.value>(t, o0, 0, i);
+                        odd<D.value>(t, o1, 1, i);
+                        even<D.value>(t, e0, true, 2, i);
+                    }
+                };
+                if (w) add(std::true_type()); else add(std::false_type());
+                sd[w] = t.value();
+            }
             if constexpr (NZM == 1) {
-                store(0, S);
+                store(0, sd[0]);
             } else {
-                const fxc D = sum<true>(comp, i);
-                store(i, cadd(S, D));
-                store(NZM - 1 - i, csub(S, D));
+                store(i, sd[0] + sd[1]);
+                store(NZM - 1 - i, sd[0] - sd[1]);
             }
         }
     }
@@ -380,9 +398,10 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     __shared__ unsigned s_r[4];   // flags, magnitudes in and out, sum of the frequencies' scales over the largest
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int ny = g.ny, nz = g.nz, Py = g.Py, nrow = 3 * nz;
-    signed char *s_sc = reinterpret_cast<signed char *>(S + nrow * g.rsy);  // [2][Py]: scale and top bit of every ky
     fxc *Wk = P.W + (long)kx * nrow * ny;
-    const fxmc *tw = P.tw_py;
+    fxmc *tw = reinterpret_cast<fxmc *>(S + nrow * g.rsy);
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + Py);  // [2][Py]: scale and top bit of every ky
+    load_twiddles_async(tw, P.tw_py, Py, Py, tt, nth);
     if (tid == 0) { s_e = FX_ZERO; s_top = FX_ZERO; }
     if (tid < 4) s_r[tid] = 0;
     __syncthreads();
@@ -418,7 +437,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
             const int d = fx_exp(P.fe1[rest]) - emax;
             if (d) v[i] = fx_scale(v[i], d);
             mag |= fx_mag(v[i]);
-            S[(c * nz + zz) * g.rsy + pidx(y)] = v[i];
+            S[(c * nz + zz) * g.rsy + spos<fxc>(y)] = v[i];
         }
         e0 += PF * nth;
         if (e0 < tot) load(e0);
@@ -427,8 +446,9 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     const int npad = Py - ny;
     for (int e = tt; e < nrow * npad; e += nth) {
         const int row = g.fd_pady.div(e), y = ny + (e - row * npad);
-        S[row * g.rsy + pidx(y)] = czero<fxc>();
+        S[row * g.rsy + spos<fxc>(y)] = czero<fxc>();
     }
+    cp_async_wait_all();
     __syncthreads();
     const int rb = tid / g.Gy, j = tid - rb * g.Gy;  // row within a batch of g.RB rows
     const bool act = rb < g.RB;
@@ -444,54 +464,62 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     constexpr int NC = 4 * ZConv<NZM>::NE + 2 * ZConv<NZM>::NO;
     e += sh + P.fek[kx] - (NZM > 1 ? 1 : 0);
     int top = FX_ZERO;
-    for (int ky = tt; ky < Py; ky += nth) {
-        const int pky = pidx(ky), kyr = ky <= hy ? ky : Py - ky;
-        const bool flip = ky > hy;   // xy and yz are odd in ky: m_y and H_y change sign
+    for (int u = tt; u < 2 * Py; u += nth) {
+        // a pair of lanes per ky: part 0 the real parts (of m_x, m_y and i m_z), part 1 the imaginary ones
+        const int ky = u >> 1, part = u & 1, kyr = ky <= hy ? ky : Py - ky;
+        const int left = 2 * Py - (u & ~31);
+        const unsigned lanes = left >= 32 ? 0xffffffffu : (1u << left) - 1;
+        fx *col = &S[spos<fxc>(ky)].x;                 // this ky's column; rows are 2 g.rsy values apart
+        const int at[3] = {part, part, 1 - part};      // where the part lies in a component's complex value
+        const bool flip[3] = {false, ky > hy, part == 0};  // xy and yz are odd in ky; i m_z and -i H_z
         ZConv<NZM> z;
         z.K = P.Nhat + (long)kx * NC * kst + kyr;
         z.kst = kst;
         int sc;
         {
-            fxc m[3][NZM];
+            fx m[3][NZM];
             unsigned mk = 0;
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
-                    m[c][n] = n < nz ? S[(c * nz + n) * g.rsy + pky] : czero<fxc>();
+                    m[c][n] = n < nz ? col[2 * (c * nz + n) * g.rsy + at[c]] : fx(0);
                     mk |= fx_mag(m[c][n]);
                 }
+            mk |= __shfl_xor_sync(lanes, mk, 1);
             sc = 59 - fx_bits(mk);
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
                     m[c][n] = fx_scale(m[c][n], sc);
-                    if (c == 1 && flip) m[c][n] = fxc{-m[c][n].x, -m[c][n].y};
+                    if (flip[c]) m[c][n] = -m[c][n];
                 }
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int i = 0; i < ZConv<NZM>::H; ++i) {
-                    const fxc a = m[c][i], b = m[c][NZM - 1 - i];
-                    z.up[c][i][0] = fx_split(NZM > 1 ? a.x + b.x : a.x);
-                    z.up[c][i][1] = fx_split(NZM > 1 ? a.y + b.y : a.y);
-                    z.um[c][i][0] = fx_split(a.x - b.x);
-                    z.um[c][i][1] = fx_split(a.y - b.y);
+                    const fx a = m[c][i], b = m[c][NZM - 1 - i];
+                    z.up[c][i] = fx_split(NZM > 1 ? a + b : a);
+                    z.um[c][i] = fx_split(a - b);
                 }
         }
         mag = 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            z.output(c, [&](int n, fxc r) {
-                if (n >= nz) return;
-                if (c == 1 && flip) r = fxc{-r.x, -r.y};
-                mag |= fx_mag(r);
-                S[(c * nz + n) * g.rsy + pky] = r;
-            });
+        auto put = [&](int c, int n, fx r) {
+            if (n >= nz) return;
+            if (c == 1 ? flip[1] : (c == 2 && part == 1)) r = -r;
+            mag |= fx_mag(r);
+            col[2 * (c * nz + n) * g.rsy + at[c]] = r;
+        };
+        z.template output<0>([&](int n, fx r) { put(0, n, r); });
+        z.template output<1>([&](int n, fx r) { put(1, n, r); });
+        z.template output<2>([&](int n, fx r) { put(2, n, r); });
+        mag |= __shfl_xor_sync(lanes, mag, 1);
         const int tk = fx_bits(mag) - sc;  // values of this ky: stored * 2^-sc, below 2^tk
-        s_sc[ky] = (signed char)sc;
-        s_sc[Py + ky] = (signed char)tk;
+        if (part == 0) {
+            s_sc[ky] = (signed char)sc;
+            s_sc[Py + ky] = (signed char)tk;
+        }
         top = max(top, tk);
     }
     fx_cta_max(&s_top, top);
@@ -514,7 +542,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     e += sh - pre - post;
     for (int i = tt; i < tot; i += nth) {
         const int c = i % 3, rest = i / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + pidx(y)], post);
+        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], post);
     }
     // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
     const int flags = (int)s_r[0];
@@ -534,7 +562,7 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<float> &P
     const int nrow = 3 * nz;
     V *Wk = P.W + (long)kx * nrow * ny;
     V *tw = S + nrow * g.rsy;
-    for (int i = tt; i < Py; i += nth) cp_async8(tw + i, P.tw_py + i);
+    load_twiddles_async(tw, P.tw_py, Py, Py, tt, nth);
 
     // Wk[z][y][c] -> row (c, z); PF loads per thread in flight before use
     constexpr int PF = 8;
@@ -640,7 +668,7 @@ __global__ void __launch_bounds__(YZBound<float>::v, 1) k_yz(Geom g, FieldPtrs<f
 }
 
 template <int PZ, int LY>
-__global__ void __launch_bounds__(YZBound<double>::v, 1) k_yz_fx(Geom g, FieldPtrs<double, fx> P)
+__global__ void __launch_bounds__(YZBound<double>::v, 2) k_yz_fx(Geom g, FieldPtrs<double, fx> P)
 {
     yz_body_fx<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
 }
@@ -908,10 +936,7 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     const bool stg = sizeof(T) == 4 && MODE == MODE_MIN && g.stage;
     T *SG = reinterpret_cast<T *>(smem_raw + stage_offset<T>(g));
     const int oZm = 3 * (TY + 2) * nx, oZp = oZm + 3 * TY * nx, oMP = oZp + 3 * TY * nx, oGQ = oMP + 3 * TY * nx;
-    for (int i = tt; i < g.Px; i += nth) {
-        if constexpr (sizeof(V) == 16) cp_async16(tw + i, P.tw_px + i);
-        else cp_async8(tw + i, P.tw_px + i);
-    }
+    load_twiddles_async(tw, P.tw_px, g.Px, g.Hx, tt, nth);
     cp_async_commit();
     if (stg) {
         stage_rows(SG, m, g, z, y0 - 1, TY + 2, tid, nth);
@@ -970,8 +995,8 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             }
             const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
             V t;
-            if constexpr (is_fx<F>) t = fx_cmul<true>(dif, tw[kk], 0);
-            else t = cmulc(dif, tw[kk]);  // conj(w^k) dif
+            if constexpr (is_fx<F>) t = fx_cmul<true>(dif, tw[tpos<TW>(kk, g.Hx)], 0);
+            else t = cmulc(dif, tw[tpos<TW>(kk, g.Hx)]);  // conj(w^k) dif
             Z.x = sum.x - t.y;
             Z.y = sum.y + t.x;
             row[spos<V>(kk)] = Z;
@@ -1256,9 +1281,9 @@ template <typename T> size_t smem_x_t(const Geom &g)
 template <typename T> size_t smem_yz_t(const Geom &g)
 {
     typedef typename cvec<typename fft_of<T>::type>::type V;
-    // the float kernel also holds the Py twiddles (the double kernel reads them from global memory)
+    // rows and Py twiddles,
     // and the block fixed-point kernel two bytes per y-frequency
-    return (size_t)3 * g.nz * g.rsy * sizeof(V) + (sizeof(T) == 4 ? (size_t)g.Py * sizeof(V) : 2 * (size_t)g.Py);
+    return ((size_t)3 * g.nz * g.rsy + g.Py) * sizeof(V) + (sizeof(T) == 4 ? 0 : 2 * (size_t)g.Py);
 }
 
 // The field kernels are compiled for a set of FFT row lengths (template
