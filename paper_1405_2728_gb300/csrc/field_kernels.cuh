@@ -694,7 +694,7 @@ template <> struct Acc<double> {
     __device__ __forceinline__ void add(const Acc &o) { v += o.v; }
     __device__ __forceinline__ void maxv(double x) { v = fmax(v, x); }
     __device__ __forceinline__ void maxv(const Acc &o) { v = fmax(v, o.v); }
-    __device__ __forceinline__ Acc shfl_down(int o) const { Acc r; r.v = __shfl_down_sync(0xffffffffu, v, o); return r; }
+    __device__ __forceinline__ Acc shfl_xor(int o) const { Acc r; r.v = __shfl_xor_sync(0xffffffffu, v, o); return r; }
     __device__ __forceinline__ double value() const { return v; }
 };
 template <> struct Acc<float> {
@@ -719,11 +719,11 @@ template <> struct Acc<float> {
     __device__ __forceinline__ void add(const Acc &o) { add(o.hi); lo += o.lo; }
     __device__ __forceinline__ void maxv(float x) { hi = fmaxf(hi, x); }
     __device__ __forceinline__ void maxv(const Acc &o) { hi = fmaxf(hi, o.hi); }
-    __device__ __forceinline__ Acc shfl_down(int o) const
+    __device__ __forceinline__ Acc shfl_xor(int o) const
     {
         Acc r;
-        r.hi = __shfl_down_sync(0xffffffffu, hi, o);
-        r.lo = __shfl_down_sync(0xffffffffu, lo, o);
+        r.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+        r.lo = __shfl_xor_sync(0xffffffffu, lo, o);
         return r;
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
@@ -743,11 +743,11 @@ template <> struct Acc<dfloat> {
         if (x.hi > v.hi || (x.hi == v.hi && x.lo > v.lo)) v = x;
     }
     __device__ __forceinline__ void maxv(const Acc &o) { maxv(o.v); }
-    __device__ __forceinline__ Acc shfl_down(int o) const
+    __device__ __forceinline__ Acc shfl_xor(int o) const
     {
         Acc r;
-        r.v.hi = __shfl_down_sync(0xffffffffu, v.hi, o);
-        r.v.lo = __shfl_down_sync(0xffffffffu, v.lo, o);
+        r.v.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+        r.v.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
         return r;
     }
     __device__ __forceinline__ double value() const { return df_to_double(v); }
@@ -760,63 +760,82 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
     return t;
 }
 
-// Last CTA of the field evaluation: sum the per-CTA partials in block order
-// (one warp; fixed order, so the result does not depend on which CTA came
-// last), then finish the iteration on lane 0.
+// b into a: the maximum for the torque slot of the minimiser, a sum otherwise
+template <int MODE, typename A> __device__ __forceinline__ void fold(A &a, const A &b, int slot)
+{
+    if (MODE == MODE_MIN && slot == SL_T2) a.maxv(b);
+    else a.add(b);
+}
+
+// The NSL = 8 slots of every working thread of the CTA reduced to totals, slot s
+// in lane s of warp 0 (in the return value; other lanes and warps get
+// something else).  In a warp, each exchange halves the slots a lane is in
+// charge of along with the lanes, 4 + 2 + 1 + 1 + 1 additions instead of 8 x 5;
+// FP64 instructions are what a small film's reduction waits for.  nw working
+// warps; `sm`: NSL values a warp of shared memory, free for use; two barriers,
+// all threads of the CTA take part.
+template <int MODE, typename A>
+__device__ __forceinline__ A reduce_slots(A (&r)[NSL], A *sm, const int tid, const int nth)
+{
+    static_assert(NSL == 8, "three exchanges leave one slot a lane");
+    const int lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+    int slot = 0;
+#pragma unroll
+    for (int n = 4, o = 16; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+        slot += up ? n : 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const A give = up ? r[i] : r[n + i];
+            A keep = up ? r[n + i] : r[i];
+            fold<MODE>(keep, give.shfl_xor(o), slot + i);
+            r[i] = keep;
+        }
+    }
+    fold<MODE>(r[0], r[0].shfl_xor(2), slot);
+    fold<MODE>(r[0], r[0].shfl_xor(1), slot);
+    if (warp < nw && (lane & 3) == 0) sm[warp * NSL + slot] = r[0];
+    __syncthreads();
+    A t;
+    t.zero();
+    if (warp == 0) {
+        const int s = lane & 7;
+        for (int w = lane >> 3; w < nw; w += 4) fold<MODE>(t, sm[w * NSL + s], s);
+        fold<MODE>(t, t.shfl_xor(8), s);
+        fold<MODE>(t, t.shfl_xor(16), s);
+    }
+    __syncthreads();
+    return t;
+}
+
+// Finish the evaluation from the totals (warp 0; `mine`: the total of slot `lane`
+// in lanes 0 .. 7).  The quotients and roots are taken by one lane each, in one
+// division and one square root: one after another they took several
+// microseconds of dependent FP64 instructions.
 template <int MODE>
-__device__ void finish_iteration(const Geom &g, double *partials, int nblk, MinState *st,
-                                 cudaGraphConditionalHandle h, int use_cond, int body_kernels)
+__device__ __forceinline__ void finish_iteration(const Geom &g, double mine, const double *hext, MinState *st,
+                                                 cudaGraphConditionalHandle h, int use_cond, int body_kernels)
 {
     const int lane = threadIdx.x & 31;
-    // lane l sums blocks l, l + 32, l + 64, ... of every slot in that order;
-    // the loads of FB blocks (all slots, 16-byte reads) are issued before any
-    // is added, so the wait is one L2 round trip per FB blocks, not one per
-    // block and slot
-    constexpr int FB = 2;
-    double v[NSL];
-#pragma unroll
-    for (int s = 0; s < NSL; ++s) v[s] = 0.0;
-    auto fold = [&](const double2 *x) {
-#pragma unroll
-        for (int s = 0; s < NSL; ++s) {
-            const double xs = (s & 1) ? x[s / 2].y : x[s / 2].x;
-            v[s] = (MODE == MODE_MIN && s == SL_T2) ? fmax(v[s], xs) : v[s] + xs;
-        }
-    };
-    int b = lane;
-    for (; b + (FB - 1) * 32 < nblk; b += FB * 32) {
-        double2 x[FB][NSL / 2];
-#pragma unroll
-        for (int i = 0; i < FB; ++i)
-#pragma unroll
-            for (int q = 0; q < NSL / 2; ++q)
-                x[i][q] = __ldcg(reinterpret_cast<const double2 *>(partials + (long)(b + 32 * i) * RED_NSLOT) + q);
-#pragma unroll
-        for (int i = 0; i < FB; ++i) fold(x[i]);
-    }
-    for (; b < nblk; b += 32) {
-        double2 x[NSL / 2];
-#pragma unroll
-        for (int q = 0; q < NSL / 2; ++q) x[q] = __ldcg(reinterpret_cast<const double2 *>(partials + (long)b * RED_NSLOT) + q);
-        fold(x);
-    }
     double tot[NSL];
 #pragma unroll
-    for (int s = 0; s < NSL; ++s) {
-        const bool isMax = (MODE == MODE_MIN && s == SL_T2);
-        double w = v[s];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double y = __shfl_down_sync(0xffffffffu, w, o);
-            w = isMax ? fmax(w, y) : w + y;
-        }
-        tot[s] = w;
-    }
-    if (lane != 0) return;
+    for (int s = 0; s < NSL; ++s) tot[s] = __shfl_sync(0xffffffffu, mine, s);
     const double V = g.dx * g.dy * g.dz, Ms = g.Ms, cE = MM_MU0 * Ms * V;
-    st->mavg[0] = tot[SL_MX] / (double)g.N;
-    st->mavg[1] = tot[SL_MY] / (double)g.N;
-    st->mavg[2] = tot[SL_MZ] / (double)g.N;
+    const double ss = tot[SL_SS], sy = tot[SL_SY], yy = tot[SL_YY];
+    enum { Q_TAU1 = 0, Q_TAU2 = 1, Q_ROOT = 2, Q_TORQUE = 3, Q_TMAX = 4, Q_M = SL_MX };
+    const bool min = MODE == MODE_MIN;
+    const double num = lane == Q_TAU1 || lane == Q_ROOT ? ss : (lane == Q_TAU2 ? sy : (lane < SL_MX ? tot[SL_T2] : mine));
+    const double den = lane == Q_TAU1 ? sy
+                       : (lane == Q_TAU2 || lane == Q_ROOT ? yy : (lane == Q_TORQUE ? Ms * Ms : (lane == Q_TMAX ? 1.0 : (double)g.N)));
+    const double quot = num / den;
+    const double root = min ? sqrt(quot) : 0.0;
+    double q[NSL];
+#pragma unroll
+    for (int s = 0; s < NSL; ++s) q[s] = __shfl_sync(0xffffffffu, min && s >= Q_ROOT && s <= Q_TMAX ? root : quot, s);
+    if (lane != 0) return;
+    st->mavg[0] = q[SL_MX];
+    st->mavg[1] = q[SL_MY];
+    st->mavg[2] = q[SL_MZ];
     if (MODE == MODE_ENERGY) {
         const double Ed = -0.5 * cE * tot[SL_ED], Eex = -0.5 * cE * tot[SL_EEX];
         const double Ean = V * tot[SL_EAN], Ez = -cE * tot[SL_EZ];
@@ -825,18 +844,20 @@ __device__ void finish_iteration(const Geom &g, double *partials, int nblk, MinS
         return;
     }
     const long k = st->k;
-    const double tmax = sqrt(tot[SL_T2]);
-    st->max_torque = tmax / Ms;
-    st->bb[0] = k > 0 ? tot[SL_SS] : 0.0;
-    st->bb[1] = k > 0 ? tot[SL_SY] : 0.0;
-    st->bb[2] = k > 0 ? tot[SL_YY] : 0.0;
-    st->energy[4] = cE * tot[SL_ET];
+    const double tmax = q[Q_TMAX];
+    st->max_torque = q[Q_TORQUE];
+    st->bb[0] = k > 0 ? ss : 0.0;
+    st->bb[1] = k > 0 ? sy : 0.0;
+    st->bb[2] = k > 0 ? yy : 0.0;
+    // the slot holds the sum of m.H - 2 K/(mu0 Ms) with per-cell K, of m.H with a uniform one
+    const double mhe = tot[SL_MX] * hext[0] + tot[SL_MY] * hext[1] + tot[SL_MZ] * hext[2];
+    st->energy[4] = cE * (-0.5 * (tot[SL_ET] + mhe)) + hext[3];
     st->evals = k + 1;
     st->launches += body_kernels;
     if (k == 0) st->t_start_ns = globaltimer_ns();
     int stop = 1;
     const bool finite = isfinite(tmax) && isfinite(st->energy[4]) &&
-                        (k == 0 || (isfinite(tot[SL_SS]) && isfinite(tot[SL_SY]) && isfinite(tot[SL_YY])));
+                        (k == 0 || (isfinite(ss) && isfinite(sy) && isfinite(yy)));
     if (!finite) {
         st->status = MMS_NONFINITE;
     } else if (tmax < st->tol_abs) {
@@ -850,12 +871,11 @@ __device__ void finish_iteration(const Geom &g, double *partials, int nblk, MinS
         if (k == 0) {
             tau = st->tau0;
         } else {
-            const double ss = tot[SL_SS], sy = tot[SL_SY], yy = tot[SL_YY];
             if (st->tau_rule == MM_TAU_ADAPTIVE)   // tau^2 when cos^2(s, y) < kappa, else tau^1
-                tau = (sy * sy < st->kappa * (ss * yy)) ? sy / yy : ss / sy;
+                tau = (sy * sy < st->kappa * (ss * yy)) ? q[Q_TAU2] : q[Q_TAU1];
             else                                   // alternation: tau^1 on odd k, tau^2 on even k
-                tau = (k & 1) ? ss / sy : sy / yy;
-            if (!(isfinite(tau) && tau > 0.0)) tau = sqrt(ss / yy);
+                tau = (k & 1) ? q[Q_TAU1] : q[Q_TAU2];
+            if (!(isfinite(tau) && tau > 0.0)) tau = q[Q_ROOT];
             if (!(isfinite(tau) && tau > 0.0)) tau = st->tau0;
         }
         st->tau = tau;
@@ -1048,7 +1068,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     const T cx = pick<T>(g.cex_x, g.fcex_x, g.wcex[0]), cy = pick<T>(g.cex_y, g.fcex_y, g.wcex[1]),
             cz = pick<T>(g.cex_z, g.fcex_z, g.wcex[2]);
     const T can = pick<T>(g.can, g.fcan, g.wcan);
-    const T kfac = (T)0.5 * can;  // 1/(mu0 Ms)
     const T Kuni = pick<T>(g.K, g.fK, g.wK), ux = pick<T>(g.u[0], g.fu[0], g.wu[0]),
             uy = pick<T>(g.u[1], g.fu[1], g.wu[1]), uz = pick<T>(g.u[2], g.fu[2], g.wu[2]);
     const T hs = (T)P.hscale;
@@ -1127,7 +1146,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             continue;
         }
         red[SL_MX].add(m0); red[SL_MY].add(m1); red[SL_MZ].add(m2);
-        const T mhe = m0 * he0 + m1 * he1 + m2 * he2;
         if (MODE == MODE_ENERGY) {
             if constexpr (sizeof(T) == 4) {
                 // float path: every per-cell product enters its sum exactly
@@ -1139,7 +1157,7 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
                 red[SL_ED].add(m0 * d0 + m1 * d1 + m2 * d2);
                 red[SL_EEX].add(m0 * e0 + m1 * e1 + m2 * e2);
                 red[SL_EAN].add(Kv * ((T)1 - mu * mu));
-                red[SL_EZ].add(mhe);
+                red[SL_EZ].add(m0 * he0 + m1 * he1 + m2 * he2);
             }
             continue;
         }
@@ -1150,14 +1168,14 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         const T mm = m0 * m0 + m1 * m1 + m2 * m2;
         const T g0 = mh * m0 - mm * H0, g1 = mh * m1 - mm * H1, g2 = mh * m2 - mm * H2;
         red[SL_T2].maxv(g0 * g0 + g1 * g1 + g2 * g2);  // |m x H|^2 = |g|^2 for |m| = 1
-        // energy density / (mu0 Ms V): -m.H/2 - m.H_ext/2 + K/(mu0 Ms)
+        // energy density / (mu0 Ms V): -(m.H + m.H_ext)/2 + K/(mu0 Ms).  The slot
+        // sums m.H; the Zeeman part follows from the sums of m, the constant of a
+        // uniform K from the cell count (finish_iteration)
         if constexpr (sizeof(T) == 4) {
-            const T h0 = (T)-0.5 * m0, h1 = (T)-0.5 * m1, h2 = (T)-0.5 * m2;  // exact halvings
-            red[SL_ET].add_prod(h0, H0); red[SL_ET].add_prod(h1, H1); red[SL_ET].add_prod(h2, H2);
-            red[SL_ET].add_prod(h0, he0); red[SL_ET].add_prod(h1, he1); red[SL_ET].add_prod(h2, he2);
-            red[SL_ET].add_prod(kfac, Kv);
+            red[SL_ET].add_prod(m0, H0); red[SL_ET].add_prod(m1, H1); red[SL_ET].add_prod(m2, H2);
+            if (P.Kc) red[SL_ET].add_prod(-can, Kv);
         } else {
-            red[SL_ET].add((T)-0.5 * (mh + mhe) + kfac * Kv);
+            red[SL_ET].add(P.Kc ? mh - can * Kv : mh);
         }
         T *gout = (k & 1) ? P.gbuf[1] : P.gbuf[0];
         if (k > 0) {
@@ -1188,41 +1206,52 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     }
     if (MODE == MODE_HEFF) return;
 
-    // CTA reduction: the FFT rows are done with; stage every thread's
-    // accumulators in shared memory and let warp s reduce slot s.
-    __syncthreads();
-    Acc<T> *stage = reinterpret_cast<Acc<T> *>(smem_raw);
-    if (tid < nth) {
-#pragma unroll
-        for (int s = 0; s < NSL; ++s) stage[s * nth + tid] = red[s];
-    }
+    // CTA reduction, in shared memory that the FFT rows no longer need
     __syncthreads();
     const int warp = tid >> 5, lane = tid & 31;
-    for (int s = (tid < nth ? warp : NSL); s < NSL; s += nth >> 5) {  // warp w reduces slots w, w + nwarps, ...
-        const bool isMax = (MODE == MODE_MIN && s == SL_T2);
-        Acc<T> a = stage[s * nth + lane];
-        for (int i = lane + 32; i < nth; i += 32) {
-            if (isMax) a.maxv(stage[s * nth + i]); else a.add(stage[s * nth + i]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const Acc<T> b = a.shfl_down(o);
-            if (isMax) a.maxv(b); else a.add(b);
-        }
-        if (lane == 0) P.partials[(long)bid * RED_NSLOT + s] = a.value();
+    {
+        const Acc<T> t = reduce_slots<MODE>(red, reinterpret_cast<Acc<T> *>(smem_raw), tid, nth);
+        if (warp == 0 && lane < NSL) P.partials[(long)bid * RED_NSLOT + lane] = t.value();
     }
     // the last CTA to arrive finishes the evaluation
     __shared__ int s_last;
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = (atomicAdd(P.counter, 1u) == (unsigned)nblk - 1);
+    if (warp == 0) {
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            s_last = (atomicAdd(P.counter, 1u) == (unsigned)nblk - 1);
+        }
     }
     __syncthreads();
-    if (s_last && warp == 0) {   // no early return: a persistent batch CTA goes on to its next work item
+    if (s_last) {   // no early return: a persistent batch CTA goes on to its next work item
+        // thread t sums the partials of CTAs t, t + nth, ...: a fixed order, so
+        // the result does not depend on which CTA came last
         __threadfence();
-        finish_iteration<MODE>(g, P.partials, nblk, st, h, use_cond, g.nbody);
-        if (lane == 0) *P.counter = 0u;
+        Acc<double> v[NSL];
+#pragma unroll
+        for (int s = 0; s < NSL; ++s) v[s].zero();
+        for (int b = tt; b < nblk; b += nth) {
+            double2 x[NSL / 2];
+#pragma unroll
+            for (int q = 0; q < NSL / 2; ++q)
+                x[q] = __ldcg(reinterpret_cast<const double2 *>(P.partials + (long)b * RED_NSLOT) + q);
+#pragma unroll
+            for (int s = 0; s < NSL; ++s) {
+                Acc<double> xs;
+                xs.v = (s & 1) ? x[s / 2].y : x[s / 2].x;
+                fold<MODE>(v[s], xs, s);
+            }
+        }
+        const Acc<double> t = reduce_slots<MODE>(v, reinterpret_cast<Acc<double> *>(smem_raw), tid, nth);
+        if (warp == 0) {
+            double fin[4] = {0.0, 0.0, 0.0, 0.0};   // external field, energy of a uniform K
+            if (MODE == MODE_MIN) {
+                fin[0] = st->Hext[0]; fin[1] = st->Hext[1]; fin[2] = st->Hext[2];
+                if (!P.Kc) fin[3] = g.K * g.dx * g.dy * g.dz * (double)g.N;
+            }
+            finish_iteration<MODE>(g, t.v, fin, st, h, use_cond, g.nbody);
+            if (lane == 0) *P.counter = 0u;
+        }
     }
 }
 
@@ -1275,7 +1304,7 @@ template <typename T> size_t smem_x_t(const Geom &g)
     typedef typename cvec<typename fft_of<T>::type>::type V;
     size_t rows = (size_t)3 * g.TY * g.rsx * sizeof(V) + (size_t)g.Px * sizeof(V);
     if (sizeof(T) == 4 && g.stage) rows = stage_offset<T>(g) + (size_t)(15 * g.TY + 6) * g.nx * sizeof(T);
-    const size_t stage = (size_t)NSL * threads_x<T>(g) * sizeof(Acc<T>);
+    const size_t stage = (size_t)NSL * (threads_x<T>(g) / 32) * 8;   // reduce_slots: 8-byte values
     return rows > stage ? rows : stage;
 }
 template <typename T> size_t smem_yz_t(const Geom &g)
