@@ -217,6 +217,12 @@ __device__ __forceinline__ float fx_pow2f(int e)
 {
     return e < -126 ? 0.0f : __int_as_float((min(e, 127) + 127) << 23);
 }
+// x * 2^e by its exponent bits; 0 for results below the normal numbers (and for x = 0)
+__device__ __forceinline__ double fx_ldexp(double x, int e)
+{
+    const int hi = __double2hiint(x), old = (hi >> 20) & 0x7ff;
+    return old == 0 || old + e <= 0 ? 0.0 : __hiloint2double(hi + (e << 20), __double2loint(x));
+}
 // 2^e as a double, 0 below the smallest normal power
 __device__ __forceinline__ double fx_pow2(int e)
 {

@@ -83,3 +83,28 @@ def test_non_finite_inputs_come_out_as_nan(mmlib, bad):
         st, _ = mmlib.mm_minimize(prob, b, (0, 0, 0), mmlib.make_opts(max_iter=5))
         assert st == mmlib.MM_ERR_NONFINITE
         assert np.array_equal(demag(mmlib, prob, m), clean)  # nothing stays behind
+
+
+@pytest.mark.parametrize("prec,bar", [("MM_FP64", 2e-15), ("MM_F32X2", 2e-14)])
+@pytest.mark.parametrize("grid", [(1, 9, 1), (9, 1, 2), (33, 18, 3), (200, 7, 4)])
+def test_exchange_on_the_integer_copy_and_beside_it(mmlib, grid, prec, bar):
+    """The whole field with exchange, anisotropy and Zeeman terms: rows of one scale (integer differences), and rows
+    whose scales differ (differences of the fields themselves) next to each other.  Bars: 2^-52 and 2^-46 times a small
+    multiple of the terms' root-sum-square."""
+    nx, ny, nz = grid
+    prob, oprob = make_pair(mmlib, nx, ny, nz, (4e-9, 3e-9, 5e-9), A=1.3e-11, K=2e4, u=(0.6, 0.0, 0.8),
+                            precision=getattr(mmlib, prec))
+    d = om.Demag(oprob)
+    m = inputs.random_unit_m(oprob.shape, 31 + nx)
+    states = [m, m * 2.0 ** -30, m * np.where(np.arange(ny) % 3 == 0, 2.0 ** -12, 1.0).reshape(1, 1, ny, 1)]
+    for s in states:
+        H = torch.empty(s.shape, dtype=torch.float64, device="cuda")
+        Hext = np.array([3e3, -2e3, 1e3]) * np.max(np.abs(s))
+        mmlib.mm_heff(prob, dev(s), Hext, H)
+        assert rel_l2(H.cpu().numpy(), om.heff(oprob, s, Hext, d)) <= bar
+        E = mmlib.mm_energy(prob, dev(s), Hext)
+        ref = om.energy(oprob, s, Hext, d)
+        keys = ["demag", "exchange", "anisotropy", "zeeman", "total"]
+        scale = max(abs(ref[k]) for k in keys)
+        for i, k in enumerate(keys):
+            assert abs(E[i] - ref[k]) <= 1e-12 * scale, k
