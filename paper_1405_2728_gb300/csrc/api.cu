@@ -184,6 +184,7 @@ int plan(mm_problem *p)
         g.rsz = f ? row_stride(g.Pz, 8) : row_stride_fx(g.Pz);
         g.fd_padx.init(g.Px - gr.nx > 0 ? g.Px - gr.nx : 1);
         g.fd_pady.init(g.Py - gr.ny > 0 ? g.Py - gr.ny : 1);
+        g.fd_padz.init(g.Pz - gr.nz > 0 ? g.Pz - gr.nz : 1);
     };
     if (P2[0] > 4096 || P2[1] > 4096 || P2[2] > 4096) return MM_ERR_UNSUPPORTED;
     lengths(P2[0], P2[1], P2[2]);

@@ -21,6 +21,9 @@
 
 namespace {
 
+// log2 of a power of two (ZB, KB)
+__device__ __forceinline__ int log2_of(int p) { return 31 - __clz(p); }
+
 template <typename V> __device__ __forceinline__ V load_cg(const V *p) { return __ldcg(p); }
 template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
 {
@@ -47,7 +50,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int ny = g.ny, nz = g.nz, Py = g.Py, ZB = g.ZB, rs = g.rsy;
+    const int ny = g.ny, nz = g.nz, Py = LY ? fft_length(LY) : g.Py, ZB = g.ZB, rs = g.rsy;
     const int kx = blockIdx.x, z0 = blockIdx.y * ZB;
     const int zb = min(ZB, nz - z0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * ZB * rs);
@@ -88,20 +91,19 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= tot) break;
-            const int c = e % 3, rest = e / 3, zl = rest / lin, y = rest - zl * lin;
+            const int c = e % 3, rest = e / 3, zl = INV ? rest / Py : g.fd_ny.div(rest), y = rest - zl * lin;
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[INV ? y / g.KB : rest]) - emax);
+                v[i] = fx_scale(v[i], fx_exp(scales[INV ? y >> log2_of(g.KB) : rest]) - emax);
                 mag |= fx_mag(v[i]);
             }
-            S[(c * ZB + zl) * rs + spos<V>(y)] = v[i];
+            S[(c * ZB + zl) * rs + rpos<V, LY>(y)] = v[i];
         }
     }
     if (!INV) {
         const int npad = Py - ny;
-        for (int e = tid; e < 3 * zb * npad; e += nth) {
-            const int r = e / npad, y = ny + (e - r * npad);
-            const int c = r / zb, zl = r - c * zb;
-            S[(c * ZB + zl) * rs + spos<V>(y)] = czero<V>();
+        for (int e = tid; e < 3 * ZB * npad; e += nth) {
+            const int r = g.fd_pady.div(e), y = ny + (e - r * npad);
+            S[r * rs + rpos<V, LY>(y)] = czero<V>();
         }
     }
     if constexpr (FX) fx_cta_or(&s_r[1], mag);
@@ -134,8 +136,8 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
     const int lout = INV ? ny : Py;
     V *dst = INV ? P.W + first * ny * 3 : P.W2 + first * Py * 3;
     for (int e = tid; e < zb * lout * 3; e += nth) {
-        const int c = e % 3, rest = e / 3, zl = rest / lout, y = rest - zl * lout;
-        V r = S[(c * ZB + zl) * rs + spos<V>(y)];
+        const int c = e % 3, rest = e / 3, zl = INV ? g.fd_ny.div(rest) : rest / Py, y = rest - zl * lout;
+        V r = S[(c * ZB + zl) * rs + rpos<V, LY>(y)];
         if constexpr (FX) r = fx_scale(r, post);
         dst[e] = r;
     }
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int nz = g.nz, Py = g.Py, Pz = g.Pz, KB = g.KB, rs = g.rsz;
+    const int nz = g.nz, Py = g.Py, Pz = LZ ? fft_length(LZ) : g.Pz, KB = g.KB, rs = g.rsz, lkb = log2_of(KB);
     const int kx = blockIdx.x, ky0 = blockIdx.y * KB;
     const int kb = min(KB, Py - ky0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * KB * rs);
@@ -176,6 +178,11 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
         __syncthreads();
         emax = s_e;
     }
+    // i = z * kb + kyl: a whole block of KB = 2^lkb frequencies, or the last one
+    auto split = [&](int i, int &kyl, int &z) {
+        if (kb == KB) { z = i >> lkb; kyl = i & (KB - 1); }
+        else { z = i / kb; kyl = i - z * kb; }
+    };
     // W2[kx][z][ky0 + kyl][c], z < nz -> row (c, kyl), element z; PF loads
     // per thread in flight before use
     V *base = P.W2 + ((long)kx * nz * Py + ky0) * 3;
@@ -188,7 +195,9 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e < tot) {
-                const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
+                const int c = e % 3;
+                int kyl, z;
+                split(e / 3, kyl, z);
                 v[i] = load_cg(base + (long)z * zs + kyl * 3 + c);
             }
         }
@@ -196,19 +205,20 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= tot) break;
-            const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
+            const int c = e % 3;
+            int kyl, z;
+            split(e / 3, kyl, z);
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[z / g.ZB]) - emax);
+                v[i] = fx_scale(v[i], fx_exp(scales[z >> log2_of(g.ZB)]) - emax);
                 mag |= fx_mag(v[i]);
             }
-            S[(c * KB + kyl) * rs + spos<V>(z)] = v[i];
+            S[(c * KB + kyl) * rs + rpos<V, LZ>(z)] = v[i];
         }
     }
     const int npad = Pz - nz;
-    for (int e = tid; e < 3 * kb * npad; e += nth) {
-        const int r = e / npad, z = nz + (e - r * npad);
-        const int c = r / kb, kyl = r - c * kb;
-        S[(c * KB + kyl) * rs + spos<V>(z)] = czero<V>();
+    for (int e = tid; e < 3 * KB * npad; e += nth) {
+        const int r = g.fd_padz.div(e), z = nz + (e - r * npad);
+        S[r * rs + rpos<V, LZ>(z)] = czero<V>();
     }
     if constexpr (FX) fx_cta_or(&s_r[1], mag);
     cp_async_wait_all();
@@ -232,12 +242,14 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
     const int hy = Py / 2, hz = Pz / 2;
     const typename coef<typename fft_of<T>::type>::type *Nk = P.Nhat + (long)kx * (hz + 1) * (hy + 1) * 6;
     for (int e = tid; e < kb * Pz; e += nth) {
-        const int kyl = e % kb, kz = e / kb, ky = ky0 + kyl;
+        int kyl, kz;
+        split(e, kyl, kz);
+        const int ky = ky0 + kyl;
         const int kyr = ky <= hy ? ky : Py - ky, kzr = kz <= hz ? kz : Pz - kz;
         const auto *n6 = Nk + ((long)kzr * (hy + 1) + kyr) * 6;
-        V *a0 = S + (0 * KB + kyl) * rs + spos<V>(kz);
-        V *a1 = S + (1 * KB + kyl) * rs + spos<V>(kz);
-        V *a2 = S + (2 * KB + kyl) * rs + spos<V>(kz);
+        V *a0 = S + (0 * KB + kyl) * rs + rpos<V, LZ>(kz);
+        V *a1 = S + (1 * KB + kyl) * rs + rpos<V, LZ>(kz);
+        V *a2 = S + (2 * KB + kyl) * rs + rpos<V, LZ>(kz);
         if constexpr (FX) {
             // one scale per frequency: inputs below 2^59, outputs below 2^59
             auto element = [&](int c, bool neg) {
@@ -267,8 +279,11 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
             *a0 = h0; *a1 = h1; *a2 = h2;
         } else {
         const T sy = ky <= hy ? (T)1 : (T)-1, sz = kz <= hz ? (T)1 : (T)-1;
-        const T nxx = __ldg(n6 + 0), nyy = __ldg(n6 + 1), nzz = __ldg(n6 + 2);
-        const T nxy = sy * __ldg(n6 + 3), nxz = sz * __ldg(n6 + 4), nyz = sy * sz * __ldg(n6 + 5);
+        // six floats from an 8-byte boundary
+        const float2 *n2 = reinterpret_cast<const float2 *>(n6);
+        const float2 n01 = __ldg(n2), n23 = __ldg(n2 + 1), n45 = __ldg(n2 + 2);
+        const T nxx = n01.x, nyy = n01.y, nzz = n23.x;
+        const T nxy = sy * n23.y, nxz = sz * n45.x, nyz = sy * sz * n45.y;
         const V m0 = *a0, m1 = *a1, m2 = *a2;
         V h0, h1, h2;
         h0.x = nxx * m0.x + nxy * m1.x + nxz * m2.x; h0.y = nxx * m0.y + nxy * m1.y + nxz * m2.y;
@@ -312,8 +327,10 @@ __global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom 
         if (tid == 0) P.feb[(long)kx * g.nkb + blockIdx.y] = fx_pack(emax + sh - pre - post, s_r[0] ? 3 : 0);
     }
     for (int e = tid; e < nz * kb * 3; e += nth) {
-        const int c = e % 3, rest = e / 3, kyl = rest % kb, z = rest / kb;
-        V r = S[(c * KB + kyl) * rs + spos<V>(z)];
+        const int c = e % 3;
+        int kyl, z;
+        split(e / 3, kyl, z);
+        V r = S[(c * KB + kyl) * rs + rpos<V, LZ>(z)];
         if constexpr (FX) r = fx_scale(r, post);
         base[(long)z * zs + kyl * 3 + c] = r;
     }

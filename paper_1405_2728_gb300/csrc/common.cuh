@@ -161,7 +161,7 @@ struct Geom {
     float fcex_x, fcex_y, fcex_z, fcan, fK, fu[3];
     dfloat wcex[3], wcan, wK, wu[3];   // and as double-word pairs for the double-word kernels
     int lty;                       // log2(TY)
-    FastDiv fd_nx, fd_ny, fd_padx, fd_pady;  // divisors nx, ny, Px - nx, Py - ny
+    FastDiv fd_nx, fd_ny, fd_padx, fd_pady, fd_padz;  // divisors nx, ny, Px - nx, Py - ny, Pz - nz
     int stage;                     // k_xinv (float) stages its stencil rows with 16-byte cp.async
     FastDiv fd_nc;                 // 16-byte chunks per x row when staging
 };

@@ -51,9 +51,20 @@ template <typename V> __host__ __device__ __forceinline__ int spos(int i)
     else if constexpr (sizeof(V) == 8) return i ^ (((i >> 4) & 7) | (((i >> 6) & 1) << 3));
     else return i + (i >> 3);
 }
+// (rows of a length with an odd part are padded like 16-byte ones: rpos)
 __host__ __device__ __forceinline__ int row_stride(int L, int esz)
 {
-    return esz == 8 ? (L <= 8 ? L : (L + 15) / 16 * 16) + 1 : padded_row(L);
+    return esz == 8 && (L & (L - 1)) == 0 ? L + 1 : padded_row(L);
+}
+// Element i of a row of a kernel compiled for LC.  The swizzle of a power of two
+// is linear over XOR, so a pass takes one XOR per access.  A length with an odd
+// part has offsets that share bits, which costs about five integer instructions an
+// access, in kernels bound by those; padding has constant offsets there.  160^3
+// cells, FP32 z pass: 533 us swizzled and with divisions by runtime block sizes, 445 without both.
+template <typename V, int LC> __host__ __device__ __forceinline__ int rpos(int i)
+{
+    if constexpr (sizeof(V) == 8 && LC > 16) return pidx(i);
+    else return spos<V>(i);
 }
 
 // the same for block fixed-point rows
@@ -223,7 +234,7 @@ __device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G
             const int step = tstep0 * (Ns == LR ? b : b & (Ns - 1));
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                v[q * R + r] = row[spos<V>(b + r * LR)];
+                v[q * R + r] = row[(LR & 7) ? pidx(b + r * LR) : pidx(b) + r * (LR + (LR >> 3))];
                 if (r > 0) {
                     const V w = tw[tpos<V>(r * step, L)];
                     v[q * R + r] = INV ? cmulc(v[q * R + r], w) : cmul(v[q * R + r], w);
@@ -242,8 +253,8 @@ __device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G
             const int k = Ns == LR ? b : b & (Ns - 1);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const int i = (b - k) * R + k + r * Ns;
-                if (!HOUT || 2 * i < L) row[spos<V>(i)] = v[q * R + r];
+                const int i0 = (b - k) * R + k, i = i0 + r * Ns;
+                if (!HOUT || 2 * i < L) row[(Ns & 7) ? pidx(i) : pidx(i0) + r * (Ns + (Ns >> 3))] = v[q * R + r];
             }
         }
     }
@@ -261,11 +272,12 @@ __device__ __forceinline__ void stockham_odd(V *row, int L, int Ns, int j, int G
 // whose padded offsets are 9 (b - k) + k + k/8 + r Ns + (r Ns)/8 for R = 8
 // (and likewise with (b - k) R for R < 8), since k < Ns and Ns divides or is
 // a multiple of 8.
-template <int R, bool INV, bool HIN, bool HOUT, typename V>
+template <int R, bool INV, bool HIN, bool HOUT, bool PAD = false, typename V>
 __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int G,
                                               const V *__restrict__ tw, int ts, bool active)
 {
     constexpr int NB = 8 / R;
+    constexpr bool XOR = sizeof(V) == 8 && !PAD;   // a swizzled float row (PAD: length with an odd part)
     V v[8];
     const int LR = L / R;
     const int ld9 = LR + (LR >> 3);       // padded stride between the inputs of a butterfly (8 | LR)
@@ -274,11 +286,11 @@ __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int 
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
             const int b = j + q * G;
-            const int p0 = pidx(b);
+            const int p0 = XOR ? spos<V>(b) : pidx(b);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (HIN && r >= R / 2) { v[q * R + r] = czero<V>(); continue; }
-                if constexpr (sizeof(V) == 8) v[q * R + r] = row[spos<V>(b + r * LR)];
+                if constexpr (XOR) v[q * R + r] = row[p0 ^ spos<V>(r * LR)];   // b < LR
                 else v[q * R + r] = row[(LR & 7) ? pidx(b + r * LR) : p0 + r * ld9];
             }
             if (Ns > 1) {
@@ -305,11 +317,11 @@ __device__ __forceinline__ void stockham_pass(V *row, int L, int Ns, int j, int 
             const int b = j + q * G;
             const int k = b & (Ns - 1);
             const int hi = (b - k) * R;                  // multiple of 8 when R == 8
-            const int s0 = (R == 8) ? hi + (hi >> 3) + k + (k >> 3) : 0;
+            const int s0 = XOR ? spos<V>(hi + k) : ((R == 8) ? hi + (hi >> 3) + k + (k >> 3) : 0);
 #pragma unroll
             for (int r = 0; r < (HOUT ? R / 2 : R); ++r) {
                 const int rn = r * Ns;
-                if constexpr (sizeof(V) == 8) row[spos<V>(hi + k + rn)] = v[q * R + r];
+                if constexpr (XOR) row[s0 ^ spos<V>(rn)] = v[q * R + r];       // hi + k has no bits of rn
                 else row[(R == 8) ? s0 + rn + (rn >> 3) : pidx(hi + k + rn)] = v[q * R + r];
             }
         }
@@ -405,18 +417,18 @@ __device__ __forceinline__ void fft_row_c(V *row, int j, const V *__restrict__ t
     static_assert(L >= 8 && L % 8 == 0, "compile-time rows have at least 8 elements");
     constexpr int LOGL = pow2_part(L), odd = L >> LOGL, G = L >> 3, rem = LOGL % 3, n8 = LOGL / 3;
     constexpr int NS0 = rem == 1 ? 2 : (rem == 2 ? 4 : 1);
-    if constexpr (rem == 1) stockham_pass<2, INV, HIN, false>(row, L, 1, j, G, tw, TS, active);
-    if constexpr (rem == 2) stockham_pass<4, INV, HIN, false>(row, L, 1, j, G, tw, TS, active);
+    if constexpr (rem == 1) stockham_pass<2, INV, HIN, false, (odd > 1)>(row, L, 1, j, G, tw, TS, active);
+    if constexpr (rem == 2) stockham_pass<4, INV, HIN, false, (odd > 1)>(row, L, 1, j, G, tw, TS, active);
 #pragma unroll
     for (int p = 0; p < n8; ++p) {
         const int Ns = NS0 << (3 * p);
         const bool last = (p == n8 - 1) && odd == 1, first = (p == 0 && rem == 0);
         if (first && HIN) {
-            if (last && HOUT) stockham_pass<8, INV, true, true>(row, L, Ns, j, G, tw, TS, active);
-            else stockham_pass<8, INV, true, false>(row, L, Ns, j, G, tw, TS, active);
+            if (last && HOUT) stockham_pass<8, INV, true, true, (odd > 1)>(row, L, Ns, j, G, tw, TS, active);
+            else stockham_pass<8, INV, true, false, (odd > 1)>(row, L, Ns, j, G, tw, TS, active);
         } else {
-            if (last && HOUT) stockham_pass<8, INV, false, true>(row, L, Ns, j, G, tw, TS, active);
-            else stockham_pass<8, INV, false, false>(row, L, Ns, j, G, tw, TS, active);
+            if (last && HOUT) stockham_pass<8, INV, false, true, (odd > 1)>(row, L, Ns, j, G, tw, TS, active);
+            else stockham_pass<8, INV, false, false, (odd > 1)>(row, L, Ns, j, G, tw, TS, active);
         }
     }
     if constexpr (odd == 25) stockham_odd<5, INV, false>(row, L, L / 25, j, G, tw, TS, active);
@@ -739,7 +751,7 @@ __device__ __forceinline__ int fft_row_fx(fxc *row, int L, int logL, int j, cons
 #define MM_LB_ODD(X) X(80) X(96) X(160) X(192) X(200) X(320) X(384) X(400) X(640) X(768) X(800)
 #define MM_LX_CASES(X) X(0) MM_LC_POW2(X) MM_LX_ODD(X)
 #define MM_LY_CASES(X) X(0) MM_LC_POW2(X) MM_LY_ODD(X)
-#define MM_LB_CASES(X) X(-1) MM_LC_POW2(X) MM_LB_ODD(X)
+#define MM_LB_CASES(X) X(0) MM_LC_POW2(X) MM_LB_ODD(X)
 __host__ __device__ inline int lc_pow2(int L, int other)
 {
     return L >= 64 && L <= 1024 && (L & (L - 1)) == 0 ? pow2_part(L) : other;
@@ -755,4 +767,4 @@ __host__ __device__ inline int lc_pow2(int L, int other)
 #define MM_LC_CASE(N) case N:
 MM_LC_OF(lx_of, MM_LX_ODD, 0)
 MM_LC_OF(ly_of, MM_LY_ODD, 0)
-MM_LC_OF(lb_of, MM_LB_ODD, -1)
+MM_LC_OF(lb_of, MM_LB_ODD, 0)

@@ -52,9 +52,10 @@ __device__ __forceinline__ int magnitude(dfloat x) { return __float_as_int(x.hi)
 __device__ __forceinline__ int magnitude(float) { return 0; }   // floats keep their own scale
 
 // real element x of a padded complex row holding Px reals
-template <typename T, typename V> __device__ __forceinline__ T &rel(V *row, int x)
+// (of a kernel compiled for LC)
+template <typename T, int LC, typename V> __device__ __forceinline__ T &rel(V *row, int x)
 {
-    return reinterpret_cast<T *>(row + spos<V>(x >> 1))[x & 1];
+    return reinterpret_cast<T *>(row + rpos<V, LC>(x >> 1))[x & 1];
 }
 
 // Rows of a field [3][nz][ny][nx] copied asynchronously into shared memory:
@@ -179,13 +180,13 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         if constexpr (is_fx<F>) {  // as they are, until the tile's scale is known
             max_xy = max(max_xy, max(magnitude(m0), magnitude(m1)));
             max_z = max(max_z, magnitude(m2));
-            rel<T>(S + (0 * TY + yl) * g.rsx, x) = m0;
-            rel<T>(S + (1 * TY + yl) * g.rsx, x) = m1;
-            rel<T>(S + (2 * TY + yl) * g.rsx, x) = m2;
+            rel<T, LX>(S + (0 * TY + yl) * g.rsx, x) = m0;
+            rel<T, LX>(S + (1 * TY + yl) * g.rsx, x) = m1;
+            rel<T, LX>(S + (2 * TY + yl) * g.rsx, x) = m2;
         } else {
-            rel<F>(S + (0 * TY + yl) * g.rsx, x) = F(m0);
-            rel<F>(S + (1 * TY + yl) * g.rsx, x) = F(m1);
-            rel<F>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
+            rel<F, LX>(S + (0 * TY + yl) * g.rsx, x) = F(m0);
+            rel<F, LX>(S + (1 * TY + yl) * g.rsx, x) = F(m1);
+            rel<F, LX>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
         }
     }
     int e1 = 0;
@@ -207,7 +208,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             const int yl = g.fd_nx.div(e), x = e - yl * nx, y = y0 + yl;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const T a = rel<T>(S + (c * TY + yl) * g.rsx, x);
+                const T a = rel<T, LX>(S + (c * TY + yl) * g.rsx, x);
                 fx q(0), q4(0);   // the transform's value, and 4 of its units for the stencil
                 if (!(c < 2 ? bad_xy : bad_z) && top > 0) {
                     if constexpr (DW) {
@@ -217,7 +218,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
                         q = fx_shr(q4, 2);
                     }
                 }
-                rel<fx>(S + (c * TY + yl) * g.rsx, x) = q;
+                rel<fx, LX>(S + (c * TY + yl) * g.rsx, x) = q;
                 if (!DW && y < ny) P.mfix[c * N + ((long)z * ny + y) * nx + x] = q4.v;
             }
         }
@@ -225,7 +226,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
     const int npad = Px - nx;
     for (int e = tt; e < 3 * TY * npad; e += nth) {
         const int row = g.fd_padx.div(e), x = nx + (e - row * npad);
-        rel<F>(S + row * g.rsx, x) = F(0);
+        rel<F, LX>(S + row * g.rsx, x) = F(0);
     }
     __syncthreads();
 
@@ -252,8 +253,8 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         const int c = e % 3, rest = e / 3, yl = rest & (TY - 1), k = rest >> g.ltyf;
         const int y = y0 + yl;
         const V *row = S + (c * TY + yl) * g.rsx;
-        const V Zk = row[spos<V>(k)];
-        const V Zm = cconj(row[spos<V>(k == 0 ? 0 : Hx - k)]);
+        const V Zk = row[rpos<V, LX>(k)];
+        const V Zm = cconj(row[rpos<V, LX>(k == 0 ? 0 : Hx - k)]);
         if constexpr (is_fx<F>) {  // 2 X is stored: |Zk|, |Zm| < 2^60.5, so |2 X| < 2^62
             const V sum = cadd(Zk, Zm), wd = fx_cmul<false>(csub(Zk, Zm), tw[tpos<TW>(k, g.Hx)], 0);
             if (y < ny) {
@@ -582,13 +583,13 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<float> &P
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-            S[(c * nz + zz) * g.rsy + spos<V>(y)] = v[i];
+            S[(c * nz + zz) * g.rsy + rpos<V, LY>(y)] = v[i];
         }
     }
     const int npad = Py - ny;
     for (int e = tt; e < nrow * npad; e += nth) {
         const int row = g.fd_pady.div(e), y = ny + (e - row * npad);
-        S[row * g.rsy + spos<V>(y)] = czero<V>();
+        S[row * g.rsy + rpos<V, LY>(y)] = czero<V>();
     }
     cp_async_wait_all();
     __syncthreads();
@@ -610,7 +611,7 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<float> &P
     const int hy = Py / 2, kst = hy + 1;
     const F *Kk = P.Nhat + (long)kx * NZM * 6 * kst;
     for (int ky = tt; ky < Py; ky += nth) {
-        const int pky = spos<V>(ky);
+        const int pky = rpos<V, LY>(ky);
         const int kyr = ky <= hy ? ky : Py - ky;
         const bool flip = ky > hy;
         V mz[3][NZM], hz[3][NZM];
@@ -660,7 +661,7 @@ __device__ __forceinline__ void yz_body(const Geom &g, const FieldPtrs<float> &P
 
     for (int e = tt; e < nrow * ny; e += nth) {
         const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-        Wk[e] = S[(c * nz + zz) * g.rsy + spos<V>(y)];
+        Wk[e] = S[(c * nz + zz) * g.rsy + rpos<V, LY>(y)];
     }
 }
 
@@ -1033,12 +1034,12 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             else t = cmulc(dif, tw[tpos<TW>(kk, g.Hx)]);  // conj(w^k) dif
             Z.x = sum.x - t.y;
             Z.y = sum.y + t.x;
-            row[spos<V>(kk)] = Z;
+            row[rpos<V, LX>(kk)] = Z;
             if constexpr (is_fx<F>) mag |= fx_mag(Z);
             if (kk != 0 && Hx - kk != kk) {
                 Z.x = sum.x + t.y;
                 Z.y = t.x - sum.y;
-                row[spos<V>(Hx - kk)] = Z;
+                row[rpos<V, LX>(Hx - kk)] = Z;
                 if constexpr (is_fx<F>) mag |= fx_mag(Z);
             }
         }
@@ -1109,8 +1110,8 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         const long n = ((long)z * ny + y) * nx + x;
         T d0, d1, d2;
         if constexpr (is_fx<F>) {
-            const fx q0 = rel<F>(S + (0 * TY + yl) * g.rsx, x), q1 = rel<F>(S + (1 * TY + yl) * g.rsx, x),
-                     q2 = rel<F>(S + (2 * TY + yl) * g.rsx, x);
+            const fx q0 = rel<F, LX>(S + (0 * TY + yl) * g.rsx, x), q1 = rel<F, LX>(S + (1 * TY + yl) * g.rsx, x),
+                     q2 = rel<F, LX>(S + (2 * TY + yl) * g.rsx, x);
             if constexpr (DW) {
                 d0 = fx_to_dfloat(q0, dscalef);
                 d1 = fx_to_dfloat(q1, dscalef);
@@ -1131,9 +1132,9 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
                 if (bad & 2) d2 = nan;
             }
         } else {
-            d0 = to_field<T>(rel<F>(S + (0 * TY + yl) * g.rsx, x));
-            d1 = to_field<T>(rel<F>(S + (1 * TY + yl) * g.rsx, x));
-            d2 = to_field<T>(rel<F>(S + (2 * TY + yl) * g.rsx, x));
+            d0 = to_field<T>(rel<F, LX>(S + (0 * TY + yl) * g.rsx, x));
+            d1 = to_field<T>(rel<F, LX>(S + (1 * TY + yl) * g.rsx, x));
+            d2 = to_field<T>(rel<F, LX>(S + (2 * TY + yl) * g.rsx, x));
         }
         // exchange: sum over present neighbours of (m_j - m_i) / d^2 (free faces)
         // (the external field starts the sums where they are not wanted apart)
