@@ -31,16 +31,20 @@ template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
     return fxc{fx(v.x), fx(v.y)};
 }
 
-template <typename T> struct BulkBound { static constexpr int v = sizeof(T) == 8 ? 384 : 512; };
-// two float CTAs of the z pass per SM: its odd radices would otherwise take 121 registers
-template <typename T> struct BulkCtas { static constexpr int v = sizeof(T) == 8 ? 1 : 2; };
+template <typename T> struct BulkBound { static constexpr int v = sizeof(T) == 8 ? 256 : 512; };
+// two CTAs of the z pass per SM: without the bound its odd radices take 121
+// registers (float: 682 -> 550 us at 160^3), and in fixed point one CTA of 384
+// threads and 127 registers had an SM to itself (64^3: 121 -> 102 us)
+constexpr int Z_CTAS = 2;
+// the y passes' register bound: 168 in fixed point (128: y-forward 28.5 -> 32.5 us)
+template <typename T> constexpr int Y_BOUND = sizeof(T) == 8 ? 384 : 512;
 
 // In block fixed point (double fields, F = fx) every CTA of a pass brings its
 // block to full magnitude when it loads it and when it stores it, with the
 // scale of a block per (kx, ZB planes) after the y passes and per (kx, KB
 // y-frequencies) after the z convolution.
 template <typename T, bool INV, int LY>
-__global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> P)
+__global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
 {
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v) k_ypass(Geom g, FieldPtrs<T> 
 }
 
 template <typename T, int LZ>
-__global__ void __launch_bounds__(BulkBound<T>::v, BulkCtas<T>::v) k_zconv(Geom g, FieldPtrs<T> P)
+__global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, FieldPtrs<T> P)
 {
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
