@@ -15,7 +15,7 @@ template <typename T, int PZ, int L>
 __device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int tid, int nth, int kx)
 {
     if constexpr (!is_fx<FA<T>>) yz_body<PZ, L>(g, P, tid, nth, kx);
-    else if constexpr (L == 0) yz_body_fx<PZ, 0>(g, P, tid, nth, kx);
+    else if constexpr (L == 0) yz_body_fx<PZ, -1>(g, P, tid, nth, kx);
 }
 
 // one problem of a grouped launch, as the grouped kernels read it
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(768) k_xfwd_group(const GFilm<T> *films, const
     }
 }
 
-// Block fixed point takes the code for any row length here: integer results do
+// Block fixed point takes the code for any row length, odd parts included, here: integer results do
 // not depend on the instance, and its compiled lengths in one kernel with
 // three layer counts took four minutes to build.
 template <typename T>

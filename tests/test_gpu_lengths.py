@@ -70,3 +70,24 @@ def test_layout_and_support_do_not_depend_on_the_padding(mmlib):
     with pytest.raises(mmlib.MMError) as e:
         mmlib.mm_setup_geometry(grid, mmlib.make_material(8e5, 1.3e-11, 500.0), mmlib.MM_F32X2)
     assert e.value.status == mmlib.MM_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("prec", ["MM_FP64", "MM_FP32"])
+def test_grouped_batch_of_such_films_equals_single_sweeps(mmlib, prec):
+    # every odd y length of films (320, 384, 640, 768), both size groups: the grouped kernels give the
+    # films' own results bit for bit
+    sizes = [(24, 150, 1), (20, 190, 2), (16, 300, 3), (12, 350, 1), (160, 130, 4)]
+    dt = torch.float32 if prec == "MM_FP32" else torch.float64
+    probs = [mmlib.mm_setup_geometry(mmlib.make_grid(*n, *CELL), mmlib.make_material(8e5, 1.3e-11, 500.0),
+                                     getattr(mmlib, prec)) for n in sizes]
+    assert [mmlib.mm_problem_info(p)["py"] for p in probs] == [320, 384, 640, 768, 320]
+    F = np.array([[2e4, 1e3, 0.0], [-1e4, 1e3, 0.0]])
+    opts = mmlib.make_opts(max_iter=6)
+    batch = mmlib.mm_batch_create(probs, mmlib.MM_BATCH_GROUPED)
+    starts = [dev(inputs.random_unit_m((nz, ny, nx), 5 + nx), dt) for nx, ny, nz in sizes]
+    ms = [m.clone() for m in starts]
+    _, mavg, _ = mmlib.mm_batch_sweep(batch, ms, F, opts=opts)
+    for i, p in enumerate(probs):
+        _, mavg1, _ = mmlib.mm_hysteresis_sweep(p, starts[i], F, opts=opts)
+        assert torch.equal(ms[i], starts[i]) and np.array_equal(mavg[i], mavg1), sizes[i]
+    batch.close()
