@@ -231,17 +231,17 @@ int plan(mm_problem *p)
         g.RB = 1;
         p->rbs[0] = 1;
         p->nrb = 1;
-        const int maxT = mm_bulk_thread_bound(p);
+        const int maxT = mm_bulk_thread_bound(p), maxTy = mm_bulk_thread_bound_y(p);
         // z planes per y-pass CTA: up to 4, as many rows as one pass of threads covers
         g.ZB = 0;
         for (int zb = 4; zb >= 1; zb /= 2)
-            if (zb <= g.nz && 3 * zb * g.Gy <= maxT && mm_bulk_smem_y(p, zb) <= smax) { g.ZB = zb; break; }
+            if (zb <= g.nz && 3 * zb * g.Gy <= maxTy && mm_bulk_smem_y(p, zb) <= smax) { g.ZB = zb; break; }
         if (!g.ZB) {
             if (mm_bulk_smem_y(p, 1) > smax) return MM_ERR_UNSUPPORTED;
             g.ZB = 1;
         }
         g.RBY = 3 * g.ZB;
-        if (g.RBY * g.Gy > maxT) g.RBY = maxT / g.Gy;
+        if (g.RBY * g.Gy > maxTy) g.RBY = maxTy / g.Gy;
         // y frequencies per z-pass CTA: runs of KB*3 complex values along y
         // coalesce; keep two CTAs per SM (<= 113 KiB each) where possible
         g.KB = 0;

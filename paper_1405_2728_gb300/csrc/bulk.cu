@@ -1,9 +1,9 @@
 // Bulk layout of the demagnetisation convolution (Section 3's zero-padded
 // FFT convolution for three-dimensional samples).
 //
-// The film kernel k_yz holds a whole padded y-z plane of one x-frequency in
+// The film kernels k_yz and k_yz_fx hold a whole padded y-z plane of one x-frequency in
 // shared memory, which bounds nz * Py.  Bulk samples (a cube of 256^3 cells
-// pads to 512 x 512 x 512) split that stage into three passes through HBM:
+// pads to 512 x 512 x 512, one of 160^3 to 320^3) split that stage into three passes through HBM:
 //
 //  k_ypass<fwd>  per (kx, ZB z-planes): FFT along y of the three components,
 //                zero padding ny -> Py, W[kx][z][y][c] -> W2[kx][z][ky][c];
@@ -15,7 +15,7 @@
 //
 // The x passes (k_xfwd with the minimiser step, k_xinv with the local terms
 // and the step-size sums) are the film kernels unchanged.  Shared-memory rows
-// use the padded Stockham layout of fft.cuh.
+// use the swizzled or padded Stockham layout of fft.cuh.
 #include "common.cuh"
 #include "fft.cuh"
 
@@ -433,6 +433,10 @@ size_t mm_bulk_smem_z(const mm_problem *p, int kb)
 int mm_bulk_thread_bound(const mm_problem *p)
 {
     return p->precision == MM_FP64 ? BulkBound<double>::v : BulkBound<float>::v;
+}
+int mm_bulk_thread_bound_y(const mm_problem *p)
+{
+    return p->precision == MM_FP64 ? Y_BOUND<double> : Y_BOUND<float>;
 }
 cudaError_t mm_bulk_configure(const mm_problem *p)
 {

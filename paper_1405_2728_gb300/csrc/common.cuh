@@ -408,7 +408,8 @@ cudaError_t mm_bulk_conv(const Geom &g, const FieldPtrs<double> &P, cudaStream_t
 cudaError_t mm_bulk_conv(const Geom &g, const FieldPtrs<float> &P, cudaStream_t s, int pass);
 size_t mm_bulk_smem_y(const mm_problem *p, int zb);
 size_t mm_bulk_smem_z(const mm_problem *p, int kb);
-int mm_bulk_thread_bound(const mm_problem *p);
+int mm_bulk_thread_bound(const mm_problem *p);    // threads of a z-pass CTA at most
+int mm_bulk_thread_bound_y(const mm_problem *p);  // and of a y-pass CTA
 cudaError_t mm_bulk_configure(const mm_problem *p);
 // implemented in newell.cu
 int mm_newell_device(const mm_grid *g, double *N_dev, cudaStream_t s);

@@ -10,7 +10,8 @@
 //             the renormalised explicit step) fused with the real-to-complex
 //             FFT along x of the three components, zero padding nx -> Px,
 //             written transposed to the spectrum W[kx][z][y][c].
-//  k_yz       per x-frequency kx: FFT along y (padding ny -> Py) in shared
+//  k_yz (float), k_yz_fx (double and double-word fields)
+//             per x-frequency kx: FFT along y (padding ny -> Py) in shared
 //             memory; then per ky, in registers, the z direction as a direct
 //             convolution with the tensor transformed along x and y
 //             (H^ = -Ms N m^, nz <= 4, normalisation folded into the tensor);
@@ -25,6 +26,9 @@
 //             CTA to finish sums them in a fixed order (deterministic), picks
 //             the step size tau^1 / tau^2 alternately (Eq. stepsize), applies
 //             the stop rule and sets the device-side loop condition.
+//
+// The transforms and the convolution run in float on the float path and in
+// 64-bit block fixed point (fixed.cuh) on the others.
 //
 // Sums are accumulated in double on the double path.  On the float path each
 // per-cell product enters its sum exactly (TwoProduct with one FMA) and the

@@ -19,6 +19,8 @@
 //                    the even/odd symmetry) of the octant kx <= Px/2,
 //                    ky <= Py/2, kz <= Pz/2, scaled by -Ms/(Px Py Pz) so that
 //                    the convolution kernels need no other normalisation.
+//  k_tensor_fixed    double and double-word problems: the spectra from doubles
+//                    to the multipliers of the block fixed-point convolution.
 #include "common.cuh"
 #include "dd.cuh"
 #include "fft.cuh"
