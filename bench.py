@@ -35,15 +35,16 @@ if ROOT not in sys.path:
 METRIC = "H_eff evals/s & hysteresis-loop time (512x256x4 film) FP32 vs FP64, %HBM peak"
 UNIT = "H_eff evals/s"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-# nominal FMA lanes per SM per clock (the measured rates come from mm_probe_fma)
-FP64_FMA_PER_SM_CLK = 2
-FP32_FMA_PER_SM_CLK = 128
 # the timed steps' field values are far from switching; a whole loop needs more evaluations there
 LOOP_NOTE = ("field values x the mean time of the timed steps; the whole loop, timed by --full-loop, takes longer: "
              "near the switching field a value needs thousands of evaluations")
+# 64-bit integer additions per SM per clock (measured, chains of independent additions): the FP64 and
+# double-word transforms run in 64-bit block fixed point on the integer units
+ADD64_PER_SM_CLK = 42
 DW_ADD_INSTRUCTIONS = 11      # FP32 instructions of one double-word (float pair) addition
+LOCAL_FLOPS = 90              # of the local terms, torque and step-size sums per cell (x-inverse stage)
 PRECISIONS = {"fp64": 0, "fp32": 1, "f32x2": 2}   # mm.MM_FP64, mm.MM_FP32, mm.MM_F32X2
-DTYPE_LABEL = {"fp64": "f64", "fp32": "f32", "f32x2": "f32x2 (double-word) fields, FFT, convolution and local terms"}
+DTYPE_LABEL = {"fp64": "f64 fields and local terms, 64-bit block fixed-point FFT and convolution", "fp32": "f32", "f32x2": "f32x2 (double-word) fields and local terms, 64-bit block fixed-point FFT and convolution"}
 
 
 def dist_env():
@@ -123,7 +124,10 @@ def algorithmic_model(info, esz):
     and writes m_{k+1} and the x-spectrum; yz reads/writes the spectrum and
     reads the tensor spectra; xinv reads the spectrum, m_{k+1}, m_k and g_k and
     writes g_{k+1} (its last CTA also sums the per-CTA partials and picks tau).  Flops: real arithmetic of the radix-8 Stockham transforms
-    with zero-padding pruning, the tensor product and the local terms."""
+    (one odd pass of 3, 5 or 25 at the lengths that have the factor) with
+    zero-padding pruning, the tensor product and the local terms; in the fixed
+    point of FP64 and double-word those of the transforms and the product are
+    integer operations."""
     nx, ny, nz, Px, Py, Pz = (info[k] for k in ("nx", "ny", "nz", "px", "py", "pz"))
     N = nx * ny * nz
     F = 3 * N * esz
@@ -135,8 +139,9 @@ def algorithmic_model(info, esz):
     def fft_flops(L, half_in, half_out):
         if L <= 1:
             return 0
-        lg = L.bit_length() - 1
-        passes = []
+        pow2 = L & -L
+        lg = pow2.bit_length() - 1
+        passes = [L // pow2] if L != pow2 else []
         if lg % 3 == 1:
             passes.append(2)
         elif lg % 3 == 2:
@@ -144,7 +149,7 @@ def algorithmic_model(info, esz):
         passes += [8] * (lg // 3)
         if L < 8:
             passes = [L]
-        dft = {2: (4, 0), 4: (16, 8), 8: (56, 40)}
+        dft = {2: (4, 0), 3: (16, 12), 4: (16, 8), 5: (40, 32), 8: (56, 40), 25: (496, 400)}
         fl = 0
         ns = 1
         for i, R in enumerate(passes):
@@ -158,7 +163,7 @@ def algorithmic_model(info, esz):
     x_rows = 3 * ny * nz
     unpack = 10 * C
     f_xfwd = x_rows * (fft_flops(Hx, True, False) + unpack) + N * 3 * 8
-    f_xinv = x_rows * (fft_flops(Hx, False, True) + unpack) + N * 90
+    f_xinv = x_rows * (fft_flops(Hx, False, True) + unpack) + N * LOCAL_FLOPS
     model = {
         "xfwd_step": {"bytes": 3 * F + W, "flops": f_xfwd},
         "xinv_local_bb": {"bytes": W + 4 * F, "flops": f_xinv},
@@ -188,9 +193,9 @@ def survey_flops(info):
     product, 200 flops per cell for the local terms, torque, step and
     step-size sums.  At 512 x 256 x 4 (padded 1024 x 512 x 8) this is
     x 0.157 + y 0.284 + z 0.189 + product 0.076 + local 0.105 = 0.81 GFLOP per
-    evaluation.  The kernels execute fewer flops (zero inputs and discarded
-    outputs pruned, the film z direction as a direct sum); this model is the
-    algorithmic count the roofline is quoted against."""
+    evaluation.  The kernels execute fewer operations (zero inputs and discarded
+    outputs pruned, the film z direction as a direct sum), and in FP64 and
+    double-word those of the transforms are integer ones."""
     import math
     nx, ny, nz, Px, Py, Pz = (info[k] for k in ("nx", "ny", "nz", "px", "py", "pz"))
     C = Px // 2 + 1
@@ -208,7 +213,7 @@ def survey_flops(info):
     return out
 
 
-KERNEL_SOURCES = ("fft.cuh", "dfloat.cuh", "field_kernels.cuh")  # the device code of the film field kernels
+KERNEL_SOURCES = ("fixed.cuh", "fft.cuh", "dfloat.cuh", "field_kernels.cuh")  # the device code of the film field kernels
 
 
 def kernel_source_hash():
@@ -838,29 +843,35 @@ def main():
         sec = kt[dom] * 1e-3
         gbs = model[dom]["bytes"] / sec / 1e9
         hbm = peaks.get("hbm_gbs")
-        if pname == "f32x2":
-            # double-word arithmetic on the FP32 pipes: one double-word add
-            # (the bulk of an FFT) takes 11 FP32 instructions, a product 6
-            peak = fma["fp32"] / 2 / DW_ADD_INSTRUCTIONS
-            ach = sflops[dom] / sec / 1e12
-            roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s (double-word)",
-                    "frac": ach / peak,
-                    "peak_source": f"measured FP32 FMA throughput {fma['fp32']:.1f} TFLOP/s = {fma['fp32'] / 2:.1f} T "
-                                   f"instructions/s, / {DW_ADD_INSTRUCTIONS} instructions per double-word add",
-                    "flop_model": "workload reference model (2.5/5 L log2 L per real/complex transform, 36 per "
-                                  "frequency, 200 per cell)",
-                    "vs_fp64_fma_peak": ach / fma["fp64"]}
-        elif pname == "fp64":
-            derived = n_sm * FP64_FMA_PER_SM_CLK * 2 * sm_mhz * 1e6 / 1e12
-            peak = fma["fp64"]
-            ach = sflops[dom] / sec / 1e12
-            roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                    "peak_source": f"measured FP64 FMA throughput (mm_probe_fma, {n_sm} SMs): {peak:.3f} TFLOP/s; "
-                                   f"nominal {n_sm} SMs x {FP64_FMA_PER_SM_CLK} FMA/clk x 2 flop at "
-                                   f"{sm_mhz:.0f} MHz = {derived:.3f}",
-                    "flop_model": "workload reference model (2.5/5 L log2 L per real/complex transform, 36 per "
-                                  "frequency, 200 per cell)",
-                    "executed_flops_frac": model[dom]["flops"] / sec / 1e12 / peak}
+        if pname != "fp32":
+            # The transforms and the tensor product run on the integer units, the
+            # local terms on the FP64 (or, as float pairs, the FP32) units, the
+            # bytes through HBM: the bound is the resource that takes longest.
+            cells = inf["nx"] * inf["ny"] * inf["nz"]
+            local = {"xfwd_step": 24, "xinv_local_bb": LOCAL_FLOPS}.get(dom, 0) * cells
+            local_rate = fma["fp64"] / 2 if pname == "fp64" else fma["fp32"] / 2 / DW_ADD_INSTRUCTIONS
+            int_rate = n_sm * ADD64_PER_SM_CLK * sm_mhz * 1e6 / 1e12
+            work = {"alu_int64": (model[dom]["flops"] - local, int_rate),
+                    "alu_local": (local, local_rate)}
+            floors = {k: v[0] / (v[1] * 1e12) for k, v in work.items()}
+            floors["hbm"] = model[dom]["bytes"] / ((hbm or 6800.0) * 1e9)
+            bound = max(floors, key=floors.get)
+            if bound == "hbm":
+                roof = {"bound": "hbm", "achieved": gbs, "peak": hbm or 6800.0, "unit": "GB/s"}
+            else:
+                roof = {"bound": bound, "achieved": work[bound][0] / sec / 1e12, "peak": work[bound][1],
+                        "unit": "T operations/s"}
+            roof.update({
+                "frac": roof["achieved"] / roof["peak"], "floor_ms": {k: 1e3 * v for k, v in floors.items()},
+                "peak_source": f"int64: {n_sm} SMs x {ADD64_PER_SM_CLK} 64-bit additions/clk at {sm_mhz:.0f} MHz, every "
+                               "operation of the transforms priced as an addition (a product takes several); local: "
+                               + (f"measured FP64 FMA rate (mm_probe_fma), {fma['fp64'] / 2:.3f} T instructions/s"
+                                  if pname == "fp64" else
+                                  f"measured FP32 FMA rate, {fma['fp32'] / 2:.1f} T instructions/s / "
+                                  f"{DW_ADD_INSTRUCTIONS} per double-word addition"),
+                # the workload's reference model (2.5/5 L log2 L per real/complex transform, 36 per frequency,
+                # 200 per cell) as a multiple of what the FP64 units can do at all
+                "reference_model_vs_fp64_fma_peak": sflops[dom] / sec / 1e12 / fma["fp64"]})
         else:
             peak = hbm or 6800.0
             roof = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
