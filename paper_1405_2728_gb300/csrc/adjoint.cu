@@ -342,21 +342,22 @@ int hvp_t(mm_problem *p, const void *m, const double Hext[3], const void *v, voi
     const long N = p->g.N;
     const size_t F = 3 * (size_t)N * sizeof(T);
     int rc;
-    if ((rc = ensure_adjoint_buffers(p))) return rc;
     T *H = (T *)p->stage_in, *Lv = (T *)p->stage_out;
     const bool odev = mm_is_device_ptr(Av);
     // device inputs are read where they are, unless the output overlaps them
     // other than cell for cell; the rest goes through the work buffers (128 x 64 x 2
-    // FP64: 131 -> 116 us without the two copies)
-    auto input = [&](const void *src, void *work, const T *&at) {
+    // FP64: 131 -> 116 us without the two copies), which are allocated when first
+    // needed (a problem's first call: 256 -> 150 us)
+    auto input = [&](const void *src, int work, const T *&at) {
         const bool dev = mm_is_device_ptr(src);
         const uintptr_t a = (uintptr_t)src, b = (uintptr_t)Av;
         if (dev && (!odev || a == b || a + F <= b || b + F <= a)) { at = (const T *)src; return (int)MM_OK; }
-        at = (const T *)work;
-        return mm_copy_user(work, src, F, true, dev, s);
+        if (const int e = ensure_adjoint_buffers(p)) return e;
+        at = (const T *)p->adj[work];
+        return mm_copy_user(p->adj[work], src, F, true, dev, s);
     };
     const T *mm_, *vv;
-    if ((rc = input(m, p->adj[0], mm_)) || (rc = input(v, p->adj[1], vv))) return rc;
+    if ((rc = input(m, 0, mm_)) || (rc = input(v, 1, vv))) return rc;
     const double zero[3] = {0.0, 0.0, 0.0};
     if ((rc = mm_launch_field(p, mm_, H, Hext, MODE_HEFF, s))) return rc;
     if ((rc = mm_launch_field(p, vv, Lv, zero, MODE_HEFF, s))) return rc;
