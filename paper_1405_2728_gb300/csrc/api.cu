@@ -136,7 +136,7 @@ void free_problem(mm_problem *p)
     mm_adjoint_invalidate(p);
     void *bufs[] = {p->mbuf[0], p->mbuf[1], p->gbuf[0], p->gbuf[1], p->W, p->Nhat, p->tw_px, p->tw_py,
                     p->tw_pz, p->W2, p->Kc, p->uc, p->partials, p->st, p->Hext_dev, p->stage_in, p->stage_out,
-                    p->rec_dev, p->counter, p->fexp, p->mfix, p->adj[0], p->adj[1], p->adj_state, p->adj_partials};
+                    p->rec_dev, p->counter, p->fexp, p->adj[0], p->adj[1], p->adj_state, p->adj_partials};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (p->st_host) cudaFreeHost(p->st_host);
@@ -433,7 +433,6 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
             (rc = dalloc(p, &p->tw_px, g.Px * vsz)) || (rc = dalloc(p, &p->tw_py, g.Py * vsz)) ||
             (rc = dalloc(p, &p->tw_pz, g.Pz * vsz)) ||
             (precision != MM_FP32 && (rc = dalloc(p, (void **)&p->fexp, sizeof(int) * mm_scale_count(g)))) ||
-            (precision == MM_FP64 && (rc = dalloc(p, (void **)&p->mfix, 3 * sizeof(long long) * (size_t)g.N))) ||
             (rc = dalloc(p, (void **)&p->partials, sizeof(double) * RED_NSLOT * (size_t)p->nblk_x)) ||
             (rc = dalloc(p, (void **)&p->st, sizeof(MinState))) ||
             (rc = dalloc(p, (void **)&p->counter, 64)) ||
@@ -447,8 +446,7 @@ extern "C" int mm_setup_geometry(const mm_grid *grid, const mm_material *mat, in
             rc = failed(ce, "cudaMemsetAsync", MM_ERR_CUDA);
             break;
         }
-        if ((p->fexp && (ce = cudaMemsetAsync(p->fexp, 0, sizeof(int) * mm_scale_count(g), s))) ||
-            (p->mfix && (ce = cudaMemsetAsync(p->mfix, 0, 3 * sizeof(long long) * (size_t)g.N, s)))) {
+        if (p->fexp && (ce = cudaMemsetAsync(p->fexp, 0, sizeof(int) * mm_scale_count(g), s))) {
             rc = failed(ce, "cudaMemsetAsync", MM_ERR_CUDA);
             break;
         }

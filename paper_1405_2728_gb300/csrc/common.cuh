@@ -270,7 +270,6 @@ struct FieldPtrs {
     const TW *tw_py;       // exp(-2 pi i t/Py), t < Py
     const TW *tw_pz;       // exp(-2 pi i t/Pz), t < Pz
     // block fixed point only (F = fx): the scales of the blocks (fx_pack)
-    long long *mfix;       // [3][N] double fields: the evaluated m as integers, 4 units of its tile's scale each
     int *fe1;              // [nz][ny] of W as the x-forward kernel writes it
     int *fea;              // [C][nzb] bulk: of W2 after the y transform
     int *feb;              // [C][nkb] bulk: of W2 after the z convolution
@@ -298,7 +297,6 @@ struct mm_problem {
     void *W;
     void *W2;              // bulk layout only
     void *Nhat;
-    long long *mfix;       // the evaluated m as integers (MM_FP64)
     int *fexp;             // block scales of the fixed-point convolution: fe1, fea, feb, fe2, fek in one buffer
     void *tw_px, *tw_py, *tw_pz;
     void *Kc, *uc;

@@ -467,13 +467,6 @@ __host__ __device__ __forceinline__ constexpr int fx_cum(int q, int t)
     return m > 3 ? m - 3 : 0;
 }
 
-// all bits shifted out of a row of length L with nothing known of its sum
-__host__ __device__ constexpr int fx_total(int L)
-{
-    const int l = pow2_part(L), odd = L >> l;
-    return fx_cum(l + (odd == 25 ? 5 : (odd == 5 ? 3 : (odd == 3 ? 2 : 0))), 64);
-}
-
 template <bool INV, bool HIN> __device__ __forceinline__ void dft8_fx(fxc *a)
 {
     // sqrt(1/2) in units of 2^-61

@@ -205,21 +205,16 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         float scalef = 0.0f;
         if constexpr (DW) scalef = top > 0 ? fx_pow2f(sc - 28) : 0.0f;
         for (int e = tt; e < TY * nx; e += nth) {  // the elements this thread stored
-            const int yl = g.fd_nx.div(e), x = e - yl * nx, y = y0 + yl;
+            const int yl = g.fd_nx.div(e), x = e - yl * nx;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const T a = rel<T, LX>(S + (c * TY + yl) * g.rsx, x);
-                fx q(0), q4(0);   // the transform's value, and 4 of its units for the stencil
+                fx q(0);
                 if (!(c < 2 ? bad_xy : bad_z) && top > 0) {
-                    if constexpr (DW) {
-                        q = fx_from(a, scalef);
-                    } else {
-                        q4 = fx(__double2ll_rn(fx_ldexp(a, sc + 2)));
-                        q = fx_shr(q4, 2);
-                    }
+                    if constexpr (DW) q = fx_from(a, scalef);
+                    else q = fx(__double2ll_rn(fx_ldexp(a, sc)));
                 }
                 rel<fx, LX>(S + (c * TY + yl) * g.rsx, x) = q;
-                if (!DW && y < ny) P.mfix[c * N + ((long)z * ny + y) * nx + x] = q4.v;
             }
         }
     }
@@ -912,26 +907,16 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     // block fixed point: largest scale and flags of the x-frequencies, the sum of their scales over the largest, and
     // the magnitude of this CTA's rows
     __shared__ int s_e;
-    __shared__ unsigned s_r[4];   // and whether the stencil's rows differ in scale
+    __shared__ unsigned s_r[3];
     unsigned mag = 0;
     const int *fe2 = nullptr;
     int emax = FX_ZERO;
-    constexpr bool INTS = std::is_same<T, double>::value;   // exchange sums over the integer copy of m, see below
     if constexpr (is_fx<F>) {
         fe2 = P.fe2 + z / g.ZB;
         if (tid == 0) s_e = FX_ZERO;
-        if (tid < 4) s_r[tid] = 0;
+        if (tid < 3) s_r[tid] = 0;
         __syncthreads();
         unsigned fl = 0;
-        unsigned differ = 0;
-        if constexpr (INTS) {   // rows y0 - 1 .. y0 + TY of planes z - 1 .. z + 1 (those that exist)
-            const int own = P.fe1[z * ny + y0];
-            differ = fx_flags(own);
-            for (int i = tt; i < 3 * (TY + 2); i += nth) {
-                const int zo = (i >= TY + 2) + (i >= 2 * (TY + 2)), zz = z - 1 + zo, y = y0 - 1 + i - zo * (TY + 2);
-                if (zz >= 0 && zz < nz && y >= 0 && y < ny) differ |= P.fe1[zz * ny + y] != own;
-            }
-        }
         for (int i = tt; i < g.C; i += nth) {
             const int p = fe2[i * g.nzb];
             emax = max(emax, fx_exp(p));
@@ -939,7 +924,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         }
         fx_cta_max(&s_e, emax);
         fx_cta_or(&s_r[0], fl);
-        if constexpr (INTS) fx_cta_or(&s_r[3], differ);
     }
 
     MinState *st = P.st;
@@ -1088,18 +1072,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             uy = pick<T>(g.u[1], g.fu[1], g.wu[1]), uz = pick<T>(g.u[2], g.fu[2], g.wu[2]);
     const T hs = (T)P.hscale;
     const T canK = can * Kuni;
-    // The exchange sums of double fields are taken over the integer copy of m
-    // where the rows share one scale and are finite: exact differences and sums
-    // on the integer pipes, converted once an axis, 18 FP64 instructions a cell
-    // instead of 36 (512 x 256 x 4: 133 -> 123 us, 64^3: 82 -> 72 us).  Double-word
-    // fields gain nothing (84 -> 86 us): their differences run on the FP32 pipes.
-    bool ints = false;
-    T cxs = 0, cys = 0, czs = 0;   // cx, cy, cz per unit of the copy
-    if constexpr (INTS) {
-        ints = s_r[3] == 0;
-        const int unit = fx_exp(P.fe1[z * ny + y0]) + 1 - fx_total(Hx) - 2;
-        cxs = fx_ldexp(cx, unit); cys = fx_ldexp(cy, unit); czs = fx_ldexp(cz, unit);
-    }
     Acc<T> red[NSL];
 #pragma unroll
     for (int s = 0; s < NSL; ++s) red[s].zero();
@@ -1137,9 +1109,7 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             d2 = to_field<T>(rel<F, LX>(S + (2 * TY + yl) * g.rsx, x));
         }
         // exchange: sum over present neighbours of (m_j - m_i) / d^2 (free faces)
-        // (the external field starts the sums where they are not wanted apart)
         T m0, m1, m2, e0 = 0, e1 = 0, e2 = 0;
-        if (MODE != MODE_ENERGY) { e0 = he0; e1 = he1; e2 = he2; }
         if (stg) {
             const int cs = (TY + 2) * nx, ct = TY * nx;    // component strides of the staged rows
             const T *r0 = SG + (yl + 1) * nx + x;          // this cell, component 0
@@ -1157,25 +1127,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             } else {
                 m0 = from_io<T>(ldg(mio + n)); m1 = from_io<T>(ldg(mio + N + n)); m2 = from_io<T>(ldg(mio + 2 * N + n));
             }
-            if (ints) {
-                if constexpr (INTS) {
-                    const int sxy = nx * ny;
-                    T *ee[3] = {&e0, &e1, &e2};
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const long long *q = P.mfix + c * N + n;
-                        const long long q0 = __ldg(q);
-                        const long long X = (x > 0 ? __ldg(q - 1) - q0 : 0) + (x < nx - 1 ? __ldg(q + 1) - q0 : 0);
-                        const long long Y = (y > 0 ? __ldg(q - nx) - q0 : 0) + (y < ny - 1 ? __ldg(q + nx) - q0 : 0);
-                        *ee[c] += cxs * __ll2double_rn(X);
-                        *ee[c] += cys * __ll2double_rn(Y);
-                        if (nz > 1) {
-                            const long long Z = (z > 0 ? __ldg(q - sxy) - q0 : 0) + (z < nz - 1 ? __ldg(q + sxy) - q0 : 0);
-                            *ee[c] += czs * __ll2double_rn(Z);
-                        }
-                    }
-                }
-            } else {
             if (x > 0)      { e0 += cx * (mval(n - 1) - m0);  e1 += cx * (mval(N + n - 1) - m1);  e2 += cx * (mval(2 * N + n - 1) - m2); }
             if (x < nx - 1) { e0 += cx * (mval(n + 1) - m0);  e1 += cx * (mval(N + n + 1) - m1);  e2 += cx * (mval(2 * N + n + 1) - m2); }
             if (y > 0)      { e0 += cy * (mval(n - nx) - m0); e1 += cy * (mval(N + n - nx) - m1); e2 += cy * (mval(2 * N + n - nx) - m2); }
@@ -1183,7 +1134,6 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             const long sxy = (long)nx * ny;
             if (z > 0)      { e0 += cz * (mval(n - sxy) - m0); e1 += cz * (mval(N + n - sxy) - m1); e2 += cz * (mval(2 * N + n - sxy) - m2); }
             if (z < nz - 1) { e0 += cz * (mval(n + sxy) - m0); e1 += cz * (mval(N + n + sxy) - m1); e2 += cz * (mval(2 * N + n + sxy) - m2); }
-            }
         }
         // uniaxial anisotropy
         const T Kv = P.Kc ? from_io<T>(P.Kc[n]) : Kuni;
@@ -1192,8 +1142,9 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         else { u0 = ux; u1 = uy; u2 = uz; }
         const T mu = m0 * u0 + m1 * u1 + m2 * u2;
         const T ka = (P.Kc ? can * Kv : canK) * mu;
-        T H0 = d0 + e0 + ka * u0, H1 = d1 + e1 + ka * u1, H2 = d2 + e2 + ka * u2;
-        if (MODE == MODE_ENERGY) { H0 += he0; H1 += he1; H2 += he2; }
+        const T H0 = d0 + e0 + ka * u0 + he0;
+        const T H1 = d1 + e1 + ka * u1 + he1;
+        const T H2 = d2 + e2 + ka * u2 + he2;
         if (MODE == MODE_HEFF) {
             P.H_out[n] = to_io(hs * H0); P.H_out[N + n] = to_io(hs * H1); P.H_out[2 * N + n] = to_io(hs * H2);
             continue;
@@ -1330,7 +1281,6 @@ template <typename T, typename F = typename fft_of<T>::type> FieldPtrs<T, F> mak
     P.gbuf[0] = (T *)p->gbuf[0]; P.gbuf[1] = (T *)p->gbuf[1];
     P.W = (V *)p->W; P.W2 = (V *)p->W2; P.Nhat = (const typename coef<F>::type *)p->Nhat;
     P.tw_px = (const TW *)p->tw_px; P.tw_py = (const TW *)p->tw_py; P.tw_pz = (const TW *)p->tw_pz;
-    P.mfix = p->mfix;
     P.fe1 = p->fexp;
     P.fea = p->fexp + (long)g.nz * g.ny;
     P.feb = P.fea + (long)g.C * g.nzb;

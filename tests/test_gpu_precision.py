@@ -1,0 +1,77 @@
+"""Terms of the field against extended precision where one of them, or one
+component, is far smaller or larger than the rest: each has to be as accurate
+as its own arithmetic, not only as the whole field's largest term."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import micromag as om
+from gpu_cases import dev, make_pair
+
+pytestmark = pytest.mark.gpu
+LD = np.longdouble
+AXES = ((3, "dx"), (2, "dy"), (1, "dz"))
+
+
+def smooth(shape, seed):
+    """Three smooth fields of order one."""
+    z, y, x = np.meshgrid(*(np.linspace(0.0, 1.0, n) for n in shape), indexing="ij")
+    r = np.random.default_rng(seed).uniform(0.5, 2.0, (3, 4))
+    return np.stack([np.cos(a * x + b * y + c * z + d) for a, b, c, d in r])
+
+
+def exchange(p, m):
+    """The exchange field in extended precision, and the sum of its terms' magnitudes."""
+    M = m.astype(LD)
+    H, mag = np.zeros_like(M), np.zeros_like(M)
+    for ax, d in AXES:
+        if m.shape[ax] < 2:
+            continue
+        c = LD(2) * LD(p.A) / (LD(om.MU0) * LD(p.Ms) * LD(getattr(p, d)) ** 2)
+        diff = c * np.diff(M, axis=ax)
+        for sign, pad in ((1, (0, 1)), (-1, (1, 0))):
+            t = np.pad(sign * diff, [pad if a == ax else (0, 0) for a in range(4)])
+            H += t
+            mag += abs(t)
+    return H, mag
+
+
+def field(mmlib, prob, m, Hext, dtype=torch.float64):
+    H = torch.empty(m.shape, dtype=dtype, device="cuda")
+    mmlib.mm_heff(prob, dev(m, dtype), Hext, H)
+    return H.cpu().numpy()
+
+
+@pytest.mark.parametrize("grid", [(1, 9, 1), (24, 7, 1), (9, 1, 2), (33, 18, 3), (9, 6, 7)])
+def test_exchange_of_a_small_component_beside_a_large_one(mmlib, grid):
+    """Differences of doubles this close are exact, so a cell's sum is off by the roundings of at most six terms: three
+    roundings each at the terms' size, 18 x 2^-53 < 2^-48 of the sum of their magnitudes.  The coefficient's own rounding
+    adds three, the demagnetisation (2^-50 Ms) nothing: the exchange field is 10^4 Ms and more here."""
+    nx, ny, nz = grid
+    prob, p = make_pair(mmlib, nx, ny, nz, (1e-9, 1.1e-9, 0.9e-9), Ms=1e3, A=1e-11, K=0.0)
+    for big in range(3):
+        m = 1e-6 * smooth(p.shape, 7 + big)
+        m[big] = 1.0
+        H = field(mmlib, prob, m, (0, 0, 0))
+        ref, mag = exchange(p, m)
+        ref = ref + om.Demag(p).field(m)
+        assert np.all(abs(H - ref) <= 2.0 ** -48 * mag + 2.0 ** -49 * p.Ms)
+
+
+@pytest.mark.parametrize("prec,dtype,h", [("MM_FP64", torch.float64, 2.0 ** 42), ("MM_FP32", torch.float32, 2.0 ** 34)])
+@pytest.mark.parametrize("grid", [(24, 7, 1), (9, 6, 3), (8, 9, 7)])
+def test_large_external_field_is_rounded_once(mmlib, grid, prec, dtype, h):
+    """The other terms (below 2^22 A/m) are summed first: a component is off by half a unit in the last place of the
+    external field and the terms' own error, at most 2^-42 (FP64) and 2^-16 (FP32) of 2^22."""
+    nx, ny, nz = grid
+    prob, p = make_pair(mmlib, nx, ny, nz, (4e-9, 3e-9, 5e-9), A=1.3e-11, K=2e4, u=(0.6, 0.0, 0.8),
+                        precision=getattr(mmlib, prec))
+    m = smooth(p.shape, 3)
+    m = (m / np.sqrt((m * m).sum(0))).astype(np.float32).astype(np.float64)
+    ref = om.heff(p, m, np.zeros(3), om.Demag(p))
+    assert np.max(abs(ref)) < 2.0 ** 22
+    Hext = np.array([1.25 * h, -1.5 * h, 1.75 * h])      # exact in either type; sums stay in the same binade
+    H = field(mmlib, prob, m, Hext, dtype).astype(LD)
+    ulp = h * 2.0 ** (-52 if prec == "MM_FP64" else -23)
+    own = 2.0 ** 22 * (2.0 ** -42 if prec == "MM_FP64" else 2.0 ** -16)
+    assert np.max(abs(H - (ref.astype(LD) + Hext.reshape(3, 1, 1, 1)))) <= 0.5 * ulp + own
