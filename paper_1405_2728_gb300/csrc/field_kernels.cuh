@@ -46,6 +46,11 @@ template <> __device__ __forceinline__ dfloat inv_sqrt<dfloat>(dfloat x) { retur
 __device__ __forceinline__ float renorm_scale(float s) { return rsqrtf(s); }
 __device__ __forceinline__ dfloat renorm_scale(dfloat s) { return df_rsqrt(s); }
 
+// a product that is not contracted into a sum: the same rounded value wherever it is used
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ dfloat mul_rn(dfloat a, dfloat b) { return a * b; }
+
 // ordered bits of |x|'s high part, at or above those of infinity if x is not finite
 __device__ __forceinline__ int magnitude(double x) { return __double2hiint(x) & 0x7fffffff; }
 __device__ __forceinline__ int magnitude(dfloat x) { return __float_as_int(x.hi) & 0x7fffffff; }
@@ -812,7 +817,7 @@ __device__ __forceinline__ A reduce_slots(A (&r)[NSL], A *sm, const int tid, con
 // division and one square root: one after another they took several
 // microseconds of dependent FP64 instructions.
 template <int MODE>
-__device__ __forceinline__ void finish_iteration(const Geom &g, double mine, const double *hext, MinState *st,
+__device__ __forceinline__ void finish_iteration(const Geom &g, double mine, MinState *st,
                                                  cudaGraphConditionalHandle h, int use_cond, int body_kernels)
 {
     const int lane = threadIdx.x & 31;
@@ -848,9 +853,7 @@ __device__ __forceinline__ void finish_iteration(const Geom &g, double mine, con
     st->bb[0] = k > 0 ? ss : 0.0;
     st->bb[1] = k > 0 ? sy : 0.0;
     st->bb[2] = k > 0 ? yy : 0.0;
-    // the slot holds the sum of m.H - 2 K/(mu0 Ms) with per-cell K, of m.H with a uniform one
-    const double mhe = tot[SL_MX] * hext[0] + tot[SL_MY] * hext[1] + tot[SL_MZ] * hext[2];
-    st->energy[4] = cE * (-0.5 * (tot[SL_ET] + mhe)) + hext[3];
+    st->energy[4] = -0.5 * cE * tot[SL_ET];
     st->evals = k + 1;
     st->launches += body_kernels;
     if (k == 0) st->t_start_ns = globaltimer_ns();
@@ -1071,7 +1074,7 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     const T Kuni = pick<T>(g.K, g.fK, g.wK), ux = pick<T>(g.u[0], g.fu[0], g.wu[0]),
             uy = pick<T>(g.u[1], g.fu[1], g.wu[1]), uz = pick<T>(g.u[2], g.fu[2], g.wu[2]);
     const T hs = (T)P.hscale;
-    const T canK = can * Kuni;
+    const T canK = mul_rn(can, Kuni);
     Acc<T> red[NSL];
 #pragma unroll
     for (int s = 0; s < NSL; ++s) red[s].zero();
@@ -1141,7 +1144,8 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         if (P.uc) { u0 = from_io<T>(P.uc[n]); u1 = from_io<T>(P.uc[N + n]); u2 = from_io<T>(P.uc[2 * N + n]); }
         else { u0 = ux; u1 = uy; u2 = uz; }
         const T mu = m0 * u0 + m1 * u1 + m2 * u2;
-        const T ka = (P.Kc ? can * Kv : canK) * mu;
+        const T kc = P.Kc ? mul_rn(can, Kv) : canK;
+        const T ka = kc * mu;
         const T H0 = d0 + e0 + ka * u0 + he0;
         const T H1 = d1 + e1 + ka * u1 + he1;
         const T H2 = d2 + e2 + ka * u2 + he2;
@@ -1172,14 +1176,16 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         const T mm = m0 * m0 + m1 * m1 + m2 * m2;
         const T g0 = mh * m0 - mm * H0, g1 = mh * m1 - mm * H1, g2 = mh * m2 - mm * H2;
         red[SL_T2].maxv(g0 * g0 + g1 * g1 + g2 * g2);  // |m x H|^2 = |g|^2 for |m| = 1
-        // energy density / (mu0 Ms V): -(m.H + m.H_ext)/2 + K/(mu0 Ms).  The slot
-        // sums m.H; the Zeeman part follows from the sums of m, the constant of a
-        // uniform K from the cell count (finish_iteration)
+        // energy density / (mu0 Ms V), times -2: m.H + m.H_ext - 2 K/(mu0 Ms), complete
+        // in every cell and with the field's own rounded 2 K/(mu0 Ms): a hard magnet's
+        // terms cancel to a small part of K there, and sums of them apart would not
+        const T mhe = m0 * he0 + m1 * he1 + m2 * he2;
         if constexpr (sizeof(T) == 4) {
             red[SL_ET].add_prod(m0, H0); red[SL_ET].add_prod(m1, H1); red[SL_ET].add_prod(m2, H2);
-            if (P.Kc) red[SL_ET].add_prod(-can, Kv);
+            red[SL_ET].add_prod(m0, he0); red[SL_ET].add_prod(m1, he1); red[SL_ET].add_prod(m2, he2);
+            red[SL_ET].add(-kc);
         } else {
-            red[SL_ET].add(P.Kc ? mh - can * Kv : mh);
+            red[SL_ET].add((mh + mhe) - kc);
         }
         T *gout = (k & 1) ? P.gbuf[1] : P.gbuf[0];
         if (k > 0) {
@@ -1248,12 +1254,7 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
         }
         const Acc<double> t = reduce_slots<MODE>(v, reinterpret_cast<Acc<double> *>(smem_raw), tid, nth);
         if (warp == 0) {
-            double fin[4] = {0.0, 0.0, 0.0, 0.0};   // external field, energy of a uniform K
-            if (MODE == MODE_MIN) {
-                fin[0] = st->Hext[0]; fin[1] = st->Hext[1]; fin[2] = st->Hext[2];
-                if (!P.Kc) fin[3] = g.K * g.dx * g.dy * g.dz * (double)g.N;
-            }
-            finish_iteration<MODE>(g, t.v, fin, st, h, use_cond, g.nbody);
+            finish_iteration<MODE>(g, t.v, st, h, use_cond, g.nbody);
             if (lane == 0) *P.counter = 0u;
         }
     }

@@ -75,3 +75,28 @@ def test_large_external_field_is_rounded_once(mmlib, grid, prec, dtype, h):
     ulp = h * 2.0 ** (-52 if prec == "MM_FP64" else -23)
     own = 2.0 ** 22 * (2.0 ** -42 if prec == "MM_FP64" else 2.0 ** -16)
     assert np.max(abs(H - (ref.astype(LD) + Hext.reshape(3, 1, 1, 1)))) <= 0.5 * ulp + own
+
+
+@pytest.mark.parametrize("prec,u,floor", [("MM_FP64", 2.0 ** -53, 2.0 ** -50), ("MM_F32X2", 2.0 ** -47, 2.0 ** -44),
+                                          ("MM_FP32", 2.0 ** -24, 2.0 ** -20)])
+@pytest.mark.parametrize("Ms,K,tilt", [(1.28e6, 4.3e6, 0.1), (3e5, 6e6, 1e-3), (8e5, 500.0, 0.1)])
+def test_energy_of_a_minimisation_with_a_large_uniform_anisotropy(mmlib, Ms, K, tilt, prec, u, floor):
+    """The cells' anisotropy terms cancel against 2 K/(mu0 Ms) before they are summed, so what is left of K V N in the
+    sum is each cell's own rounding: about 4 u K V, of either sign, 16 u K V N / sqrt(N) at four standard deviations.
+    `floor` covers the other terms."""
+    nx, ny, nz = 256, 128, 2
+    N = nx * ny * nz
+    cell = (4e-9, 4e-9, 5e-9)
+    single = prec == "MM_FP32"
+    Hext = np.array([5e4, 0.0, 2e4])
+    m = tilt * np.random.default_rng(5).standard_normal((3, nz, ny, nx))
+    m[0] += 1.0
+    m /= np.sqrt((m * m).sum(0))
+    m = m.astype(np.float32).astype(np.float64) if single else m
+    prob, p = make_pair(mmlib, nx, ny, nz, cell, Ms=Ms, A=1e-11, K=K, precision=getattr(mmlib, prec))
+    _, r = mmlib.mm_minimize(prob, dev(m, torch.float32 if single else torch.float64), Hext, mmlib.make_opts(max_iter=0))
+    double, _ = make_pair(mmlib, nx, ny, nz, cell, Ms=Ms, A=1e-11, K=K)
+    M, V, c = m.astype(LD), LD(cell[0]) * LD(cell[1]) * LD(cell[2]), LD(om.MU0) * LD(Ms)
+    ref = LD(mmlib.mm_energy(double, dev(m), Hext)[0]) - c * V / 2 * (M * exchange(p, m)[0]).sum()
+    ref += LD(K) * V * (1 - M[0] ** 2).sum() - c * V * (M * Hext.astype(LD).reshape(3, 1, 1, 1)).sum()
+    assert abs(r.energy - ref) <= 16 * u * float(K * V) * N ** 0.5 + floor * float(abs(ref))
