@@ -24,6 +24,9 @@ namespace {
 // log2 of a power of two (ZB, KB)
 __device__ __forceinline__ int log2_of(int p) { return 31 - __clz(p); }
 
+// the tensor couples all components: no axis of one cell
+__host__ __device__ __forceinline__ bool coupled(const Geom &g) { return g.nx > 1 && g.ny > 1 && g.nz > 1; }
+
 template <typename V> __device__ __forceinline__ V load_cg(const V *p) { return __ldcg(p); }
 template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
 {
@@ -40,17 +43,18 @@ constexpr int Z_CTAS = 2;
 template <typename T> constexpr int Y_BOUND = sizeof(T) == 8 ? 384 : 512;
 
 // In block fixed point (double fields, F = fx) every CTA of a pass brings its
-// block to full magnitude when it loads it and when it stores it, with the
-// scale of a block per (kx, ZB planes) after the y passes and per (kx, KB
-// y-frequencies) after the z convolution.
+// block to full magnitude when it loads it and when it stores it, component by
+// component, with the scales of a block per (kx, ZB planes) after the y passes
+// and per (kx, KB y-frequencies) after the z convolution.
 template <typename T, bool INV, int LY>
 __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
 {
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
     constexpr bool FX = std::is_same<V, fxc>::value;
-    __shared__ int s_e;
-    __shared__ unsigned s_r[3];  // flags, magnitudes in and out
+    __shared__ int s_e[3];
+    __shared__ unsigned s_r[7];  // flags, magnitudes in and out
+    unsigned *s_fl = s_r, *s_in = s_r + 1, *s_out = s_r + 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -59,24 +63,15 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
     const int zb = min(ZB, nz - z0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * ZB * rs);
     load_twiddles_async(tw, P.tw_py, Py, Py, tid, nth);
-    int emax = FX_ZERO;
-    unsigned mag = 0;
-    const int *scales = nullptr;   // of the values read: one per (z, y) row of W, or per KB y-frequencies of W2
+    fx3 mags;
+    const int *scales = nullptr;   // of the values read: of every (z, y) row of W, or of KB y-frequencies of W2
     if constexpr (FX) {
-        if (tid == 0) s_e = FX_ZERO;
-        if (tid < 3) s_r[tid] = 0;
+        if (tid < 3) s_e[tid] = FX_ZERO;
+        if (tid < 7) s_r[tid] = 0;
         __syncthreads();
-        scales = INV ? P.feb + (long)kx * g.nkb : P.fe1 + (long)z0 * ny;
-        const int n = INV ? g.nkb : zb * ny;
-        unsigned fl = 0;
-        for (int i = tid; i < n; i += nth) {
-            emax = max(emax, fx_exp(scales[i]));
-            fl |= fx_flags(scales[i]);
-        }
-        fx_cta_max(&s_e, emax);
-        fx_cta_or(&s_r[0], fl);
+        scales = INV ? P.feb + (long)kx * g.nkb * 3 : P.fe1 + (long)z0 * ny * 3;
+        fx_cta_scales(scales, INV ? g.nkb : zb * ny, 3, tid, nth, s_e, s_fl);
         __syncthreads();
-        emax = s_e;
     }
     const long first = (long)kx * nz + z0;  // first (kx, z) row pair of this CTA
     const int lin = INV ? Py : ny;           // input length per (z, c) row
@@ -97,8 +92,8 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zl = INV ? rest / Py : g.fd_ny.div(rest), y = rest - zl * lin;
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[INV ? y >> log2_of(g.KB) : rest]) - emax);
-                mag |= fx_mag(v[i]);
+                v[i] = fx_scale(v[i], fx_exp(scales[INV ? (y >> log2_of(g.KB)) * 3 + c : e]) - s_e[c]);
+                mags.or_in(c, fx_mag(v[i]));
             }
             S[(c * ZB + zl) * rs + rpos<V, LY>(y)] = v[i];
         }
@@ -110,39 +105,39 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             S[r * rs + rpos<V, LY>(y)] = czero<V>();
         }
     }
-    if constexpr (FX) fx_cta_or(&s_r[1], mag);
+    if constexpr (FX) mags.cta_or(s_in);
     cp_async_wait_all();
     __syncthreads();
     const int Gy = g.Gy, RB = g.RBY;
     const int rb = tid / Gy, j = tid - rb * Gy;
-    const int pre = FX ? (INV ? 58 : 59) - fx_bits(s_r[1]) : 0;
+    auto pre = [&](int c) { return (INV ? 58 : 59) - fx_bits(s_in[c]); };
     int sh = 0;
-    mag = 0;
+    mags = fx3();
     for (int r0 = 0; r0 < 3 * ZB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * ZB && (r % ZB) < zb;
-        if constexpr (FX)
-            sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, pre, 64, mag);
-        else
+        if constexpr (FX) {
+            const int c = act ? r >> log2_of(ZB) : 0;
+            unsigned mag = 0;
+            sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, pre(c), 64, mag);
+            mags.or_in(c, mag);
+        } else
             fft_row<INV, !INV, INV, 1, LY>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act);
     }
-    int post = 0;
+    auto post = [&](int c) { return 60 - fx_bits(s_out[c]); };
+    if constexpr (FX) mags.cta_or(s_out);
+    __syncthreads();
     if constexpr (FX) {
-        fx_cta_or(&s_r[2], mag);
-        __syncthreads();
-        post = 60 - fx_bits(s_r[2]);
-        if (tid == 0)
-            (INV ? P.fe2 : P.fea)[(long)kx * g.nzb + blockIdx.y] =
-                fx_pack(emax - pre + sh - post, s_r[0] ? 3 : 0);  // the tensor mixes all components
-    } else {
-        __syncthreads();
+        if (tid < 3)
+            (INV ? P.fe2 : P.fea)[((long)kx * g.nzb + blockIdx.y) * 3 + tid] =
+                fx_pack(s_e[tid] - pre(tid) + sh - post(tid), *s_fl >> tid & 1);
     }
     const int lout = INV ? ny : Py;
     V *dst = INV ? P.W + first * ny * 3 : P.W2 + first * Py * 3;
     for (int e = tid; e < zb * lout * 3; e += nth) {
         const int c = e % 3, rest = e / 3, zl = INV ? g.fd_ny.div(rest) : rest / Py, y = rest - zl * lout;
         V r = S[(c * ZB + zl) * rs + rpos<V, LY>(y)];
-        if constexpr (FX) r = fx_scale(r, post);
+        if constexpr (FX) r = fx_scale(r, post(c));
         dst[e] = r;
     }
 }
@@ -153,9 +148,10 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
     constexpr bool FX = std::is_same<V, fxc>::value;
-    __shared__ int s_e;
-    __shared__ int s_top;
-    __shared__ unsigned s_r[4];  // flags, magnitudes in and out, sum of the frequencies' scales over the largest
+    __shared__ int s_e[3], s_top[3];
+    // magnitudes in and out, sums of the frequencies' scales over the largest, flags
+    __shared__ unsigned s_r[10];
+    unsigned *s_in = s_r, *s_out = s_r + 3, *s_sum = s_r + 6, *s_fl = s_r + 9;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -164,23 +160,15 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     const int kb = min(KB, Py - ky0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * KB * rs);
     load_twiddles_async(tw, P.tw_pz, Pz, Pz, tid, nth);
-    int emax = FX_ZERO;
-    unsigned mag = 0;
+    fx3 mags;
     const int *scales = nullptr;
     if constexpr (FX) {
-        if (tid == 0) { s_e = FX_ZERO; s_top = FX_ZERO; }
-        if (tid < 4) s_r[tid] = 0;
+        if (tid < 3) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
+        if (tid < 10) s_r[tid] = 0;
         __syncthreads();
-        scales = P.fea + (long)kx * g.nzb;
-        unsigned fl = 0;
-        for (int i = tid; i < g.nzb; i += nth) {
-            emax = max(emax, fx_exp(scales[i]));
-            fl |= fx_flags(scales[i]);
-        }
-        fx_cta_max(&s_e, emax);
-        fx_cta_or(&s_r[0], fl);
+        scales = P.fea + (long)kx * g.nzb * 3;
+        fx_cta_scales(scales, g.nzb, 3, tid, nth, s_e, s_fl);
         __syncthreads();
-        emax = s_e;
     }
     // i = z * kb + kyl: a whole block of KB = 2^lkb frequencies, or the last one
     auto split = [&](int i, int &kyl, int &z) {
@@ -213,8 +201,8 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             int kyl, z;
             split(e / 3, kyl, z);
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[z >> log2_of(g.ZB)]) - emax);
-                mag |= fx_mag(v[i]);
+                v[i] = fx_scale(v[i], fx_exp(scales[(z >> log2_of(g.ZB)) * 3 + c]) - s_e[c]);
+                mags.or_in(c, fx_mag(v[i]));
             }
             S[(c * KB + kyl) * rs + rpos<V, LZ>(z)] = v[i];
         }
@@ -224,23 +212,38 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         const int r = g.fd_padz.div(e), z = nz + (e - r * npad);
         S[r * rs + rpos<V, LZ>(z)] = czero<V>();
     }
-    if constexpr (FX) fx_cta_or(&s_r[1], mag);
+    if constexpr (FX) mags.cta_or(s_in);
     cp_async_wait_all();
     __syncthreads();
     const int Gz = g.Gz, RB = g.RBZ;
     const int rb = tid / Gz, j = tid - rb * Gz;
-    signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));  // [2][KB][Pz]: scale and top bit of a frequency
-    int pre = FX ? 59 - fx_bits(s_r[1]) : 0, sh = 0, top = FX_ZERO;
+    // scales [1 or 3][KB][Pz] and top bits [3][KB][Pz] of the frequencies: components that are all coupled share the scales
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));
+    const int own_sc = coupled(g) ? 0 : KB * Pz;   // from one component's scales to the next's
+    signed char *s_tk = s_sc + 2 * own_sc + KB * Pz;
+    int sh = 0;
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
-        if constexpr (FX)
-            sh = fft_row_fx<false, true, false, 1, LZ, false>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, pre, 64, mag);
-        else
+        if constexpr (FX) {
+            unsigned none = 0;
+            sh = fft_row_fx<false, true, false, 1, LZ, false>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act,
+                                                              59 - fx_bits(s_in[act ? r >> lkb : 0]), 64, none);
+        } else {
             fft_row<false, true, false, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
+        }
     }
     __syncthreads();
-    if constexpr (FX) emax += sh - pre + P.fek[kx];
+    int eb[3], d[3], top[3] = {FX_ZERO, FX_ZERO, FX_ZERO};   // a component's scale where it is mixed, its own over that
+    const FxCouple couple{g.nx > 1 && g.ny > 1, g.nx > 1 && nz > 1, g.ny > 1 && nz > 1};
+    if constexpr (FX) {
+        int own[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) eb[c] = own[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+        couple.join(eb[0], eb[1], eb[2]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = own[c] - eb[c];
+    }
     // tensor product per (ky, kz); octant storage [kx][kzr][kyr][6] with the
     // off-diagonal signs of the reflected frequencies
     const int hy = Py / 2, hz = Pz / 2;
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         V *a1 = S + (1 * KB + kyl) * rs + rpos<V, LZ>(kz);
         V *a2 = S + (2 * KB + kyl) * rs + rpos<V, LZ>(kz);
         if constexpr (FX) {
-            // one scale per frequency: inputs below 2^59, outputs below 2^59
+            // one scale per frequency and coupled components: inputs below 2^59, outputs below 2^59
             auto element = [&](int c, bool neg) {
                 const int2 w = __ldg(reinterpret_cast<const int2 *>(n6 + c));
                 return fxk(fxk(fxm{w.x, w.y}), neg);
@@ -263,8 +266,11 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             const fxk k[6] = {element(0, false), element(1, false), element(2, false), element(3, ky > hy),
                               element(4, kz > hz), element(5, (ky > hy) != (kz > hz))};
             fxc m0 = *a0, m1 = *a1, m2 = *a2;
-            const int sc = 59 - fx_bits(fx_mag(m0) | fx_mag(m1) | fx_mag(m2));
-            m0 = fx_scale(m0, sc); m1 = fx_scale(m1, sc); m2 = fx_scale(m2, sc);
+            int sc[3] = {fx_bits(fx_mag(m0)) + d[0], fx_bits(fx_mag(m1)) + d[1], fx_bits(fx_mag(m2)) + d[2]};
+            couple.join(sc[0], sc[1], sc[2]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sc[c] = 59 - sc[c];
+            m0 = fx_scale(m0, sc[0] + d[0]); m1 = fx_scale(m1, sc[1] + d[1]); m2 = fx_scale(m2, sc[2] + d[2]);
             auto row = [&](const fxk &p, const fxk &q, const fxk &r, fx x, fx y, fx z) {
                 fxdot h;
                 h.zero();
@@ -276,10 +282,13 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             const fxc h0{row(k[0], k[3], k[4], m0.x, m1.x, m2.x), row(k[0], k[3], k[4], m0.y, m1.y, m2.y)};
             const fxc h1{row(k[3], k[1], k[5], m0.x, m1.x, m2.x), row(k[3], k[1], k[5], m0.y, m1.y, m2.y)};
             const fxc h2{row(k[4], k[5], k[2], m0.x, m1.x, m2.x), row(k[4], k[5], k[2], m0.y, m1.y, m2.y)};
-            const int tk = fx_bits(fx_mag(h0) | fx_mag(h1) | fx_mag(h2)) - sc;
-            s_sc[kyl * Pz + kz] = (signed char)sc;
-            s_sc[(KB + kyl) * Pz + kz] = (signed char)tk;
-            top = max(top, tk);
+            const int tk[3] = {fx_bits(fx_mag(h0)) - sc[0], fx_bits(fx_mag(h1)) - sc[1], fx_bits(fx_mag(h2)) - sc[2]};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                s_sc[c * own_sc + kyl * Pz + kz] = (signed char)sc[c];
+                s_tk[(c * KB + kyl) * Pz + kz] = (signed char)tk[c];
+                top[c] = max(top[c], tk[c]);
+            }
             *a0 = h0; *a1 = h1; *a2 = h2;
         } else {
         const T sy = ky <= hy ? (T)1 : (T)-1, sz = kz <= hz ? (T)1 : (T)-1;
@@ -296,46 +305,58 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         *a0 = h0; *a1 = h1; *a2 = h2;
         }
     }
-    int t = 64;
-    if constexpr (FX) fx_cta_max(&s_top, top);
+    if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_cta_max(&s_top[c], top[c]);
+    }
     __syncthreads();
     if constexpr (FX) {
         // no partial sum of an inverse transform exceeds the sum of the largest moduli over kz
-        top = s_top;
-        unsigned sum = 0;
+        unsigned sum[3] = {0, 0, 0};
         for (int e = tid; e < Pz; e += nth) {
-            int tk = FX_ZERO;
-            for (int kyl = 0; kyl < kb; ++kyl) tk = max(tk, (int)s_sc[(KB + kyl) * Pz + e]);
-            sum += ((1u << 18) >> min(top - tk, 18)) + 1;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                int tk = FX_ZERO;
+                for (int kyl = 0; kyl < kb; ++kyl) tk = max(tk, (int)s_tk[(c * KB + kyl) * Pz + e]);
+                sum[c] += ((1u << 18) >> min(s_top[c] - tk, 18)) + 1;
+            }
         }
-        fx_cta_add(&s_r[3], sum);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
         __syncthreads();
-        pre = 58 - top;
-        t = max(0, fx_log2_up(s_r[3]) - 18);
-        mag = 0;
+        mags = fx3();
     }
+    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
-        if constexpr (FX)
-            sh = fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, pre, t,
-                                                                  mag, s_sc + (act ? r % KB : 0) * Pz);
-        else
+        if constexpr (FX) {
+            const int c = act ? r >> lkb : 0;
+            unsigned mag = 0;
+            fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, 58 - s_top[c],
+                                                             bound(c), mag,
+                                                             s_sc + c * own_sc + (act ? r & (KB - 1) : 0) * Pz);
+            mags.or_in(c, mag);
+        } else {
             fft_row<true, false, true, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
+        }
     }
-    if constexpr (FX) fx_cta_or(&s_r[2], mag);
+    auto post = [&](int c) { return 60 - fx_bits(s_out[c]); };
+    if constexpr (FX) mags.cta_or(s_out);
     __syncthreads();
-    int post = 0;
     if constexpr (FX) {
-        post = 60 - fx_bits(s_r[2]);
-        if (tid == 0) P.feb[(long)kx * g.nkb + blockIdx.y] = fx_pack(emax + sh - pre - post, s_r[0] ? 3 : 0);
+        if (tid < 3) {
+            const int c = tid, e = (c == 0 ? eb[0] : (c == 1 ? eb[1] : eb[2])) + P.fek[kx] +
+                                   fx_cum(fx_log(Pz), bound(c)) - (58 - s_top[c]) - post(c);
+            P.feb[((long)kx * g.nkb + blockIdx.y) * 3 + c] = fx_pack(e, *s_fl ? 1 : 0);  // the tensor mixes all components
+        }
     }
     for (int e = tid; e < nz * kb * 3; e += nth) {
         const int c = e % 3;
         int kyl, z;
         split(e / 3, kyl, z);
         V r = S[(c * KB + kyl) * rs + rpos<V, LZ>(z)];
-        if constexpr (FX) r = fx_scale(r, post);
+        if constexpr (FX) r = fx_scale(r, post(c));
         base[(long)z * zs + kyl * 3 + c] = r;
     }
 }
@@ -350,8 +371,8 @@ template <typename T> size_t smem_y_t(const Geom &g, int zb)
 template <typename T> size_t smem_z_t(const Geom &g, int kb)
 {
     typedef typename cvec<T>::type V;
-    // and two bytes per frequency of a block fixed-point transform
-    return ((size_t)3 * kb * g.rsz + tw_slots(g.Pz)) * sizeof(V) + (sizeof(T) == 8 ? (size_t)2 * kb * g.Pz : 0);
+    // and the bytes per frequency of a block fixed-point transform: scales, and a top bit per component
+    return ((size_t)3 * kb * g.rsz + tw_slots(g.Pz)) * sizeof(V) + (sizeof(T) == 8 ? (size_t)(coupled(g) ? 4 : 6) * kb * g.Pz : 0);
 }
 
 template <typename T> cudaError_t bulk_conv_t(const Geom &g, const FieldPtrs<T> &P, cudaStream_t s, int pass)

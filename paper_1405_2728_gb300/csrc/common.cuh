@@ -269,11 +269,11 @@ struct FieldPtrs {
     const TW *tw_px;       // exp(-2 pi i t/Px), t < Px
     const TW *tw_py;       // exp(-2 pi i t/Py), t < Py
     const TW *tw_pz;       // exp(-2 pi i t/Pz), t < Pz
-    // block fixed point only (F = fx): the scales of the blocks (fx_pack)
-    int *fe1;              // [nz][ny] of W as the x-forward kernel writes it
-    int *fea;              // [C][nzb] bulk: of W2 after the y transform
-    int *feb;              // [C][nkb] bulk: of W2 after the z convolution
-    int *fe2;              // [C][nzb] of W as the y-z stage leaves it
+    // block fixed point only (F = fx): the scales of the blocks (fx_pack), one per component
+    int *fe1;              // [nz][ny][3] of W as the x-forward kernel writes it
+    int *fea;              // [C][nzb][3] bulk: of W2 after the y transform
+    int *feb;              // [C][nkb][3] bulk: of W2 after the z convolution
+    int *fe2;              // [C][nzb][3] of W as the y-z stage leaves it
     const int *fek;        // [C] exponents of the tensor
     const IO *Kc;          // per-cell K or NULL
     const IO *uc;          // per-cell axis [3][N] or NULL
@@ -369,11 +369,9 @@ inline int mm_film_coefs(const Geom &g, int precision)
     return nzm == 1 ? 4 : (nzm == 2 ? 10 : 32);
 }
 
-// ints of mm_problem::fexp
-inline size_t mm_scale_count(const Geom &g)
-{
-    return (size_t)g.nz * g.ny + (size_t)g.C * (2 * g.nzb + g.nkb + 1);
-}
+// ints of mm_problem::fexp: three per block, and where fek (one per x-frequency) starts
+inline size_t mm_scale_fek(const Geom &g) { return 3 * ((size_t)g.nz * g.ny + (size_t)g.C * (2 * g.nzb + g.nkb)); }
+inline size_t mm_scale_count(const Geom &g) { return mm_scale_fek(g) + g.C; }
 
 // launchers implemented in heff.cu
 int mm_launch_min_body(mm_problem *p, cudaGraphConditionalHandle h, cudaStream_t s, int use_cond);

@@ -467,6 +467,13 @@ __host__ __device__ __forceinline__ constexpr int fx_cum(int q, int t)
     return m > 3 ? m - 3 : 0;
 }
 
+// q of a whole row of length L
+__host__ __device__ constexpr int fx_log(int L)
+{
+    const int l = pow2_part(L), odd = L >> l;
+    return l + (odd == 25 ? 5 : (odd == 5 ? 3 : (odd == 3 ? 2 : 0)));
+}
+
 template <bool INV, bool HIN> __device__ __forceinline__ void dft8_fx(fxc *a)
 {
     // sqrt(1/2) in units of 2^-61

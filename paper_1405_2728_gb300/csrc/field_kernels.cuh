@@ -115,10 +115,10 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
     const long N = g.N;
     TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);  // Px twiddles exp(-2 pi i t / Px)
     for (int i = tt; i < Px; i += nth) tw[tpos<TW>(i, g.Hx)] = P.tw_px[i];
-    __shared__ int s_max[2];       // block fixed point: high words of the tile's largest |m_x|, |m_y| and |m_z|
-    int max_xy = 0, max_z = 0;
+    __shared__ int s_max[3];       // block fixed point: high words of the tile's largest components
+    int mmax[3] = {0, 0, 0};
     if constexpr (is_fx<F>) {
-        if (tid < 2) s_max[tid] = 0;
+        if (tid < 3) s_max[tid] = 0;
         __syncthreads();
     }
 
@@ -183,8 +183,9 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             }
         }
         if constexpr (is_fx<F>) {  // as they are, until the tile's scale is known
-            max_xy = max(max_xy, max(magnitude(m0), magnitude(m1)));
-            max_z = max(max_z, magnitude(m2));
+            mmax[0] = max(mmax[0], magnitude(m0));
+            mmax[1] = max(mmax[1], magnitude(m1));
+            mmax[2] = max(mmax[2], magnitude(m2));
             rel<T, LX>(S + (0 * TY + yl) * g.rsx, x) = m0;
             rel<T, LX>(S + (1 * TY + yl) * g.rsx, x) = m1;
             rel<T, LX>(S + (2 * TY + yl) * g.rsx, x) = m2;
@@ -194,30 +195,37 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             rel<F, LX>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
         }
     }
-    int e1 = 0;
+    int e1[3] = {0, 0, 0};
     if constexpr (is_fx<F>) {
-        // the tile's scale 2^s: its largest component becomes 2^57 .. 2^58 (one up to 1 + 2^-8 counts as 1, so that
-        // unit vectors and their rounding share one scale); non-finite components are taken as zero and flagged
-        fx_cta_max(&s_max[0], max_xy);
-        fx_cta_max(&s_max[1], max_z);
+        // the tile's scales 2^s, one per component: its largest value becomes 2^57 .. 2^58 (one up to 1 + 2^-8 counts
+        // as 1, so that unit vectors and their rounding share one scale); a non-finite component is taken as zero and
+        // flagged
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_cta_max(&s_max[c], mmax[c]);
         __syncthreads();
         constexpr bool DW = std::is_same<T, dfloat>::value;
         constexpr int inf = DW ? 0x7f800000 : 0x7ff00000, mant = DW ? 23 : 20, bias = DW ? 126 : 1022;
-        const bool bad_xy = s_max[0] >= inf, bad_z = s_max[1] >= inf;
-        const int top = max(bad_xy ? 0 : s_max[0], bad_z ? 0 : s_max[1]);
-        const int top_e = ((top - (1 << (mant - 8))) >> mant) - bias, sc = min(58 - top_e, DW ? 150 : 1000);
-        e1 = fx_pack(top > 0 ? -sc - 1 : FX_ZERO, (bad_xy ? 1 : 0) | (bad_z ? 2 : 0));
-        float scalef = 0.0f;
-        if constexpr (DW) scalef = top > 0 ? fx_pow2f(sc - 28) : 0.0f;
+        int sc[3];
+        float scalef[3];
+        bool use[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const bool bad = s_max[c] >= inf;
+            const int top = bad ? 0 : s_max[c], top_e = ((top - (1 << (mant - 8))) >> mant) - bias;
+            sc[c] = min(58 - top_e, DW ? 150 : 1000);
+            use[c] = top > 0;
+            scalef[c] = DW ? fx_pow2f(sc[c] - 28) : 0.0f;
+            e1[c] = fx_pack(top > 0 ? -sc[c] - 1 : FX_ZERO, bad ? 1 : 0);
+        }
         for (int e = tt; e < TY * nx; e += nth) {  // the elements this thread stored
             const int yl = g.fd_nx.div(e), x = e - yl * nx;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const T a = rel<T, LX>(S + (c * TY + yl) * g.rsx, x);
                 fx q(0);
-                if (!(c < 2 ? bad_xy : bad_z) && top > 0) {
-                    if constexpr (DW) q = fx_from(a, scalef);
-                    else q = fx(__double2ll_rn(fx_ldexp(a, sc)));
+                if (use[c]) {
+                    if constexpr (DW) q = fx_from(a, scalef[c]);
+                    else q = fx(__double2ll_rn(fx_ldexp(a, sc[c])));
                 }
                 rel<fx, LX>(S + (c * TY + yl) * g.rsx, x) = q;
             }
@@ -236,9 +244,12 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
         const bool act = row < 3 * TY;
         if constexpr (is_fx<F>) {
             unsigned none = 0;
-            e1 += fx_pack(fft_row_fx<false, true, false, 2, LX, false>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j,
-                                                                       tw, act, 0, 64, none), 0);
-            if (tid < TY && y0 + tid < ny) P.fe1[z * ny + y0 + tid] = e1;
+            const int sh = fft_row_fx<false, true, false, 2, LX, false>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j,
+                                                                        tw, act, 0, 64, none);
+            if (tid < TY && y0 + tid < ny) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) P.fe1[(z * ny + y0 + tid) * 3 + c] = e1[c] + fx_pack(sh, 0);
+            }
         } else {
             fft_row<false, true, false, 2, LX>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j, tw, act);
         }
@@ -388,26 +399,29 @@ template <int NZM> struct ZConv {
     }
 };
 
-// The same stage in block fixed point (F = fx), one scale per x-frequency.
-// The plane is brought to full magnitude when it is loaded, before the inverse
-// transform and when it is stored; the z convolution, where the tensor scales
-// each frequency differently, has a scale per ky.
+// The same stage in block fixed point (F = fx), one scale per x-frequency and
+// component.  The plane is brought to full magnitude when it is loaded, before
+// the inverse transform and when it is stored; the z convolution, where the
+// tensor scales each frequency differently, has a scale per ky, which the
+// components that the tensor couples share.
 template <int PZ, int LY>
 __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double, fx> &P, const int tid, const int nth,
                                            const int kx)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fxc *S = reinterpret_cast<fxc *>(smem_raw);
-    __shared__ int s_e, s_top;
-    __shared__ unsigned s_r[4];   // flags, magnitudes in and out, sum of the frequencies' scales over the largest
+    __shared__ int s_e[3], s_top[3];
+    // magnitudes in and out, sums of the frequencies' scales over the largest, flags
+    __shared__ unsigned s_r[10];
+    unsigned *s_in = s_r, *s_out = s_r + 3, *s_sum = s_r + 6, *s_fl = s_r + 9;
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int ny = g.ny, nz = g.nz, Py = g.Py, nrow = 3 * nz;
     fxc *Wk = P.W + (long)kx * nrow * ny;
     fxmc *tw = reinterpret_cast<fxmc *>(S + nrow * g.rsy);
-    signed char *s_sc = reinterpret_cast<signed char *>(tw + Py);  // [2][Py]: scale and top bit of every ky
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + Py);  // [2][3][Py]: scale and top bit of every ky
     load_twiddles_async(tw, P.tw_py, Py, Py, tt, nth);
-    if (tid == 0) { s_e = FX_ZERO; s_top = FX_ZERO; }
-    if (tid < 4) s_r[tid] = 0;
+    if (tid < 3) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
+    if (tid < 10) s_r[tid] = 0;
     __syncthreads();
 
     // Wk[z][y][c] -> row (c, z); the first loads are issued before the rows' scales are looked at
@@ -420,33 +434,24 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
             if (e0 + i * nth < tot) v[i] = ld_cg(Wk + e0 + i * nth);
     };
     if (tt < tot) load(tt);
-    int emax = FX_ZERO;
-    unsigned fl = 0;
-    for (int i = tt; i < nz * ny; i += nth) {
-        const int p = P.fe1[i];
-        emax = max(emax, fx_exp(p));
-        fl |= fx_flags(p);
-    }
-    fx_cta_max(&s_e, emax);
-    fx_cta_or(&s_r[0], fl);
+    fx_cta_scales(P.fe1, nz * ny, 3, tt, nth, s_e, s_fl);
     __syncthreads();
-    emax = s_e;
-    unsigned mag = 0;
+    fx3 mags;
     for (int e0 = tt; e0 < tot;) {
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-            const int d = fx_exp(P.fe1[rest]) - emax;
+            const int d = fx_exp(P.fe1[e]) - s_e[c];
             if (d) v[i] = fx_scale(v[i], d);
-            mag |= fx_mag(v[i]);
+            mags.or_in(c, fx_mag(v[i]));
             S[(c * nz + zz) * g.rsy + spos<fxc>(y)] = v[i];
         }
         e0 += PF * nth;
         if (e0 < tot) load(e0);
     }
-    fx_cta_or(&s_r[1], mag);
+    mags.cta_or(s_in);
     const int npad = Py - ny;
     for (int e = tt; e < nrow * npad; e += nth) {
         const int row = g.fd_pady.div(e), y = ny + (e - row * npad);
@@ -456,18 +461,31 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     __syncthreads();
     const int rb = tid / g.Gy, j = tid - rb * g.Gy;  // row within a batch of g.RB rows
     const bool act = rb < g.RB;
-    int pre = 59 - fx_bits(s_r[1]), e = emax - pre, sh = 0;
-    for (int r0 = 0; r0 < nrow; r0 += g.RB)
-        sh = fft_row_fx<false, true, false, 1, LY, false>(S + (act ? r0 + rb : 0) * g.rsy, Py, g.lpy, j, tw, act, pre,
-                                                          64, mag);
+    auto comp = [&](int r) { return (r >= nz) + (r >= 2 * nz); };  // of a row
+    int sh = 0;
+    unsigned none = 0;
+    for (int r0 = 0; r0 < nrow; r0 += g.RB) {
+        const int r = act ? r0 + rb : 0;
+        sh = fft_row_fx<false, true, false, 1, LY, false>(S + r * g.rsy, Py, g.lpy, j, tw, act,
+                                                          59 - fx_bits(s_in[comp(r)]), 64, none);
+    }
     // z convolution: inputs of a ky below 2^59, so sums and differences below
     // 2^60; outputs below 2^60 (the tensor's terms of an output sum to less
     // than 2^62 units, and the factor 2)
     constexpr int NZM = PZ > 1 ? PZ / 2 : 1;
     const int hy = Py / 2, kst = hy + 1;
     constexpr int NC = 4 * ZConv<NZM>::NE + 2 * ZConv<NZM>::NO;
-    e += sh + P.fek[kx] - (NZM > 1 ? 1 : 0);
-    int top = FX_ZERO;
+    const FxCouple couple{g.nx > 1 && ny > 1, NZM > 1 && g.nx > 1, NZM > 1 && ny > 1};
+    int eb[3], d[3];   // a component's scale where it is mixed, and its own over that
+    {
+        int own[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) eb[c] = own[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+        couple.join(eb[0], eb[1], eb[2]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d[c] = own[c] - eb[c];
+    }
+    int top[3] = {FX_ZERO, FX_ZERO, FX_ZERO};
     for (int u = tt; u < 2 * Py; u += nth) {
         // a pair of lanes per ky: part 0 the real parts (of m_x, m_y and i m_z), part 1 the imaginary ones
         const int ky = u >> 1, part = u & 1, kyr = ky <= hy ? ky : Py - ky;
@@ -479,26 +497,29 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
         ZConv<NZM> z;
         z.K = P.Nhat + (long)kx * NC * kst + kyr;
         z.kst = kst;
-        int sc;
+        int sc[3];
         {
             fx m[3][NZM];
-            unsigned mk = 0;
+            unsigned mk[3] = {0, 0, 0};
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
                     m[c][n] = n < nz ? col[2 * (c * nz + n) * g.rsy + at[c]] : fx(0);
-                    mk |= fx_mag(m[c][n]);
+                    mk[c] |= fx_mag(m[c][n]);
                 }
-            mk |= __shfl_xor_sync(lanes, mk, 1);
-            sc = 59 - fx_bits(mk);
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
+            for (int c = 0; c < 3; ++c) sc[c] = fx_bits(mk[c] | __shfl_xor_sync(lanes, mk[c], 1)) + d[c];
+            couple.join(sc[0], sc[1], sc[2]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                sc[c] = 59 - sc[c];
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
-                    m[c][n] = fx_scale(m[c][n], sc);
+                    m[c][n] = fx_scale(m[c][n], sc[c] + d[c]);
                     if (flip[c]) m[c][n] = -m[c][n];
                 }
+            }
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -508,49 +529,64 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
                     z.um[c][i] = fx_split(a - b);
                 }
         }
-        mag = 0;
+        unsigned mag = 0;
         auto put = [&](int c, int n, fx r) {
             if (n >= nz) return;
             if (c == 1 ? flip[1] : (c == 2 && part == 1)) r = -r;
             mag |= fx_mag(r);
             col[2 * (c * nz + n) * g.rsy + at[c]] = r;
         };
+        auto done = [&](int c) {
+            // values of this ky and component: stored * 2^-sc, below 2^tk
+            const int tk = fx_bits(mag | __shfl_xor_sync(lanes, mag, 1)) - sc[c];
+            if (part == 0) {
+                s_sc[c * Py + ky] = (signed char)sc[c];
+                s_sc[(3 + c) * Py + ky] = (signed char)tk;
+            }
+            top[c] = max(top[c], tk);
+            mag = 0;
+        };
         z.template output<0>([&](int n, fx r) { put(0, n, r); });
+        done(0);
         z.template output<1>([&](int n, fx r) { put(1, n, r); });
+        done(1);
         z.template output<2>([&](int n, fx r) { put(2, n, r); });
-        mag |= __shfl_xor_sync(lanes, mag, 1);
-        const int tk = fx_bits(mag) - sc;  // values of this ky: stored * 2^-sc, below 2^tk
-        if (part == 0) {
-            s_sc[ky] = (signed char)sc;
-            s_sc[Py + ky] = (signed char)tk;
-        }
-        top = max(top, tk);
+        done(2);
     }
-    fx_cta_max(&s_top, top);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fx_cta_max(&s_top[c], top[c]);
     __syncthreads();
-    top = s_top;
     // no partial sum of an inverse transform exceeds the sum of the largest moduli over ky
-    unsigned sum = 0;
-    for (int ky = tt; ky < Py; ky += nth) sum += ((1u << 18) >> min(top - s_sc[Py + ky], 18)) + 1;
-    fx_cta_add(&s_r[3], sum);
+    unsigned sum[3] = {0, 0, 0};
+    for (int ky = tt; ky < Py; ky += nth) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sum[c] += ((1u << 18) >> min(s_top[c] - s_sc[(3 + c) * Py + ky], 18)) + 1;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
     __syncthreads();
-    pre = 58 - top;
-    const int t = max(0, fx_log2_up(s_r[3]) - 18);
-    mag = 0;
-    for (int r0 = 0; r0 < nrow; r0 += g.RB)
-        sh = fft_row_fx<true, false, true, 1, LY, true, true>(S + (act ? r0 + rb : 0) * g.rsy, Py, g.lpy, j, tw, act, pre,
-                                                              t, mag, s_sc);
-    fx_cta_or(&s_r[2], mag);
+    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
+    mags = fx3();
+    for (int r0 = 0; r0 < nrow; r0 += g.RB) {
+        const int r = act ? r0 + rb : 0, c = comp(r);
+        unsigned mag = 0;
+        fft_row_fx<true, false, true, 1, LY, true, true>(S + r * g.rsy, Py, g.lpy, j, tw, act, 58 - s_top[c], bound(c),
+                                                         mag, s_sc + c * Py);
+        mags.or_in(c, mag);
+    }
+    mags.cta_or(s_out);
     __syncthreads();
-    const int post = 60 - fx_bits(s_r[2]);
-    e += sh - pre - post;
     for (int i = tt; i < tot; i += nth) {
         const int c = i % 3, rest = i / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], post);
+        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], 60 - fx_bits(s_out[c]));
     }
-    // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
-    const int flags = (int)s_r[0];
-    if (tid == 0) P.fe2[kx] = fx_pack(e, (nz == 1 || !flags) ? flags : 3);
+    if (tid < 3) {
+        // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
+        const int c = tid, fl = (int)*s_fl, hit = nz > 1 ? 7 : (c == 2 ? 4 : 3);
+        const int e = (c == 0 ? eb[0] : (c == 1 ? eb[1] : eb[2])) + P.fek[kx] - (NZM > 1 ? 1 : 0) +
+                      fx_cum(fx_log(Py), bound(c)) - (58 - s_top[c]) - (60 - fx_bits(s_out[c]));
+        P.fe2[kx * 3 + c] = fx_pack(e, fl & hit ? 1 : 0);
+    }
 }
 
 template <int PZ, int LY>
@@ -907,26 +943,20 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     const int nx = g.nx, ny = g.ny, nz = g.nz, Hx = g.Hx;
     const long N = g.N;
     TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);
-    // block fixed point: largest scale and flags of the x-frequencies, the sum of their scales over the largest, and
-    // the magnitude of this CTA's rows
-    __shared__ int s_e;
-    __shared__ unsigned s_r[3];
-    unsigned mag = 0;
+    // block fixed point, per component: the x-frequencies' largest scale, the sum of their scales over the largest, and
+    // the magnitude of this CTA's rows; and the flags
+    __shared__ int s_e[3];
+    __shared__ unsigned s_r[7];
+    unsigned *s_fl = s_r, *s_sum = s_r + 1, *s_mag = s_r + 4;
+    fx3 mags;
     const int *fe2 = nullptr;
-    int emax = FX_ZERO;
+    const int fst = 3 * g.nzb;     // ints from one x-frequency's scales to the next's
     if constexpr (is_fx<F>) {
-        fe2 = P.fe2 + z / g.ZB;
-        if (tid == 0) s_e = FX_ZERO;
-        if (tid < 3) s_r[tid] = 0;
+        fe2 = P.fe2 + 3 * (z / g.ZB);
+        if (tid < 3) s_e[tid] = FX_ZERO;
+        if (tid < 7) s_r[tid] = 0;
         __syncthreads();
-        unsigned fl = 0;
-        for (int i = tt; i < g.C; i += nth) {
-            const int p = fe2[i * g.nzb];
-            emax = max(emax, fx_exp(p));
-            fl |= fx_flags(p);
-        }
-        fx_cta_max(&s_e, emax);
-        fx_cta_or(&s_r[0], fl);
+        fx_cta_scales(fe2, g.C, fst, tt, nth, s_e, s_fl);
     }
 
     MinState *st = P.st;
@@ -997,10 +1027,13 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             cp_async_wait_group<1>();
             __syncthreads();
             if constexpr (is_fx<F>) {
-                emax = s_e;
-                unsigned sum = 0;
-                for (int i = tt; i < g.C; i += nth) sum += ((1u << 18) >> min(emax - fx_exp(fe2[i * g.nzb]), 18)) + 1;
-                fx_cta_add(&s_r[1], sum);
+                unsigned sum[3] = {0, 0, 0};
+                for (int i = tt; i < g.C; i += nth) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) sum[c] += ((1u << 18) >> min(s_e[c] - fx_exp(fe2[i * fst + c]), 18)) + 1;
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
             }
         }
 #pragma unroll
@@ -1012,8 +1045,8 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             V Z;
             V Xk = xa[i], Xm = cconj(xb[i]);
             if constexpr (is_fx<F>) {  // components below 2^60: |Z| < 2^62
-                Xk = fx_scale(Xk, fx_exp(fe2[kk * g.nzb]) - emax);
-                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * g.nzb]) - emax);
+                Xk = fx_scale(Xk, fx_exp(fe2[kk * fst + c]) - s_e[c]);
+                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * fst + c]) - s_e[c]);
             }
             const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
             V t;
@@ -1022,39 +1055,49 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             Z.x = sum.x - t.y;
             Z.y = sum.y + t.x;
             row[rpos<V, LX>(kk)] = Z;
-            if constexpr (is_fx<F>) mag |= fx_mag(Z);
+            if constexpr (is_fx<F>) mags.or_in(c, fx_mag(Z));
             if (kk != 0 && Hx - kk != kk) {
                 Z.x = sum.x + t.y;
                 Z.y = t.x - sum.y;
                 row[rpos<V, LX>(Hx - kk)] = Z;
-                if constexpr (is_fx<F>) mag |= fx_mag(Z);
+                if constexpr (is_fx<F>) mags.or_in(c, fx_mag(Z));
             }
         }
     }
-    if constexpr (is_fx<F>) fx_cta_or(&s_r[2], mag);
+    if constexpr (is_fx<F>) mags.cta_or(s_mag);
     __syncthreads();
+    // the moduli of a row sum to at most 2^62 times the frequencies' scales over the largest
+    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18 + 62 - fx_bits(s_mag[c])); };
     {
         const int row = tid / g.Gx, j = tid - row * g.Gx;
         const bool act = row < 3 * TY;
         if constexpr (is_fx<F>) {
-            // the moduli of a row sum to at most 2^62 times the frequencies' scales over the largest
-            const int bits = fx_bits(s_r[2]), pre = 58 - bits;
+            const int c = act ? row >> g.lty : 0;
             unsigned none = 0;
-            emax += fft_row_fx<true, false, true, 2, LX, false>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act, pre,
-                                                                max(0, fx_log2_up(s_r[1]) - 18 + 62 - bits), none) - pre;
+            fft_row_fx<true, false, true, 2, LX, false>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act,
+                                                        58 - fx_bits(s_mag[c]), bound(c), none);
         } else {
             fft_row<true, false, true, 2, LX>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act);
         }
     }
     constexpr bool DW = std::is_same<T, dfloat>::value;
-    double dscale = 0.0;   // block fixed point: one unit of the rows' values, in A/m
-    float dscalef = 0.0f, dtiny = 1.0f;   // (in two factors below the range of one)
+    // block fixed point: one unit of a component's values, in A/m (of double-words in two factors below the range of one)
+    double dscale[3];
+    float dscalef[3], dtiny[3];
     int bad = 0;
     if constexpr (is_fx<F>) {
-        if (DW && emax < -100) { emax += 64; dtiny = 5.42101086e-20f; }   // 2^-64
-        if constexpr (DW) dscalef = fx_pow2f(emax);
-        else dscale = fx_pow2(emax);
-        bad = (int)s_r[0];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int e = s_e[c] + fx_cum(fx_log(Hx), bound(c)) - (58 - fx_bits(s_mag[c]));
+            const bool tiny = DW && e < -100;
+            if constexpr (DW) {
+                dscalef[c] = fx_pow2f(tiny ? e + 64 : e);
+                dtiny[c] = tiny ? 5.42101086e-20f : 1.0f;   // 2^-64
+            } else {
+                dscale[c] = fx_pow2(e);
+            }
+        }
+        bad = (int)*s_fl;
     }
     cp_async_wait_all();
     if (stg) __syncthreads();
@@ -1088,23 +1131,24 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             const fx q0 = rel<F, LX>(S + (0 * TY + yl) * g.rsx, x), q1 = rel<F, LX>(S + (1 * TY + yl) * g.rsx, x),
                      q2 = rel<F, LX>(S + (2 * TY + yl) * g.rsx, x);
             if constexpr (DW) {
-                d0 = fx_to_dfloat(q0, dscalef);
-                d1 = fx_to_dfloat(q1, dscalef);
-                d2 = fx_to_dfloat(q2, dscalef);
-                if (dtiny != 1.0f) {
-                    d0.hi *= dtiny; d0.lo *= dtiny; d1.hi *= dtiny; d1.lo *= dtiny; d2.hi *= dtiny; d2.lo *= dtiny;
-                }
+                d0 = fx_to_dfloat(q0, dscalef[0]);
+                d1 = fx_to_dfloat(q1, dscalef[1]);
+                d2 = fx_to_dfloat(q2, dscalef[2]);
+                d0.hi *= dtiny[0]; d0.lo *= dtiny[0];
+                d1.hi *= dtiny[1]; d1.lo *= dtiny[1];
+                d2.hi *= dtiny[2]; d2.lo *= dtiny[2];
             } else {
-                d0 = __ll2double_rn(q0.v) * dscale;
-                d1 = __ll2double_rn(q1.v) * dscale;
-                d2 = __ll2double_rn(q2.v) * dscale;
+                d0 = __ll2double_rn(q0.v) * dscale[0];
+                d1 = __ll2double_rn(q1.v) * dscale[1];
+                d2 = __ll2double_rn(q2.v) * dscale[2];
             }
             if (bad) {  // uniform over the CTA
                 T nan;
                 if constexpr (DW) nan = dfloat(__int_as_float(0x7fc00000), 0.0f);
                 else nan = __longlong_as_double(0x7ff8000000000000ll);
-                if (bad & 1) d0 = d1 = nan;
-                if (bad & 2) d2 = nan;
+                if (bad & 1) d0 = nan;
+                if (bad & 2) d1 = nan;
+                if (bad & 4) d2 = nan;
             }
         } else {
             d0 = to_field<T>(rel<F, LX>(S + (0 * TY + yl) * g.rsx, x));
@@ -1283,10 +1327,10 @@ template <typename T, typename F = typename fft_of<T>::type> FieldPtrs<T, F> mak
     P.W = (V *)p->W; P.W2 = (V *)p->W2; P.Nhat = (const typename coef<F>::type *)p->Nhat;
     P.tw_px = (const TW *)p->tw_px; P.tw_py = (const TW *)p->tw_py; P.tw_pz = (const TW *)p->tw_pz;
     P.fe1 = p->fexp;
-    P.fea = p->fexp + (long)g.nz * g.ny;
-    P.feb = P.fea + (long)g.C * g.nzb;
-    P.fe2 = P.feb + (long)g.C * g.nkb;
-    P.fek = P.fe2 + (long)g.C * g.nzb;
+    P.fea = p->fexp + 3 * (long)g.nz * g.ny;
+    P.feb = P.fea + 3 * (long)g.C * g.nzb;
+    P.fe2 = P.feb + 3 * (long)g.C * g.nkb;
+    P.fek = P.fe2 + 3 * (long)g.C * g.nzb;   // mm_scale_fek
     typedef typename io_of<T>::type IO;
     P.Kc = (const IO *)p->Kc; P.uc = (const IO *)p->uc;
     P.partials = p->partials; P.st = p->st; P.counter = p->counter;
@@ -1316,8 +1360,8 @@ template <typename T> size_t smem_yz_t(const Geom &g)
 {
     typedef typename cvec<typename fft_of<T>::type>::type V;
     // rows and Py twiddles,
-    // and the block fixed-point kernel two bytes per y-frequency
-    return ((size_t)3 * g.nz * g.rsy + g.Py) * sizeof(V) + (sizeof(T) == 4 ? 0 : 2 * (size_t)g.Py);
+    // and the block fixed-point kernel two bytes per y-frequency and component
+    return ((size_t)3 * g.nz * g.rsy + g.Py) * sizeof(V) + (sizeof(T) == 4 ? 0 : 6 * (size_t)g.Py);
 }
 
 // The field kernels are compiled for a set of FFT row lengths (template

@@ -38,9 +38,14 @@ struct __align__(16) fxmc {
     fxm x, y;
 };
 
-// Scale of a block as the kernels hand it on: e * 4 + flags.  Non-finite
-// inputs have no place in a block; their components are taken as zero and
-// flagged (1: x or y, 2: z), and come out as NaN where the field would.
+// The three components have scales of their own: where the tensor does not
+// couple them (axes of one cell), or where one is not mixed with the others yet,
+// a component is as accurate as its own size allows.  (With one scale for the
+// three, the in-plane field of a one-layer film magnetised along z with a tilt of
+// 1e-8 was off by 1e-8 of itself.)
+// Scale of a block as the kernels hand it on: e * 4 + flag.  Non-finite inputs
+// have no place in a block; their component is taken as zero and flagged (1),
+// and comes out as NaN where the field would.
 #define FX_ZERO (-100000)   // exponent of an all-zero block
 __host__ __device__ __forceinline__ constexpr int fx_pack(int e, int flags) { return e * 4 + flags; }
 __host__ __device__ __forceinline__ constexpr int fx_exp(int p) { return p >> 2; }
@@ -209,6 +214,50 @@ __device__ __forceinline__ void fx_cta_add(unsigned *dst, unsigned v)
     v = __reduce_add_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) atomicAdd(dst, v);
 }
+// one value per component, added to by component number
+struct fx3 {
+    unsigned v[3] = {0, 0, 0};
+    __device__ __forceinline__ void or_in(int c, unsigned x)
+    {
+        v[0] |= c == 0 ? x : 0; v[1] |= c == 1 ? x : 0; v[2] |= c == 2 ? x : 0;
+    }
+    __device__ __forceinline__ void cta_or(unsigned *dst) const
+    {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_cta_or(dst + c, v[c]);
+    }
+};
+// Largest exponent of each component, and the flags (bit c), of the scales
+// p[i * stride + c], i < n, over the CTA; a barrier makes them visible
+__device__ __forceinline__ void fx_cta_scales(const int *p, int n, long stride, int tt, int nth, int *s_e,
+                                              unsigned *s_fl)
+{
+    int e[3] = {FX_ZERO, FX_ZERO, FX_ZERO};
+    unsigned fl = 0;
+    for (int i = tt; i < n; i += nth) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int q = p[i * stride + c];
+            e[c] = max(e[c], fx_exp(q));
+            fl |= (unsigned)fx_flags(q) << c;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fx_cta_max(s_e + c, e[c]);
+    fx_cta_or(s_fl, fl);
+}
+// Components that the tensor couples (pairs of axes that both have more than
+// one cell) share a scale where they are mixed: the largest of theirs.  All
+// pairs are coupled, one, or none.
+struct FxCouple {
+    bool xy, xz, yz;
+    __device__ __forceinline__ void join(int &a, int &b, int &c) const
+    {
+        const int x = max(a, max(xy ? b : a, xz ? c : a)), y = max(b, max(xy ? a : b, yz ? c : b)),
+                  z = max(c, max(xz ? a : c, yz ? b : c));
+        a = x; b = y; c = z;
+    }
+};
 // least t >= 0 with 2^t >= v
 __device__ __forceinline__ int fx_log2_up(unsigned v) { return v > 1 ? 32 - __clz((int)(v - 1)) : 0; }
 __device__ __forceinline__ int fx_bits(unsigned mag) { return 64 - __clz((int)mag); }  // 32 + bits of mag

@@ -335,7 +335,7 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
     if (!e && p->precision != MM_FP32) {
         const int hy = g.Py / 2;
         fxm *out = (fxm *)p->Nhat;
-        int *ek = p->fexp + ((long)g.nz * g.ny + (long)g.C * (2 * g.nzb + g.nkb));
+        int *ek = p->fexp + mm_scale_fek(g);
         if (g.bulk) {
             const int n = (g.Pz / 2 + 1) * (hy + 1);
             k_tensor_fixed<0><<<g.C, 256, 0, s>>>((const double *)K64, (long)n * 6, out, (long)n * 6, n, ek);

@@ -100,3 +100,32 @@ def test_energy_of_a_minimisation_with_a_large_uniform_anisotropy(mmlib, Ms, K, 
     ref = LD(mmlib.mm_energy(double, dev(m), Hext)[0]) - c * V / 2 * (M * exchange(p, m)[0]).sum()
     ref += LD(K) * V * (1 - M[0] ** 2).sum() - c * V * (M * Hext.astype(LD).reshape(3, 1, 1, 1)).sum()
     assert abs(r.energy - ref) <= 16 * u * float(K * V) * N ** 0.5 + floor * float(abs(ref))
+
+
+def coupled(shape, a, b):
+    """Whether the tensor mixes components a and b: the cells of an axis lie on both sides of one another."""
+    n = shape[::-1]
+    return a == b or (n[a] > 1 and n[b] > 1)
+
+
+@pytest.mark.parametrize("prec,bar", [("MM_FP64", 2e-15), ("MM_F32X2", 1e-13)])
+@pytest.mark.parametrize("grid", [(24, 20, 1), (1, 36, 1), (300, 1, 1), (24, 1, 3), (1, 20, 2), (257, 9, 1), (12, 1, 9),
+                                  (1, 1, 24), (1, 9, 70)])
+def test_components_of_different_size(mmlib, grid, prec, bar):
+    """A magnetisation tilted by little from an axis: the field of the components that the tensor does not mix with the
+    large one is as accurate as that of components of their own size (the bars of random states, relative to Ms times
+    the mixed components: the field itself can be a small difference).  The tilts stay far above the oracle's tensor
+    entries of pairs that do not mix, 1e-33 in place of 0."""
+    nx, ny, nz = grid
+    if prec == "MM_F32X2" and nz > 4:
+        pytest.skip("double-word problems are films")
+    prob, p = make_pair(mmlib, nx, ny, nz, (4e-9, 3e-9, 5e-9), A=0.0, K=0.0, precision=getattr(mmlib, prec))
+    d = om.Demag(p)
+    for big in range(3):
+        for tilt in (1e-3, 1e-8, 1e-12):
+            m = tilt * smooth(p.shape, 11 + big)
+            m[big] = 1.0
+            H, ref = field(mmlib, prob, m, (0, 0, 0)), d.field(m)
+            for c in range(3):
+                mixed = np.sqrt(sum(np.sum(m[a] ** 2) for a in range(3) if coupled(p.shape, a, c)))
+                assert np.linalg.norm(H[c] - ref[c]) <= bar * p.Ms * mixed, (big, tilt, c)
