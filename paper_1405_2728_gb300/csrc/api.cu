@@ -168,6 +168,7 @@ int plan(mm_problem *p)
     Geom &g = p->g;
     const mm_grid &gr = p->grid;
     g.nx = gr.nx; g.ny = gr.ny; g.nz = gr.nz;
+    g.sep = mm_separate(g);
     // what is supported, and in which layout, is decided on powers of two
     const int P2[3] = {next_pow2(2 * gr.nx - 1), next_pow2(2 * gr.ny - 1), next_pow2(2 * gr.nz - 1)};
     auto lengths = [&](int Px, int Py, int Pz) {
@@ -261,7 +262,7 @@ int plan(mm_problem *p)
     // y rows per CTA in the x kernels: powers of two up to 16 (and up to the
     // next power of two of ny) within 768 threads and the shared-memory cap
     p->nty = 0;
-    for (int ty = 1; ty <= 16 && ty <= next_pow2(gr.ny); ty *= 2)
+    for (int ty = 1; ty <= MM_MAX_TILE && ty <= next_pow2(gr.ny); ty *= 2)
         if (3 * ty * g.Gx <= 768 && mm_smem_x_for(p, ty) <= smax) p->tys[p->nty++] = ty;
     if (!p->nty) return MM_ERR_UNSUPPORTED;
     // untuned problems (below the autotuner's size) take the smallest tile:

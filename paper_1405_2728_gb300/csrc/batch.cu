@@ -44,12 +44,14 @@
     const void *mm_group_xinv_##SFX();
 MM_DECLARE_GROUP(fp64)
 MM_DECLARE_GROUP(fp32)
+const void *mm_group_yz_sep_fp64();
 
 namespace {
 
+enum { STAGE_YZ_SEP = 3 };   // the y-z stage's second kernel (group_sep)
 template <typename T> const void *group_kernel(int stage)
 {
-    if constexpr (sizeof(T) == 8) return stage == 0 ? mm_group_xfwd_fp64() : (stage == 1 ? mm_group_yz_fp64() : mm_group_xinv_fp64());
+    if constexpr (sizeof(T) == 8) return stage == STAGE_YZ_SEP ? mm_group_yz_sep_fp64() : stage == 0 ? mm_group_xfwd_fp64() : (stage == 1 ? mm_group_yz_fp64() : mm_group_xinv_fp64());
     else return stage == 0 ? mm_group_xfwd_fp32() : (stage == 1 ? mm_group_yz_fp32() : mm_group_xinv_fp32());
 }
 
@@ -201,6 +203,7 @@ struct Group {
     int n_xf = 0, n_yz = 0, n_x = 0;
     int thr_xf = 32, thr_yz = 32, thr_x = 32;
     size_t sm_xf = 0, sm_yz = 0, sm_x = 0;
+    bool any_sep = false;
 };
 
 } // namespace
@@ -319,6 +322,7 @@ template <typename T> cudaError_t build_group(mm_batch *b, Group<T> &G)
         G.sm_xf = std::max(G.sm_xf, smem_xf_t<T>(g));
         G.sm_x = std::max(G.sm_x, smem_x_t<T>(g));
         G.sm_yz = std::max(G.sm_yz, smem_yz_t<T>(g));
+        G.any_sep = G.any_sep || group_sep<T>(g);
         const int gxf = (g.ny + g.TYF - 1) / g.TYF, gx = d.gx_x;
         first[0 * nf + f] = d.first[0] = (int)ixf.size();
         for (int z = 0; z < g.nz; ++z)
@@ -346,6 +350,9 @@ template <typename T> cudaError_t build_group(mm_batch *b, Group<T> &G)
     if ((e = cudaFuncSetAttribute(group_kernel<T>(0), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
         (e = cudaFuncSetAttribute(group_kernel<T>(1), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)) ||
         (e = cudaFuncSetAttribute(group_kernel<T>(2), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)))
+        return e;
+    if (G.any_sep &&
+        (e = cudaFuncSetAttribute(group_kernel<T>(STAGE_YZ_SEP), cudaFuncAttributeMaxDynamicSharedMemorySize, MM_SMEM_CAP)))
         return e;
     // persistent grids: as many CTAs as are resident on all SMs at once
     int r0 = 0, r1 = 0, r2 = 0;
@@ -382,6 +389,7 @@ template <typename T> void launch_group(const Group<T> &G, cudaStream_t s)
     };
     launch(0, G.grid_xf, G.thr_xf, G.sm_xf, G.items_xf);
     launch(1, G.grid_yz, G.thr_yz, G.sm_yz, G.items_yz);
+    if (G.any_sep) launch(STAGE_YZ_SEP, G.grid_yz, G.thr_yz, G.sm_yz, G.items_yz);
     launch(2, G.grid_x, G.thr_x, G.sm_x, G.items_x);
 }
 

@@ -11,12 +11,15 @@ namespace {
 
 // the FFT arithmetic of a group's fields, and its y-z stage
 template <typename T> using FA = typename fft_of<T>::type;
-template <typename T, int PZ, int L>
+template <typename T, int PZ, int L, bool SEP>
 __device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int tid, int nth, int kx)
 {
     if constexpr (!is_fx<FA<T>>) yz_body<PZ, L>(g, P, tid, nth, kx);
-    else if constexpr (L == 0) yz_body_fx<PZ, -1>(g, P, tid, nth, kx);
+    else if constexpr (L == 0 && !(SEP && PZ == 1)) yz_body_fx<PZ, -1, (SEP || PZ == 1)>(g, P, tid, nth, kx);
 }
+// double grids of one column or row with several layers: a kernel of their own (SEP), launched if a batch has one, as
+// both kinds in one kernel spill 2 KB a thread
+template <typename T> __host__ __device__ inline bool group_sep(const Geom &g) { return is_fx<FA<T>> && g.sep && g.Pz > 1; }
 
 // one problem of a grouped launch, as the grouped kernels read it
 template <typename T>
@@ -94,15 +97,16 @@ __global__ void __launch_bounds__(768) k_xfwd_group(const GFilm<T> *films, const
 // Block fixed point takes the code for any row length, odd parts included, here: integer results do
 // not depend on the instance, and its compiled lengths in one kernel with
 // three layer counts took four minutes to build.
-template <typename T>
+template <typename T, bool SEP>
 __global__ void __launch_bounds__(YZBound<T>::v) k_yz_group(const GFilm<T> *films, const GItem *items,
                                                             const int *first_of, GActive A)
 {
     MM_GROUP_LOOP(1)
+    if (group_sep<T>(f.g) != SEP) continue;
     switch (f.g.Pz * 1024 + (is_fx<FA<T>> ? 0 : ly_of(f.g.Py))) {
-#define C(L) case 1 * 1024 + L: yz_of<T, 1, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 4 * 1024 + L: yz_of<T, 4, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
-             case 8 * 1024 + L: yz_of<T, 8, L>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break;
+#define C(L) case 1 * 1024 + L: yz_of<T, 1, L, SEP>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
+             case 4 * 1024 + L: yz_of<T, 4, L, SEP>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break; \
+             case 8 * 1024 + L: yz_of<T, 8, L, SEP>(f.g, f.P, threadIdx.x, f.nth_yz, it.bx); break;
         MM_LY_CASES(C)
 #undef C
     }

@@ -24,9 +24,6 @@ namespace {
 // log2 of a power of two (ZB, KB)
 __device__ __forceinline__ int log2_of(int p) { return 31 - __clz(p); }
 
-// the tensor couples all components: no axis of one cell
-__host__ __device__ __forceinline__ bool coupled(const Geom &g) { return g.nx > 1 && g.ny > 1 && g.nz > 1; }
-
 template <typename V> __device__ __forceinline__ V load_cg(const V *p) { return __ldcg(p); }
 template <> __device__ __forceinline__ fxc load_cg(const fxc *p)
 {
@@ -63,14 +60,19 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
     const int zb = min(ZB, nz - z0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * ZB * rs);
     load_twiddles_async(tw, P.tw_py, Py, Py, tid, nth);
-    fx3 mags;
+    FxMags<3> mags;
     const int *scales = nullptr;   // of the values read: of every (z, y) row of W, or of KB y-frequencies of W2
+    const bool sep = g.sep;
+    const int ns = sep ? 3 : 1;
+    auto own = [&](int c) { return sep ? c : 0; };   // which of the scales is a component's
     if constexpr (FX) {
         if (tid < 3) s_e[tid] = FX_ZERO;
         if (tid < 7) s_r[tid] = 0;
         __syncthreads();
-        scales = INV ? P.feb + (long)kx * g.nkb * 3 : P.fe1 + (long)z0 * ny * 3;
-        fx_cta_scales(scales, INV ? g.nkb : zb * ny, 3, tid, nth, s_e, s_fl);
+        scales = INV ? P.feb + (long)kx * g.nkb * ns : P.fe1 + (long)z0 * ny * ns;
+        const int n = INV ? g.nkb : zb * ny;
+        if (sep) fx_cta_scales<3>(scales, n, 3, tid, nth, s_e, s_fl);
+        else fx_cta_scales<1>(scales, n, 1, tid, nth, s_e, s_fl);
         __syncthreads();
     }
     const long first = (long)kx * nz + z0;  // first (kx, z) row pair of this CTA
@@ -92,8 +94,8 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zl = INV ? rest / Py : g.fd_ny.div(rest), y = rest - zl * lin;
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[INV ? (y >> log2_of(g.KB)) * 3 + c : e]) - s_e[c]);
-                mags.or_in(c, fx_mag(v[i]));
+                v[i] = fx_scale(v[i], fx_exp(scales[(INV ? y >> log2_of(g.KB) : rest) * ns + own(c)]) - s_e[own(c)]);
+                mags.or_in(own(c), fx_mag(v[i]));
             }
             S[(c * ZB + zl) * rs + rpos<V, LY>(y)] = v[i];
         }
@@ -105,19 +107,24 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             S[r * rs + rpos<V, LY>(y)] = czero<V>();
         }
     }
-    if constexpr (FX) mags.cta_or(s_in);
+    auto cta_mags = [&](unsigned *dst) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (c == 0 || sep) fx_cta_or(dst + c, mags.v[c]);
+    };
+    if constexpr (FX) cta_mags(s_in);
     cp_async_wait_all();
     __syncthreads();
     const int Gy = g.Gy, RB = g.RBY;
     const int rb = tid / Gy, j = tid - rb * Gy;
     auto pre = [&](int c) { return (INV ? 58 : 59) - fx_bits(s_in[c]); };
     int sh = 0;
-    mags = fx3();
+    mags = FxMags<3>();
     for (int r0 = 0; r0 < 3 * ZB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * ZB && (r % ZB) < zb;
         if constexpr (FX) {
-            const int c = act ? r >> log2_of(ZB) : 0;
+            const int c = act ? own(r >> log2_of(ZB)) : 0;
             unsigned mag = 0;
             sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, pre(c), 64, mag);
             mags.or_in(c, mag);
@@ -125,11 +132,11 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             fft_row<INV, !INV, INV, 1, LY>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act);
     }
     auto post = [&](int c) { return 60 - fx_bits(s_out[c]); };
-    if constexpr (FX) mags.cta_or(s_out);
+    if constexpr (FX) cta_mags(s_out);
     __syncthreads();
     if constexpr (FX) {
-        if (tid < 3)
-            (INV ? P.fe2 : P.fea)[((long)kx * g.nzb + blockIdx.y) * 3 + tid] =
+        if (tid < ns)
+            (INV ? P.fe2 : P.fea)[((long)kx * g.nzb + blockIdx.y) * ns + tid] =
                 fx_pack(s_e[tid] - pre(tid) + sh - post(tid), *s_fl >> tid & 1);
     }
     const int lout = INV ? ny : Py;
@@ -137,37 +144,39 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
     for (int e = tid; e < zb * lout * 3; e += nth) {
         const int c = e % 3, rest = e / 3, zl = INV ? g.fd_ny.div(rest) : rest / Py, y = rest - zl * lout;
         V r = S[(c * ZB + zl) * rs + rpos<V, LY>(y)];
-        if constexpr (FX) r = fx_scale(r, post(c));
+        if constexpr (FX) r = fx_scale(r, post(own(c)));
         dst[e] = r;
     }
 }
 
-template <typename T, int LZ>
+// SEP: block fixed point with scales per component (Geom::sep)
+template <typename T, int LZ, bool SEP>
 __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, FieldPtrs<T> P)
 {
     typedef typename FieldPtrs<T>::V V;
     typedef typename FieldPtrs<T>::TW TW;
     constexpr bool FX = std::is_same<V, fxc>::value;
-    __shared__ int s_e[3], s_top[3];
+    constexpr int NS = SEP ? 3 : 1;
+    __shared__ int s_e[NS], s_top[NS];
     // magnitudes in and out, sums of the frequencies' scales over the largest, flags
-    __shared__ unsigned s_r[10];
-    unsigned *s_in = s_r, *s_out = s_r + 3, *s_sum = s_r + 6, *s_fl = s_r + 9;
+    __shared__ unsigned s_r[3 * NS + 1];
+    unsigned *s_in = s_r, *s_out = s_r + NS, *s_sum = s_r + 2 * NS, *s_fl = s_r + 3 * NS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *S = reinterpret_cast<V *>(smem_raw);
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int nz = g.nz, Py = g.Py, Pz = LZ ? fft_length(LZ) : g.Pz, KB = g.KB, rs = g.rsz, lkb = log2_of(KB);
+    const int nz = g.nz, Py = g.Py, Pz = LZ > 0 ? fft_length(LZ) : g.Pz, KB = g.KB, rs = g.rsz, lkb = log2_of(KB);
     const int kx = blockIdx.x, ky0 = blockIdx.y * KB;
     const int kb = min(KB, Py - ky0);
     TW *tw = reinterpret_cast<TW *>(S + 3 * KB * rs);
     load_twiddles_async(tw, P.tw_pz, Pz, Pz, tid, nth);
-    fx3 mags;
+    FxMags<NS> mags;
     const int *scales = nullptr;
     if constexpr (FX) {
-        if (tid < 3) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
-        if (tid < 10) s_r[tid] = 0;
+        if (tid < NS) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
+        if (tid < 3 * NS + 1) s_r[tid] = 0;
         __syncthreads();
-        scales = P.fea + (long)kx * g.nzb * 3;
-        fx_cta_scales(scales, g.nzb, 3, tid, nth, s_e, s_fl);
+        scales = P.fea + (long)kx * g.nzb * NS;
+        fx_cta_scales<NS>(scales, g.nzb, NS, tid, nth, s_e, s_fl);
         __syncthreads();
     }
     // i = z * kb + kyl: a whole block of KB = 2^lkb frequencies, or the last one
@@ -201,7 +210,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             int kyl, z;
             split(e / 3, kyl, z);
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[(z >> log2_of(g.ZB)) * 3 + c]) - s_e[c]);
+                v[i] = fx_scale(v[i], fx_exp(scales[(z >> log2_of(g.ZB)) * NS + (SEP ? c : 0)]) - s_e[SEP ? c : 0]);
                 mags.or_in(c, fx_mag(v[i]));
             }
             S[(c * KB + kyl) * rs + rpos<V, LZ>(z)] = v[i];
@@ -217,10 +226,8 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     __syncthreads();
     const int Gz = g.Gz, RB = g.RBZ;
     const int rb = tid / Gz, j = tid - rb * Gz;
-    // scales [1 or 3][KB][Pz] and top bits [3][KB][Pz] of the frequencies: components that are all coupled share the scales
-    signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));
-    const int own_sc = coupled(g) ? 0 : KB * Pz;   // from one component's scales to the next's
-    signed char *s_tk = s_sc + 2 * own_sc + KB * Pz;
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));  // [2][NS][KB][Pz]: scale and top bit of a frequency
+    signed char *s_tk = s_sc + NS * KB * Pz;
     int sh = 0;
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
@@ -228,21 +235,23 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         if constexpr (FX) {
             unsigned none = 0;
             sh = fft_row_fx<false, true, false, 1, LZ, false>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act,
-                                                              59 - fx_bits(s_in[act ? r >> lkb : 0]), 64, none);
+                                                              59 - fx_bits(s_in[SEP && act ? r >> lkb : 0]), 64, none);
         } else {
             fft_row<false, true, false, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
         }
     }
     __syncthreads();
-    int eb[3], d[3], top[3] = {FX_ZERO, FX_ZERO, FX_ZERO};   // a component's scale where it is mixed, its own over that
+    int eb[NS], d[NS], top[NS];   // a component's scale where it is mixed, its own over that, the largest output
     const FxCouple couple{g.nx > 1 && g.ny > 1, g.nx > 1 && nz > 1, g.ny > 1 && nz > 1};
     if constexpr (FX) {
-        int own[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) eb[c] = own[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
-        couple.join(eb[0], eb[1], eb[2]);
+        for (int c = 0; c < NS; ++c) {
+            eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+            top[c] = FX_ZERO;
+        }
+        couple.join(eb);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) d[c] = own[c] - eb[c];
+        for (int c = 0; c < NS; ++c) d[c] -= eb[c];
     }
     // tensor product per (ky, kz); octant storage [kx][kzr][kyr][6] with the
     // off-diagonal signs of the reflected frequencies
@@ -266,11 +275,20 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             const fxk k[6] = {element(0, false), element(1, false), element(2, false), element(3, ky > hy),
                               element(4, kz > hz), element(5, (ky > hy) != (kz > hz))};
             fxc m0 = *a0, m1 = *a1, m2 = *a2;
-            int sc[3] = {fx_bits(fx_mag(m0)) + d[0], fx_bits(fx_mag(m1)) + d[1], fx_bits(fx_mag(m2)) + d[2]};
-            couple.join(sc[0], sc[1], sc[2]);
+            auto mags_of = [](const fxc &x, const fxc &y, const fxc &z) {
+                FxMags<NS> k;
+                k.or_in(0, fx_mag(x)); k.or_in(1, fx_mag(y)); k.or_in(2, fx_mag(z));
+                return k;
+            };
+            const FxMags<NS> mk = mags_of(m0, m1, m2);
+            int sc[NS];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) sc[c] = 59 - sc[c];
-            m0 = fx_scale(m0, sc[0] + d[0]); m1 = fx_scale(m1, sc[1] + d[1]); m2 = fx_scale(m2, sc[2] + d[2]);
+            for (int c = 0; c < NS; ++c) sc[c] = fx_bits(mk.v[c]) + d[c];
+            couple.join(sc);
+#pragma unroll
+            for (int c = 0; c < NS; ++c) sc[c] = 59 - sc[c];
+            constexpr int c1 = SEP ? 1 : 0, c2 = SEP ? 2 : 0;
+            m0 = fx_scale(m0, sc[0] + d[0]); m1 = fx_scale(m1, sc[c1] + d[c1]); m2 = fx_scale(m2, sc[c2] + d[c2]);
             auto row = [&](const fxk &p, const fxk &q, const fxk &r, fx x, fx y, fx z) {
                 fxdot h;
                 h.zero();
@@ -282,12 +300,13 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             const fxc h0{row(k[0], k[3], k[4], m0.x, m1.x, m2.x), row(k[0], k[3], k[4], m0.y, m1.y, m2.y)};
             const fxc h1{row(k[3], k[1], k[5], m0.x, m1.x, m2.x), row(k[3], k[1], k[5], m0.y, m1.y, m2.y)};
             const fxc h2{row(k[4], k[5], k[2], m0.x, m1.x, m2.x), row(k[4], k[5], k[2], m0.y, m1.y, m2.y)};
-            const int tk[3] = {fx_bits(fx_mag(h0)) - sc[0], fx_bits(fx_mag(h1)) - sc[1], fx_bits(fx_mag(h2)) - sc[2]};
+            const FxMags<NS> hk = mags_of(h0, h1, h2);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                s_sc[c * own_sc + kyl * Pz + kz] = (signed char)sc[c];
-                s_tk[(c * KB + kyl) * Pz + kz] = (signed char)tk[c];
-                top[c] = max(top[c], tk[c]);
+            for (int c = 0; c < NS; ++c) {
+                const int tk = fx_bits(hk.v[c]) - sc[c];
+                s_sc[(c * KB + kyl) * Pz + kz] = (signed char)sc[c];
+                s_tk[(c * KB + kyl) * Pz + kz] = (signed char)tk;
+                top[c] = max(top[c], tk);
             }
             *a0 = h0; *a1 = h1; *a2 = h2;
         } else {
@@ -307,35 +326,37 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     }
     if constexpr (FX) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) fx_cta_max(&s_top[c], top[c]);
+        for (int c = 0; c < NS; ++c) fx_cta_max(&s_top[c], top[c]);
     }
     __syncthreads();
     if constexpr (FX) {
         // no partial sum of an inverse transform exceeds the sum of the largest moduli over kz
-        unsigned sum[3] = {0, 0, 0};
+        unsigned sum[NS];
+#pragma unroll
+        for (int c = 0; c < NS; ++c) sum[c] = 0;
         for (int e = tid; e < Pz; e += nth) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
+            for (int c = 0; c < NS; ++c) {
                 int tk = FX_ZERO;
                 for (int kyl = 0; kyl < kb; ++kyl) tk = max(tk, (int)s_tk[(c * KB + kyl) * Pz + e]);
                 sum[c] += ((1u << 18) >> min(s_top[c] - tk, 18)) + 1;
             }
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
+        for (int c = 0; c < NS; ++c) fx_cta_add(&s_sum[c], sum[c]);
         __syncthreads();
-        mags = fx3();
+        mags = FxMags<NS>();
     }
     auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
         if constexpr (FX) {
-            const int c = act ? r >> lkb : 0;
+            const int c = SEP && act ? r >> lkb : 0;
             unsigned mag = 0;
             fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, 58 - s_top[c],
                                                              bound(c), mag,
-                                                             s_sc + c * own_sc + (act ? r & (KB - 1) : 0) * Pz);
+                                                             s_sc + (c * KB + (act ? r & (KB - 1) : 0)) * Pz);
             mags.or_in(c, mag);
         } else {
             fft_row<true, false, true, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
@@ -345,10 +366,10 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     if constexpr (FX) mags.cta_or(s_out);
     __syncthreads();
     if constexpr (FX) {
-        if (tid < 3) {
-            const int c = tid, e = (c == 0 ? eb[0] : (c == 1 ? eb[1] : eb[2])) + P.fek[kx] +
+        if (tid < NS) {
+            const int c = tid, e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] +
                                    fx_cum(fx_log(Pz), bound(c)) - (58 - s_top[c]) - post(c);
-            P.feb[((long)kx * g.nkb + blockIdx.y) * 3 + c] = fx_pack(e, *s_fl ? 1 : 0);  // the tensor mixes all components
+            P.feb[((long)kx * g.nkb + blockIdx.y) * NS + c] = fx_pack(e, *s_fl ? 1 : 0);  // the tensor mixes all components
         }
     }
     for (int e = tid; e < nz * kb * 3; e += nth) {
@@ -356,7 +377,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         int kyl, z;
         split(e / 3, kyl, z);
         V r = S[(c * KB + kyl) * rs + rpos<V, LZ>(z)];
-        if constexpr (FX) r = fx_scale(r, post(c));
+        if constexpr (FX) r = fx_scale(r, post(SEP ? c : 0));
         base[(long)z * zs + kyl * 3 + c] = r;
     }
 }
@@ -371,8 +392,9 @@ template <typename T> size_t smem_y_t(const Geom &g, int zb)
 template <typename T> size_t smem_z_t(const Geom &g, int kb)
 {
     typedef typename cvec<T>::type V;
-    // and the bytes per frequency of a block fixed-point transform: scales, and a top bit per component
-    return ((size_t)3 * kb * g.rsz + tw_slots(g.Pz)) * sizeof(V) + (sizeof(T) == 8 ? (size_t)(coupled(g) ? 4 : 6) * kb * g.Pz : 0);
+    // and two bytes per frequency (and component) of a block fixed-point transform
+    return ((size_t)3 * kb * g.rsz + tw_slots(g.Pz)) * sizeof(V) +
+           (sizeof(T) == 8 ? (size_t)(g.sep ? 6 : 2) * kb * g.Pz : 0);
 }
 
 template <typename T> cudaError_t bulk_conv_t(const Geom &g, const FieldPtrs<T> &P, cudaStream_t s, int pass)
@@ -390,11 +412,16 @@ template <typename T> cudaError_t bulk_conv_t(const Geom &g, const FieldPtrs<T> 
         }
     }
     if (pass < 0 || pass == 1) {
-        switch (lz) {
-#define C(L) case L: k_zconv<T, L><<<gz, tz, sz, s>>>(g, P); break;
-            MM_LB_CASES(C)
+        if constexpr (sizeof(T) == 8) {
+            if (g.sep) k_zconv<T, -1, true><<<gz, tz, sz, s>>>(g, P);  // rare: the code for any length
+        }
+        if (sizeof(T) == 4 || !g.sep) {
+            switch (lz) {
+#define C(L) case L: k_zconv<T, L, false><<<gz, tz, sz, s>>>(g, P); break;
+                MM_LB_CASES(C)
 #undef C
-        default: return cudaErrorInvalidValue;
+            default: return cudaErrorInvalidValue;
+            }
         }
     }
     if (pass < 0 || pass == 2) {
@@ -424,8 +451,11 @@ template <typename T> cudaError_t configure_t(const Geom &g)
         MM_LB_CASES(C)
 #undef C
     }
+    if constexpr (sizeof(T) == 8) {
+        if (g.sep) return smem_attr(k_zconv<T, -1, true>, sz);
+    }
     switch (lb_of(g.Pz)) {
-#define C(L) case L: return smem_attr(k_zconv<T, L>, sz);
+#define C(L) case L: return smem_attr(k_zconv<T, L, false>, sz);
         MM_LB_CASES(C)
 #undef C
     }

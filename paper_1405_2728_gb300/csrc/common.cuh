@@ -176,6 +176,7 @@ struct Geom {
     int RBZ;               // z rows transformed at once in the z pass
     int nzb, nkb;          // blocks of ZB z planes (film layout: one block of all), of KB y frequencies
     int lpz, Gz, rsz;      // likewise of Pz, threads per z row, smem stride of a z row
+    int sep;               // block fixed point: components have scales of their own (mm_separate)
     int nbody;             // kernels per minimiser iteration (3 film, 5 bulk)
     long N;                // cells
     double dx, dy, dz;
@@ -269,11 +270,12 @@ struct FieldPtrs {
     const TW *tw_px;       // exp(-2 pi i t/Px), t < Px
     const TW *tw_py;       // exp(-2 pi i t/Py), t < Py
     const TW *tw_pz;       // exp(-2 pi i t/Pz), t < Pz
-    // block fixed point only (F = fx): the scales of the blocks (fx_pack), one per component
-    int *fe1;              // [nz][ny][3] of W as the x-forward kernel writes it
-    int *fea;              // [C][nzb][3] bulk: of W2 after the y transform
-    int *feb;              // [C][nkb][3] bulk: of W2 after the z convolution
-    int *fe2;              // [C][nzb][3] of W as the y-z stage leaves it
+    // block fixed point only (F = fx): the scales of the blocks (fx_pack), ns = 3 per block, one per component, with
+    // Geom::sep, ns = 1 without
+    int *fe1;              // [nz][ny][ns] of W as the x-forward kernel writes it
+    int *fea;              // [C][nzb][ns] bulk: of W2 after the y transform
+    int *feb;              // [C][nkb][ns] bulk: of W2 after the z convolution
+    int *fe2;              // [C][nzb][ns] of W as the y-z stage leaves it
     const int *fek;        // [C] exponents of the tensor
     const IO *Kc;          // per-cell K or NULL
     const IO *uc;          // per-cell axis [3][N] or NULL
@@ -350,6 +352,9 @@ MM_DECLARE_FIELD_ENTRIES(fp64)
 MM_DECLARE_FIELD_ENTRIES(fp32)
 MM_DECLARE_FIELD_ENTRIES(f32x2)
 
+// y rows per CTA of the x kernels, at most
+#define MM_MAX_TILE 16
+
 // Largest dynamic shared memory any field-kernel launch may use (the
 // planner keeps every launch shape within it).  Kernels get this limit as
 // their MaxDynamicSharedMemorySize attribute once and for all: the attribute
@@ -358,6 +363,12 @@ MM_DECLARE_FIELD_ENTRIES(f32x2)
 // problems configured before it.  It only permits launches; nothing is
 // reserved by it.
 #define MM_SMEM_CAP (200 * 1024)
+
+// Whether the components keep scales of their own in block fixed point: an axis
+// of one cell, whose pairs the tensor does not mix.  A grid's kernels that share
+// one are faster (k_yz_fx at 512 x 256 x 4: 121 us, with three scales 130; the z
+// pass of 64^3: 102 and 112 us).
+__host__ __device__ inline bool mm_separate(const Geom &g) { return g.nx == 1 || g.ny == 1 || g.nz == 1; }
 
 // tensor elements per (kx, ky) of the film layout: six components at
 // max(1, Pz/2) z offsets, or the combinations of them that the block
@@ -369,7 +380,7 @@ inline int mm_film_coefs(const Geom &g, int precision)
     return nzm == 1 ? 4 : (nzm == 2 ? 10 : 32);
 }
 
-// ints of mm_problem::fexp: three per block, and where fek (one per x-frequency) starts
+// ints of mm_problem::fexp: up to three per block, and where fek (one per x-frequency) starts
 inline size_t mm_scale_fek(const Geom &g) { return 3 * ((size_t)g.nz * g.ny + (size_t)g.C * (2 * g.nzb + g.nkb)); }
 inline size_t mm_scale_count(const Geom &g) { return mm_scale_fek(g) + g.C; }
 

@@ -115,11 +115,9 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
     const long N = g.N;
     TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);  // Px twiddles exp(-2 pi i t / Px)
     for (int i = tt; i < Px; i += nth) tw[tpos<TW>(i, g.Hx)] = P.tw_px[i];
-    __shared__ int s_max[3];       // block fixed point: high words of the tile's largest components
-    int mmax[3] = {0, 0, 0};
+    __shared__ int s_max[3 * MM_MAX_TILE];   // block fixed point: high words of the rows' largest values
     if constexpr (is_fx<F>) {
-        if (tid < 3) s_max[tid] = 0;
-        __syncthreads();
+        if (tid < 3 * TY) s_max[tid] = 0;
     }
 
     typedef typename io_of<T>::type IO;
@@ -182,10 +180,7 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
                 dst[n] = m0; dst[N + n] = m1; dst[2 * N + n] = m2;
             }
         }
-        if constexpr (is_fx<F>) {  // as they are, until the tile's scale is known
-            mmax[0] = max(mmax[0], magnitude(m0));
-            mmax[1] = max(mmax[1], magnitude(m1));
-            mmax[2] = max(mmax[2], magnitude(m2));
+        if constexpr (is_fx<F>) {  // as they are, until the rows' scales are known
             rel<T, LX>(S + (0 * TY + yl) * g.rsx, x) = m0;
             rel<T, LX>(S + (1 * TY + yl) * g.rsx, x) = m1;
             rel<T, LX>(S + (2 * TY + yl) * g.rsx, x) = m2;
@@ -195,39 +190,48 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             rel<F, LX>(S + (2 * TY + yl) * g.rsx, x) = F(m2);
         }
     }
-    int e1[3] = {0, 0, 0};
+    int e1 = 0;
     if constexpr (is_fx<F>) {
-        // the tile's scales 2^s, one per component: its largest value becomes 2^57 .. 2^58 (one up to 1 + 2^-8 counts
-        // as 1, so that unit vectors and their rounding share one scale); a non-finite component is taken as zero and
-        // flagged
-#pragma unroll
-        for (int c = 0; c < 3; ++c) fx_cta_max(&s_max[c], mmax[c]);
-        __syncthreads();
+        // The scale 2^s of a row's three components, or with Geom::sep of each: the largest value becomes 2^57 .. 2^58
+        // (one up to 1 + 2^-8 counts as 1, so that unit vectors and their rounding share one scale); non-finite
+        // components are taken as zero and flagged.  By row, because the tile is chosen by timing and results must not
+        // depend on it.  The Gx threads that transform a row convert it.
         constexpr bool DW = std::is_same<T, dfloat>::value;
         constexpr int inf = DW ? 0x7f800000 : 0x7ff00000, mant = DW ? 23 : 20, bias = DW ? 126 : 1022;
-        int sc[3];
-        float scalef[3];
-        bool use[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const bool bad = s_max[c] >= inf;
-            const int top = bad ? 0 : s_max[c], top_e = ((top - (1 << (mant - 8))) >> mant) - bias;
-            sc[c] = min(58 - top_e, DW ? 150 : 1000);
-            use[c] = top > 0;
-            scalef[c] = DW ? fx_pow2f(sc[c] - 28) : 0.0f;
-            e1[c] = fx_pack(top > 0 ? -sc[c] - 1 : FX_ZERO, bad ? 1 : 0);
+        __syncthreads();
+        const int row = tid / g.Gx, j = tid - row * g.Gx;
+        const bool act = row < 3 * TY;
+        V *const R = S + row * g.rsx;
+        int top = 0;
+        if (act) {
+            for (int x = j; x < nx; x += g.Gx) top = max(top, magnitude(rel<T, LX>(R, x)));
+            if (top) atomicMax(&s_max[row], top);
         }
-        for (int e = tt; e < TY * nx; e += nth) {  // the elements this thread stored
-            const int yl = g.fd_nx.div(e), x = e - yl * nx;
+        __syncthreads();
+        if (act) {
+            auto finite = [&](int t) { return t < inf ? t : 0; };
+            const int own = s_max[row], yl = row & (TY - 1);
+            int all = own;   // the largest of those that share the scale, finite or not
+            top = finite(own);
+            if (!g.sep) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const T a = rel<T, LX>(S + (c * TY + yl) * g.rsx, x);
-                fx q(0);
-                if (use[c]) {
-                    if constexpr (DW) q = fx_from(a, scalef[c]);
-                    else q = fx(__double2ll_rn(fx_ldexp(a, sc[c])));
+                for (int c = 0; c < 3; ++c) {
+                    all = max(all, s_max[c * TY + yl]);
+                    top = max(top, finite(s_max[c * TY + yl]));
                 }
-                rel<fx, LX>(S + (c * TY + yl) * g.rsx, x) = q;
+            }
+            const int top_e = ((top - (1 << (mant - 8))) >> mant) - bias, sc = min(58 - top_e, DW ? 150 : 1000);
+            e1 = fx_pack(top > 0 ? -sc - 1 : FX_ZERO, all < inf ? 0 : 1);
+            const float scalef = DW ? fx_pow2f(sc - 28) : 0.0f;
+            const bool use = top > 0 && own < inf;
+            for (int x = j; x < nx; x += g.Gx) {
+                const T a = rel<T, LX>(R, x);
+                fx q(0);
+                if (use) {
+                    if constexpr (DW) q = fx_from(a, scalef);
+                    else q = fx(__double2ll_rn(fx_ldexp(a, sc)));
+                }
+                rel<fx, LX>(R, x) = q;
             }
         }
     }
@@ -246,10 +250,8 @@ __device__ __forceinline__ void xfwd_body(const Geom &g, const FieldPtrs<T, F> &
             unsigned none = 0;
             const int sh = fft_row_fx<false, true, false, 2, LX, false>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j,
                                                                         tw, act, 0, 64, none);
-            if (tid < TY && y0 + tid < ny) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) P.fe1[(z * ny + y0 + tid) * 3 + c] = e1[c] + fx_pack(sh, 0);
-            }
+            const int c = row >> g.ltyf, y = y0 + (row & (TY - 1));
+            if (act && j == 0 && y < ny && (c == 0 || g.sep)) P.fe1[(z * ny + y) * (g.sep ? 3 : 1) + c] = e1 + fx_pack(sh, 0);
         } else {
             fft_row<false, true, false, 2, LX>(S + (act ? row : 0) * g.rsx, g.Hx, g.lhx, j, tw, act);
         }
@@ -399,29 +401,30 @@ template <int NZM> struct ZConv {
     }
 };
 
-// The same stage in block fixed point (F = fx), one scale per x-frequency and
-// component.  The plane is brought to full magnitude when it is loaded, before
-// the inverse transform and when it is stored; the z convolution, where the
-// tensor scales each frequency differently, has a scale per ky, which the
-// components that the tensor couples share.
-template <int PZ, int LY>
+// The same stage in block fixed point (F = fx), one scale per x-frequency, or
+// with SEP one per x-frequency and component.  The plane is brought to full
+// magnitude when it is loaded, before the inverse transform and when it is
+// stored; the z convolution, where the tensor scales each frequency differently,
+// has a scale per ky, which components that the tensor couples share.
+template <int PZ, int LY, bool SEP>
 __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double, fx> &P, const int tid, const int nth,
                                            const int kx)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fxc *S = reinterpret_cast<fxc *>(smem_raw);
-    __shared__ int s_e[3], s_top[3];
+    constexpr int NS = SEP ? 3 : 1;
+    __shared__ int s_e[NS], s_top[NS];
     // magnitudes in and out, sums of the frequencies' scales over the largest, flags
-    __shared__ unsigned s_r[10];
-    unsigned *s_in = s_r, *s_out = s_r + 3, *s_sum = s_r + 6, *s_fl = s_r + 9;
+    __shared__ unsigned s_r[3 * NS + 1];
+    unsigned *s_in = s_r, *s_out = s_r + NS, *s_sum = s_r + 2 * NS, *s_fl = s_r + 3 * NS;
     const int tt = tid < nth ? tid : MM_IDLE_START;
     const int ny = g.ny, nz = g.nz, Py = g.Py, nrow = 3 * nz;
     fxc *Wk = P.W + (long)kx * nrow * ny;
     fxmc *tw = reinterpret_cast<fxmc *>(S + nrow * g.rsy);
-    signed char *s_sc = reinterpret_cast<signed char *>(tw + Py);  // [2][3][Py]: scale and top bit of every ky
+    signed char *s_sc = reinterpret_cast<signed char *>(tw + Py);  // [2][NS][Py]: scale and top bit of every ky
     load_twiddles_async(tw, P.tw_py, Py, Py, tt, nth);
-    if (tid < 3) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
-    if (tid < 10) s_r[tid] = 0;
+    if (tid < NS) { s_e[tid] = FX_ZERO; s_top[tid] = FX_ZERO; }
+    if (tid < 3 * NS + 1) s_r[tid] = 0;
     __syncthreads();
 
     // Wk[z][y][c] -> row (c, z); the first loads are issued before the rows' scales are looked at
@@ -434,16 +437,16 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
             if (e0 + i * nth < tot) v[i] = ld_cg(Wk + e0 + i * nth);
     };
     if (tt < tot) load(tt);
-    fx_cta_scales(P.fe1, nz * ny, 3, tt, nth, s_e, s_fl);
+    fx_cta_scales<NS>(P.fe1, nz * ny, NS, tt, nth, s_e, s_fl);
     __syncthreads();
-    fx3 mags;
+    FxMags<NS> mags;
     for (int e0 = tt; e0 < tot;) {
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-            const int d = fx_exp(P.fe1[e]) - s_e[c];
+            const int d = fx_exp(P.fe1[SEP ? e : rest]) - s_e[SEP ? c : 0];
             if (d) v[i] = fx_scale(v[i], d);
             mags.or_in(c, fx_mag(v[i]));
             S[(c * nz + zz) * g.rsy + spos<fxc>(y)] = v[i];
@@ -461,7 +464,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     __syncthreads();
     const int rb = tid / g.Gy, j = tid - rb * g.Gy;  // row within a batch of g.RB rows
     const bool act = rb < g.RB;
-    auto comp = [&](int r) { return (r >= nz) + (r >= 2 * nz); };  // of a row
+    auto comp = [&](int r) { return SEP ? (r >= nz) + (r >= 2 * nz) : 0; };  // of a row
     int sh = 0;
     unsigned none = 0;
     for (int r0 = 0; r0 < nrow; r0 += g.RB) {
@@ -476,16 +479,15 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     const int hy = Py / 2, kst = hy + 1;
     constexpr int NC = 4 * ZConv<NZM>::NE + 2 * ZConv<NZM>::NO;
     const FxCouple couple{g.nx > 1 && ny > 1, NZM > 1 && g.nx > 1, NZM > 1 && ny > 1};
-    int eb[3], d[3];   // a component's scale where it is mixed, and its own over that
-    {
-        int own[3];
+    int eb[NS], d[NS], top[NS];   // a component's scale where it is mixed, its own over that, the largest output
 #pragma unroll
-        for (int c = 0; c < 3; ++c) eb[c] = own[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
-        couple.join(eb[0], eb[1], eb[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) d[c] = own[c] - eb[c];
+    for (int c = 0; c < NS; ++c) {
+        eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+        top[c] = FX_ZERO;
     }
-    int top[3] = {FX_ZERO, FX_ZERO, FX_ZERO};
+    couple.join(eb);
+#pragma unroll
+    for (int c = 0; c < NS; ++c) d[c] -= eb[c];
     for (int u = tt; u < 2 * Py; u += nth) {
         // a pair of lanes per ky: part 0 the real parts (of m_x, m_y and i m_z), part 1 the imaginary ones
         const int ky = u >> 1, part = u & 1, kyr = ky <= hy ? ky : Py - ky;
@@ -497,26 +499,27 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
         ZConv<NZM> z;
         z.K = P.Nhat + (long)kx * NC * kst + kyr;
         z.kst = kst;
-        int sc[3];
+        int sc[NS];
         {
             fx m[3][NZM];
-            unsigned mk[3] = {0, 0, 0};
+            FxMags<NS> mk;
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
                     m[c][n] = n < nz ? col[2 * (c * nz + n) * g.rsy + at[c]] : fx(0);
-                    mk[c] |= fx_mag(m[c][n]);
+                    mk.or_in(c, fx_mag(m[c][n]));
                 }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) sc[c] = fx_bits(mk[c] | __shfl_xor_sync(lanes, mk[c], 1)) + d[c];
-            couple.join(sc[0], sc[1], sc[2]);
+            for (int c = 0; c < NS; ++c) sc[c] = fx_bits(mk.v[c] | __shfl_xor_sync(lanes, mk.v[c], 1)) + d[c];
+            couple.join(sc);
+#pragma unroll
+            for (int c = 0; c < NS; ++c) sc[c] = 59 - sc[c];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                sc[c] = 59 - sc[c];
 #pragma unroll
                 for (int n = 0; n < NZM; ++n) {
-                    m[c][n] = fx_scale(m[c][n], sc[c] + d[c]);
+                    m[c][n] = fx_scale(m[c][n], sc[SEP ? c : 0] + d[SEP ? c : 0]);
                     if (flip[c]) m[c][n] = -m[c][n];
                 }
             }
@@ -541,32 +544,34 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
             const int tk = fx_bits(mag | __shfl_xor_sync(lanes, mag, 1)) - sc[c];
             if (part == 0) {
                 s_sc[c * Py + ky] = (signed char)sc[c];
-                s_sc[(3 + c) * Py + ky] = (signed char)tk;
+                s_sc[(NS + c) * Py + ky] = (signed char)tk;
             }
             top[c] = max(top[c], tk);
             mag = 0;
         };
         z.template output<0>([&](int n, fx r) { put(0, n, r); });
-        done(0);
+        if (SEP) done(0);
         z.template output<1>([&](int n, fx r) { put(1, n, r); });
-        done(1);
+        if (SEP) done(SEP ? 1 : 0);
         z.template output<2>([&](int n, fx r) { put(2, n, r); });
-        done(2);
+        done(SEP ? 2 : 0);
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) fx_cta_max(&s_top[c], top[c]);
+    for (int c = 0; c < NS; ++c) fx_cta_max(&s_top[c], top[c]);
     __syncthreads();
     // no partial sum of an inverse transform exceeds the sum of the largest moduli over ky
-    unsigned sum[3] = {0, 0, 0};
+    unsigned sum[NS];
+#pragma unroll
+    for (int c = 0; c < NS; ++c) sum[c] = 0;
     for (int ky = tt; ky < Py; ky += nth) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sum[c] += ((1u << 18) >> min(s_top[c] - s_sc[(3 + c) * Py + ky], 18)) + 1;
+        for (int c = 0; c < NS; ++c) sum[c] += ((1u << 18) >> min(s_top[c] - s_sc[(NS + c) * Py + ky], 18)) + 1;
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
+    for (int c = 0; c < NS; ++c) fx_cta_add(&s_sum[c], sum[c]);
     __syncthreads();
     auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
-    mags = fx3();
+    mags = FxMags<NS>();
     for (int r0 = 0; r0 < nrow; r0 += g.RB) {
         const int r = act ? r0 + rb : 0, c = comp(r);
         unsigned mag = 0;
@@ -578,14 +583,14 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     __syncthreads();
     for (int i = tt; i < tot; i += nth) {
         const int c = i % 3, rest = i / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], 60 - fx_bits(s_out[c]));
+        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], 60 - fx_bits(s_out[SEP ? c : 0]));
     }
-    if (tid < 3) {
+    if (tid < NS) {
         // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
         const int c = tid, fl = (int)*s_fl, hit = nz > 1 ? 7 : (c == 2 ? 4 : 3);
-        const int e = (c == 0 ? eb[0] : (c == 1 ? eb[1] : eb[2])) + P.fek[kx] - (NZM > 1 ? 1 : 0) +
+        const int e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] - (NZM > 1 ? 1 : 0) +
                       fx_cum(fx_log(Py), bound(c)) - (58 - s_top[c]) - (60 - fx_bits(s_out[c]));
-        P.fe2[kx * 3 + c] = fx_pack(e, fl & hit ? 1 : 0);
+        P.fe2[kx * NS + c] = fx_pack(e, (SEP ? fl & hit : fl) ? 1 : 0);
     }
 }
 
@@ -707,10 +712,10 @@ __global__ void __launch_bounds__(YZBound<float>::v, 1) k_yz(Geom g, FieldPtrs<f
     yz_body<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
 }
 
-template <int PZ, int LY>
+template <int PZ, int LY, bool SEP>
 __global__ void __launch_bounds__(YZBound<double>::v, 2) k_yz_fx(Geom g, FieldPtrs<double, fx> P)
 {
-    yz_body_fx<PZ, LY>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
+    yz_body_fx<PZ, LY, SEP>(g, P, threadIdx.x, blockDim.x, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -943,20 +948,26 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     const int nx = g.nx, ny = g.ny, nz = g.nz, Hx = g.Hx;
     const long N = g.N;
     TW *tw = reinterpret_cast<TW *>(S + 3 * TY * g.rsx);
-    // block fixed point, per component: the x-frequencies' largest scale, the sum of their scales over the largest, and
-    // the magnitude of this CTA's rows; and the flags
+    // block fixed point: the x-frequencies' largest scale and the sum of their scales over the largest, per component,
+    // and the flags; the magnitude of each row and the scale of its transform, by row for the reason given in xfwd_body
     __shared__ int s_e[3];
-    __shared__ unsigned s_r[7];
-    unsigned *s_fl = s_r, *s_sum = s_r + 1, *s_mag = s_r + 4;
-    fx3 mags;
+    __shared__ unsigned s_r[4];
+    __shared__ unsigned s_mag[3 * MM_MAX_TILE];
+    __shared__ double s_scale[3 * MM_MAX_TILE];
+    unsigned *s_fl = s_r, *s_sum = s_r + 1;
+    unsigned mag = 0;
     const int *fe2 = nullptr;
-    const int fst = 3 * g.nzb;     // ints from one x-frequency's scales to the next's
+    const int ns = g.sep ? 3 : 1, fst = ns * g.nzb;   // ints from one x-frequency's scales to the next's
+    const bool sep = g.sep;
+    auto own = [&](int c) { return sep ? c : 0; };   // which of the scales is a component's
     if constexpr (is_fx<F>) {
-        fe2 = P.fe2 + 3 * (z / g.ZB);
+        fe2 = P.fe2 + ns * (z / g.ZB);
         if (tid < 3) s_e[tid] = FX_ZERO;
-        if (tid < 7) s_r[tid] = 0;
+        if (tid < 4) s_r[tid] = 0;
+        if (tid < 3 * TY) s_mag[tid] = 0;
         __syncthreads();
-        fx_cta_scales(fe2, g.C, fst, tt, nth, s_e, s_fl);
+        if (sep) fx_cta_scales<3>(fe2, g.C, fst, tt, nth, s_e, s_fl);
+        else fx_cta_scales<1>(fe2, g.C, fst, tt, nth, s_e, s_fl);
     }
 
     MinState *st = P.st;
@@ -1005,22 +1016,22 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
     // With sum and dif the two brackets and t = conj(w^k) dif, Z[k] = sum + i t and
     // (w^Hx = -1) Z[Hx-k] = sum* + i t*: one item per pair k = 0..Hx/2 loads X[k] and
     // X[Hx-k] once.  The loads of PF items per thread are issued before any is used.
+    // A thread's items are all of one row (c, yl): it takes every ks-th k.
     constexpr int PF = sizeof(V) == 8 ? 8 : 4;
-    const int hh = Hx >> 1;
-    const int nel = TY * 3 * (hh + 1);
+    const int hh = Hx >> 1, ks = nth / (3 * TY), k0 = tid / (3 * TY), q = tid - k0 * 3 * TY, c = q % 3, yl = q / 3;
+    const bool mine = k0 < ks;
     const long strideK = (long)3 * nz * ny;
-    for (int g0 = 0; g0 < nel; g0 += PF * nth) {  // trip count uniform over the CTA (barrier inside)
-        const int e0 = g0 + tt;
+    V *const row = S + (c * TY + yl) * g.rsx;
+    const V *const Wrow = P.W + ((long)z * ny + y0 + yl) * 3 + c;
+    for (int g0 = 0; g0 <= hh; g0 += PF * ks) {  // trip count uniform over the CTA (barrier inside)
         V xa[PF], xb[PF];
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
-            const int e = e0 + i * nth;
-            const int c = e % 3, rest = e / 3, yl = rest & (TY - 1), kk = rest >> g.lty;
+            const int kk = g0 + k0 + i * ks;
             xa[i] = czero<V>(); xb[i] = czero<V>();
-            if (e < nel && y0 + yl < ny) {
-                const long base = ((long)z * ny + y0 + yl) * 3 + c;
-                xa[i] = ld_nc(P.W + (long)kk * strideK + base);
-                xb[i] = ld_nc(P.W + (long)(Hx - kk) * strideK + base);
+            if (mine && kk <= hh && y0 + yl < ny) {
+                xa[i] = ld_nc(Wrow + (long)kk * strideK);
+                xb[i] = ld_nc(Wrow + (long)(Hx - kk) * strideK);
             }
         }
         if (g0 == 0) {  // the twiddles (first commit group) are needed from here on
@@ -1030,23 +1041,23 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
                 unsigned sum[3] = {0, 0, 0};
                 for (int i = tt; i < g.C; i += nth) {
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) sum[c] += ((1u << 18) >> min(s_e[c] - fx_exp(fe2[i * fst + c]), 18)) + 1;
+                    for (int a = 0; a < 3; ++a)
+                        if (a == 0 || sep) sum[a] += ((1u << 18) >> min(s_e[a] - fx_exp(fe2[i * fst + a]), 18)) + 1;
                 }
 #pragma unroll
-                for (int c = 0; c < 3; ++c) fx_cta_add(&s_sum[c], sum[c]);
+                for (int a = 0; a < 3; ++a)
+                    if (a == 0 || sep) fx_cta_add(&s_sum[a], sum[a]);
             }
         }
 #pragma unroll
         for (int i = 0; i < PF; ++i) {
-            const int e = e0 + i * nth;
-            if (e >= nel) break;
-            const int c = e % 3, rest = e / 3, yl = rest & (TY - 1), kk = rest >> g.lty;
-            V *row = S + (c * TY + yl) * g.rsx;
+            const int kk = g0 + k0 + i * ks;
+            if (!mine || kk > hh) break;
             V Z;
             V Xk = xa[i], Xm = cconj(xb[i]);
             if constexpr (is_fx<F>) {  // components below 2^60: |Z| < 2^62
-                Xk = fx_scale(Xk, fx_exp(fe2[kk * fst + c]) - s_e[c]);
-                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * fst + c]) - s_e[c]);
+                Xk = fx_scale(Xk, fx_exp(fe2[kk * fst + own(c)]) - s_e[own(c)]);
+                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * fst + own(c)]) - s_e[own(c)]);
             }
             const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
             V t;
@@ -1055,50 +1066,47 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             Z.x = sum.x - t.y;
             Z.y = sum.y + t.x;
             row[rpos<V, LX>(kk)] = Z;
-            if constexpr (is_fx<F>) mags.or_in(c, fx_mag(Z));
+            if constexpr (is_fx<F>) mag |= fx_mag(Z);
             if (kk != 0 && Hx - kk != kk) {
                 Z.x = sum.x + t.y;
                 Z.y = t.x - sum.y;
                 row[rpos<V, LX>(Hx - kk)] = Z;
-                if constexpr (is_fx<F>) mags.or_in(c, fx_mag(Z));
+                if constexpr (is_fx<F>) mag |= fx_mag(Z);
             }
         }
     }
-    if constexpr (is_fx<F>) mags.cta_or(s_mag);
+    constexpr bool DW = std::is_same<T, dfloat>::value;
+    if constexpr (is_fx<F>) {
+        if (mine && mag) atomicOr(&s_mag[c * TY + yl], mag);
+    }
     __syncthreads();
     // the moduli of a row sum to at most 2^62 times the frequencies' scales over the largest
-    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18 + 62 - fx_bits(s_mag[c])); };
+    auto bound = [&](int r) { return max(0, fx_log2_up(s_sum[own(r >> g.lty)]) - 18 + 62 - fx_bits(s_mag[r])); };
+    if constexpr (is_fx<F>) {
+        if (tid < 3 * TY) {
+            // one unit of the row's values after its transform, in A/m (of double-words in two factors below the range of one)
+            const int e = s_e[own(tid >> g.lty)] + fx_cum(fx_log(Hx), bound(tid)) - (58 - fx_bits(s_mag[tid]));
+            if constexpr (DW)
+                *reinterpret_cast<float2 *>(&s_scale[tid]) = make_float2(fx_pow2f(e < -100 ? e + 64 : e),
+                                                                         e < -100 ? 5.42101086e-20f : 1.0f);   // 2^-64
+            else
+                s_scale[tid] = fx_pow2(e);
+        }
+    }
     {
         const int row = tid / g.Gx, j = tid - row * g.Gx;
         const bool act = row < 3 * TY;
         if constexpr (is_fx<F>) {
-            const int c = act ? row >> g.lty : 0;
+            const int r = act ? row : 0;
             unsigned none = 0;
-            fft_row_fx<true, false, true, 2, LX, false>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act,
-                                                        58 - fx_bits(s_mag[c]), bound(c), none);
+            fft_row_fx<true, false, true, 2, LX, false>(S + r * g.rsx, Hx, g.lhx, j, tw, act, 58 - fx_bits(s_mag[r]),
+                                                        bound(r), none);
         } else {
             fft_row<true, false, true, 2, LX>(S + (act ? row : 0) * g.rsx, Hx, g.lhx, j, tw, act);
         }
     }
-    constexpr bool DW = std::is_same<T, dfloat>::value;
-    // block fixed point: one unit of a component's values, in A/m (of double-words in two factors below the range of one)
-    double dscale[3];
-    float dscalef[3], dtiny[3];
     int bad = 0;
-    if constexpr (is_fx<F>) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int e = s_e[c] + fx_cum(fx_log(Hx), bound(c)) - (58 - fx_bits(s_mag[c]));
-            const bool tiny = DW && e < -100;
-            if constexpr (DW) {
-                dscalef[c] = fx_pow2f(tiny ? e + 64 : e);
-                dtiny[c] = tiny ? 5.42101086e-20f : 1.0f;   // 2^-64
-            } else {
-                dscale[c] = fx_pow2(e);
-            }
-        }
-        bad = (int)*s_fl;
-    }
+    if constexpr (is_fx<F>) bad = sep || !*s_fl ? (int)*s_fl : 7;
     cp_async_wait_all();
     if (stg) __syncthreads();
 
@@ -1131,16 +1139,18 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             const fx q0 = rel<F, LX>(S + (0 * TY + yl) * g.rsx, x), q1 = rel<F, LX>(S + (1 * TY + yl) * g.rsx, x),
                      q2 = rel<F, LX>(S + (2 * TY + yl) * g.rsx, x);
             if constexpr (DW) {
-                d0 = fx_to_dfloat(q0, dscalef[0]);
-                d1 = fx_to_dfloat(q1, dscalef[1]);
-                d2 = fx_to_dfloat(q2, dscalef[2]);
-                d0.hi *= dtiny[0]; d0.lo *= dtiny[0];
-                d1.hi *= dtiny[1]; d1.lo *= dtiny[1];
-                d2.hi *= dtiny[2]; d2.lo *= dtiny[2];
+                dfloat *d[3] = {&d0, &d1, &d2};
+                const fx q[3] = {q0, q1, q2};
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float2 f = *reinterpret_cast<const float2 *>(&s_scale[c * TY + yl]);
+                    *d[c] = fx_to_dfloat(q[c], f.x);
+                    if (f.y != 1.0f) { d[c]->hi *= f.y; d[c]->lo *= f.y; }
+                }
             } else {
-                d0 = __ll2double_rn(q0.v) * dscale[0];
-                d1 = __ll2double_rn(q1.v) * dscale[1];
-                d2 = __ll2double_rn(q2.v) * dscale[2];
+                d0 = __ll2double_rn(q0.v) * s_scale[yl];
+                d1 = __ll2double_rn(q1.v) * s_scale[TY + yl];
+                d2 = __ll2double_rn(q2.v) * s_scale[2 * TY + yl];
             }
             if (bad) {  // uniform over the CTA
                 T nan;
@@ -1361,7 +1371,7 @@ template <typename T> size_t smem_yz_t(const Geom &g)
     typedef typename cvec<typename fft_of<T>::type>::type V;
     // rows and Py twiddles,
     // and the block fixed-point kernel two bytes per y-frequency and component
-    return ((size_t)3 * g.nz * g.rsy + g.Py) * sizeof(V) + (sizeof(T) == 4 ? 0 : 6 * (size_t)g.Py);
+    return ((size_t)3 * g.nz * g.rsy + g.Py) * sizeof(V) + (sizeof(T) == 4 ? 0 : (g.sep ? 6 : 2) * (size_t)g.Py);
 }
 
 // The field kernels are compiled for a set of FFT row lengths (template

@@ -38,11 +38,12 @@ struct __align__(16) fxmc {
     fxm x, y;
 };
 
-// The three components have scales of their own: where the tensor does not
-// couple them (axes of one cell), or where one is not mixed with the others yet,
-// a component is as accurate as its own size allows.  (With one scale for the
-// three, the in-plane field of a one-layer film magnetised along z with a tilt of
-// 1e-8 was off by 1e-8 of itself.)
+// The three components have scales of their own where they are not all mixed by
+// the tensor (Geom::sep): a component is then as accurate as its own size allows.
+// (With one scale for the three, the in-plane field of a one-layer film
+// magnetised along z with a tilt of 1e-8 was off by 1e-8 of itself.)  Where all
+// are mixed, a field component gathers the rounding of the largest in any
+// arithmetic, and they share one.
 // Scale of a block as the kernels hand it on: e * 4 + flag.  Non-finite inputs
 // have no place in a block; their component is taken as zero and flagged (1),
 // and comes out as NaN where the field would.
@@ -214,36 +215,44 @@ __device__ __forceinline__ void fx_cta_add(unsigned *dst, unsigned v)
     v = __reduce_add_sync(0xffffffffu, v);
     if ((threadIdx.x & 31) == 0) atomicAdd(dst, v);
 }
-// one value per component, added to by component number
-struct fx3 {
-    unsigned v[3] = {0, 0, 0};
+// N = 3: one value per component, added to by component number; N = 1: one for all
+template <int N> struct FxMags {
+    unsigned v[N];
+    __device__ __forceinline__ FxMags()
+    {
+#pragma unroll
+        for (int c = 0; c < N; ++c) v[c] = 0;
+    }
     __device__ __forceinline__ void or_in(int c, unsigned x)
     {
-        v[0] |= c == 0 ? x : 0; v[1] |= c == 1 ? x : 0; v[2] |= c == 2 ? x : 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] |= N == 1 || c == i ? x : 0;
     }
     __device__ __forceinline__ void cta_or(unsigned *dst) const
     {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) fx_cta_or(dst + c, v[c]);
+        for (int c = 0; c < N; ++c) fx_cta_or(dst + c, v[c]);
     }
 };
-// Largest exponent of each component, and the flags (bit c), of the scales
-// p[i * stride + c], i < n, over the CTA; a barrier makes them visible
-__device__ __forceinline__ void fx_cta_scales(const int *p, int n, long stride, int tt, int nth, int *s_e,
-                                              unsigned *s_fl)
+// Largest exponents and the flags (bit c) of the scales p[i * stride + c], i < n,
+// c < N, over the CTA; a barrier makes them visible
+template <int N> __device__ __forceinline__ void fx_cta_scales(const int *p, int n, long stride, int tt, int nth, int *s_e,
+                                                               unsigned *s_fl)
 {
-    int e[3] = {FX_ZERO, FX_ZERO, FX_ZERO};
+    int e[N];
+#pragma unroll
+    for (int c = 0; c < N; ++c) e[c] = FX_ZERO;
     unsigned fl = 0;
     for (int i = tt; i < n; i += nth) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < N; ++c) {
             const int q = p[i * stride + c];
             e[c] = max(e[c], fx_exp(q));
             fl |= (unsigned)fx_flags(q) << c;
         }
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) fx_cta_max(s_e + c, e[c]);
+    for (int c = 0; c < N; ++c) fx_cta_max(s_e + c, e[c]);
     fx_cta_or(s_fl, fl);
 }
 // Components that the tensor couples (pairs of axes that both have more than
@@ -251,12 +260,14 @@ __device__ __forceinline__ void fx_cta_scales(const int *p, int n, long stride, 
 // pairs are coupled, one, or none.
 struct FxCouple {
     bool xy, xz, yz;
-    __device__ __forceinline__ void join(int &a, int &b, int &c) const
+    __device__ __forceinline__ void join(int (&e)[3]) const
     {
-        const int x = max(a, max(xy ? b : a, xz ? c : a)), y = max(b, max(xy ? a : b, yz ? c : b)),
-                  z = max(c, max(xz ? a : c, yz ? b : c));
-        a = x; b = y; c = z;
+        const int a = e[0], b = e[1], c = e[2];
+        e[0] = max(a, max(xy ? b : a, xz ? c : a));
+        e[1] = max(b, max(xy ? a : b, yz ? c : b));
+        e[2] = max(c, max(xz ? a : c, yz ? b : c));
     }
+    __device__ __forceinline__ void join(int (&)[1]) const {}
 };
 // least t >= 0 with 2^t >= v
 __device__ __forceinline__ int fx_log2_up(unsigned v) { return v > 1 ? 32 - __clz((int)(v - 1)) : 0; }

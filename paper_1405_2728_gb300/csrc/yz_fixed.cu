@@ -6,10 +6,16 @@
 
 namespace {
 
+// One layer never has all components coupled.  With more, a grid of one column or
+// row is the exception, and takes the code for any length.
 template <int PZ> cudaError_t launch(const Geom &g, const FieldPtrs<double, fx> &P, cudaStream_t s)
 {
+    if (PZ > 1 && g.sep) {
+        k_yz_fx<PZ, -1, true><<<g.C, threads_yz<double>(g), smem_yz_t<double>(g), s>>>(g, P);
+        return cudaGetLastError();
+    }
     switch (ly_of(g.Py)) {
-#define C(L) case L: k_yz_fx<PZ, L><<<g.C, threads_yz<double>(g), smem_yz_t<double>(g), s>>>(g, P); break;
+#define C(L) case L: k_yz_fx<PZ, L, PZ == 1><<<g.C, threads_yz<double>(g), smem_yz_t<double>(g), s>>>(g, P); break;
         MM_LY_CASES(C)
 #undef C
     default: return cudaErrorInvalidValue;
@@ -19,8 +25,9 @@ template <int PZ> cudaError_t launch(const Geom &g, const FieldPtrs<double, fx> 
 
 template <int PZ> cudaError_t configure(const Geom &g, size_t smem)
 {
+    if (PZ > 1 && g.sep) return smem_attr(k_yz_fx<PZ, -1, true>, smem);
     switch (ly_of(g.Py)) {
-#define C(L) case L: return smem_attr(k_yz_fx<PZ, L>, smem);
+#define C(L) case L: return smem_attr(k_yz_fx<PZ, L, PZ == 1>, smem);
         MM_LY_CASES(C)
 #undef C
     }

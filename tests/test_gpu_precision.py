@@ -129,3 +129,37 @@ def test_components_of_different_size(mmlib, grid, prec, bar):
             for c in range(3):
                 mixed = np.sqrt(sum(np.sum(m[a] ** 2) for a in range(3) if coupled(p.shape, a, c)))
                 assert np.linalg.norm(H[c] - ref[c]) <= bar * p.Ms * mixed, (big, tilt, c)
+
+
+def test_grouped_batch_with_grids_of_one_row_or_column_equals_single_sweeps(mmlib):
+    sizes = [(24, 1, 3), (1, 20, 2), (16, 9, 2), (40, 1, 1), (1, 150, 4), (12, 10, 4)]
+    probs = [make_pair(mmlib, *n, (4e-9, 3e-9, 5e-9))[0] for n in sizes]
+    F = np.array([[2e4, 1e3, 0.0], [-1e4, 1e3, 0.0]])
+    opts = mmlib.make_opts(max_iter=6)
+    batch = mmlib.mm_batch_create(probs, mmlib.MM_BATCH_GROUPED)
+    starts = [smooth((nz, ny, nx), 5 + nx) for nx, ny, nz in sizes]
+    starts = [dev(m / np.sqrt((m * m).sum(0))) for m in starts]
+    ms = [m.clone() for m in starts]
+    _, mavg, _ = mmlib.mm_batch_sweep(batch, ms, F, opts=opts)
+    for i, p in enumerate(probs):
+        _, mavg1, _ = mmlib.mm_hysteresis_sweep(p, starts[i], F, opts=opts)
+        assert torch.equal(ms[i], starts[i]) and np.array_equal(mavg[i], mavg1), sizes[i]
+    batch.close()
+
+
+@pytest.mark.parametrize("prec,bar", [("MM_FP64", 2e-15), ("MM_F32X2", 1e-13)])
+def test_field_does_not_depend_on_the_tile_chosen_by_timing(mmlib, prec, bar):
+    """Rows of very different magnitude (as the Hessian product and the adjoint evaluate): problems of one grid, whose
+    tiles are timed anew at each setup, and a repeated evaluation give the same bits, and the rows' scales the accuracy
+    of one scale."""
+    grid = (130, 128, 4)   # above the size from which tiles are timed
+    m = smooth((4, 128, 130), 9) * 2.0 ** (-3.0 * (np.arange(128) % 13)).reshape(1, 1, 128, 1)
+    fields, tiles = [], set()
+    for _ in range(6):
+        prob, p = make_pair(mmlib, *grid, (4e-9, 3e-9, 5e-9), A=0.0, K=0.0, precision=getattr(mmlib, prec))
+        tiles.add(mmlib.mm_problem_info(prob)["x_fwd_tile_rows"])
+        fields += [field(mmlib, prob, m, (0, 0, 0)) for _ in range(2)]
+        prob.close()
+    assert all(np.array_equal(f, fields[0]) for f in fields), tiles
+    ref = om.Demag(p).field(m)
+    assert np.linalg.norm(fields[0] - ref) <= bar * p.Ms * np.linalg.norm(m)
