@@ -168,7 +168,7 @@ int plan(mm_problem *p)
     Geom &g = p->g;
     const mm_grid &gr = p->grid;
     g.nx = gr.nx; g.ny = gr.ny; g.nz = gr.nz;
-    g.sep = mm_separate(g);
+    g.sep = mm_separate(gr);
     // what is supported, and in which layout, is decided on powers of two
     const int P2[3] = {next_pow2(2 * gr.nx - 1), next_pow2(2 * gr.ny - 1), next_pow2(2 * gr.nz - 1)};
     auto lengths = [&](int Px, int Py, int Pz) {

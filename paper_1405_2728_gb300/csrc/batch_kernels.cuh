@@ -17,7 +17,7 @@ __device__ __forceinline__ void yz_of(const Geom &g, const FieldPtrs<T> &P, int 
     if constexpr (!is_fx<FA<T>>) yz_body<PZ, L>(g, P, tid, nth, kx);
     else if constexpr (L == 0 && !(SEP && PZ == 1)) yz_body_fx<PZ, -1, (SEP || PZ == 1)>(g, P, tid, nth, kx);
 }
-// double grids of one column or row with several layers: a kernel of their own (SEP), launched if a batch has one, as
+// double grids of several layers with scales per component: a kernel of their own (SEP), launched if a batch has one, as
 // both kinds in one kernel spill 2 KB a thread
 template <typename T> __host__ __device__ inline bool group_sep(const Geom &g) { return is_fx<FA<T>> && g.sep && g.Pz > 1; }
 

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     if constexpr (FX) {
 #pragma unroll
         for (int c = 0; c < NS; ++c) {
-            eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+            eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh + (SEP ? g.tsc[c] : 0);
             top[c] = FX_ZERO;
         }
         couple.join(eb);
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     if constexpr (FX) {
         if (tid < NS) {
             const int c = tid, e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] +
-                                   fx_cum(fx_log(Pz), bound(c)) - (58 - s_top[c]) - post(c);
+                                   fx_cum(fx_log(Pz), bound(c)) - (58 - s_top[c]) - post(c) + (SEP ? g.tsc[c] : 0);
             P.feb[((long)kx * g.nkb + blockIdx.y) * NS + c] = fx_pack(e, *s_fl ? 1 : 0);  // the tensor mixes all components
         }
     }

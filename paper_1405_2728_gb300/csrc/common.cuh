@@ -176,7 +176,8 @@ struct Geom {
     int RBZ;               // z rows transformed at once in the z pass
     int nzb, nkb;          // blocks of ZB z planes (film layout: one block of all), of KB y frequencies
     int lpz, Gz, rsz;      // likewise of Pz, threads per z row, smem stride of a z row
-    int sep;               // block fixed point: components have scales of their own (mm_separate)
+    int sep;               // block fixed point: components have scales of their own (mm_separate),
+    int tsc[3];            // and the tensor's element ab is held over 2^(tsc[a] + tsc[b]) (mm_tensor_spectrum; else 0)
     int nbody;             // kernels per minimiser iteration (3 film, 5 bulk)
     long N;                // cells
     double dx, dy, dz;
@@ -365,10 +366,17 @@ MM_DECLARE_FIELD_ENTRIES(f32x2)
 #define MM_SMEM_CAP (200 * 1024)
 
 // Whether the components keep scales of their own in block fixed point: an axis
-// of one cell, whose pairs the tensor does not mix.  A grid's kernels that share
-// one are faster (k_yz_fx at 512 x 256 x 4: 121 us, with three scales 130; the z
-// pass of 64^3: 102 and 112 us).
-__host__ __device__ inline bool mm_separate(const Geom &g) { return g.nx == 1 || g.ny == 1 || g.nz == 1; }
+// of one cell, whose pairs the tensor does not mix, or cells flatter than 1:16,
+// whose tensor has elements much smaller than its largest (N_xx of a film of cells
+// 1:10^4 is 10^-4 of N_zz).  Grids whose kernels share one scale are faster (k_yz_fx at
+// 512 x 256 x 4: 123 us, with three scales 130; the z pass of 64^3: 102 and 112
+// us), and lose nothing: at 1:16 an element is still held to 2^-57 of itself.
+inline bool mm_separate(const mm_grid &g)
+{
+    const double lo = g.dx < g.dy ? (g.dx < g.dz ? g.dx : g.dz) : (g.dy < g.dz ? g.dy : g.dz);
+    const double hi = g.dx > g.dy ? (g.dx > g.dz ? g.dx : g.dz) : (g.dy > g.dz ? g.dy : g.dz);
+    return g.nx == 1 || g.ny == 1 || g.nz == 1 || hi > 16.0 * lo;
+}
 
 // tensor elements per (kx, ky) of the film layout: six components at
 // max(1, Pz/2) z offsets, or the combinations of them that the block

@@ -482,7 +482,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     int eb[NS], d[NS], top[NS];   // a component's scale where it is mixed, its own over that, the largest output
 #pragma unroll
     for (int c = 0; c < NS; ++c) {
-        eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh;
+        eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh + (SEP ? g.tsc[c] : 0);
         top[c] = FX_ZERO;
     }
     couple.join(eb);
@@ -589,7 +589,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
         // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
         const int c = tid, fl = (int)*s_fl, hit = nz > 1 ? 7 : (c == 2 ? 4 : 3);
         const int e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] - (NZM > 1 ? 1 : 0) +
-                      fx_cum(fx_log(Py), bound(c)) - (58 - s_top[c]) - (60 - fx_bits(s_out[c]));
+                      fx_cum(fx_log(Py), bound(c)) - (58 - s_top[c]) - (60 - fx_bits(s_out[c])) + (SEP ? g.tsc[c] : 0);
         P.fe2[kx * NS + c] = fx_pack(e, (SEP ? fl & hit : fl) ? 1 : 0);
     }
 }

@@ -39,7 +39,7 @@ struct __align__(16) fxmc {
 };
 
 // The three components have scales of their own where they are not all mixed by
-// the tensor (Geom::sep): a component is then as accurate as its own size allows.
+// the tensor, or unequally (Geom::sep): a component is then as accurate as its own size allows.
 // (With one scale for the three, the in-plane field of a one-layer film
 // magnetised along z with a tilt of 1e-8 was off by 1e-8 of itself.)  Where all
 // are mixed, a field component gathers the rounding of the largest in any

@@ -21,6 +21,9 @@
 //                    the convolution kernels need no other normalisation.
 //  k_tensor_fixed    double and double-word problems: the spectra from doubles
 //                    to the multipliers of the block fixed-point convolution.
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
 #include "dd.cuh"
 #include "fft.cuh"
@@ -174,13 +177,17 @@ __global__ void k_extract_film(int c, int Px, int Py, int nz, int nzf, const dou
 // that the magnitudes of the terms of any one output value sum to less than 1:
 // over the sources' components and, for films, z offsets (offset 0 once, the
 // others on both sides).
+// Element ab is first divided by 2^(tsc[a] + tsc[b]) (balance[c], an exact power of two).
 // Bulk (NZM = 0), in place: K[i * 6 + c], i < n frequencies.
 // Film, from K[(dz * 6 + c) * n + i] to out[coefficient * n + i], i < n ky
 // values: the combinations of the offsets that ZConv multiplies with, formed
 // from the rounded elements so that they are exact.
+struct Balance {
+    double f[6];
+};
 template <int NZM>
 __global__ void __launch_bounds__(256) k_tensor_fixed(const double *K, long per_kx, fxm *out, long out_kx, int n,
-                                                      int *ek)
+                                                      int *ek, Balance bal)
 {
     const double *Kx = K + blockIdx.x * per_kx;
     fxm *Ox = out + blockIdx.x * out_kx;
@@ -190,7 +197,7 @@ __global__ void __launch_bounds__(256) k_tensor_fixed(const double *K, long per_
         double r0 = 0.0, r1 = 0.0, r2 = 0.0;
         for (int dz = 0; dz < (NZM ? NZM : 1); ++dz) {
             double k[6];
-            for (int c = 0; c < 6; ++c) k[c] = fabs(NZM ? Kx[((long)dz * 6 + c) * n + i] : Kx[(long)i * 6 + c]);
+            for (int c = 0; c < 6; ++c) k[c] = bal.f[c] * fabs(NZM ? Kx[((long)dz * 6 + c) * n + i] : Kx[(long)i * 6 + c]);
             const double w = dz ? 2.0 : 1.0;
             r0 += w * (k[0] + k[3] + k[4]);
             r1 += w * (k[3] + k[1] + k[5]);
@@ -209,13 +216,14 @@ __global__ void __launch_bounds__(256) k_tensor_fixed(const double *K, long per_
     const int e = top > 0.0 && isfinite(top) ? ilogb(top) + 2 : 0;
     if (threadIdx.x == 0) ek[blockIdx.x] = e;
     if constexpr (NZM == 0) {
-        for (long q = threadIdx.x; q < per_kx; q += 256) Ox[q] = fx_multiplier(__double2ll_rn(scalbn(Kx[q], 62 - e)));
+        for (long q = threadIdx.x; q < per_kx; q += 256)
+            Ox[q] = fx_multiplier(__double2ll_rn(scalbn(bal.f[q % 6] * Kx[q], 62 - e)));
     } else {
         for (int i = threadIdx.x; i < n; i += 256) {
             fxm *o = Ox + i;
             for (int c = 0; c < 6; ++c) {
                 long long k[4] = {0, 0, 0, 0};
-                for (int dz = 0; dz < NZM; ++dz) k[dz] = __double2ll_rn(scalbn(Kx[((long)dz * 6 + c) * n + i], 62 - e));
+                for (int dz = 0; dz < NZM; ++dz) k[dz] = __double2ll_rn(scalbn(bal.f[c] * Kx[((long)dz * 6 + c) * n + i], 62 - e));
                 auto put = [&](long long v) { *o = fx_multiplier(v); o += n; };
                 if (c < 4) {  // even in z
                     if (NZM == 1) put(k[0]);
@@ -269,6 +277,22 @@ int mm_newell_device(const mm_grid *gr, double *N_dev, cudaStream_t s)
 int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
 {
     const Geom &g = p->g;
+    // Block fixed point with scales per component: the tensor is balanced by powers of two, so that elements between
+    // components of small self-demagnetisation (flat cells) keep their bits beside those of large: N_ab is at most about
+    // sqrt(N_aa N_bb), and the self terms stand for N_aa.
+    Balance bal;
+    for (int c = 0; c < 6; ++c) bal.f[c] = 1.0;
+    if (p->precision != MM_FP32 && g.sep) {
+        double self[3] = {0.0, 0.0, 0.0};
+        cudaError_t e = cudaSuccess;
+        for (int c = 0; c < 3 && !e; ++c)
+            e = cudaMemcpyAsync(&self[c], N_dev + c * g.N, sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (!e) e = cudaStreamSynchronize(s);
+        if (e) { mm_set_cuda_error(e, "tensor self terms"); return MM_ERR_CUDA; }
+        const int ab[6][2] = {{0, 0}, {1, 1}, {2, 2}, {0, 1}, {0, 2}, {1, 2}};
+        for (int c = 0; c < 3; ++c) p->g.tsc[c] = self[c] > 0.0 && self[c] < 1.0 ? std::max(ilogb(self[c]) / 2, -60) : 0;
+        for (int c = 0; c < 6; ++c) bal.f[c] = ldexp(1.0, -(g.tsc[ab[c][0]] + g.tsc[ab[c][1]]));
+    }
     const long tot = (long)g.Px * g.Py * g.Pz;
     double2 *F = nullptr, *tw = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&F, sizeof(double2) * tot, s);
@@ -338,11 +362,11 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
         int *ek = p->fexp + mm_scale_fek(g);
         if (g.bulk) {
             const int n = (g.Pz / 2 + 1) * (hy + 1);
-            k_tensor_fixed<0><<<g.C, 256, 0, s>>>((const double *)K64, (long)n * 6, out, (long)n * 6, n, ek);
+            k_tensor_fixed<0><<<g.C, 256, 0, s>>>((const double *)K64, (long)n * 6, out, (long)n * 6, n, ek, bal);
         } else {
             const long in = (long)nzf * 6 * (hy + 1), no = (long)mm_film_coefs(g, p->precision) * (hy + 1);
             auto *k = nzf == 1 ? k_tensor_fixed<1> : (nzf == 2 ? k_tensor_fixed<2> : k_tensor_fixed<4>);
-            k<<<g.C, 256, 0, s>>>((const double *)K64, in, out, no, hy + 1, ek);
+            k<<<g.C, 256, 0, s>>>((const double *)K64, in, out, no, hy + 1, ek, bal);
         }
         e = cudaGetLastError();
     }

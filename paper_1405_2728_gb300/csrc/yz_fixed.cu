@@ -7,7 +7,7 @@
 namespace {
 
 // One layer never has all components coupled.  With more, a grid of one column or
-// row is the exception, and takes the code for any length.
+// row or of very flat cells is the exception, and takes the code for any length.
 template <int PZ> cudaError_t launch(const Geom &g, const FieldPtrs<double, fx> &P, cudaStream_t s)
 {
     if (PZ > 1 && g.sep) {

@@ -163,3 +163,26 @@ def test_field_does_not_depend_on_the_tile_chosen_by_timing(mmlib, prec, bar):
     assert all(np.array_equal(f, fields[0]) for f in fields), tiles
     ref = om.Demag(p).field(m)
     assert np.linalg.norm(fields[0] - ref) <= bar * p.Ms * np.linalg.norm(m)
+
+
+@pytest.mark.parametrize("prec,bar", [("MM_FP64", 2e-15), ("MM_F32X2", 1e-13)])
+@pytest.mark.parametrize("cell", [(4e-9, 4e-9, 4e-13), (4e-13, 3e-9, 4e-9), (4e-9, 2e-10, 5e-9)])
+@pytest.mark.parametrize("grid", [(24, 20, 1), (40, 1, 1), (18, 12, 2), (12, 10, 4), (1, 20, 3), (8, 9, 7), (12, 1, 9)])
+def test_flat_cells(mmlib, grid, cell, prec, bar):
+    """Cells whose tensor has elements far below its largest: every component is accurate to the products that form it.
+    The bars are those of random states, relative to the sum over the components of the largest modulus of the element's
+    transform times the component."""
+    nx, ny, nz = grid
+    if prec == "MM_F32X2" and nz > 4:
+        pytest.skip("double-word problems are films")
+    prob, p = make_pair(mmlib, nx, ny, nz, cell, A=0.0, K=0.0, precision=getattr(mmlib, prec))
+    d = om.Demag(p)
+    top = [[p.Ms * np.max(abs(N)) for N in row] for row in om._sym(d.Nhat)]
+    for big in range(3):
+        for tilt in (0.3, 1e-8):
+            m = tilt * smooth(p.shape, 11 + big)
+            m[big] = 1.0
+            H, ref = field(mmlib, prob, m, (0, 0, 0)), d.field(m)
+            for c in range(3):
+                terms = sum(top[c][b] * np.linalg.norm(m[b]) for b in range(3) if coupled(p.shape, b, c))
+                assert np.linalg.norm(H[c] - ref[c]) <= bar * terms, (big, tilt, c)
