@@ -283,8 +283,10 @@ MM_API int mm_energy_gradient(mm_problem *prob, const void *m, const double Hext
  * tangent field v (units A/m; times mu0 Ms V it is the Riemannian Hessian of U):
  *   Av = P_m((m.H) v - L v)  (= (m.H) v - P_m(L v) for tangent v),  H = H_eff(m),
  *   L v = H_eff(v) without the external field,  P_m w = w - (m.w) m.
- * m, v, Av: host or device [3][nz][ny][nx].  Overwrites the minimiser's work
- * buffers (a later mm_minimize / mm_hysteresis_sweep starts from its own m).
+ * m, v, Av: host or device [3][nz][ny][nx].  Inputs on the problem's device are
+ * read where they are; others, unaligned ones and ones that Av overlaps other
+ * than cell for cell are copied first.  Overwrites the minimiser's work buffers
+ * (a later mm_minimize / mm_hysteresis_sweep starts from its own m).
  */
 MM_API int mm_hessian_vec(mm_problem *prob, const void *m, const double Hext[3], const void *v, void *Av,
                           void *stream);

@@ -345,16 +345,17 @@ int hvp_t(mm_problem *p, const void *m, const double Hext[3], const void *v, voi
     T *H = (T *)p->stage_in, *Lv = (T *)p->stage_out;
     const bool odev = mm_is_device_ptr(Av);
     // device inputs are read where they are, unless the output overlaps them
-    // other than cell for cell; the rest goes through the work buffers (128 x 64 x 2
+    // other than cell for cell, they are not aligned to their type, or another
+    // device holds them; the rest goes through the work buffers (128 x 64 x 2
     // FP64: 131 -> 116 us without the two copies), which are allocated when first
     // needed (a problem's first call: 256 -> 150 us)
     auto input = [&](const void *src, int work, const T *&at) {
-        const bool dev = mm_is_device_ptr(src);
         const uintptr_t a = (uintptr_t)src, b = (uintptr_t)Av;
-        if (dev && (!odev || a == b || a + F <= b || b + F <= a)) { at = (const T *)src; return (int)MM_OK; }
+        const bool apart = !odev || a == b || a + F <= b || b + F <= a;
+        if (apart && a % sizeof(T) == 0 && mm_is_local_ptr(p, src)) { at = (const T *)src; return (int)MM_OK; }
         if (const int e = ensure_adjoint_buffers(p)) return e;
         at = (const T *)p->adj[work];
-        return mm_copy_user(p->adj[work], src, F, true, dev, s);
+        return mm_copy_user(p->adj[work], src, F, true, mm_is_device_ptr(src), s);
     };
     const T *mm_, *vv;
     if ((rc = input(m, 0, mm_)) || (rc = input(v, 1, vv))) return rc;

@@ -432,6 +432,8 @@ int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s);
 
 // helpers (api.cu)
 bool mm_is_device_ptr(const void *ptr);
+// and does the problem's own device hold it (or is it managed)?
+bool mm_is_local_ptr(const mm_problem *p, const void *ptr);
 // fields of this problem are double (MM_FP64, MM_F32X2) rather than float
 inline bool mm_double_fields(const mm_problem *p) { return p->precision != MM_FP32; }
 // options of a minimisation within range (finite tolerances, known rules)
