@@ -131,14 +131,27 @@ template <typename T, typename F> cudaError_t configure_t(const Geom &g, size_t 
 }
 
 // Launch-shape autotuner: time every admissible rows-per-tile of the
-// x-forward kernel and, separately, of the x-inverse kernel (the two are
-// independent: the spectrum layout does not depend on the tile), and every
-// rows-per-batch RB of the y-z kernel, on this problem's own buffers
-// (MM_TUNE_REPS repetitions, best taken: candidates within a few percent of
-// each other otherwise swap places from run to run); keep the fastest of each.
-// The kernels run in their minimiser modes on the zeroed state of a fresh
-// problem.
+// x-forward kernel, every rows-per-batch RB of the y-z kernel, and every
+// rows-per-tile of the x-inverse kernel (the three are independent: the spectrum
+// layout does not depend on them), on this problem's own buffers (MM_TUNE_REPS
+// repetitions, best taken: candidates within a few percent of each other
+// otherwise swap places from run to run); keep the fastest of each.  The
+// kernels run in their minimiser modes on a state past its first iteration, so
+// that the step and the step-size sums are part of what is timed, and on a
+// tilted unit field: the block fixed point's work depends on the values (of an
+// all-zero row nothing is converted, and equal scales are not shifted).
 #define MM_TUNE_REPS 5
+template <typename T> __global__ void k_tune_field(T *m, long N)
+{
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < N; i += (long)gridDim.x * blockDim.x) {
+        const unsigned h = (unsigned)i * 2654435761u;   // a scrambled cell number: tilts up to 0.1
+        const float y = (float)(h >> 16) * (0.2f / 65536.0f) - 0.1f, z = (float)(h & 0xffffu) * (0.2f / 65536.0f) - 0.1f;
+        const float s = rsqrtf(1.0f + y * y + z * z);
+        m[i] = T(s);
+        m[N + i] = T(y * s);
+        m[2 * N + i] = T(z * s);
+    }
+}
 template <typename T, typename F> cudaError_t autotune_t(mm_problem *p, const int *tys, int nty, const int *rbs, int nrb,
                                              cudaStream_t s)
 {
@@ -149,9 +162,6 @@ template <typename T, typename F> cudaError_t autotune_t(mm_problem *p, const in
     P.H_out = (IO *)p->gbuf[0];
     cudaEvent_t a, b;
     cudaError_t e;
-    // a minimiser state past its first iteration, so that the step and the
-    // step-size sums are part of what is timed (the zeroed buffers make it
-    // arithmetic on zeros and NaNs, which costs the same)
     MinState ms;
     memset(&ms, 0, sizeof ms);
     ms.k = 1;
@@ -160,51 +170,49 @@ template <typename T, typename F> cudaError_t autotune_t(mm_problem *p, const in
     ms.tauw = dfloat(1e-9);
     ms.max_iter = 1L << 40;
     ms.status = MMS_RUNNING;
+    // iterate 0 in mbuf[0], which the x-forward kernel steps from (with the zeroed gradient)
+    k_tune_field<T><<<mm_grid_for(g.N, 256, 8), 256, 0, s>>>((T *)p->mbuf[0], g.N);
+    if ((e = cudaGetLastError())) return e;
     if ((e = cudaMemcpyAsync(p->st, &ms, sizeof ms, cudaMemcpyHostToDevice, s)) || (e = cudaStreamSynchronize(s)))
         return e;
     if ((e = cudaEventCreate(&a))) return e;
     if ((e = cudaEventCreate(&b))) { cudaEventDestroy(a); return e; }
-    for (int which = 0; which < 2 && !e; ++which) {
+    // best of n candidates: set(i) takes one, before() runs untimed, run() is timed
+    auto best_of = [&](int n, auto set, auto before, auto run) {
         float best = 1e30f;
-        int bty = tys[0];
-        for (int i = 0; i < nty && !e; ++i) {
-            if (which == 0) { g.TYF = tys[i]; g.ltyf = mm_ilog2(g.TYF); }
-            else { g.TY = tys[i]; g.lty = mm_ilog2(g.TY); }
+        int at = 0;
+        for (int i = 0; i < n && !e; ++i) {
+            set(i);
             float tmin = 1e30f;
             for (int r = 0; r < MM_TUNE_REPS && !e; ++r) {
+                if ((e = before())) break;
                 cudaEventRecord(a, s);
-                if (which == 0) launch_xfwd<T, F, true>(g, P, s);
-                else launch_xinv<T, F, MODE_MIN>(g, P, s, nullptr, 0, 0);
+                e = run();
                 cudaEventRecord(b, s);
-                if ((e = cudaGetLastError()) || (e = cudaEventSynchronize(b))) break;
+                if (e || (e = cudaEventSynchronize(b))) break;
                 float t = 0;
                 cudaEventElapsedTime(&t, a, b);
                 if (t < tmin) tmin = t;
             }
-            if (tmin < best) { best = tmin; bty = tys[i]; }
+            if (tmin < best) { best = tmin; at = i; }
         }
-        if (which == 0) { g.TYF = bty; g.ltyf = mm_ilog2(bty); }
-        else { g.TY = bty; g.lty = mm_ilog2(bty); }
-    }
-    float best = 1e30f;
-    int brb = rbs[0];
-    for (int i = 0; i < nrb && !e && !g.bulk; ++i) {
-        g.RB = rbs[i];
-        float tmin = 1e30f;
-        for (int r = 0; r < MM_TUNE_REPS && !e; ++r) {
-            cudaEventRecord(a, s);
-            e = launch_yz_any<T, F>(g, P, s);
-            cudaEventRecord(b, s);
-            if (e || (e = cudaEventSynchronize(b))) break;
-            float t = 0;
-            cudaEventElapsedTime(&t, a, b);
-            if (t < tmin) tmin = t;
-        }
-        if (tmin < best) { best = tmin; brb = rbs[i]; }
-    }
-    g.RB = brb;
+        set(at);
+    };
+    auto nothing = [] { return cudaSuccess; };
+    auto xfwd = [&] { return launch_xfwd<T, F, true>(g, P, s); };
+    best_of(nty, [&](int i) { g.TYF = tys[i]; g.ltyf = mm_ilog2(g.TYF); }, nothing, xfwd);
+    if (!g.bulk) best_of(nrb, [&](int i) { g.RB = rbs[i]; }, xfwd, [&] { return launch_yz_any<T, F>(g, P, s); });
+    if (!e) e = xfwd();
+    if (!e) e = launch_conv<T, F>(g, P, s);
+    best_of(nty, [&](int i) { g.TY = tys[i]; g.lty = mm_ilog2(g.TY); }, nothing,
+            [&] { return launch_xinv<T, F, MODE_MIN>(g, P, s, nullptr, 0, 0); });
     cudaEventDestroy(a);
     cudaEventDestroy(b);
+    const size_t bytes = 3 * (size_t)g.N * p->esz;
+    for (int i = 0; i < 2; ++i) {
+        if (!e) e = cudaMemsetAsync(p->mbuf[i], 0, bytes, s);
+        if (!e) e = cudaMemsetAsync(p->gbuf[i], 0, bytes, s);
+    }
     if (!e) e = cudaMemsetAsync(p->st, 0, sizeof(MinState), s);
     if (!e) e = cudaMemsetAsync(p->counter, 0, 64, s);
     if (!e) p->g = g;

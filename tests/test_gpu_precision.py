@@ -186,3 +186,16 @@ def test_flat_cells(mmlib, grid, cell, prec, bar):
             for c in range(3):
                 terms = sum(top[c][b] * np.linalg.norm(m[b]) for b in range(3) if coupled(p.shape, b, c))
                 assert np.linalg.norm(H[c] - ref[c]) <= bar * terms, (big, tilt, c)
+
+
+@pytest.mark.parametrize("prec", ["MM_FP64", "MM_FP32", "MM_F32X2"])
+def test_nothing_of_the_timed_state_stays_behind(mmlib, prec):
+    """Launch shapes are timed at setup on a field of the tuner's own: a new problem holds zeros."""
+    dt = torch.float32 if prec == "MM_FP32" else torch.float64
+    prob, p = make_pair(mmlib, 130, 128, 4, (4e-9, 3e-9, 5e-9), precision=getattr(mmlib, prec))
+    bufs = [torch.ones((3,) + p.shape, dtype=dt, device="cuda") for _ in range(4)]
+    st = mmlib.mm_min_inspect(prob, *bufs)
+    assert all(not b.any() for b in bufs)
+    info = mmlib.mm_problem_info(prob)
+    assert info["x_tile_rows"] in (1, 2, 4, 8, 16) and info["x_fwd_tile_rows"] in (1, 2, 4, 8, 16)
+    assert 12 % info["yz_batch_rows"] == 0 and st is not None
