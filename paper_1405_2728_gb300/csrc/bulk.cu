@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zl = INV ? rest / Py : g.fd_ny.div(rest), y = rest - zl * lin;
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[(INV ? y >> log2_of(g.KB) : rest) * ns + own(c)]) - s_e[own(c)]);
+                v[i] = fx_down(v[i], s_e[own(c)] - fx_exp(scales[(INV ? y >> log2_of(g.KB) : rest) * ns + own(c)]));
                 mags.or_in(own(c), fx_mag(v[i]));
             }
             S[(c * ZB + zl) * rs + rpos<V, LY>(y)] = v[i];
@@ -117,8 +117,11 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
     __syncthreads();
     const int Gy = g.Gy, RB = g.RBY;
     const int rb = tid / Gy, j = tid - rb * Gy;
-    auto pre = [&](int c) { return (INV ? 58 : 59) - fx_bits(s_in[c]); };
-    int sh = 0;
+    int sh = 0, pre[3] = {0, 0, 0}, post[3] = {0, 0, 0};
+    if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) pre[c] = (INV ? 58 : 59) - fx_bits(s_in[own(c)]);
+    }
     mags = FxMags<3>();
     for (int r0 = 0; r0 < 3 * ZB; r0 += RB) {
         const int r = r0 + rb;
@@ -126,25 +129,27 @@ __global__ void __launch_bounds__(Y_BOUND<T>) k_ypass(Geom g, FieldPtrs<T> P)
         if constexpr (FX) {
             const int c = act ? own(r >> log2_of(ZB)) : 0;
             unsigned mag = 0;
-            sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, pre(c), 64, mag);
+            sh = fft_row_fx<INV, !INV, INV, 1, LY, true>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act, fx_of(pre, c), 64,
+                                                         mag);
             mags.or_in(c, mag);
         } else
             fft_row<INV, !INV, INV, 1, LY>(S + (act ? r : 0) * rs, Py, g.lpy, j, tw, act);
     }
-    auto post = [&](int c) { return 60 - fx_bits(s_out[c]); };
     if constexpr (FX) cta_mags(s_out);
     __syncthreads();
     if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) post[c] = 60 - fx_bits(s_out[own(c)]);
         if (tid < ns)
             (INV ? P.fe2 : P.fea)[((long)kx * g.nzb + blockIdx.y) * ns + tid] =
-                fx_pack(s_e[tid] - pre(tid) + sh - post(tid), *s_fl >> tid & 1);
+                fx_pack(s_e[tid] - fx_of(pre, tid) + sh - fx_of(post, tid), *s_fl >> tid & 1);
     }
     const int lout = INV ? ny : Py;
     V *dst = INV ? P.W + first * ny * 3 : P.W2 + first * Py * 3;
     for (int e = tid; e < zb * lout * 3; e += nth) {
         const int c = e % 3, rest = e / 3, zl = INV ? g.fd_ny.div(rest) : rest / Py, y = rest - zl * lout;
         V r = S[(c * ZB + zl) * rs + rpos<V, LY>(y)];
-        if constexpr (FX) r = fx_scale(r, post(own(c)));
+        if constexpr (FX) r = fx_scale(r, fx_of(post, c));
         dst[e] = r;
     }
 }
@@ -210,7 +215,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
             int kyl, z;
             split(e / 3, kyl, z);
             if constexpr (FX) {
-                v[i] = fx_scale(v[i], fx_exp(scales[(z >> log2_of(g.ZB)) * NS + (SEP ? c : 0)]) - s_e[SEP ? c : 0]);
+                v[i] = fx_down(v[i], s_e[SEP ? c : 0] - fx_exp(scales[(z >> log2_of(g.ZB)) * NS + (SEP ? c : 0)]));
                 mags.or_in(c, fx_mag(v[i]));
             }
             S[(c * KB + kyl) * rs + rpos<V, LZ>(z)] = v[i];
@@ -228,14 +233,18 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     const int rb = tid / Gz, j = tid - rb * Gz;
     signed char *s_sc = reinterpret_cast<signed char *>(tw + tw_slots(Pz));  // [2][NS][KB][Pz]: scale and top bit of a frequency
     signed char *s_tk = s_sc + NS * KB * Pz;
-    int sh = 0;
+    int sh = 0, pre[NS], t[NS], post[NS];
+    if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < NS; ++c) pre[c] = 59 - fx_bits(s_in[c]);
+    }
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
         if constexpr (FX) {
             unsigned none = 0;
             sh = fft_row_fx<false, true, false, 1, LZ, false>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act,
-                                                              59 - fx_bits(s_in[SEP && act ? r >> lkb : 0]), 64, none);
+                                                              fx_of(pre, act ? r >> lkb : 0), 64, none);
         } else {
             fft_row<false, true, false, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
         }
@@ -246,7 +255,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
     if constexpr (FX) {
 #pragma unroll
         for (int c = 0; c < NS; ++c) {
-            eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh + (SEP ? g.tsc[c] : 0);
+            eb[c] = d[c] = s_e[c] - pre[c] + sh + (SEP ? g.tsc[c] : 0);
             top[c] = FX_ZERO;
         }
         couple.join(eb);
@@ -346,29 +355,34 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         for (int c = 0; c < NS; ++c) fx_cta_add(&s_sum[c], sum[c]);
         __syncthreads();
         mags = FxMags<NS>();
+#pragma unroll
+        for (int c = 0; c < NS; ++c) {
+            pre[c] = 58 - s_top[c];
+            t[c] = max(0, fx_log2_up(s_sum[c]) - 18);
+        }
     }
-    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
     for (int r0 = 0; r0 < 3 * KB; r0 += RB) {
         const int r = r0 + rb;
         const bool act = rb < RB && r < 3 * KB && (r % KB) < kb;
         if constexpr (FX) {
             const int c = SEP && act ? r >> lkb : 0;
             unsigned mag = 0;
-            fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, 58 - s_top[c],
-                                                             bound(c), mag,
+            fft_row_fx<true, false, true, 1, LZ, true, true>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act, fx_of(pre, c),
+                                                             fx_of(t, c), mag,
                                                              s_sc + (c * KB + (act ? r & (KB - 1) : 0)) * Pz);
             mags.or_in(c, mag);
         } else {
             fft_row<true, false, true, 1, LZ>(S + (act ? r : 0) * rs, Pz, g.lpz, j, tw, act);
         }
     }
-    auto post = [&](int c) { return 60 - fx_bits(s_out[c]); };
     if constexpr (FX) mags.cta_or(s_out);
     __syncthreads();
     if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < NS; ++c) post[c] = 60 - fx_bits(s_out[c]);
         if (tid < NS) {
-            const int c = tid, e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] +
-                                   fx_cum(fx_log(Pz), bound(c)) - (58 - s_top[c]) - post(c) + (SEP ? g.tsc[c] : 0);
+            const int c = tid, e = fx_of(eb, c) + P.fek[kx] + fx_cum(fx_log(Pz), fx_of(t, c)) - fx_of(pre, c) -
+                                   fx_of(post, c) + (SEP ? g.tsc[c] : 0);
             P.feb[((long)kx * g.nkb + blockIdx.y) * NS + c] = fx_pack(e, *s_fl ? 1 : 0);  // the tensor mixes all components
         }
     }
@@ -377,7 +391,7 @@ __global__ void __launch_bounds__(BulkBound<T>::v, Z_CTAS) k_zconv(Geom g, Field
         int kyl, z;
         split(e / 3, kyl, z);
         V r = S[(c * KB + kyl) * rs + rpos<V, LZ>(z)];
-        if constexpr (FX) r = fx_scale(r, post(SEP ? c : 0));
+        if constexpr (FX) r = fx_scale(r, fx_of(post, c));
         base[(long)z * zs + kyl * 3 + c] = r;
     }
 }

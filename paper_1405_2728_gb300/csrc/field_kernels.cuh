@@ -428,7 +428,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     __syncthreads();
 
     // Wk[z][y][c] -> row (c, z); the first loads are issued before the rows' scales are looked at
-    constexpr int PF = 4;
+    constexpr int PF = LY == 0 ? 2 : 4;   // (short rows: fewer instructions to fetch)
     const int tot = nrow * ny;
     fxc v[PF];
     auto load = [&](int e0) {
@@ -446,8 +446,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
             const int e = e0 + i * nth;
             if (e >= tot) break;
             const int c = e % 3, rest = e / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-            const int d = fx_exp(P.fe1[SEP ? e : rest]) - s_e[SEP ? c : 0];
-            if (d) v[i] = fx_scale(v[i], d);
+            v[i] = fx_down(v[i], s_e[SEP ? c : 0] - fx_exp(P.fe1[SEP ? e : rest]));
             mags.or_in(c, fx_mag(v[i]));
             S[(c * nz + zz) * g.rsy + spos<fxc>(y)] = v[i];
         }
@@ -465,12 +464,14 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     const int rb = tid / g.Gy, j = tid - rb * g.Gy;  // row within a batch of g.RB rows
     const bool act = rb < g.RB;
     auto comp = [&](int r) { return SEP ? (r >= nz) + (r >= 2 * nz) : 0; };  // of a row
-    int sh = 0;
+    int sh = 0, pre[NS];
+#pragma unroll
+    for (int c = 0; c < NS; ++c) pre[c] = 59 - fx_bits(s_in[c]);
     unsigned none = 0;
     for (int r0 = 0; r0 < nrow; r0 += g.RB) {
         const int r = act ? r0 + rb : 0;
-        sh = fft_row_fx<false, true, false, 1, LY, false>(S + r * g.rsy, Py, g.lpy, j, tw, act,
-                                                          59 - fx_bits(s_in[comp(r)]), 64, none);
+        sh = fft_row_fx<false, true, false, 1, LY, false>(S + r * g.rsy, Py, g.lpy, j, tw, act, fx_of(pre, comp(r)), 64,
+                                                          none);
     }
     // z convolution: inputs of a ky below 2^59, so sums and differences below
     // 2^60; outputs below 2^60 (the tensor's terms of an output sum to less
@@ -482,7 +483,7 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
     int eb[NS], d[NS], top[NS];   // a component's scale where it is mixed, its own over that, the largest output
 #pragma unroll
     for (int c = 0; c < NS; ++c) {
-        eb[c] = d[c] = s_e[c] - (59 - fx_bits(s_in[c])) + sh + (SEP ? g.tsc[c] : 0);
+        eb[c] = d[c] = s_e[c] - pre[c] + sh + (SEP ? g.tsc[c] : 0);
         top[c] = FX_ZERO;
     }
     couple.join(eb);
@@ -570,26 +571,33 @@ __device__ __forceinline__ void yz_body_fx(const Geom &g, const FieldPtrs<double
 #pragma unroll
     for (int c = 0; c < NS; ++c) fx_cta_add(&s_sum[c], sum[c]);
     __syncthreads();
-    auto bound = [&](int c) { return max(0, fx_log2_up(s_sum[c]) - 18); };
+    int t[NS], post[NS];
+#pragma unroll
+    for (int c = 0; c < NS; ++c) {
+        pre[c] = 58 - s_top[c];
+        t[c] = max(0, fx_log2_up(s_sum[c]) - 18);
+    }
     mags = FxMags<NS>();
     for (int r0 = 0; r0 < nrow; r0 += g.RB) {
         const int r = act ? r0 + rb : 0, c = comp(r);
         unsigned mag = 0;
-        fft_row_fx<true, false, true, 1, LY, true, true>(S + r * g.rsy, Py, g.lpy, j, tw, act, 58 - s_top[c], bound(c),
+        fft_row_fx<true, false, true, 1, LY, true, true>(S + r * g.rsy, Py, g.lpy, j, tw, act, fx_of(pre, c), fx_of(t, c),
                                                          mag, s_sc + c * Py);
         mags.or_in(c, mag);
     }
     mags.cta_or(s_out);
     __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NS; ++c) post[c] = 60 - fx_bits(s_out[c]);
     for (int i = tt; i < tot; i += nth) {
         const int c = i % 3, rest = i / 3, zz = g.fd_ny.div(rest), y = rest - zz * ny;
-        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], 60 - fx_bits(s_out[SEP ? c : 0]));
+        Wk[i] = fx_scale(S[(c * nz + zz) * g.rsy + spos<fxc>(y)], fx_of(post, c));
     }
     if (tid < NS) {
         // with one layer the field along z depends on m_z alone, the others on m_x and m_y alone
         const int c = tid, fl = (int)*s_fl, hit = nz > 1 ? 7 : (c == 2 ? 4 : 3);
-        const int e = (c == 0 ? eb[0] : (c == 1 ? eb[SEP ? 1 : 0] : eb[SEP ? 2 : 0])) + P.fek[kx] - (NZM > 1 ? 1 : 0) +
-                      fx_cum(fx_log(Py), bound(c)) - (58 - s_top[c]) - (60 - fx_bits(s_out[c])) + (SEP ? g.tsc[c] : 0);
+        const int e = fx_of(eb, c) + P.fek[kx] - (NZM > 1 ? 1 : 0) + fx_cum(fx_log(Py), fx_of(t, c)) - fx_of(pre, c) -
+                      fx_of(post, c) + (SEP ? g.tsc[c] : 0);
         P.fe2[kx * NS + c] = fx_pack(e, (SEP ? fl & hit : fl) ? 1 : 0);
     }
 }
@@ -1056,8 +1064,8 @@ __device__ __forceinline__ void xinv_body(const Geom &g, const FieldPtrs<T, F> &
             V Z;
             V Xk = xa[i], Xm = cconj(xb[i]);
             if constexpr (is_fx<F>) {  // components below 2^60: |Z| < 2^62
-                Xk = fx_scale(Xk, fx_exp(fe2[kk * fst + own(c)]) - s_e[own(c)]);
-                Xm = fx_scale(Xm, fx_exp(fe2[(Hx - kk) * fst + own(c)]) - s_e[own(c)]);
+                Xk = fx_down(Xk, s_e[own(c)] - fx_exp(fe2[kk * fst + own(c)]));
+                Xm = fx_down(Xm, s_e[own(c)] - fx_exp(fe2[(Hx - kk) * fst + own(c)]));
             }
             const V sum = cadd(Xk, Xm), dif = csub(Xk, Xm);
             V t;

@@ -181,6 +181,14 @@ __device__ __forceinline__ fxc fx_scale(fxc a, int d)
     r.y = fx_scale(a.y, d);
     return r;
 }
+// v / 2^s rounded, s >= 0 (fx_scale's right shift alone: half the code where small
+// films wait for instructions)
+__device__ __forceinline__ fxc fx_down(fxc a, int s)
+{
+    if (s == 0) return a;
+    if (s > 61) return fxc{fx(0), fx(0)};
+    return fxc{fx_shr(a.x, s), fx_shr(a.y, s)};
+}
 // bits of the high word's magnitude, to be OR-ed over a block; with b the
 // number of bits of the result, every |v| of the block is below 2^(32 + b) + 1
 __device__ __forceinline__ unsigned fx_mag(fx a)
@@ -234,6 +242,12 @@ template <int N> struct FxMags {
         for (int c = 0; c < N; ++c) fx_cta_or(dst + c, v[c]);
     }
 };
+// element c of a register array (N = 1: the one for all components)
+template <int N> __device__ __forceinline__ int fx_of(const int (&a)[N], int c)
+{
+    if constexpr (N == 1) return a[0];
+    else return c == 0 ? a[0] : (c == 1 ? a[1] : a[2]);
+}
 // Largest exponents and the flags (bit c) of the scales p[i * stride + c], i < n,
 // c < N, over the CTA; a barrier makes them visible
 template <int N> __device__ __forceinline__ void fx_cta_scales(const int *p, int n, long stride, int tt, int nth, int *s_e,
