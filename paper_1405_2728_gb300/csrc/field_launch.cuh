@@ -202,9 +202,16 @@ template <typename T, typename F> cudaError_t autotune_t(mm_problem *p, const in
     auto xfwd = [&] { return launch_xfwd<T, F, true>(g, P, s); };
     best_of(nty, [&](int i) { g.TYF = tys[i]; g.ltyf = mm_ilog2(g.TYF); }, nothing, xfwd);
     if (!g.bulk) best_of(nrb, [&](int i) { g.RB = rbs[i]; }, xfwd, [&] { return launch_yz_any<T, F>(g, P, s); });
-    if (!e) e = xfwd();
-    if (!e) e = launch_conv<T, F>(g, P, s);
-    best_of(nty, [&](int i) { g.TY = tys[i]; g.lty = mm_ilog2(g.TY); }, nothing,
+    // the x-inverse kernel after the others, as in an iteration: alone it finds its inputs in L2.  (512 x 256 x 4 double-word:
+    // timed alone 4 rows won, 87 to 90 us in the iteration, where 1 or 2 take 85.)  Large grids, whose inputs do not fit there, run
+    // the others once: an iteration of theirs takes milliseconds.
+    auto others = [&] {
+        const cudaError_t r = xfwd();
+        return r ? r : launch_conv<T, F>(g, P, s);
+    };
+    const bool chain = g.N <= 1L << 20;
+    if (!e) e = others();
+    best_of(nty, [&](int i) { g.TY = tys[i]; g.lty = mm_ilog2(g.TY); }, [&] { return chain ? others() : cudaSuccess; },
             [&] { return launch_xinv<T, F, MODE_MIN>(g, P, s, nullptr, 0, 0); });
     cudaEventDestroy(a);
     cudaEventDestroy(b);
