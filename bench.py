@@ -41,8 +41,12 @@ LOOP_NOTE = ("field values x the mean time of the timed steps; the whole loop, t
 # 64-bit integer additions per SM per clock (measured, chains of independent additions): the FP64 and
 # double-word transforms run in 64-bit block fixed point on the integer units
 ADD64_PER_SM_CLK = 42
-DW_ADD_INSTRUCTIONS = 11      # FP32 instructions of one double-word (float pair) addition
-LOCAL_FLOPS = 90              # of the local terms, torque and step-size sums per cell (x-inverse stage)
+LOCAL_FLOPS = {"xfwd_step": 24, "xinv_local_bb": 90}   # of the step, and of the local terms, torque and sums, per cell
+# What the kernels execute for them, per cell, conversions to and from fixed point included: FP64-pipe instructions of
+# FP64, FP32 instructions of double-word (float pairs).  Counted on the device at 256x128x4 after the first iteration
+# (smsp__inst_executed_pipe_fp64; smsp__sass_thread_inst_executed_op_fadd, fmul and ffma).
+LOCAL_INSTRUCTIONS = {"fp64": {"xfwd_step": 23, "xinv_local_bb": 103},
+                      "f32x2": {"xfwd_step": 312, "xinv_local_bb": 1254}}
 PRECISIONS = {"fp64": 0, "fp32": 1, "f32x2": 2}   # mm.MM_FP64, mm.MM_FP32, mm.MM_F32X2
 DTYPE_LABEL = {"fp64": "f64 fields and local terms, 64-bit block fixed-point FFT and convolution", "fp32": "f32", "f32x2": "f32x2 (double-word) fields and local terms, 64-bit block fixed-point FFT and convolution"}
 
@@ -162,8 +166,8 @@ def algorithmic_model(info, esz):
 
     x_rows = 3 * ny * nz
     unpack = 10 * C
-    f_xfwd = x_rows * (fft_flops(Hx, True, False) + unpack) + N * 3 * 8
-    f_xinv = x_rows * (fft_flops(Hx, False, True) + unpack) + N * LOCAL_FLOPS
+    f_xfwd = x_rows * (fft_flops(Hx, True, False) + unpack) + N * LOCAL_FLOPS["xfwd_step"]
+    f_xinv = x_rows * (fft_flops(Hx, False, True) + unpack) + N * LOCAL_FLOPS["xinv_local_bb"]
     model = {
         "xfwd_step": {"bytes": 3 * F + W, "flops": f_xfwd},
         "xinv_local_bb": {"bytes": W + 4 * F, "flops": f_xinv},
@@ -214,6 +218,17 @@ def survey_flops(info):
 
 
 KERNEL_SOURCES = ("fixed.cuh", "fft.cuh", "dfloat.cuh", "field_kernels.cuh")  # the device code of the film field kernels
+
+
+def fixed_point_work(model, info, stage, precision, fma, int_rate):
+    """Work and rate (T/s) of a stage's two instruction streams in FP64 or
+    double-word: the transforms and the product on the integer units (every
+    operation priced as a 64-bit addition), the local terms on the FP64 or FP32
+    units as counted."""
+    cells = info["nx"] * info["ny"] * info["nz"]
+    return {"alu_int64": (model[stage]["flops"] - LOCAL_FLOPS.get(stage, 0) * cells, int_rate),
+            "alu_local": (LOCAL_INSTRUCTIONS[precision].get(stage, 0) * cells,
+                          fma["fp64" if precision == "fp64" else "fp32"] / 2)}
 
 
 def kernel_source_hash():
@@ -844,15 +859,8 @@ def main():
         gbs = model[dom]["bytes"] / sec / 1e9
         hbm = peaks.get("hbm_gbs")
         if pname != "fp32":
-            # The transforms and the tensor product run on the integer units, the
-            # local terms on the FP64 (or, as float pairs, the FP32) units, the
-            # bytes through HBM: the bound is the resource that takes longest.
-            cells = inf["nx"] * inf["ny"] * inf["nz"]
-            local = {"xfwd_step": 24, "xinv_local_bb": LOCAL_FLOPS}.get(dom, 0) * cells
-            local_rate = fma["fp64"] / 2 if pname == "fp64" else fma["fp32"] / 2 / DW_ADD_INSTRUCTIONS
-            int_rate = n_sm * ADD64_PER_SM_CLK * sm_mhz * 1e6 / 1e12
-            work = {"alu_int64": (model[dom]["flops"] - local, int_rate),
-                    "alu_local": (local, local_rate)}
+            # The bound is the resource that takes longest: the integer units, those of the local terms, or HBM
+            work = fixed_point_work(model, inf, dom, pname, fma, n_sm * ADD64_PER_SM_CLK * sm_mhz * 1e6 / 1e12)
             floors = {k: v[0] / (v[1] * 1e12) for k, v in work.items()}
             floors["hbm"] = model[dom]["bytes"] / ((hbm or 6800.0) * 1e9)
             bound = max(floors, key=floors.get)
@@ -865,10 +873,8 @@ def main():
                 "frac": roof["achieved"] / roof["peak"], "floor_ms": {k: 1e3 * v for k, v in floors.items()},
                 "peak_source": f"int64: {n_sm} SMs x {ADD64_PER_SM_CLK} 64-bit additions/clk at {sm_mhz:.0f} MHz, every "
                                "operation of the transforms priced as an addition (a product takes several); local: "
-                               + (f"measured FP64 FMA rate (mm_probe_fma), {fma['fp64'] / 2:.3f} T instructions/s"
-                                  if pname == "fp64" else
-                                  f"measured FP32 FMA rate, {fma['fp32'] / 2:.1f} T instructions/s / "
-                                  f"{DW_ADD_INSTRUCTIONS} per double-word addition"),
+                               f"instructions as counted on the device, at the measured {'FP64' if pname == 'fp64' else 'FP32'} "
+                               f"FMA rate (mm_probe_fma), {work['alu_local'][1]:.3f} T instructions/s",
                 # the workload's reference model (2.5/5 L log2 L per real/complex transform, 36 per frequency,
                 # 200 per cell) as a multiple of what the FP64 units can do at all
                 "reference_model_vs_fp64_fma_peak": sflops[dom] / sec / 1e12 / fma["fp64"]})
