@@ -163,7 +163,7 @@ def _ptr(a, dtype=None, shape=None, what="array"):
             raise ValueError(f"{what} must be contiguous")
         if dtype is not None and _dtype_name(a.dtype) != _dtype_name(dtype):
             raise TypeError(f"{what} has dtype {a.dtype}, expected {np.dtype(dtype).name}")
-        if shape is not None and a.shape != shape:
+        if shape is not None and a.shape != shape and tuple(a.shape) != tuple(shape):
             raise ValueError(f"{what} has shape {tuple(a.shape)}, expected {tuple(shape)}")
         return c_void_p(a.data_ptr())
     if isinstance(a, np.ndarray):
