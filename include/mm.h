@@ -71,8 +71,12 @@ typedef enum {
 
 /* Element type and arithmetic of the field path.  MM_FP64: double fields,
  * local terms, step and sums; the FFTs and the demagnetisation convolution run
- * in 64-bit block fixed point on the integer pipes, with a smaller error than
- * the same transforms in double.  MM_F32X2 (an extension): the caller's arrays
+ * in 64-bit block fixed point on the integer pipes.  Its error relative to the
+ * field is smaller than that of the same transforms in double, and so is each
+ * component's: components that the tensor does not mix (axes of one cell) or
+ * mixes unequally (cells flatter than 1:16) have scales of their own, so a small
+ * one beside a large one is as accurate as alone.  Like a double transform's, the
+ * error is spread over the cells of a component.  MM_F32X2 (an extension): the caller's arrays
  * are double as for MM_FP64; inside, the iterates, the local terms, the step
  * and the per-CTA sums use double-float arithmetic (pairs of floats, about 48
  * significant bits, run on the FP32 pipes), the FFTs and the convolution the
@@ -143,12 +147,11 @@ MM_API int mm_newell_static(const mm_grid *grid, double *N_dev, void *stream);
  * allocates device workspaces, computes the Newell tensor (as mm_newell), its
  * Fourier spectrum on the zero-padded grid (padded size per axis: the power of
  * two P >= 2n-1 (and >= 2 along x) or a shorter length
- * >= 2n-1: 5/8 or 3/4 of P = 512 or 1024 along x and along y of films, 5/8, 3/4
- * or 25/32 of P = 128 .. 1024 along y and z of bulk grids), times the admissible launch
+ * >= 2n-1: 5/8 or 3/4 of P = 512 or 1024 along x and along y of films, 5/8 or 3/4
+ * of P = 128 .. 1024 and 25/32 of P = 256 .. 1024 along y and z of bulk grids), times the admissible launch
  * shapes of the field kernels on this problem and keeps the fastest, and
- * captures the minimiser's CUDA graph.  precision = MM_FP64 or MM_FP32: element type of m/H and of the FFT
- * and stencil arithmetic; MM_F32X2: double arrays, double-float arithmetic
- * (see the enum).  The reductions (step-size sums, energies,
+ * captures the minimiser's CUDA graph.  precision: element type of m/H, arithmetic of the local terms and of the
+ * transforms (see the enum).  The reductions (step-size sums, energies,
  * averages) are combined across CTAs in double and the step size is chosen in
  * double.  Within a CTA the MM_FP64 path accumulates in double; the MM_FP32
  * path adds every per-cell product exactly (an FMA-split product) into a
@@ -156,8 +159,8 @@ MM_API int mm_newell_static(const mm_grid *grid, double *N_dev, void *stream);
  * lets callers check against their own double reduction; the MM_F32X2 path
  * accumulates in double-float pairs.
  * Two layouts of the y-z stage of the convolution.  Film layout (nz <= 4 and
- * the padded y-z plane of one x-frequency, about 3 * nz * 9/8 * Py complex
- * values, within 200 KiB of shared memory; e.g. 512 x 256 x 4 in FP64 or
+ * the padded y-z plane of one x-frequency with its twiddles, about (3 * nz + 1) * Py
+ * complex values of 16 (FP32: 8) bytes, within 200 KiB of shared memory; e.g. 512 x 256 x 4 in FP64 or
  * 1024 x 512 x 4 in FP32): one kernel per x-frequency.  Bulk layout (every
  * other grid, e.g. 256^3 cubes): separate y, z and inverse-y passes through
  * an extra spectrum buffer of C * nz * Py * 3 complex values.

@@ -155,10 +155,11 @@ void free_problem(mm_problem *p)
 // the first of 5/8, 3/4 and 25/32 of P that reaches 2n - 1 (bulk y and z: P from
 // 128 to 1024, 25/32 too; x and the film y-z kernel: 320, 384, 640 and 768).
 // Work and traffic of an axis go with its padded length: a 160^3 cube's z pass
-// takes 2045 us at 512 x 512 x 512 and 550 us at 320 x 320 x 320 (FP32).  Films
-// of up to 128 cells an axis stay on powers of two, their kernels being bound by
-// latency, and 25/32 loses there: its 25 x 8 points take five passes' barriers
-// (200 x 100 x 2, FP64 y-z stage: 20.6 us at 256, 31.8 us at 200).
+// took 2045 us at 512 x 512 x 512 and takes 440 us at 320 x 320 x 320 (FP32).
+// Film axes of up to 128 cells, and 25/32 of films, stay on powers of two: with
+// the code for any length, the only one tried there, the y-z stage lost (200 x
+// 100 x 2 in FP64: 20.6 us at 256 points, 31.8 us at 200; 50 x 35 in FP32: 8.1
+// and 12.3 us).  Compiled instances of those lengths have not been measured.
 int padded_length(int n, bool bulk_axis)
 {
     const int P = next_pow2(2 * n - 1);

@@ -266,8 +266,8 @@ struct FieldPtrs {
     V *W;                  // spectrum [C][nz][ny][3] (x-frequency slowest, component fastest)
     V *W2;                 // bulk layout only: y-transformed spectrum [C][nz][Py][3]
     const typename coef<F>::type *Nhat;  // tensor: film [C][max(1,Pz/2)][6][Py/2+1] (x-y transform at real z offsets, scaled by
-                           // -Ms/(Px Py)); bulk [C][Pz/2+1][Py/2+1][6] (octant of the 3-D spectrum,
-                           // scaled by -Ms/(Px Py Pz))
+                           // -Ms/(Px Py)), in block fixed point [C][mm_film_coefs][Py/2+1] (ZConv's combinations of
+                           // them); bulk [C][Pz/2+1][Py/2+1][6] (octant of the 3-D spectrum, scaled by -Ms/(Px Py Pz))
     const TW *tw_px;       // exp(-2 pi i t/Px), t < Px
     const TW *tw_py;       // exp(-2 pi i t/Py), t < Py
     const TW *tw_pz;       // exp(-2 pi i t/Pz), t < Pz

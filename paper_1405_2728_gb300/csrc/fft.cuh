@@ -44,7 +44,7 @@ __host__ __device__ __forceinline__ int padded_row(int L) { return L + (L >> 3) 
 // Block fixed-point rows (16-byte elements, 8 per wavefront) are swizzled
 // within aligned groups of 8 for the same reason, which leaves room for the
 // twiddles of the y-z kernel beside its rows: 12 rows of 512 and the table take
-// 108 KiB, two CTAs an SM.
+// 105 KiB, two CTAs an SM.
 template <typename V> __host__ __device__ __forceinline__ int spos(int i)
 {
     if constexpr (std::is_same<V, fxc>::value) return i ^ ((i >> 3) & 7);
@@ -81,8 +81,8 @@ __host__ __device__ constexpr int pow2_part(int L)
 // Twiddle t of a table in shared memory lives at tpos(t, L), L the row length.
 // A pass reads multiples of L/(Ns R) r; unswizzled, the eight different ones of
 // a pass with Ns = 8 over a power of two lie 128 bytes apart, in one bank group
-// (512 x 256 x 4: FP32 y-z kernel 37 -> 32.5 us,
-// x-forward 20.7 -> 19.5 us).  Lengths with an odd part
+// (512 x 256 x 4, two measurements: FP32 y-z kernel 37 and 38.5 -> 32.5 us,
+// x-forward 20.7 and 20.4 -> 19.5 us).  Lengths with an odd part
 // spread by themselves.  Double tables (the tensor setup) stay in global
 // memory, in order.
 template <typename W> __host__ __device__ __forceinline__ int tpos(int t, int L)

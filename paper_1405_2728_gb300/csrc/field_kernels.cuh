@@ -314,7 +314,8 @@ template <typename T> struct YZBound { static constexpr int v = sizeof(T) == 8 ?
 // m_z and -i H_z in that of H_z its matrix is real,
 //   [xx xy xz; xy yy yz; xz yz -zz],
 // and the real and the imaginary part are convolved apart, by two threads: half
-// the registers, which lets the kernel run 24 warps an SM instead of 16.
+// the values and sums a thread, within the 128 registers that two CTAs of 256
+// threads (16 warps an SM) leave.
 // Along z the tensor is a Toeplitz matrix, even (xx, yy, zz, xy) or odd (xz,
 // yz) in z - z', so with up_j = m_j + m_{NZM-1-j} and um_j = m_j - m_{NZM-1-j} the
 // sums S_i and differences D_i of the outputs i and NZM-1-i come from half-size

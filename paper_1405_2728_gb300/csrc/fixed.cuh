@@ -1,6 +1,6 @@
 // Block fixed-point arithmetic of the MM_FP64 and MM_F32X2 convolution: 64-bit integers
-// with one power-of-two scale per block of values (a tile of rows, an
-// x-frequency), run on the integer pipes.
+// with power-of-two scales per block of values (a row, an x-frequency), run on
+// the integer pipes.
 //
 // Why: this GPU has 2 FP64 lanes per SM (measured 1.68 FMA per clock and SM),
 // against 42 64-bit integer additions and 24-32 wide multiply-adds per clock

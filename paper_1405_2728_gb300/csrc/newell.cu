@@ -273,7 +273,8 @@ int mm_newell_device(const mm_grid *gr, double *N_dev, cudaStream_t s)
 // Tensor spectra into p->Nhat in the precision of p: bulk layout
 // [Px/2+1][Pz/2+1][Py/2+1][6] (3-D transform, octant); film layout
 // [Px/2+1][max(1, Pz/2)][6][Py/2+1] (x-y transform at real z offsets,
-// k_extract_film).
+// k_extract_film), from which double and double-word problems keep
+// [Px/2+1][mm_film_coefs][Py/2+1] (k_tensor_fixed).
 int mm_tensor_spectrum(mm_problem *p, const double *N_dev, cudaStream_t s)
 {
     const Geom &g = p->g;
