@@ -72,8 +72,8 @@ typedef enum {
 /* Element type and arithmetic of the field path.  MM_FP64: double fields,
  * local terms, step and sums; the FFTs and the demagnetisation convolution run
  * in 64-bit block fixed point on the integer pipes.  Its error relative to the
- * field is smaller than that of the same transforms in double, and so is each
- * component's: components that the tensor does not mix (axes of one cell) or
+ * field is smaller than that of the same transforms in double, and each
+ * component's is no larger: components that the tensor does not mix (axes of one cell) or
  * mixes unequally (cells flatter than 1:16) have scales of their own, so a small
  * one beside a large one is as accurate as alone.  Like a double transform's, the
  * error is spread over the cells of a component.  MM_F32X2 (an extension): the caller's arrays
